@@ -97,14 +97,186 @@ static int launch_zgemm(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZVie
   return 0;
 }
 
+// Products too small to fill the GPU with output tiles: the K loop is spread
+// over the lanes (or the warps) of a CTA instead, so that the 256 x 256
+// product of one plane wave runs on hundreds of warps rather than on two CTAs
+// of a serial K loop (N = 256, one column: 300 us in k_zgemm, 4.7 us here).
+// What bounds them is the FP64 pipe for 4 and more columns, the latency of
+// one pass over A below that.  Sums are formed in a fixed order.
+//
+// k_zgemm_rows: K contiguous in A (A.cs == 1): one warp per row, lanes over K,
+// NC columns per pass, shuffle reduction.
+template <int NC>
+__global__ void __launch_bounds__(128) k_zgemm_rows(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B,
+                                                    zd beta, zd* __restrict__ C, int64_t ldc) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5), j0 = (int64_t)blockIdx.y * NC;
+  if (i >= m) return;
+  zd acc[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) acc[c] = mkz(0.0);
+  const zd* a = A.p + i * A.rs;
+#pragma unroll 2
+  for (int64_t t = lane; t < k; t += 32) {
+    zd v = a[t];
+    if (A.conj) v.y = -v.y;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (j0 + c < n) {
+        zd w = B.p[t * B.rs + (j0 + c) * B.cs];
+        if (B.conj) w.y = -w.y;
+        zfma(acc[c], v, w);
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, o);
+      acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, o);
+    }
+  // lane c stores column c
+  zd r = acc[0];
+#pragma unroll
+  for (int c = 1; c < NC; ++c)
+    if (lane == c) r = acc[c];
+  if (lane < NC && j0 + lane < n) {
+    zd* o = C + (j0 + lane) * ldc + i;
+    r = alpha * r;
+    if (!(beta.x == 0.0 && beta.y == 0.0)) r += beta * (*o);
+    *o = r;
+  }
+}
+
+// k_zgemm_cols: rows contiguous in A (A.rs == 1): lanes over 32 rows, the 16
+// warps of a CTA over K, their sums joined through shared memory in order.
+template <int NC>
+__global__ void __launch_bounds__(512) k_zgemm_cols(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B,
+                                                    zd beta, zd* __restrict__ C, int64_t ldc) {
+  __shared__ zd part[16][NC][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i = (int64_t)blockIdx.x * 32 + lane, j0 = (int64_t)blockIdx.y * NC;
+  zd acc[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) acc[c] = mkz(0.0);
+  if (i < m) {
+#pragma unroll 2
+    for (int64_t t = warp; t < k; t += 16) {
+      zd v = A.p[i + t * A.cs];
+      if (A.conj) v.y = -v.y;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (j0 + c < n) {
+          zd w = B.p[t * B.rs + (j0 + c) * B.cs];
+          if (B.conj) w.y = -w.y;
+          zfma(acc[c], v, w);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) part[warp][c][lane] = acc[c];
+  __syncthreads();
+  for (int c = warp; c < NC; c += 16) {
+    zd r = part[0][c][lane];
+#pragma unroll
+    for (int w = 1; w < 16; ++w) r += part[w][c][lane];
+    if (i < m && j0 + c < n) {
+      zd* o = C + (j0 + c) * ldc + i;
+      r = alpha * r;
+      if (!(beta.x == 0.0 && beta.y == 0.0)) r += beta * (*o);
+      *o = r;
+    }
+  }
+}
+
+template <int NC>
+static void launch_zgemm_small(bool rows, int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C,
+                               int64_t ldc, cudaStream_t s) {
+  if (rows) {
+    dim3 g((unsigned)((m + 3) / 4), (unsigned)((n + NC - 1) / NC));
+    k_zgemm_rows<NC><<<g, 128, 0, s>>>(m, n, k, alpha, A, B, beta, C, ldc);
+  } else {
+    dim3 g((unsigned)((m + 31) / 32), (unsigned)((n + NC - 1) / NC));
+    k_zgemm_cols<NC><<<g, 512, 0, s>>>(m, n, k, alpha, A, B, beta, C, ldc);
+  }
+  note_launch();
+}
+
+// The spread kernels serve up to 8 columns of any length (every column pass
+// reads A once) and wider products of up to 2^22 complex multiply-adds, for
+// which the tile kernel has too few tiles (64 x 64 x 64: one CTA).  Columns
+// per pass: the most that leaves about two CTAs per SM.
+static bool zgemm_small(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
+                        cudaStream_t s) {
+  const bool rows = (A.cs == 1);
+  if (!rows && A.rs != 1) return false;
+  if (n > 8 && (double)m * (double)n * (double)k > 4194304.0) return false;
+  if (n > 65535) return false;
+  const int64_t tiles = rows ? (m + 3) / 4 : (m + 31) / 32;
+  int nc = 8;
+  while (nc > 1 && (nc / 2 >= n || tiles * ((n + nc - 1) / nc) < 304)) nc /= 2;
+  switch (nc) {
+    case 8: launch_zgemm_small<8>(rows, m, n, k, alpha, A, B, beta, C, ldc, s); break;
+    case 4: launch_zgemm_small<4>(rows, m, n, k, alpha, A, B, beta, C, ldc, s); break;
+    case 2: launch_zgemm_small<2>(rows, m, n, k, alpha, A, B, beta, C, ldc, s); break;
+    default: launch_zgemm_small<1>(rows, m, n, k, alpha, A, B, beta, C, ldc, s); break;
+  }
+  return true;
+}
+
+// One thread per output, K in order: the summation order of k_zgemm, for
+// products whose difference is taken afterwards (central differences of the
+// far-field map), where the roundings of both have to be alike.  Bound by the
+// chain of 2 K dependent FP64 FMAs (45 x 8 x 1024: 1.17 ms in k_zgemm's two
+// CTAs of staged tiles).
+__global__ void __launch_bounds__(128) k_zgemm_serial(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B,
+                                                      zd beta, zd* __restrict__ C, int64_t ldc) {
+  const int64_t i = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31), j = (int64_t)blockIdx.y * 4 + (threadIdx.x >> 5);
+  if (i >= m || j >= n) return;
+  const zd* a = A.p + i * A.rs;
+  const zd* b = B.p + j * B.cs;
+  zd acc = mkz(0.0);
+#pragma unroll 8
+  for (int64_t t = 0; t < k; ++t) {
+    zd v = a[t * A.cs], w = b[t * B.rs];
+    if (A.conj) v.y = -v.y;
+    if (B.conj) w.y = -w.y;
+    zfma(acc, v, w);
+  }
+  zd r = alpha * acc;
+  zd* o = C + j * ldc + i;
+  if (!(beta.x == 0.0 && beta.y == 0.0)) r += beta * (*o);
+  *o = r;
+}
+
+int zgemm_ordered(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
+                  cudaStream_t s) {
+  if (m <= 0 || n <= 0) return 0;
+  // enough outputs for the staged tiles to fill the GPU: they load A and B once
+  if (m * n > 65536) {
+    const int r = launch_zgemm<16, 16, 4, 4>(m, n, k, alpha, A, B, beta, C, ldc, s);
+    if (r) return r;
+  } else {
+    dim3 g((unsigned)((m + 31) / 32), (unsigned)((n + 3) / 4));
+    k_zgemm_serial<<<g, 128, 0, s>>>(m, n, k, alpha, A, B, beta, C, ldc);
+    note_launch();
+  }
+  cudaError_t err = cudaGetLastError();
+  if (err != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(err)); return 3; }
+  return 0;
+}
+
 int zgemm(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
           cudaStream_t s) {
   if (m <= 0 || n <= 0) return 0;
-  int r;
-  if (n <= 8) r = launch_zgemm<32, 8, 4, 1>(m, n, k, alpha, A, B, beta, C, ldc, s);          // 128 x 8 tiles
-  else if (n <= 16) r = launch_zgemm<16, 16, 4, 1>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 64 x 16
-  else if (n <= 32) r = launch_zgemm<16, 16, 4, 2>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 64 x 32
-  else r = launch_zgemm<16, 16, 4, 4>(m, n, k, alpha, A, B, beta, C, ldc, s);                // 64 x 64
+  int r = 0;
+  if (!zgemm_small(m, n, k, alpha, A, B, beta, C, ldc, s)) {
+    if (n <= 16) r = launch_zgemm<16, 16, 4, 1>(m, n, k, alpha, A, B, beta, C, ldc, s);        // 64 x 16 tiles
+    else if (n <= 32) r = launch_zgemm<16, 16, 4, 2>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 64 x 32
+    else r = launch_zgemm<16, 16, 4, 4>(m, n, k, alpha, A, B, beta, C, ldc, s);                // 64 x 64
+  }
   if (r) return r;
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(err)); return 3; }

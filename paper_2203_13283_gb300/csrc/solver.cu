@@ -2374,7 +2374,8 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
       wcs_ctx* t = sgn == 0 ? tp.t : tm.t;
       TRY(farfield_matrix(t->near, t->quad.wn, t->quad.xn, t->opt.q_near, N, t->h, t->k, phd.d(), nphi, E.z(),
                           nphi, c->s));
-      TRY(zgemm(nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), Wf.z(), nphi, c->s));
+      TRY(zgemm_ordered(nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), Wf.z(), nphi,
+                        c->s));
       TRY(column_dotc(F.z(), nphi, Wf.z(), nphi, nphi, B, dots.z(), c->s));
       cudaMemcpyAsync(hd.data(), dots.p, sizeof(zd) * B, cudaMemcpyDeviceToHost, c->s);
       TRY(sync(c));
