@@ -114,19 +114,33 @@ void build_quad_tables(QuadTables& q) {
   std::vector<ld_t> IX, IW;
   gl_ld(n + 1, IX, IW);
 
+  // The basis at the points of each inner rule, formed once for all (p, r): an
+  // evaluation is n - 1 long-double divisions, which Arm hosts do in software
+  // (evaluated per pair, the tables of n = 12 took 350 ms of every context).
+  const int ni = n + 1;
+  auto basis = [&](std::vector<ld_t>& out, int m, int g, ld_t t) {
+    for (int p = 0; p < n; ++p) out[((size_t)p * J + m) * ni + g] = lagrange(xs, p, t);
+  };
+  std::vector<ld_t> b0((size_t)n * J * ni), b1(b0.size()), wi((size_t)J * ni);
+  auto at = [&](const std::vector<ld_t>& v, int p, int m, int g) { return v[((size_t)p * J + m) * ni + g]; };
+
   // --- self: d = |xi - eta|.  W_pq = int_0^1 log t Q_pq(t) dt,
   //     Q_pq(t) = int_0^{1-t} [l_p(y + t) l_q(y) + l_p(y) l_q(y + t)] dy
   q.wlog[0].assign(n * n, 0.0);
+  for (int m = 0; m < J; ++m)
+    for (int g = 0; g < ni; ++g) {
+      const ld_t t = tg[m], L = 1 - t, y = L * (IX[g] + 1) / 2;
+      wi[(size_t)m * ni + g] = L * IW[g] / 2;
+      basis(b0, m, g, y);
+      basis(b1, m, g, y + t);
+    }
   for (int p = 0; p < n; ++p)
     for (int r = 0; r < n; ++r) {
       std::vector<ld_t> vals(J);
       for (int m = 0; m < J; ++m) {
-        ld_t t = tg[m], L = 1 - t, acc = 0;
-        for (int g = 0; g < n + 1; ++g) {
-          ld_t y = L * (IX[g] + 1) / 2, wy = L * IW[g] / 2;
-          acc += wy * (lagrange(xs, p, y + t) * lagrange(xs, r, y) +
-                       lagrange(xs, p, y) * lagrange(xs, r, y + t));
-        }
+        ld_t acc = 0;
+        for (int g = 0; g < ni; ++g)
+          acc += wi[(size_t)m * ni + g] * (at(b1, p, m, g) * at(b0, r, m, g) + at(b0, p, m, g) * at(b1, r, m, g));
         vals[m] = acc;
       }
       q.wlog[0][p * n + r] = (double)log_moment_integral(tg, wg, vals);
@@ -135,27 +149,32 @@ void build_quad_tables(QuadTables& q) {
   // --- touching: V_ij = int int l_i(a) l_j(b) log(a + b), a, b in [0, 1].
   //     With v = a + b: on v in [0,1] Q(v) = int_0^v l_i(a) l_j(v - a) da (log moments),
   //     on v in [1,2] log v is smooth (plain Gauss with J nodes).
-  std::vector<ld_t> V(n * n, 0);
+  std::vector<ld_t> V(n * n, 0), c0(b0.size()), c1(b0.size()), wj(wi.size());
+  for (int m = 0; m < J; ++m)
+    for (int g = 0; g < ni; ++g) {
+      const ld_t v = tg[m], a = v * (IX[g] + 1) / 2;
+      wi[(size_t)m * ni + g] = v * IW[g] / 2;
+      basis(b0, m, g, a);
+      basis(b1, m, g, v - a);
+      const ld_t v2 = 1 + tg[m], lo = v2 - 1, L = 1 - lo, a2 = lo + L * (IX[g] + 1) / 2;   // a in [v - 1, 1]
+      wj[(size_t)m * ni + g] = L * IW[g] / 2;
+      basis(c0, m, g, a2);
+      basis(c1, m, g, v2 - a2);
+    }
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) {
       std::vector<ld_t> vals(J);
       for (int m = 0; m < J; ++m) {
-        ld_t v = tg[m], acc = 0;
-        for (int g = 0; g < n + 1; ++g) {
-          ld_t a = v * (IX[g] + 1) / 2, wa = v * IW[g] / 2;
-          acc += wa * lagrange(xs, i, a) * lagrange(xs, j, v - a);
-        }
+        ld_t acc = 0;
+        for (int g = 0; g < ni; ++g) acc += wi[(size_t)m * ni + g] * at(b0, i, m, g) * at(b1, j, m, g);
         vals[m] = acc;
       }
       ld_t part1 = log_moment_integral(tg, wg, vals);
       ld_t part2 = 0;
       for (int m = 0; m < J; ++m) {
-        ld_t v = 1 + tg[m], acc = 0;   // a in [v - 1, 1]
-        ld_t lo = v - 1, L = 1 - lo;
-        for (int g = 0; g < n + 1; ++g) {
-          ld_t a = lo + L * (IX[g] + 1) / 2, wa = L * IW[g] / 2;
-          acc += wa * lagrange(xs, i, a) * lagrange(xs, j, v - a);
-        }
+        const ld_t v = 1 + tg[m];
+        ld_t acc = 0;
+        for (int g = 0; g < ni; ++g) acc += wj[(size_t)m * ni + g] * at(c0, i, m, g) * at(c1, j, m, g);
         part2 += wg[m] * logl(v) * acc;
       }
       V[i * n + j] = part1 + part2;
