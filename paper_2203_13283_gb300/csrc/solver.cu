@@ -19,6 +19,7 @@
 #include "internal.h"
 #include "gemm_tc.h"
 #include "exact.h"
+#include "fxgemm.h"
 
 namespace wcs {
 std::atomic<unsigned long long> g_launches{0};
@@ -81,6 +82,7 @@ struct wcs_ctx {
   DevBuf w1, w2, w3, w4, w5;              // N x chunk scratch
   DevBuf small;                           // small scratch
   DevBuf gwork;                           // work of the Gram inverse (N x cols)
+  DevBuf fx;                              // fixed-point slices and partials of the FP64 products (zgemm_fx)
   // mixed-precision form
   bool mixed = false;
   int planes = 2, rhs_planes = 2;
@@ -175,6 +177,18 @@ static int ensure_tcerr(wcs_ctx* c) {
   TRY(c->tcerr.ensure(sizeof(int)));
   cudaMemsetAsync(c->tcerr.p, 0, sizeof(int), c->s);
   return 0;
+}
+
+// Complex FP64 product C = alpha A B + beta C: on the tensor cores through
+// fixed-point slices where the shape is worth it, else (or when their
+// workspace does not fit the device) on the FP64 pipe.
+static int cz(wcs_ctx* c, int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc) {
+  if (zgemm_fx_wanted(m, n, k) && !ensure_tcerr(c)) {
+    if (!c->fx.ensure(zgemm_fx_bytes(m, n, k)))
+      return zgemm_fx(m, n, k, alpha, A, B, beta, C, ldc, c->fx.p, (int*)c->tcerr.p, c->s);
+    (void)cudaGetLastError();   // out of memory: not an error of this call
+  }
+  return zgemm(m, n, k, alpha, A, B, beta, C, ldc, c->s);
 }
 
 static int ensure_stage(wcs_ctx* c, int64_t cols) {
@@ -290,7 +304,7 @@ static int check_tc(wcs_ctx* c) {
 static int cgemm(wcs_ctx* c, int64_t m, int64_t n, int64_t k, zd alpha, ZView A, const zd* X, int64_t ldx,
                  zd beta, zd* C, int64_t ldc, bool accurate = false) {
   if (m <= 0 || n <= 0) return 0;
-  if (!c->mixed || k < 64) return zgemm(m, n, k, alpha, A, blk(X, ldx), beta, C, ldc, c->s);
+  if (!c->mixed || k < 64) return cz(c, m, n, k, alpha, A, blk(X, ldx), beta, C, ldc);
   // fast: two planes, one accumulator; accurate: three planes, the drained
   // accumulation of the refinement residual
   const int P = accurate ? 3 : 2;
@@ -483,24 +497,24 @@ static int apply_C(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ldy, int
   const zd one = mkz(1.0), zero = mkz(0.0), mone = mkz(-1.0);
   if (!adj) {
     // T1 = (G/2 - D) X, T2 = N X
-    TRY(zgemm(N, cols, N, mone, op_view(c->D, c->ld, false), blk(X, ldx), zero, T1, N, c->s));
+    TRY(cz(c, N, cols, N, mone, op_view(c->D, c->ld, false), blk(X, ldx), zero, T1, N));
     TRY(gram_apply(X, ldx, T1, N, N, cols, c->h, 0.5, 1.0, c->s));
-    TRY(zgemm(N, cols, N, one, op_view(c->Nk, c->ld, false), blk(X, ldx), zero, T2, N, c->s));
+    TRY(cz(c, N, cols, N, one, op_view(c->Nk, c->ld, false), blk(X, ldx), zero, T2, N));
     TRY(ginv(c, T1, N, T1, N, cols));
     TRY(ginv(c, T2, N, T2, N, cols));
     // Y = (G/2 + D~) T1 + S~ T2
-    TRY(zgemm(N, cols, N, one, op_view(c->Dt, c->ld, false), blk(T1, N), zero, Y, ldy, c->s));
-    TRY(zgemm(N, cols, N, one, op_view(c->S, c->ld, false), blk(T2, N), one, Y, ldy, c->s));
+    TRY(cz(c, N, cols, N, one, op_view(c->Dt, c->ld, false), blk(T1, N), zero, Y, ldy));
+    TRY(cz(c, N, cols, N, one, op_view(c->S, c->ld, false), blk(T2, N), one, Y, ldy));
     TRY(gram_apply(T1, N, Y, ldy, N, cols, c->h, 0.5, 1.0, c->s));
   } else {
     // C^H = (G/2 - D)^H G^{-1} (G/2 + D~)^H + N^H G^{-1} S~^H   (G real symmetric)
-    TRY(zgemm(N, cols, N, one, op_view(c->Dt, c->ld, true), blk(X, ldx), zero, T1, N, c->s));
+    TRY(cz(c, N, cols, N, one, op_view(c->Dt, c->ld, true), blk(X, ldx), zero, T1, N));
     TRY(gram_apply(X, ldx, T1, N, N, cols, c->h, 0.5, 1.0, c->s));
-    TRY(zgemm(N, cols, N, one, op_view(c->S, c->ld, true), blk(X, ldx), zero, T2, N, c->s));
+    TRY(cz(c, N, cols, N, one, op_view(c->S, c->ld, true), blk(X, ldx), zero, T2, N));
     TRY(ginv(c, T1, N, T1, N, cols));
     TRY(ginv(c, T2, N, T2, N, cols));
-    TRY(zgemm(N, cols, N, mone, op_view(c->D, c->ld, true), blk(T1, N), zero, Y, ldy, c->s));
-    TRY(zgemm(N, cols, N, one, op_view(c->Nk, c->ld, true), blk(T2, N), one, Y, ldy, c->s));
+    TRY(cz(c, N, cols, N, mone, op_view(c->D, c->ld, true), blk(T1, N), zero, Y, ldy));
+    TRY(cz(c, N, cols, N, one, op_view(c->Nk, c->ld, true), blk(T2, N), one, Y, ldy));
     TRY(gram_apply(T1, N, Y, ldy, N, cols, c->h, 0.5, 1.0, c->s));
   }
   return 0;
@@ -830,7 +844,7 @@ int wcs_destroy(wcs_ctx* c) {
   free_mesh(c);
   c->xf.release(); c->xn.release(); c->wn.release(); c->wlog.release();
   c->w1.release(); c->w2.release(); c->w3.release(); c->w4.release(); c->w5.release();
-  c->small.release(); c->tcerr.release(); c->gwork.release();
+  c->small.release(); c->tcerr.release(); c->gwork.release(); c->fx.release();
   delete c;
   return WCS_OK;
 }
@@ -1228,11 +1242,11 @@ int wcs_apply(wcs_ctx* c, int op, int64_t B, const double* X, int64_t ldx, doubl
           break;
         }
         if (op != WCS_OP_S) goto fp64_ops;
-        TRY(zgemm(N, cc, N, mkz(1.0), op_view(c->S, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy, c->s)); break;
+        TRY(cz(c, N, cc, N, mkz(1.0), op_view(c->S, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy)); break;
       fp64_ops:
-        if (op == WCS_OP_D) { TRY(zgemm(N, cc, N, mkz(1.0), op_view(c->D, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy, c->s)); break; }
-        if (op == WCS_OP_DT) { TRY(zgemm(N, cc, N, mkz(1.0), op_view(c->Dt, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy, c->s)); break; }
-        TRY(zgemm(N, cc, N, mkz(1.0), op_view(c->Nk, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy, c->s));
+        if (op == WCS_OP_D) { TRY(cz(c, N, cc, N, mkz(1.0), op_view(c->D, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy)); break; }
+        if (op == WCS_OP_DT) { TRY(cz(c, N, cc, N, mkz(1.0), op_view(c->Dt, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy)); break; }
+        TRY(cz(c, N, cc, N, mkz(1.0), op_view(c->Nk, c->ld, false), blk(xc, ldx), mkz(0.0), yc, ldy));
         break;
       case WCS_OP_G: TRY(gram_apply(xc, ldx, yc, ldy, N, cc, c->h, 1.0, 0.0, c->s)); break;
       case WCS_OP_GINV: TRY(ginv(c, xc, ldx, yc, ldy, cc)); break;
@@ -1382,7 +1396,7 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
     const int64_t cc = std::min<int64_t>(wide, ell - c0);
     TRY(apply_remainder(c, Q + c0 * N, N, c->Vw.z() + c0 * N, N, cc, true, PREC_PERIODIC));
   }
-  TRY(sync(c));
+  TRY(check_tc(c));
   if (rank_out) *rank_out = (int)ell;
   c->Wt.release(); c->Kinv.release(); c->Wa.release();
   c->stage = ST_SKELETON;
@@ -1548,7 +1562,7 @@ int wcs_factor(wcs_ctx* c) {
     }
     // Wt = W K^{-1}
     TRY(cgemm(c, N, r, r, mkz(1.0), blk(Wb.z(), N), Kinv.z(), r, mkz(0.0), c->Wt.z(), N));
-    TRY(sync(c));
+    TRY(check_tc(c));
   }
   c->stage = ST_FACTORED;
   return WCS_OK;
@@ -1841,8 +1855,8 @@ static int precondition(wcs_ctx* c, const zd* e, const zd* hv, int64_t ld, zd* b
     TRY(tc_apply(c, 0, false, c->stage1, cc, mkz(0.0, -c->k), mkz(0.0), b, ldb, mode));
     TRY(tc_apply(c, 2, false, c->stage2, cc, mkz(-1.0), mkz(1.0), b, ldb, mode));
   } else {
-    TRY(zgemm(N, cc, N, mkz(0.0, -c->k), op_view(c->S, c->ld, false), blk(T1, N), mkz(0.0), b, ldb, c->s));
-    TRY(zgemm(N, cc, N, mkz(-1.0), op_view(c->Dt, c->ld, false), blk(T2, N), mkz(1.0), b, ldb, c->s));
+    TRY(cz(c, N, cc, N, mkz(0.0, -c->k), op_view(c->S, c->ld, false), blk(T1, N), mkz(0.0), b, ldb));
+    TRY(cz(c, N, cc, N, mkz(-1.0), op_view(c->Dt, c->ld, false), blk(T2, N), mkz(1.0), b, ldb));
   }
   TRY(gram_apply(T2, N, b, ldb, N, cc, c->h, -0.5, 1.0, c->s));
   return 0;
@@ -2050,6 +2064,7 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
     }
   }
   nb.release();
+  TRY(check_tc(c));
   finish(worst);
   return (worst <= c->opt.refine_tol) ? 0 : WCS_ERR_NOT_CONVERGED;
 }
@@ -2188,7 +2203,7 @@ static int sum_parts(wcs_ctx* c, const double* part, int n, zd* out) {
 static int op_apply(wcs_ctx* c, int which, bool adj, const zd* X, int64_t ldx, int64_t cols, zd* Y, int64_t ldy) {
   if (!c->mixed) {
     const zd* ops[4] = {c->S, c->D, c->Dt, c->Nk};
-    return zgemm(c->N, cols, c->N, mkz(1.0), op_view(ops[which], c->ld, adj), blk(X, ldx), mkz(0.0), Y, ldy, c->s);
+    return cz(c, c->N, cols, c->N, mkz(1.0), op_view(ops[which], c->ld, adj), blk(X, ldx), mkz(0.0), Y, ldy);
   }
   TRY(ensure_stage(c, cols));
   TRY(stage(c, c->stage0, X, ldx, cols, adj ? 1 : 0));
@@ -2299,7 +2314,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
   else if (r) return r;
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, N, c->h, c->k, phd.d(), nphi, E.z(),
                       nphi, c->s));
-  TRY(zgemm(nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), F.z(), nphi, c->s));
+  TRY(cz(c, nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), F.z(), nphi));
   std::vector<zd> hd(4 * B);
   TRY(column_dotc(F.z(), nphi, F.z(), nphi, nphi, B, dots.z(), c->s));
   cudaMemcpyAsync(hd.data(), dots.p, sizeof(zd) * B, cudaMemcpyDeviceToHost, c->s);
@@ -2309,7 +2324,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
   *J_out = J;
   if (i1 == i0) return status;
   // adjoint: lam = C^-H E^H F
-  TRY(zgemm(N, B, nphi, mkz(1.0), ZView{E.z(), nphi, 1, true}, blk(F.z(), nphi), mkz(0.0), G.z(), N, c->s));
+  TRY(cz(c, N, B, nphi, mkz(1.0), ZView{E.z(), nphi, 1, true}, blk(F.z(), nphi), mkz(0.0), G.z(), N));
   r = solve_general(c, B, G.d(), N, lam.d(), N, &si, true);
   if (r == WCS_ERR_NOT_CONVERGED) status = r;
   else if (r) return r;
@@ -2354,7 +2369,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
     const double sgn[4] = {-1.0, 1.0, -1.0, -1.0};
     for (int X = 0; X < 4; ++X) {
       zd* Wx = Wb.z() + (int64_t)X * N * N;
-      TRY(zgemm(N, N, B, mkz(sgn[X]), ZView{V[X], 1, N, false}, ZView{U[X], N, 1, true}, mkz(0.0), Wx, N, c->s));
+      TRY(cz(c, N, N, B, mkz(sgn[X]), ZView{V[X], 1, N, false}, ZView{U[X], N, 1, true}, mkz(0.0), Wx, N));
       W[X] = Wx;
     }
   }
@@ -2420,8 +2435,8 @@ int wcs_shape_operator_forms(wcs_ctx* c, int op, int64_t B, const double* u_dev,
   cudaMemsetAsync(Wb.p, 0, Wb.bytes, c->s);
   const zd* W[4];
   for (int X = 0; X < 4; ++X) W[X] = Wb.z() + (int64_t)X * N * N;
-  TRY(zgemm(N, N, B, mkz(1.0), ZView{(const zd*)v_dev, 1, ld, false}, ZView{(const zd*)u_dev, ld, 1, true}, mkz(0.0),
-            Wb.z() + (int64_t)op * N * N, N, c->s));
+  TRY(cz(c, N, N, B, mkz(1.0), ZView{(const zd*)v_dev, 1, ld, false}, ZView{(const zd*)u_dev, ld, 1, true}, mkz(0.0),
+            Wb.z() + (int64_t)op * N * N, N));
   CtxGuard tp, tm;
   TRY(make_scratch(c, tp));
   TRY(make_scratch(c, tm));
@@ -2495,9 +2510,9 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
   cudaMemcpyAsync(ang.p, phi, sizeof(double) * nphi, cudaMemcpyHostToDevice, c->s);
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, c->N, c->h, c->k, ang.d(),
                       nphi, E.z(), nphi, c->s));
-  TRY(zgemm(nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
-            (zd*)F, ldf, c->s));
-  int r = sync(c);
+  TRY(cz(c, nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
+         (zd*)F, ldf));
+  int r = check_tc(c);
   E.release();
   ang.release();
   return r;
