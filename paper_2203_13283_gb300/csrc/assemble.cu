@@ -23,8 +23,10 @@
 #include <cstring>
 #include <vector>
 
+#include "farpair.cuh"
 #include "hankel.cuh"
 #include "internal.h"
+#include "split.cuh"
 
 namespace wcs {
 
@@ -224,254 +226,36 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
 }
 
 
-// ---------------------------------------------------------------------------
-// Far element pairs in the mixed form.  With element centres c_e, c_f and
-// point offsets o = r - c (|o| < h), R = |d0 + o_p - o_r| with d0 = c_e - c_f:
-// R0 = |d0| and the phase k R0 mod 2 pi are formed in float-float once per
-// pair; R - R0 = (2 d0.(o_p - o_r) + |o_p - o_r|^2) / (R + R0) is small, so
-// the phase k R = (k R0 mod 2 pi) + k (R - R0) keeps ~1e-7 absolute accuracy
-// even for k R ~ 1e4.  The Hankel functions use the large-argument expansion
-// (DLMF 10.17.5) with ten terms (z >= 9 gives < 1e-7), for k and for
-// k~ = k + i beta (exp(i k~ R) = exp(i k R - beta R)).
-//
-// Roundings that repeat identically in every element pair act like one
-// perturbation of the whole operator and are not averaged out: the products
-// of quadrature weights and hat values, the wavenumber constants, the point
-// offsets and the normals.  So the weights come from float-float tables
-// (the tensor rule is separable: an inner sum over the source points r with
-// weights w_r phi_b(xi_r), an outer sum over the target points p with
-// w_p phi_a(xi_p)), offsets and normals carry float-float tails, and every
-// constant factor of a kernel is left out of the FP32 sums and applied in
-// FP64 when the entry is stored (AsmArgs::fS .. fN, kk2h2).  What remains in
-// FP32 varies from pair to pair (the rounding of R, the Hankel series, the
-// sums), so its effect on the solution averages down.
-// ---------------------------------------------------------------------------
-__constant__ float c_a0[10], c_a1[10];   // a_k(0), a_k(1) of the Hankel expansion
-__constant__ float c_fwt[2][16][2];      // w_r phi_b(xi_r) as float-float [b][r][hi, lo]
-__constant__ float c_fw[16][2];          // w_r as float-float
-
-struct cf {
-  float x, y;
-};
-__device__ __forceinline__ cf cmul(cf a, cf b) { return {fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x)}; }
-__device__ __forceinline__ cf cscale(cf a, float s) { return {a.x * s, a.y * s}; }
-// acc += (hi + lo) v, the small term first
-__device__ __forceinline__ void cfma2(cf& acc, float hi, float lo, cf v) {
-  acc.x = fmaf(hi, v.x, fmaf(lo, v.x, acc.x));
-  acc.y = fmaf(hi, v.y, fmaf(lo, v.y, acc.y));
-}
-__device__ __forceinline__ void cadd(cf& acc, cf v) { acc.x += v.x; acc.y += v.y; }
-
-// Reduced sums of one element pair, [a * 2 + b]:
-//   0  S~ / fS     1  D / fD     2  D~ / fD~
-//   3  N, k^2 h^2 (n.n') part     4  N, derivative part (signs s_a s_b applied)
-// with N = fN (v[4] - k^2 h^2 v[3]).
-struct PairOutF {
-  cf v[5][4];
-};
-
-__device__ void pair_fast_f(const AsmArgs& A, int64_t e, int64_t f, PairOutF& out);
-
-__device__ __forceinline__ zd zf2d(cf a) { return mkz((double)a.x, (double)a.y); }
-
-// The four operators of a far pair from the reduced FP32 sums (FP64 factors).
-__device__ void pair_fast(const AsmArgs& A, int64_t e, int64_t f, PairOut& out) {
-  PairOutF o;
-  pair_fast_f(A, e, f, o);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    out.v[0][j] = A.fS * zf2d(o.v[0][j]);
-    out.v[1][j] = A.fD * zf2d(o.v[1][j]);
-    out.v[2][j] = A.fDt * zf2d(o.v[2][j]);
-    out.v[3][j] = A.fN * (zf2d(o.v[4][j]) - A.kk2h2 * zf2d(o.v[3][j]));
-  }
-}
-
-// Float-float arithmetic (value = hi + lo, ~48 bits; Dekker/Knuth error-free
-// transformations).  The far-pair phase k |c_e - c_f| mod 2 pi needs ~1e-7
-// absolute accuracy at k R ~ 2e4; float-float gives ~1e-10 without touching
-// the FP64 pipe, which runs at 1/64 of the FP32 rate on this GPU.
-struct ff {
-  float hi, lo;
-};
-__device__ __forceinline__ ff ff_quick(float a, float b) {
-  const float s = a + b;
-  return {s, b - (s - a)};
-}
-__device__ __forceinline__ ff ff_two_sum(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ ff ff_two_prod(float a, float b) {
-  const float p = a * b;
-  return {p, fmaf(a, b, -p)};
-}
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-  const ff s = ff_two_sum(a.hi, b.hi);
-  return ff_quick(s.hi, s.lo + (a.lo + b.lo));
-}
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-  ff p = ff_two_prod(a.hi, b.hi);
-  return ff_quick(p.hi, p.lo + fmaf(a.hi, b.lo, a.lo * b.hi));
-}
-__device__ __forceinline__ ff ff_sqrt(ff a) {
-  // one Newton step from the FP32 root: x + (a - x^2) / (2x)
-  const float x = sqrtf(a.hi);
-  const ff d = ff_add(a, ff_neg(ff_two_prod(x, x)));
-  return ff_quick(x, d.hi * (0.5f / x));
-}
-
-__device__ void pair_fast_f(const AsmArgs& A, int64_t e, int64_t f, PairOutF& out) {
+// The four operators of a far pair in FP64 from its float-float sums (farpair.cuh).
+__device__ __noinline__ void pair_far(const AsmArgs& A, int64_t e, int64_t f, PairOut& out) {
+  FarPair o;
   const int q = A.q_far;
-  const FastConsts& F = A.fk;
-  const float4 ce = A.cff[e], cf_ = A.cff[f];   // (x hi, x lo, y hi, y lo)
-  const ff dx = ff_add(ff_two_sum(ce.x, -cf_.x), ff_two_sum(ce.y, -cf_.y));
-  const ff dy = ff_add(ff_two_sum(ce.z, -cf_.z), ff_two_sum(ce.w, -cf_.w));
-  const ff R0 = ff_sqrt(ff_add(ff_mul(dx, dx), ff_mul(dy, dy)));
-  const ff kR0 = ff_mul({F.k_hi, F.k_lo}, R0);
-  // kR0 - n 2pi with 2pi = t1 + t2 + t3 (24 + 24 + 24 bits); n < 2^13 so n t1, n t2 are exact products
-  const float n = rintf(kR0.hi * 0.15915494309189535f);
-  ff t = ff_add(kR0, ff_neg(ff_two_prod(n, F.twopi[0])));
-  t = ff_add(t, ff_neg(ff_two_prod(n, F.twopi[1])));
-  // ph0 = k R0 - pi/4 reduced, kept in float-float (|ph0| <= 5 pi / 4);
-  // -pi/4 = -0.785398185 + 2.18556941e-8 (float head, float tail)
-  const ff ph0 = ff_add(ff_add(t, {-n * F.twopi[2], 0.f}), {-0.785398185f, 2.18556941e-08f});
-  const float fdx0 = dx.hi, fdy0 = dy.hi, fR0 = R0.hi;
-  const ff twoR0 = {2.f * R0.hi, 2.f * R0.lo};
-  const ff kff = {F.k_hi, F.k_lo};
-  const float ldx0 = dx.lo, ldy0 = dy.lo;
-  const float k = F.kf, beta = F.beta, beta_lo = F.beta_lo;
-  const cf ik = {F.ik[0], F.ik[1]};      // i / k~
-  cf vS[4], vD[4], vDt[4], vNb[4], vNd = {0.f, 0.f};
+  if (q == 4) far_pair<4>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+  else far_pair<0>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+  const zd fac[4] = {A.fS, A.fD, A.fDt, A.fN};
 #pragma unroll
-  for (int j = 0; j < 4; ++j) vS[j] = vD[j] = vDt[j] = vNb[j] = cf{0.f, 0.f};
-  for (int p = 0; p < q; ++p) {
-    const int64_t ip = e * q + p;
-    const float oxp = A.ox[ip], oyp = A.oy[ip], oxlp = A.oxl[ip], oylp = A.oyl[ip];
-    const float nxt = A.nxf[ip], nyt = A.nyf[ip], nxtl = A.nxl[ip], nytl = A.nyl[ip];
-    cf uS[2], uD[2], uDt[2], uNb[2], uNd = {0.f, 0.f};
+  for (int op = 0; op < 4; ++op)
 #pragma unroll
-    for (int b = 0; b < 2; ++b) uS[b] = uD[b] = uDt[b] = uNb[b] = cf{0.f, 0.f};
-    for (int r = 0; r < q; ++r) {
-      const int64_t ir = f * q + r;
-      // D = o_p - o_r in float-float (the offsets' tails included)
-      ff Dx = ff_two_sum(oxp, -A.ox[ir]), Dy = ff_two_sum(oyp, -A.oy[ir]);
-      Dx = ff_quick(Dx.hi, Dx.lo + (oxlp - A.oxl[ir]));
-      Dy = ff_quick(Dy.hi, Dy.lo + (oylp - A.oyl[ir]));
-      const float nxs = A.nxf[ir], nys = A.nyf[ir], nxsl = A.nxl[ir], nysl = A.nyl[ir];
-      const float a = 2.f * (fdx0 * Dx.hi + fdy0 * Dy.hi) + Dx.hi * Dx.hi + Dy.hi * Dy.hi;
-      const float R = sqrtf(fR0 * fR0 + a);
-      const float iR = 1.f / R;
-      // n . n' with the normals' tails (a rounded normal would repeat in every pair of its point)
-      const float nd = fmaf(nxt, nxs, nyt * nys) + (fmaf(nxtl, nxs, nxt * nxsl) + fmaf(nytl, nys, nyt * nysl));
-      // phase k R - pi/4 = ph0 + k (R - R0) in float-float: R - R0 = a / (2 R0 + (R - R0))
-      // with a = 2 d0.D + |D|^2 from error-free products; the denominator
-      // takes the FP32 estimate of R - R0, whose error enters only relative to 2 R0
-      // (r - r').n' in float-float: on the flat parts of a contour it cancels to
-      // ~curvature R^2, far below the FP32 rounding of its terms (~6e-8 R)
-      const ff rx = ff_add(ff{fdx0, ldx0}, Dx), ry = ff_add(ff{fdy0, ldy0}, Dy);
-      const ff dn = ff_add(ff_mul(rx, ff{nxs, nxsl}), ff_mul(ry, ff{nys, nysl}));
-      const float gg = (dn.hi + dn.lo) * iR;
-      const ff a_ff = ff_add(ff_add(ff_add(ff_two_prod(2.f * Dx.hi, fdx0), ff_two_prod(2.f * Dy.hi, fdy0)),
-                                    ff_add(ff_two_prod(Dx.hi, Dx.hi), ff_two_prod(Dy.hi, Dy.hi))),
-                             ff{2.f * (Dx.hi * ldx0 + Dy.hi * ldy0 + Dx.lo * (fdx0 + Dx.hi) + Dy.lo * (fdy0 + Dy.hi)),
-                                0.f});
-      const ff den = ff_add(twoR0, ff{a / (fR0 + R), 0.f});
-      const float q0 = a_ff.hi / den.hi;
-      const ff rem = ff_add(a_ff, ff_neg(ff_mul(ff{q0, 0.f}, den)));
-      const ff th = ff_add(ph0, ff_mul(kff, ff_quick(q0, rem.hi / den.hi)));
-      float sn, cs;
-      sincosf(th.hi, &sn, &cs);
-      const float sq = sqrtf(iR);
-      // e^{i(kR - pi/4)} / sqrt(R)
-      const cf E1 = {fmaf(-sn, th.lo, cs) * sq, fmaf(cs, th.lo, sn) * sq};
-      // real wavenumber: P + iQ = sum (i t)^k a_k, t = 1/(kR)
-      const float tt = iR / k, t2 = tt * tt;
-      float P0 = c_a0[8], Q0 = c_a0[9], P1 = c_a1[8], Q1 = c_a1[9];
-#pragma unroll
-      for (int m = 3; m >= 0; --m) {
-        P0 = fmaf(-t2, P0, c_a0[2 * m]);
-        Q0 = fmaf(-t2, Q0, c_a0[2 * m + 1]);
-        P1 = fmaf(-t2, P1, c_a1[2 * m]);
-        Q1 = fmaf(-t2, Q1, c_a1[2 * m + 1]);
-      }
-      Q0 *= tt;
-      Q1 *= tt;
-      const cf H0 = cmul(E1, {P0, Q0});                         // H0(kR) / sqrt(2 / (pi k))
-      const cf H1g = cscale(cmul(E1, {Q1, -P1}), gg);           // H1(kR) gg / sqrt(2 / (pi k))
-      // complex wavenumber: w = i/(k~ R)
-      const cf w = cscale(ik, iR);
-      cf s0 = {c_a0[9], 0.f}, s1 = {c_a1[9], 0.f};
-#pragma unroll
-      for (int m = 8; m >= 0; --m) {
-        s0 = cmul(s0, w); s0.x += c_a0[m];
-        s1 = cmul(s1, w); s1.x += c_a1[m];
-      }
-      // exp(-Im k~ R); expf, not the fast intrinsic: its error grows with |beta R| (up to ~12 here)
-      const float damp = expf(-beta * R) * fmaf(-beta_lo, R, 1.f);
-      const cf Et = cscale(E1, damp);
-      const cf Ht0 = cmul(Et, s0);                              // H0(k~R) / sqrt(2 / (pi k~))
-      const cf Ht1g = cscale(cmul(Et, {s1.y, -s1.x}), gg);      // H1(k~R) gg / sqrt(2 / (pi k~))
-      const cf HN = cscale(H0, nd);
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const float wh = c_fwt[b][r][0], wl = c_fwt[b][r][1];
-        cfma2(uS[b], wh, wl, Ht0);
-        cfma2(uD[b], wh, wl, H1g);
-        cfma2(uDt[b], wh, wl, Ht1g);
-        cfma2(uNb[b], wh, wl, HN);
-      }
-      cfma2(uNd, c_fw[r][0], c_fw[r][1], H0);
+    for (int j = 0; j < 4; ++j) {
+      const ffc v = o.value(op, j);
+      out.v[op][j] = fac[op] * mkz((double)v.x.hi + (double)v.x.lo, (double)v.y.hi + (double)v.y.lo);
     }
-#pragma unroll
-    for (int aa = 0; aa < 2; ++aa) {
-      const float wh = c_fwt[aa][p][0], wl = c_fwt[aa][p][1];
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        cfma2(vS[aa * 2 + b], wh, wl, uS[b]);
-        cfma2(vD[aa * 2 + b], wh, wl, uD[b]);
-        cfma2(vDt[aa * 2 + b], wh, wl, uDt[b]);
-        cfma2(vNb[aa * 2 + b], wh, wl, uNb[b]);
-      }
-    }
-    cfma2(vNd, c_fw[p][0], c_fw[p][1], uNd);
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    out.v[0][j] = vS[j];
-    out.v[1][j] = vD[j];
-    out.v[2][j] = vDt[j];
-    out.v[3][j] = vNb[j];
-    // derivative part of the Maue form: phi_a' phi_b' h^2 = s_a s_b, + on the diagonal of the 2x2 block
-    out.v[4][j] = (j == 0 || j == 3) ? vNd : cf{-vNd.x, -vNd.y};
-  }
 }
 
-__device__ __forceinline__ bool fast_ok(const AsmArgs& A, int64_t e, int64_t f) {
-  if (periodic_dist(e, f, A.N) <= A.near_band) return false;
-  const float4 ce = A.cff[e], cf_ = A.cff[f];
-  const float dx0 = ce.x - cf_.x, dy0 = ce.z - cf_.z;
-  return A.fk.kf * A.fk.kf * (dx0 * dx0 + dy0 * dy0) >= A.fk.zfast2;
+__device__ __forceinline__ bool pair_is_far(const AsmArgs& A, int64_t e, int64_t f) {
+  return periodic_dist(e, f, A.N) > A.near_band && far_ok(A.fc, A.fe[e].c, A.fe[f].c);
 }
-
-__device__ __forceinline__ void pair_any(const AsmArgs& A, int64_t e, int64_t f, PairOut& o) {
-  if (A.mixed && fast_ok(A, e, f)) { pair_fast(A, e, f, o); return; }
-  pair_integrals(A, e, f, o);
-}
-
-__device__ __forceinline__ void split_store(double x, int planes, uint16_t* const* P, int64_t off);
 
 constexpr int TILE = 32;
 constexpr int ASM_THREADS = 256;
+constexpr int FAR_CTAS = 1;
 
+// One tile of node pairs from FP64 pair integrals: the 33 x 33 element pairs
+// that touch it, accumulated in acc[4][TILE][TILE].  MIXED: pairs far enough for
+// the FP32 route take it.
 template <int MIXED>
-__global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A) {
-  extern __shared__ zd acc[];  // [4][TILE][TILE]
+__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc) {
   const int64_t N = A.N;
-  const int64_t i0 = (int64_t)blockIdx.y * TILE, j0 = (int64_t)blockIdx.x * TILE;
-  if (MIXED && A.tile_flags && !A.tile_flags[(int64_t)blockIdx.y * gridDim.x + blockIdx.x]) return;
   for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) acc[t] = mkz(0.0);
   __syncthreads();
   const int span = TILE + 1;
@@ -488,7 +272,8 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A) {
     if (rowok && colok) {
       const int64_t e = ((i0 - 1 + el) % N + N) % N;
       const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-      if (MIXED) pair_any(A, e, f, o); else pair_integrals(A, e, f, o);
+      if (MIXED && pair_is_far(A, e, f)) pair_far(A, e, f, o);
+      else pair_integrals(A, e, f, o);
     }
 #pragma unroll
     for (int ph = 0; ph < 4; ++ph) {
@@ -503,38 +288,52 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A) {
       __syncthreads();
     }
   }
-  if constexpr (!MIXED) {
-    zd* outs[4] = {A.S, A.D, A.Dt, A.Nk};
-    for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) {
-      const int op = t / (TILE * TILE), rem = t - op * TILE * TILE;
-      const int li = rem / TILE, lj = rem - (rem / TILE) * TILE;
-      if (i0 + li < N && j0 + lj < N) outs[op][(i0 + li) * A.ld + j0 + lj] = acc[t];
-    }
-  } else {
-  // planes: layout 0 row i0+li holds (re, im) of column j0+lj at 2(j0+lj);
-  // layout 1 (transpose) row j0+lj holds entry (i0+li, j0+lj) at 2(i0+li)
-  for (int t = threadIdx.x; t < 4 * TILE * TILE * 2; t += blockDim.x) {
-    const int comp = t & 1;
-    const int u = t >> 1;
-    const int op = u / (TILE * TILE), rem = u - op * TILE * TILE;
+}
+
+// FP64 form: every tile, dense complex output
+__global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A) {
+  extern __shared__ zd acc[];  // [4][TILE][TILE]
+  const int64_t N = A.N;
+  const int64_t i0 = (int64_t)blockIdx.y * TILE, j0 = (int64_t)blockIdx.x * TILE;
+  tile_sums<0>(A, i0, j0, acc);
+  zd* outs[4] = {A.S, A.D, A.Dt, A.Nk};
+  for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) {
+    const int op = t / (TILE * TILE), rem = t - op * TILE * TILE;
     const int li = rem / TILE, lj = rem - (rem / TILE) * TILE;
-    if (i0 + li < N && j0 + lj < N) {
-      const zd v = acc[(op * TILE + li) * TILE + lj];
-      const double x = comp ? v.y : v.x;
-      split_store(x, A.planes, A.P[op][0], (i0 + li) * A.ldp + 2 * (j0 + lj) + comp);
-    }
+    if (i0 + li < N && j0 + lj < N) outs[op][(i0 + li) * A.ld + j0 + lj] = acc[t];
   }
-  for (int t = threadIdx.x; t < 4 * TILE * TILE * 2; t += blockDim.x) {
-    const int comp = t & 1;
-    const int u = t >> 1;
-    const int op = u / (TILE * TILE), rem = u - op * TILE * TILE;
-    const int lj = rem / TILE, li = rem - (rem / TILE) * TILE;   // consecutive threads walk i
-    if (i0 + li < N && j0 + lj < N) {
-      const zd v = acc[(op * TILE + li) * TILE + lj];
-      const double x = comp ? v.y : v.x;
-      split_store(x, A.planes, A.P[op][1], (j0 + lj) * A.ldp + 2 * (i0 + li) + comp);
+}
+
+// Mixed form: the tiles that k_assemble_far listed (those holding an element
+// pair nearer than its route), as split-bf16 planes in both layouts.
+__global__ void __launch_bounds__(ASM_THREADS) k_assemble_near(AsmArgs A, int64_t nt) {
+  extern __shared__ zd acc[];  // [4][TILE][TILE]
+  const int64_t N = A.N;
+  const int count = A.tile_list[0];
+  for (int u = blockIdx.x; u < count; u += gridDim.x) {
+    const int64_t tile = A.tile_list[1 + u];
+    const int64_t i0 = (tile / nt) * TILE, j0 = (tile % nt) * TILE;
+    tile_sums<1>(A, i0, j0, acc);
+    // layout 0: row i0 + li holds (re, im) of column j0 + lj at 2 (j0 + lj);
+    // layout 1 (transpose): row j0 + lj holds entry (i0 + li, j0 + lj) at 2 (i0 + li);
+    // consecutive threads walk the contiguous index
+    for (int lay = 0; lay < 2; ++lay) {
+      for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) {
+        const int op = t / (TILE * TILE), rem = t - op * TILE * TILE;
+        const int x = rem / TILE, y = rem - (rem / TILE) * TILE;
+        const int li = lay ? y : x, lj = lay ? x : y;
+        if (i0 + li < N && j0 + lj < N) {
+          const zd v = acc[(op * TILE + li) * TILE + lj];
+          uint16_t re[3] = {0, 0, 0}, im[3] = {0, 0, 0};
+          split3_bits(v.x, A.planes, &re[0], &re[1], &re[2]);
+          split3_bits(v.y, A.planes, &im[0], &im[1], &im[2]);
+          const int64_t off = lay ? (j0 + lj) * A.ldp + 2 * (i0 + li) : (i0 + li) * A.ldp + 2 * (j0 + lj);
+          for (int q = 0; q < A.planes; ++q)
+            *(uint32_t*)(A.P[op][lay][q] + off) = (uint32_t)re[q] | ((uint32_t)im[q] << 16);
+        }
+      }
     }
-  }
+    __syncthreads();
   }
 }
 
@@ -628,114 +427,27 @@ static int upload_rules(const AsmArgs& A) {
   if (cudaMemcpyToSymbol(c_wf, wf, sizeof(double) * A.q_far) != cudaSuccess) return 3;
   if (cudaMemcpyToSymbol(c_xn, xn, sizeof(double) * A.q_near) != cudaSuccess) return 3;
   if (cudaMemcpyToSymbol(c_wn, wn, sizeof(double) * A.q_near) != cudaSuccess) return 3;
-  // float-float weights of the FP32 far path: w_r phi_b(xi_r) and w_r
-  float fwt[2][16][2], fw[16][2];
-  std::memset(fwt, 0, sizeof(fwt));
-  std::memset(fw, 0, sizeof(fw));
-  for (int i = 0; i < A.q_far; ++i) {
-    const double v[3] = {wf[i] * (1.0 - xf[i]), wf[i] * xf[i], wf[i]};
-    float* dst[3] = {fwt[0][i], fwt[1][i], fw[i]};
-    for (int t = 0; t < 3; ++t) {
-      dst[t][0] = (float)v[t];
-      dst[t][1] = (float)(v[t] - (double)dst[t][0]);
-    }
-  }
-  if (cudaMemcpyToSymbol(c_fwt, fwt, sizeof(fwt)) != cudaSuccess) return 3;
-  if (cudaMemcpyToSymbol(c_fw, fw, sizeof(fw)) != cudaSuccess) return 3;
   return 0;
 }
 
 int assemble_dense(const AsmArgs& A, cudaStream_t s) {
   if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const size_t smem = sizeof(zd) * 4 * TILE * TILE;
-  cudaFuncSetAttribute(k_assemble<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t nt = (A.N + TILE - 1) / TILE;
   dim3 grid((unsigned)nt, (unsigned)nt);
-  k_assemble<0><<<grid, ASM_THREADS, smem, s>>>(A);
+  k_assemble<<<grid, ASM_THREADS, smem, s>>>(A);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("assemble: ") + cudaGetErrorString(err)); return 3; }
   return 0;
 }
 
-__device__ __forceinline__ void split_store(double x, int planes, uint16_t* const* P, int64_t off) {
-  __nv_bfloat16 h0 = __double2bfloat16(x);
-  double r = x - (double)__bfloat162float(h0);
-  P[0][off] = __bfloat16_as_ushort(h0);
-  if (planes > 1) {
-    __nv_bfloat16 h1 = __double2bfloat16(r);
-    r -= (double)__bfloat162float(h1);
-    P[1][off] = __bfloat16_as_ushort(h1);
-    if (planes > 2) P[2][off] = __bfloat16_as_ushort(__double2bfloat16(r));
-  }
-}
-
-// FP32 values: x - hi and (x - hi) - mid are exact in FP32, so the planes
-// equal those of split_store((double)x)
-__device__ __forceinline__ void split_store_f(float x, int planes, uint16_t* const* P, int64_t off) {
-  const __nv_bfloat16 h0 = __float2bfloat16_rn(x);
-  float r = x - __bfloat162float(h0);
-  P[0][off] = __bfloat16_as_ushort(h0);
-  if (planes > 1) {
-    const __nv_bfloat16 h1 = __float2bfloat16_rn(r);
-    r -= __bfloat162float(h1);
-    P[1][off] = __bfloat16_as_ushort(h1);
-    if (planes > 2) P[2][off] = __bfloat16_as_ushort(__float2bfloat16_rn(r));
-  }
-}
-
-static int upload_hankel_coefficients() {
-  float a0[10], a1[10];
-  double t0 = 1.0, t1 = 1.0;
-  a0[0] = 1.f;
-  a1[0] = 1.f;
-  for (int kk = 1; kk < 10; ++kk) {
-    const double o = 2.0 * kk - 1.0;
-    t0 *= (0.0 - o * o) / (8.0 * kk);
-    t1 *= (4.0 - o * o) / (8.0 * kk);
-    a0[kk] = (float)t0;
-    a1[kk] = (float)t1;
-  }
-  if (cudaMemcpyToSymbol(c_a0, a0, sizeof(a0)) != cudaSuccess) return 3;
-  if (cudaMemcpyToSymbol(c_a1, a1, sizeof(a1)) != cudaSuccess) return 3;
-  return 0;
-}
-
-// flag[t] = 1 when tile t holds an element pair outside the FP32 fast path
-__global__ void k_tile_flags(AsmArgs A, int64_t nt, uint8_t* flag) {
-  const int64_t t = blockIdx.x;
-  const int64_t ti = t / nt, tj = t - (t / nt) * nt;
-  __shared__ int any;
-  if (threadIdx.x == 0) any = 0;
-  __syncthreads();
-  const int span = TILE + 1;
-  for (int u = threadIdx.x; u < span * span; u += blockDim.x) {
-    const int el = u / span, fl = u - (u / span) * span;
-    const int64_t e = ((ti * TILE - 1 + el) % A.N + A.N) % A.N;
-    const int64_t f = ((tj * TILE - 1 + fl) % A.N + A.N) % A.N;
-    if (!fast_ok(A, e, f)) any = 1;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) flag[t] = (uint8_t)any;
-}
-
-// Tiles whose element pairs all take the FP32 path: the reduced sums of
-// pair_fast_f accumulated per node pair in shared memory (FP32, four
-// conflict-free phases), then scaled by their FP64 factors, combined (N) and
-// written as split-bf16 planes.
-// float-float helpers for the epilogue of k_assemble_fast
+// float-float helpers for the epilogue of k_assemble_far
 struct ff2 {
   ff r, i;
 };
-__device__ __forceinline__ ff ff_of(double x) {
-  const float h = (float)x;
-  return ff{h, (float)(x - (double)h)};
-}
 __device__ __forceinline__ ff2 ff2_of(zd z) { return ff2{ff_of(z.x), ff_of(z.y)}; }
-__device__ __forceinline__ ff ff_mul_f(ff a, float b) {
-  const ff p = ff_two_prod(a.hi, b);
-  return ff_quick(p.hi, fmaf(a.lo, b, p.lo));
-}
 // bf16 planes of a float-float value: hi - bf16(hi) is exact in FP32, so the
 // second residual carries the value to ~2^-24 of the first plane's scale
 __device__ __forceinline__ void ff_planes(ff x, uint16_t (&p)[3]) {
@@ -755,27 +467,42 @@ __device__ __forceinline__ void split_store_ff2(ff re, ff im, int planes, uint16
   for (int q = 0; q < planes; ++q) *(uint32_t*)(P[q] + off) = (uint32_t)a[q] | ((uint32_t)b[q] << 16);
 }
 
-__global__ void __launch_bounds__(ASM_THREADS) k_assemble_fast(AsmArgs A, int64_t nt, const uint8_t* flag) {
+// Tiles whose element pairs all take the FP32 route of farpair.cuh; a tile with
+// a nearer pair is put on the list of k_assemble_near instead.  One thread per
+// element pair, the pair's values added into float-float sums per node pair in
+// shared memory in four conflict-free phases, then multiplied by their FP64
+// factors (as float-float) and written as split-bf16 planes in both layouts.
+template <int Q>
+__global__ void __launch_bounds__(ASM_THREADS, FAR_CTAS) k_assemble_far(AsmArgs A, int64_t nt) {
+  extern __shared__ float4 facc[];   // [4][TILE][TILE] (re hi, re lo, im hi, im lo)
   const int64_t ti = blockIdx.y, tj = blockIdx.x;
-  if (flag[ti * nt + tj]) return;
-  __shared__ cf acc[5 * TILE * TILE];
   const int64_t N = A.N;
   const int64_t i0 = ti * TILE, j0 = tj * TILE;
-  for (int t = threadIdx.x; t < 5 * TILE * TILE; t += blockDim.x) acc[t] = {0.f, 0.f};
-  __syncthreads();
   const int span = TILE + 1;
   const int npairs = span * span;
+  int near = 0;
+  for (int u = threadIdx.x; u < npairs; u += blockDim.x) {
+    const int el = u / span, fl = u - (u / span) * span;
+    const int64_t e = ((i0 - 1 + el) % N + N) % N, f = ((j0 - 1 + fl) % N + N) % N;
+    if (!pair_is_far(A, e, f)) near = 1;
+  }
+  for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) facc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (__syncthreads_or(near)) {
+    if (threadIdx.x == 0) A.tile_list[1 + atomicAdd(A.tile_list, 1)] = (int)(ti * nt + tj);
+    return;
+  }
   for (int base = 0; base < npairs; base += blockDim.x) {
     const int idx = base + threadIdx.x;
     const int el = idx / span, fl = idx - (idx / span) * span;
     const bool valid = idx < npairs;
     const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N));
     const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
-    PairOutF o;
+    FarPair o;
     if (rowok && colok) {
       const int64_t e = ((i0 - 1 + el) % N + N) % N;
       const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-      pair_fast_f(A, e, f, o);
+      const int q = Q ? Q : A.q_far;
+      far_pair<Q>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
     }
 #pragma unroll
     for (int ph = 0; ph < 4; ++ph) {
@@ -784,116 +511,87 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble_fast(AsmArgs A, int64_
         const int li = el - 1 + a, lj = fl - 1 + b;
         if (li >= 0 && li < TILE && lj >= 0 && lj < TILE && i0 + li < N && j0 + lj < N) {
 #pragma unroll
-          for (int op = 0; op < 5; ++op) cadd(acc[(op * TILE + li) * TILE + lj], o.v[op][ph]);
+          for (int op = 0; op < 4; ++op) {
+            const ffc v = o.value(op, ph);
+            float4 s = facc[(op * TILE + li) * TILE + lj];
+            const ff x = ff_two_sum(s.x, v.x.hi), y = ff_two_sum(s.z, v.y.hi);
+            s.x = x.hi;
+            s.y += x.lo + v.x.lo;
+            s.z = y.hi;
+            s.w += y.lo + v.y.lo;
+            facc[(op * TILE + li) * TILE + lj] = s;
+          }
         }
       }
       __syncthreads();
     }
   }
-  // Entries: the FP64 run factors times the FP32 tile sums, in float-float
-  // on the FP32 pipe (the factors as hi + lo; products by TwoProd), split
-  // into bf16 planes from the float-float value.  The result carries ~44
-  // bits, far beyond the 24 of the FP32 sums, without touching the FP64
-  // pipe (64 times slower), which the FP64 form of this epilogue saturated.
-  const ff2 fS = ff2_of(A.fS), fD = ff2_of(A.fD), fDt = ff2_of(A.fDt), fN = ff2_of(A.fN);
-  const ff kk = ff_of(A.kk2h2);
-  auto entry = [&](int op, int t, ff& re, ff& im) {
-    if (op == 3) {
-      // N = fN (Nd - k^2 h^2 Nb)
-      const cf nb = acc[3 * TILE * TILE + t], nd = acc[4 * TILE * TILE + t];
-      const ff dr = ff_add(ff{nd.x, 0.f}, ff_neg(ff_mul_f(kk, nb.x)));
-      const ff di = ff_add(ff{nd.y, 0.f}, ff_neg(ff_mul_f(kk, nb.y)));
-      re = ff_add(ff_mul(fN.r, dr), ff_neg(ff_mul(fN.i, di)));
-      im = ff_add(ff_mul(fN.r, di), ff_mul(fN.i, dr));
-      return;
-    }
-    const ff2& f = (op == 0) ? fS : (op == 1) ? fD : fDt;
-    const cf a = acc[op * TILE * TILE + t];
-    re = ff_add(ff_mul_f(f.r, a.x), ff_neg(ff_mul_f(f.i, a.y)));
-    im = ff_add(ff_mul_f(f.r, a.y), ff_mul_f(f.i, a.x));
-  };
-  // layout 0: rows i (consecutive threads along j); layout 1: rows j
+  // entries: the FP64 run factors times the tile sums, in float-float on the
+  // FP32 pipe (~44 bits; the FP64 pipe is 64 times slower)
+  const ff2 fac[4] = {ff2_of(A.fS), ff2_of(A.fD), ff2_of(A.fDt), ff2_of(A.fN)};
   for (int lay = 0; lay < 2; ++lay) {
-    for (int u = threadIdx.x; u < 4 * TILE * TILE; u += blockDim.x) {
-      const int op = u / (TILE * TILE), rem = u - op * TILE * TILE;
-      const int a = rem / TILE, b = rem - (rem / TILE) * TILE;
-      const int li = lay ? b : a, lj = lay ? a : b;
-      if (i0 + li < N && j0 + lj < N) {
-        ff re, im;
-        entry(op, li * TILE + lj, re, im);
-        const int64_t off = lay ? (j0 + lj) * A.ldp + 2 * (i0 + li) : (i0 + li) * A.ldp + 2 * (j0 + lj);
-        split_store_ff2(re, im, A.planes, A.P[op][lay], off);
+#pragma unroll
+    for (int op = 0; op < 4; ++op) {
+      for (int u = threadIdx.x; u < TILE * TILE; u += blockDim.x) {
+        const int x = u / TILE, y = u - (u / TILE) * TILE;
+        const int li = lay ? y : x, lj = lay ? x : y;
+        if (i0 + li < N && j0 + lj < N) {
+          const float4 s = facc[(op * TILE + li) * TILE + lj];
+          const ff ar = ff_quick(s.x, s.y), ai = ff_quick(s.z, s.w);
+          const ff re = ff_add(ff_mul(fac[op].r, ar), ff_neg(ff_mul(fac[op].i, ai)));
+          const ff im = ff_add(ff_mul(fac[op].r, ai), ff_mul(fac[op].i, ar));
+          const int64_t off = lay ? (j0 + lj) * A.ldp + 2 * (i0 + li) : (i0 + li) * A.ldp + 2 * (j0 + lj);
+          split_store_ff2(re, im, A.planes, A.P[op][lay], off);
+        }
       }
     }
   }
 }
 
 int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t* fp64_tiles, int64_t* tiles) {
-  if (upload_rules(A) || upload_hankel_coefficients()) { set_error("uploading quadrature rules failed"); return 3; }
-  const size_t smem = sizeof(zd) * 4 * TILE * TILE;
-  cudaFuncSetAttribute(k_assemble<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
+  const size_t smem = sizeof(zd) * 4 * TILE * TILE;   // float-float and FP64 sums take the same room
+  cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_assemble_far<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_assemble_far<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t nt = (A.N + TILE - 1) / TILE;
-  uint8_t* flag = nullptr;
-  if (cudaMalloc(&flag, nt * nt) != cudaSuccess) { set_error("oom (tile flags)"); return 4; }
-  k_tile_flags<<<(unsigned)(nt * nt), 256, 0, s>>>(A, nt, flag);
-  note_launch();
+  cudaMemsetAsync(A.tile_list, 0, sizeof(int), s);
   dim3 grid((unsigned)nt, (unsigned)nt);
-  k_assemble_fast<<<grid, ASM_THREADS, 0, s>>>(A, nt, flag);
+  if (A.q_far == 4) k_assemble_far<4><<<grid, ASM_THREADS, smem, s>>>(A, nt);
+  else k_assemble_far<0><<<grid, ASM_THREADS, smem, s>>>(A, nt);
   note_launch();
   if (mid) { cudaEventRecord(mid[0], s); cudaEventRecord(mid[1], s); }
-  AsmArgs B = A;
-  B.tile_flags = flag;
-  k_assemble<1><<<grid, ASM_THREADS, smem, s>>>(B);
+  k_assemble_near<<<(unsigned)std::min<int64_t>(nt * nt, 152 * 3), ASM_THREADS, smem, s>>>(A, nt);
   note_launch();
   if (fp64_tiles) {   // the tiles that took the FP64 kernel (for the work count of each kernel)
-    std::vector<uint8_t> h((size_t)(nt * nt));
-    cudaMemcpyAsync(h.data(), flag, h.size(), cudaMemcpyDeviceToHost, s);
+    int n = 0;
+    cudaMemcpyAsync(&n, A.tile_list, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
-    int64_t n = 0;
-    for (uint8_t v : h) n += v;
     *fp64_tiles = n;
     *tiles = nt * nt;
   }
-  cudaStreamSynchronize(s);
-  cudaFree(flag);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("assemble (planes): ") + cudaGetErrorString(err)); return 3; }
   return 0;
 }
 
-__global__ void k_far_offsets(Points far, const double* cx, const double* cy, int64_t N, int q, float* ox,
-                              float* oy, float* nxf, float* nyf, float* nxl, float* nyl, float* oxl, float* oyl) {
+__global__ void k_far_tables(Points far, Points cen, int64_t N, int q, double h, FarElem* fe, FarPoint* fp) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * q) return;
   const int64_t e = t / q;
-  const double dxo = far.x[t] - cx[e], dyo = far.y[t] - cy[e];
-  ox[t] = (float)dxo;
-  oy[t] = (float)dyo;
-  oxl[t] = (float)(dxo - (double)ox[t]);   // float-float tails of the offsets
-  oyl[t] = (float)(dyo - (double)oy[t]);
-  nxf[t] = (float)far.nx[t];
-  nyf[t] = (float)far.ny[t];
-  nxl[t] = (float)(far.nx[t] - (double)nxf[t]);   // float-float tails of the normals
-  nyl[t] = (float)(far.ny[t] - (double)nyf[t]);
+  const int p = (int)(t - e * q);
+  fp[t] = far_point(cen.x[e], cen.y[e], cen.nx[e], cen.ny[e], far.x[t], far.y[t], far.nx[t], far.ny[t], h,
+                    c_xf[p] - 0.5);
+  if (p == 0) fe[e] = far_elem(cen.x[e], cen.y[e], cen.nx[e], cen.ny[e]);
 }
 
-__global__ void k_centres_ff(const double* cx, const double* cy, int64_t N, float4* cff) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= N) return;
-  const float xh = (float)cx[e], yh = (float)cy[e];
-  cff[e] = make_float4(xh, (float)(cx[e] - (double)xh), yh, (float)(cy[e] - (double)yh));
-}
-
-int far_offsets(const Points& far, const double* cx, const double* cy, int64_t N, int q, float* ox,
-                float* oy, float* nxf, float* nyf, float* nxl, float* nyl, float* oxl, float* oyl, float4* cff,
-                cudaStream_t s) {
-  k_far_offsets<<<(unsigned)((N * q + 255) / 256), 256, 0, s>>>(far, cx, cy, N, q, ox, oy, nxf, nyf, nxl, nyl,
-                                                                oxl, oyl);
-  note_launch();
-  k_centres_ff<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(cx, cy, N, cff);
+int far_tables(const AsmArgs& A, const Points& cen, FarElem* fe, FarPoint* fp, cudaStream_t s) {
+  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
+  const int64_t n = A.N * A.q_far;
+  k_far_tables<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(A.far, cen, A.N, A.q_far, A.h, fe, fp);
   note_launch();
   cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) { set_error(std::string("far offsets: ") + cudaGetErrorString(err)); return 3; }
+  if (err != cudaSuccess) { set_error(std::string("far tables: ") + cudaGetErrorString(err)); return 3; }
   return 0;
 }
 

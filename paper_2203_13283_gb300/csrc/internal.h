@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "farpair.cuh"
 
 namespace wcs {
 
@@ -81,20 +82,6 @@ void gauss_legendre01(int n, double* x, double* w);
 void build_quad_tables(QuadTables& q);
 
 // ---------------------------------------------------------------- assembly
-// FP32 constants of the far-pair path, formed once on the host
-struct FastConsts {
-  float kf = 0.f, beta = 0.f;      // k, Im k~
-  float ck[2] = {0.f, 0.f};        // sqrt(2 / (pi k~))
-  float ik[2] = {0.f, 0.f};        // i / k~
-  float kt4[2] = {0.f, 0.f};       // i k~ / 4
-  float ampk = 0.f;                // sqrt(2 / (pi k))
-  float kk2h2 = 0.f, h2 = 0.f;     // k^2 h^2, h^2
-  float beta_lo = 0.f;             // Im k~ - beta (float-float tail)
-  float zfast2 = 0.f;              // zfast^2 (pair test k^2 |c_e - c_f|^2 >= zfast^2)
-  float k_hi = 0.f, k_lo = 0.f;    // k as a float-float pair
-  float twopi[3] = {0.f, 0.f, 0.f};   // 2 pi = twopi[0] + twopi[1] + twopi[2]
-};
-
 struct AsmArgs {
   int64_t N;
   double h, k;
@@ -107,42 +94,32 @@ struct AsmArgs {
   const double* wlog;              // 3 * q_near^2 product weights (device)
   zd *S, *D, *Dt, *Nk;             // outputs
   int64_t ld;                      // row-major leading dimension
-  // mixed-precision form: far pairs with k R >= zfast are integrated in FP32
-  // around the FP64 element-centre distance; output written as split-bf16
-  // planes [op][layout][plane] (layout 0: X, layout 1: X^T; each row-major
+  // mixed-precision form: far pairs on the FP32 pipe (farpair.cuh); output
+  // written as split-bf16 planes [op][layout][plane] (layout 0: X, layout 1: X^T; each row-major
   // complex as real N x 2N, leading dimension ldp).
-  int mixed = 0;
   int planes = 0;
   uint16_t* P[4][2][3];
   int64_t ldp = 0;
-  const double *cx = nullptr, *cy = nullptr;     // element centres (xi = 1/2)
-  const float *ox = nullptr, *oy = nullptr;      // far points minus their element centre
-  const float *nxf = nullptr, *nyf = nullptr;    // far-point normals (FP32)
-  const float *nxl = nullptr, *nyl = nullptr;    // their float-float tails
-  const float *oxl = nullptr, *oyl = nullptr;    // float-float tails of the offsets
-  // FP64 factors of the FP32 far-pair path, applied once per stored entry (a
+  const FarElem* fe = nullptr;     // element centres and tangents, far points relative to them
+  const FarPoint* fp = nullptr;
+  FarConsts fc;
+  // FP64 factors of the far pairs' float-float sums, applied once per stored entry (a
   // constant rounded to FP32 would bias every far entry of an operator alike)
-  zd fS, fD, fDt, fN;              // S~, D, D~, N (see pair_fast_f)
-  double kk2h2 = 0.0;              // k^2 h^2 of the Maue form
-  const float4* cff = nullptr;                   // element centres as float-float (x hi, x lo, y hi, y lo)
-  double zfast = 1e300;
-  FastConsts fk;
-  const uint8_t* tile_flags = nullptr;           // mixed tile kernel: only flagged tiles
+  zd fS, fD, fDt, fN;              // S~, D, D~, N (see FarPair)
+  int* tile_list = nullptr;        // count, then the tiles that hold a pair nearer than the far route (1 + tiles)
 };
 // Fill kp.asym for kp.t and the term-count thresholds kp.xth for relative
 // tolerance tol (host).
 void fill_asymptotic(KtPair& kp, double tol);
 int assemble_dense(const AsmArgs& a, cudaStream_t s);
 // Mixed form: the same operators written as split-bf16 planes (see AsmArgs):
-// the FP32 far-pair kernel over the tiles it can take, then the FP64 kernel
+// the far-pair kernel over the tiles it can take, then the FP64 kernel
 // over the rest.  mid (optional, two events) is recorded between the two;
 // fp64_tiles and tiles (optional) receive the tile counts.
 int assemble_planes(const AsmArgs& a, cudaStream_t s, cudaEvent_t* mid = nullptr, int64_t* fp64_tiles = nullptr,
                     int64_t* tiles = nullptr);
-// FP32 offset tables of the far points relative to element centres.
-int far_offsets(const Points& far, const double* cx, const double* cy, int64_t N, int q, float* ox,
-                float* oy, float* nxf, float* nyf, float* nxl, float* nyl, float* oxl, float* oyl, float4* cff,
-                cudaStream_t s);
+// Tables of the far route: N elements, N q_far points (cen: element centres, xi = 1/2).
+int far_tables(const AsmArgs& a, const Points& cen, FarElem* fe, FarPoint* fp, cudaStream_t s);
 // First row of the four circulant operators on the circle (row 0, N entries each).
 int assemble_circle_row(const AsmArgs& a, cudaStream_t s);
 // Sampled entries (row, col) of the four operators, computed point-wise.

@@ -88,7 +88,8 @@ struct wcs_ctx {
   int planes = 2, rhs_planes = 2;
   int64_t ldp = 0;                        // plane leading dimension (bf16 elements)
   DevBuf opplanes;                        // [op][layout][plane] N x ldp bf16
-  DevBuf centres, offs;                   // element centres (FP64), far offsets (FP32)
+  DevBuf centres, offs;                   // element centres (FP64), tables of the far route
+  DevBuf tiles;                           // list of the tiles assembled in FP64
   DevBuf stage0, stage1, stage2;          // staged right-hand blocks (bf16 planes)
   int64_t stage_cols = 0;
   DevBuf tcerr;
@@ -827,7 +828,7 @@ static void free_mesh(wcs_ctx* c) {
   cudaFree(c->arc_c.cum); c->arc_c.cum = nullptr;
   c->pts_far.release(); c->pts_near.release(); c->pts_far_c.release(); c->pts_near_c.release();
   c->ops.release(); c->mu.release();
-  c->opplanes.release(); c->centres.release(); c->offs.release();
+  c->opplanes.release(); c->centres.release(); c->offs.release(); c->tiles.release();
   c->stage0.release(); c->stage1.release(); c->stage2.release(); c->stage_cols = 0;
   c->gA.release(); c->gB.release(); c->gW.release(); c->qh.release(); c->qt.release();
   c->U.release(); c->Vw.release(); c->Wt.release(); c->Kinv.release(); c->Wa.release();
@@ -1004,38 +1005,25 @@ static AsmArgs asm_args(wcs_ctx* c, bool circle) {
   return A;
 }
 
-// FP32 constants of the mixed form's far-pair path (after A.zfast is set)
-static void set_fast_consts(AsmArgs& A) {
-  const std::complex<double> kt(A.kt.x, A.kt.y);
-  const std::complex<double> ck = std::sqrt((2.0 / WCS_PI) / kt), ik = std::complex<double>(0.0, 1.0) / kt;
-  const std::complex<double> kt4 = std::complex<double>(0.0, 0.25) * kt;
-  FastConsts& F = A.fk;
-  F.kf = (float)A.k;
-  F.beta = (float)A.kt.y;
-  F.beta_lo = (float)(A.kt.y - (double)F.beta);
-  F.ck[0] = (float)ck.real(); F.ck[1] = (float)ck.imag();
-  F.ik[0] = (float)ik.real(); F.ik[1] = (float)ik.imag();
-  F.kt4[0] = (float)kt4.real(); F.kt4[1] = (float)kt4.imag();
-  F.ampk = (float)std::sqrt(2.0 / (WCS_PI * A.k));
-  F.kk2h2 = (float)(A.k * A.k * A.h * A.h);
-  F.h2 = (float)(A.h * A.h);
-  F.zfast2 = (A.zfast < 1e18) ? (float)(A.zfast * A.zfast) : INFINITY;
-  F.k_hi = (float)A.k;
-  F.k_lo = (float)(A.k - (double)F.k_hi);
-  // FP64 factors of the reduced FP32 sums (see pair_fast_f)
-  const std::complex<double> I4(0.0, 0.25);
+// Constants of the mixed form's far-pair route.  Pairs take it from k R0 = 20 on
+// (where its Hankel series holds) when k h <= 0.9: entries then carry ~5e-9, as
+// the FP64 quadrature's do after their split into bf16 planes (2.6e-9).  On
+// coarser meshes its corrections are larger (5e-8 at k h = 2.5) and it only
+// takes the pairs beyond zfast.  zfast <= 0: every pair in FP64.
+static void set_far_consts(wcs_ctx* c, AsmArgs& A) {
+  const double kh = A.k * A.h;
+  double xmin = 1e300;
+  if (c->opt.zfast > 0.0 && A.kt_pair)
+    xmin = (kh <= 0.9) ? 20.0 + kh : std::max(20.0 + kh, c->opt.zfast + 2.0 * kh);
+  far_consts(A.fc, A.q_far, c->quad.xf, c->quad.wf, A.k, A.kt.y, A.h, xmin);
+  const std::complex<double> kt(A.kt.x, A.kt.y), I4(0.0, 0.25);
+  const std::complex<double> ck = std::sqrt((2.0 / WCS_PI) / kt);
   const double ampk = std::sqrt(2.0 / (WCS_PI * A.k)), h2 = A.h * A.h;
   const std::complex<double> fS = I4 * ck * h2, fD = I4 * ampk * A.k * h2, fDt = I4 * kt * ck * h2, fN = I4 * ampk;
   A.fS = mkz(fS.real(), fS.imag());
   A.fD = mkz(fD.real(), fD.imag());
   A.fDt = mkz(fDt.real(), fDt.imag());
   A.fN = mkz(fN.real(), fN.imag());
-  A.kk2h2 = A.k * A.k * h2;
-  const double tp = 2.0 * WCS_PI;   // 2 pi to ~72 bits: double plus its float-float residual
-  const double tp_lo = 2.4492935982947064e-16;
-  F.twopi[0] = (float)tp;
-  F.twopi[1] = (float)(tp - (double)F.twopi[0]);
-  F.twopi[2] = (float)((tp - (double)F.twopi[0] - (double)F.twopi[1]) + tp_lo);
 }
 
 __global__ void k_geom_sample_dummy() {}
@@ -1082,7 +1070,7 @@ int wcs_assemble(wcs_ctx* c) {
     c->ldp = ((2 * N + 63) / 64) * 64;
     TRY(c->opplanes.ensure(sizeof(uint16_t) * (size_t)8 * c->planes * N * c->ldp));
     if (c->ldp != 2 * N) cudaMemsetAsync(c->opplanes.p, 0, c->opplanes.bytes, c->s);   // zero the padding columns
-    // element centres (xi = 1/2) and FP32 offsets of the far points
+    // element centres (xi = 1/2) and the far points relative to them
     const int qf = c->opt.q_far;
     TRY(c->centres.ensure(sizeof(double) * 6 * N));
     double* half = c->centres.d() + 5 * N;
@@ -1091,27 +1079,22 @@ int wcs_assemble(wcs_ctx* c) {
     Points cp;
     cp.x = c->centres.d(); cp.y = cp.x + N; cp.nx = cp.y + N; cp.ny = cp.nx + N; cp.kappa = nullptr; cp.n = N;
     TRY(points_build(c->contour, c->arc, N, c->h, half, 1, cp, c->s));
-    const int64_t cff_off = ((8 * N * qf + 3) / 4) * 4;   // floats; float4 table 16-byte aligned
-    TRY(c->offs.ensure(sizeof(float) * cff_off + sizeof(float4) * N));
-    float* of = (float*)c->offs.p;
-    float4* cff = (float4*)(of + cff_off);
-    TRY(far_offsets(c->far, cp.x, cp.y, N, qf, of, of + N * qf, of + 2 * N * qf, of + 3 * N * qf, of + 4 * N * qf,
-                    of + 5 * N * qf, of + 6 * N * qf, of + 7 * N * qf, cff, c->s));
+    TRY(c->offs.ensure(sizeof(FarElem) * N + sizeof(FarPoint) * N * qf));
+    FarElem* fe = (FarElem*)c->offs.p;
+    FarPoint* fp = (FarPoint*)(fe + N);
     AsmArgs A = asm_args(c, false);
-    A.mixed = 1;
+    TRY(far_tables(A, cp, fe, fp, c->s));
     A.planes = c->planes;
     A.ldp = c->ldp;
     for (int op = 0; op < 4; ++op)
       for (int l = 0; l < 2; ++l)
         for (int p = 0; p < 3; ++p) A.P[op][l][p] = (p < c->planes) ? plane_ptr(c, op, l, p) : nullptr;
-    A.cx = cp.x; A.cy = cp.y;
-    A.ox = of; A.oy = of + N * qf; A.nxf = of + 2 * N * qf; A.nyf = of + 3 * N * qf;
-    A.nxl = of + 4 * N * qf; A.nyl = of + 5 * N * qf;
-    A.oxl = of + 6 * N * qf; A.oyl = of + 7 * N * qf;
-    A.cff = cff;
-    // zfast <= 0: every pair in FP64 (the FP32 path is off)
-    A.zfast = (c->opt.zfast > 0.0) ? c->opt.zfast + 2.0 * c->k * c->h : 1e300;
-    set_fast_consts(A);
+    A.fe = fe;
+    A.fp = fp;
+    const int64_t nt = (N + 31) / 32;
+    TRY(c->tiles.ensure(sizeof(int) * (1 + nt * nt)));
+    A.tile_list = (int*)c->tiles.p;
+    set_far_consts(c, A);
     if (!c->profile) {
       TRY(assemble_planes(A, c->s));
     } else {
