@@ -190,7 +190,7 @@ struct ZView {
 // C (m x n, column-major ldc) = alpha * A (m x k) * B (k x n) + beta * C.
 int zgemm(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
           cudaStream_t s);
-// The same with every entry summed over k in order (products whose difference is taken).
+// The same with every entry summed over k in order, whatever the shape.
 int zgemm_ordered(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
                   cudaStream_t s);
 // Y = G^{-1} X for the cyclic Gram matrix of hats (h/6 [1 4 1]), column-major; may alias.

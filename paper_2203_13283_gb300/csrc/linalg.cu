@@ -226,43 +226,54 @@ static bool zgemm_small(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZVie
   return true;
 }
 
-// One thread per output, K in order: the summation order of k_zgemm, for
-// products whose difference is taken afterwards (central differences of the
-// far-field map), where the roundings of both have to be alike.  Bound by the
-// chain of 2 K dependent FP64 FMAs (45 x 8 x 1024: 1.17 ms in k_zgemm's two
-// CTAs of staged tiles).
+// K in order, for up to eight columns: a half-warp's 16 lanes form the real and
+// the other 16 the imaginary parts of 16 rows of one column, with the operations
+// of zfma in k_zgemm's order (the same bits).  Bound by the FP64 pipe, whose
+// quarter of an SM issues one warp instruction in 64 clocks: 2 K of them a warp.
 __global__ void __launch_bounds__(128) k_zgemm_serial(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B,
                                                       zd beta, zd* __restrict__ C, int64_t ldc) {
-  const int64_t i = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31), j = (int64_t)blockIdx.y * 4 + (threadIdx.x >> 5);
-  if (i >= m || j >= n) return;
-  const zd* a = A.p + i * A.rs;
+  const int lane = threadIdx.x & 31, half = lane >> 4;
+  const int64_t i = (int64_t)blockIdx.x * 16 + (lane & 15), j = (int64_t)blockIdx.y * 4 + (threadIdx.x >> 5);
+  if (j >= n) return;
+  const zd* a = A.p + min(i, m - 1) * A.rs;
   const zd* b = B.p + j * B.cs;
-  zd acc = mkz(0.0);
+  double acc = 0.0;
 #pragma unroll 8
   for (int64_t t = 0; t < k; ++t) {
     zd v = a[t * A.cs], w = b[t * B.rs];
     if (A.conj) v.y = -v.y;
     if (B.conj) w.y = -w.y;
-    zfma(acc, v, w);
+    // re: fma(a.x, b.x, fma(-a.y, b.y, re)); im: fma(a.x, b.y, fma(a.y, b.x, im))
+    acc = fma(v.x, half ? w.y : w.x, fma(half ? v.y : -v.y, half ? w.x : w.y, acc));
   }
-  zd r = alpha * acc;
+  const double im = __shfl_down_sync(0xffffffffu, acc, 16);
+  if (half || i >= m) return;
+  zd r = alpha * mkz(acc, im);
   zd* o = C + j * ldc + i;
   if (!(beta.x == 0.0 && beta.y == 0.0)) r += beta * (*o);
   *o = r;
 }
 
+// Every tile shape sums an entry over k in the same order, so the tile follows
+// the shape: the largest that still gives two CTAs per SM (N = 1024, 32
+// columns: 16 CTAs of 64 x 64 tiles took 1.2 ms, 128 of 16 x 16 take 0.2).
 int zgemm_ordered(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
                   cudaStream_t s) {
   if (m <= 0 || n <= 0) return 0;
-  // enough outputs for the staged tiles to fill the GPU: they load A and B once
-  if (m * n > 65536) {
-    const int r = launch_zgemm<16, 16, 4, 4>(m, n, k, alpha, A, B, beta, C, ldc, s);
-    if (r) return r;
-  } else {
-    dim3 g((unsigned)((m + 31) / 32), (unsigned)((n + 3) / 4));
+  int r = 0;
+  auto tiles = [&](int64_t t) { return ((m + t - 1) / t) * ((n + t - 1) / t); };
+  if (n <= 8) {
+    dim3 g((unsigned)((m + 15) / 16), (unsigned)((n + 3) / 4));
     k_zgemm_serial<<<g, 128, 0, s>>>(m, n, k, alpha, A, B, beta, C, ldc);
     note_launch();
+  } else if (tiles(64) >= 304 || m > 65535 * 32) {
+    r = launch_zgemm<16, 16, 4, 4>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 64 x 64
+  } else if (tiles(32) >= 304 || m > 65535 * 16) {
+    r = launch_zgemm<16, 16, 2, 2>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 32 x 32
+  } else {
+    r = launch_zgemm<16, 16, 1, 1>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 16 x 16
   }
+  if (r) return r;
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(err)); return 3; }
   return 0;
@@ -271,13 +282,7 @@ int zgemm_ordered(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, z
 int zgemm(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc,
           cudaStream_t s) {
   if (m <= 0 || n <= 0) return 0;
-  int r = 0;
-  if (!zgemm_small(m, n, k, alpha, A, B, beta, C, ldc, s)) {
-    if (n <= 16) r = launch_zgemm<16, 16, 4, 1>(m, n, k, alpha, A, B, beta, C, ldc, s);        // 64 x 16 tiles
-    else if (n <= 32) r = launch_zgemm<16, 16, 4, 2>(m, n, k, alpha, A, B, beta, C, ldc, s);   // 64 x 32
-    else r = launch_zgemm<16, 16, 4, 4>(m, n, k, alpha, A, B, beta, C, ldc, s);                // 64 x 64
-  }
-  if (r) return r;
+  if (!zgemm_small(m, n, k, alpha, A, B, beta, C, ldc, s)) return zgemm_ordered(m, n, k, alpha, A, B, beta, C, ldc, s);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(err)); return 3; }
   return 0;

@@ -84,6 +84,7 @@ struct wcs_ctx {
   DevBuf gwork;                           // work of the Gram inverse (N x cols)
   DevBuf fx;                              // fixed-point slices and partials of the FP64 products (zgemm_fx)
   // mixed-precision form
+  bool ordered = false;                   // FP64 products sum over k in order (see OrderedScope)
   bool mixed = false;
   int planes = 2, rhs_planes = 2;
   int64_t ldp = 0;                        // plane leading dimension (bf16 elements)
@@ -180,10 +181,24 @@ static int ensure_tcerr(wcs_ctx* c) {
   return 0;
 }
 
+// While it lives, the context's FP64 products sum every entry over k in order
+// (zgemm_ordered) instead of taking the fastest route for their shape.  The
+// shape gradient differences quantities formed from the solution (step delta,
+// 1e-6 by default), which amplifies their roundings by 1 / delta: another
+// summation order moves its results by 1e-10 to 1e-8.  So it and what it builds
+// on, the skeleton and the factors, keep one order on every shape.
+struct OrderedScope {
+  wcs_ctx* c;
+  bool was;
+  explicit OrderedScope(wcs_ctx* c_) : c(c_), was(c_->ordered) { c->ordered = true; }
+  ~OrderedScope() { c->ordered = was; }
+};
+
 // Complex FP64 product C = alpha A B + beta C: on the tensor cores through
 // fixed-point slices where the shape is worth it, else (or when their
 // workspace does not fit the device) on the FP64 pipe.
 static int cz(wcs_ctx* c, int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc) {
+  if (c->ordered) return zgemm_ordered(m, n, k, alpha, A, B, beta, C, ldc, c->s);
   if (zgemm_fx_wanted(m, n, k) && !ensure_tcerr(c)) {
     if (!c->fx.ensure(zgemm_fx_bytes(m, n, k)))
       return zgemm_fx(m, n, k, alpha, A, B, beta, C, ldc, c->fx.p, (int*)c->tcerr.p, c->s);
@@ -1255,6 +1270,7 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   if (c->stage < ST_ASSEMBLED) { set_error("assemble first"); return WCS_ERR_STATE; }
   if (!(tol >= 0)) { set_error("tolerance must be >= 0"); return WCS_ERR_ARG; }
   const int64_t N = c->N;
+  OrderedScope ordered(c);
   const int64_t cap = (max_rank <= 0 || max_rank > N) ? N : max_rank;
   const int b = c->opt.block;
   ProfScope whole(c, CAT_SKELETON, 0.0, 0.0);
@@ -1433,6 +1449,7 @@ int wcs_factor(wcs_ctx* c) {
   if (!c) { set_error("null context"); return WCS_ERR_ARG; }
   if (c->stage < ST_SKELETON) { set_error("skeleton first"); return WCS_ERR_STATE; }
   const int64_t N = c->N, r = c->rank;
+  OrderedScope ordered(c);
   c->kinv_res = -1.0;
   ProfScope whole(c, CAT_FACTOR, 8.0 / 3.0 * r * (double)r * r, 0.0);
   if (r > 0) {
@@ -2278,6 +2295,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
   TRY(check_angles(nphi, phi, "shape_gradient (observation angles)"));
   if (!(delta > 0)) delta = 1e-6;
   const int64_t N = c->N;
+  OrderedScope ordered(c);
   DevBuf j, lam, E, F, G, ang, phd, dots;
   TRY(j.ensure(sizeof(zd) * N * B));
   TRY(lam.ensure(sizeof(zd) * N * B));
@@ -2372,8 +2390,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
       wcs_ctx* t = sgn == 0 ? tp.t : tm.t;
       TRY(farfield_matrix(t->near, t->quad.wn, t->quad.xn, t->opt.q_near, N, t->h, t->k, phd.d(), nphi, E.z(),
                           nphi, c->s));
-      TRY(zgemm_ordered(nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), Wf.z(), nphi,
-                        c->s));
+      TRY(cz(c, nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), Wf.z(), nphi));
       TRY(column_dotc(F.z(), nphi, Wf.z(), nphi, nphi, B, dots.z(), c->s));
       cudaMemcpyAsync(hd.data(), dots.p, sizeof(zd) * B, cudaMemcpyDeviceToHost, c->s);
       TRY(sync(c));
@@ -2413,6 +2430,7 @@ int wcs_shape_operator_forms(wcs_ctx* c, int op, int64_t B, const double* u_dev,
   }
   if (!(delta > 0)) delta = 1e-6;
   const int64_t N = c->N;
+  OrderedScope ordered(c);
   DevBuf Wb;
   TRY(Wb.ensure(sizeof(zd) * 4 * N * N));
   cudaMemsetAsync(Wb.p, 0, Wb.bytes, c->s);
