@@ -25,12 +25,14 @@
 
 #include "farpair.cuh"
 #include "hankel.cuh"
+#include "hankeltab.cuh"
 #include "internal.h"
 #include "split.cuh"
 
 namespace wcs {
 
 __constant__ double c_xf[16], c_wf[16], c_xn[16], c_wn[16];
+static int upload_rules(const AsmArgs& A);
 
 struct PairOut {
   zd v[4][4];  // [operator S~, D, D~, N][a * 2 + b]
@@ -246,6 +248,302 @@ __device__ __forceinline__ bool pair_is_far(const AsmArgs& A, int64_t e, int64_t
   return periodic_dist(e, f, A.N) > A.near_band && far_ok(A.fc, A.fe[e].c, A.fe[f].c);
 }
 
+// ----------------------------------------------------------------------------- tables (hankeltab.cuh)
+void hankel_tab_args(double t, HankelTabArgs& a) {
+  typedef std::complex<double> cd;
+  a.t = t;
+  const cd c[2] = {cd(1.0, 0.0), cd(1.0, t)};
+  for (int w = 0; w < 2; ++w) {
+    cd a0 = 1.0, a1 = 0.5 * c[w];   // (-c^2 / 4)^m / m!^2, (c / 2) (-c^2 / 4)^m / (m! (m + 1)!)
+    double H = 0.0;
+    for (int m = 0; m < HT_M; ++m) {
+      if (m > 0) {
+        a0 *= -0.25 * c[w] * c[w] / ((double)m * m);
+        a1 *= -0.25 * c[w] * c[w] / ((double)m * (m + 1));
+        H += 1.0 / m;
+      }
+      const cd v[4] = {a0, a1, -H * a0, (2.0 * H + 1.0 / (m + 1) - 2.0 * WCS_EULER_GAMMA) * a1};
+      for (int j = 0; j < 4; ++j) {
+        if (w == 0) a.series[m * 12 + j] = v[j].real();
+        else { a.series[m * 12 + 4 + 2 * j] = v[j].real(); a.series[m * 12 + 5 + 2 * j] = v[j].imag(); }
+      }
+    }
+  }
+  const cd lc = std::log(c[1]), ic = 1.0 / c[1];
+  a.tail[0] = lc.real(); a.tail[1] = lc.imag(); a.tail[2] = ic.real(); a.tail[3] = ic.imag();
+  // interpolation at the Chebyshev nodes, as monomials: sum_n (2 - [n = 0]) / D T_n(node_j) T_n(u)
+  double T[HT_D][HT_D] = {};   // T[n][power]
+  T[0][0] = 1.0;
+  T[1][1] = 1.0;
+  for (int n = 2; n < HT_D; ++n)
+    for (int k = 0; k < HT_D; ++k) T[n][k] = (k > 0 ? 2.0 * T[n - 1][k - 1] : 0.0) - T[n - 2][k];
+  for (int j = 0; j < HT_D; ++j) {
+    const double th = WCS_PI * (2 * j + 1) / (2.0 * HT_D);
+    a.node[j] = std::cos(th);
+    for (int k = 0; k < HT_D; ++k) {
+      double v = 0.0;
+      for (int n = 0; n < HT_D; ++n) v += (n == 0 ? 1.0 : 2.0) / HT_D * std::cos(n * th) * T[n][k];
+      a.conv[k * HT_D + j] = v;
+    }
+  }
+}
+
+// J0, J1, Y0, Y1 by the backward recurrence from n = 76 (x < 24), as bessel01_miller_real
+__device__ Bessel01 bessel01_long(double x) {
+  double jp1 = 0.0, j = 1e-30, norm = 0.0, s0 = 0.0, s1 = 0.0, J1 = 0.0;
+  const double iz2 = 2.0 / x;
+  for (int n = 76; n > 0; --n) {
+    if ((n & 1) == 0) {
+      const int k = n >> 1;
+      norm += 2.0 * j;
+      s0 += ((k & 1) ? -c_recip[k] : c_recip[k]) * j;
+    } else {
+      const int kp = (n + 1) >> 1, km = (n - 1) >> 1;
+      s1 += ((kp & 1) ? -c_recip[kp] : c_recip[kp]) * j;
+      if (km >= 1) s1 -= ((km & 1) ? -c_recip[km] : c_recip[km]) * j;
+      if (n == 1) J1 = j;
+    }
+    const double jm = ((double)n * iz2) * j - jp1;
+    jp1 = j;
+    j = jm;
+  }
+  const double inv = 1.0 / (norm + j), lz = log(0.5 * x) + WCS_EULER_GAMMA;
+  Bessel01 b;
+  b.J0 = j * inv;
+  b.J1 = J1 * inv;
+  b.Y0 = (2.0 / WCS_PI) * (lz * b.J0 - 2.0 * (s0 * inv));
+  b.Y1 = (2.0 / WCS_PI) * (lz * b.J1 - b.J0 * (0.5 * iz2) + s1 * inv);
+  return b;
+}
+
+// one block per interval, the last one copies the series
+__global__ void __launch_bounds__(96) k_hankel_table(const __grid_constant__ HankelTabArgs a, double* T) {
+  const int b = blockIdx.x, t = threadIdx.x;
+  if (b == HT_N) {
+    for (int i = t; i < HT_SERIES; i += 96) T[i] = a.series[i];
+    if (t < 4) T[HT_SERIES + t] = a.tail[t];
+    return;
+  }
+  __shared__ double v[HT_D][8];
+  if (t < HT_D) {
+    const double x = HT_X0 + 0.25 + 0.5 * b + 0.25 * a.node[t];
+    const Bessel01 f = bessel01_long(x);
+    const Hankel01 h = bessel01_shift(x, x * a.t, f);
+    v[t][0] = f.J0; v[t][1] = f.Y0; v[t][2] = f.J1; v[t][3] = f.Y1;
+    v[t][4] = h.H0.x; v[t][5] = h.H0.y; v[t][6] = h.H1.x; v[t][7] = h.H1.y;
+  }
+  __syncthreads();
+  const int k = t >> 3, fn = t & 7;
+  double s = 0.0;
+  for (int j = 0; j < HT_D; ++j) s = fma(a.conv[k * HT_D + j], v[j][fn], s);
+  T[HT_SERIES + 4 + ((int64_t)b * HT_D + k) * 8 + fn] = s;
+}
+
+int64_t hankel_table_doubles() { return HT_SIZE; }
+
+int hankel_table(double t, double* T, cudaStream_t s) {
+  HankelTabArgs a;
+  hankel_tab_args(t, a);
+  k_hankel_table<<<HT_N + 1, 96, 0, s>>>(a, T);
+  note_launch();
+  cudaError_t err = cudaGetLastError();
+  if (err != cudaSuccess) { set_error(std::string("hankel table: ") + cudaGetErrorString(err)); return 3; }
+  return 0;
+}
+
+// Near-band element pairs (d <= near_band) of the elements e0 .. e0 + ne - 1
+// (mod N): the 2 x 2 blocks of the four operators, 32 doubles per pair, pair
+// (offset + near_band) * ne + (e - e0).  One warp per pair, the q^2 points over
+// its lanes, so that every lane runs the same branch (a thread per pair left 9 of
+// 33 lanes of a diagonal tile's warps on the heaviest path in the program, 60 ms
+// of FP64 pipe per tile); the 32 sums are joined by a halving exchange that
+// leaves sum l in lane l.  Bound: FP64 pipe, ~300 operations a point.
+__global__ void __launch_bounds__(128) k_near_band(AsmArgs A, int64_t e0, int64_t ne, double* out) {
+  const int64_t N = A.N;
+  const int64_t pair = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, nb = A.near_band;
+  if (pair >= ne * (2 * nb + 1)) return;
+  const int off = (int)(pair / ne) - nb;
+  const int64_t e = (e0 + pair % ne) % N, f = ((e + off) % N + N) % N;
+  const int q = A.q_near;
+  const double h = A.h, k = A.k, kk2h2 = k * k * h * h, lh = log(h);
+  const zd kt = A.kt;
+  const int d = periodic_dist(e, f, N);
+  const int kind = d == 0 ? 0 : (d == 1 ? (((e + 1) % N) == f ? 1 : 2) : -1);
+  double v[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = 0.0;
+  for (int pt = lane; pt < q * q; pt += 32) {
+    const int p = pt / q, r = pt - p * q;
+    const int64_t ip = e * q + p, ir = f * q + r;
+    const double xip = c_xn[p], xir = c_xn[r], w = c_wn[p] * c_wn[r];
+    const double dx = A.near.x[ip] - A.near.x[ir], dy = A.near.y[ip] - A.near.y[ir];
+    const double nxs = A.near.nx[ir], nys = A.near.ny[ir];
+    const double nd = A.near.nx[ip] * nxs + A.near.ny[ip] * nys;
+    zd kS, kD, kDt, kN, aS = mkz(0.0), aD = mkz(0.0), aDt = mkz(0.0), aN = mkz(0.0);
+    double lw = 0.0;
+    if (kind >= 0) lw = A.wlog[kind * q * q + pt] + w * lh;
+    if (kind == 0 && p == r) {
+      // coincident points: limits of B = K - A log|s - s'| at R = 0
+      const double kap = A.near.kappa[ip];
+      kS = mkz(0.0, 0.25) - (1.0 / (2.0 * WCS_PI)) * (zlog(0.5 * kt) + mkz(WCS_EULER_GAMMA));
+      kN = mkz(-(1.0 / (2.0 * WCS_PI)) * (log(0.5 * k) + WCS_EULER_GAMMA), 0.25);
+      kD = mkz(-kap / (4.0 * WCS_PI));
+      kDt = kD;
+      aS = mkz(-1.0 / (2.0 * WCS_PI));
+      aN = aS;
+    } else {
+      const double R2 = dx * dx + dy * dy, ri = rsqrt(R2), R = R2 * ri, gg = (dx * nxs + dy * nys) * ri, x = k * R;
+      Hankel01 Hk, Ht;
+      if (x < HT_X0) {
+        hankel_tab_series(A.htab, x, log(0.5 * x), Hk, Ht);
+      } else if (kind >= 0 || x >= HT_X1) {
+        hankel01_pair(x, A.ktp, Hk, Ht);
+      } else {
+        hankel_tab_poly(A.htab, x, Hk.H0, Hk.H1, Ht.H0, Ht.H1);
+      }
+      kN = i4(Hk.H0);
+      kS = i4(Ht.H0);
+      kD = (k * gg) * i4(Hk.H1);
+      kDt = gg * (kt * i4(Ht.H1));
+      if (kind >= 0) {
+        const double dl = (kind == 0) ? fabs(xip - xir) : ((kind == 1) ? (1.0 - xip + xir) : (xip + 1.0 - xir));
+        const double lg = lh + log(dl);  // log |s - s'|
+        aS = (-1.0 / (2.0 * WCS_PI)) * Ht.J0;
+        aN = (-1.0 / (2.0 * WCS_PI)) * Hk.J0;
+        aD = (-(k * gg) / (2.0 * WCS_PI)) * Hk.J1;
+        aDt = (-gg / (2.0 * WCS_PI)) * (kt * Ht.J1);
+        kS -= lg * aS;
+        kN -= lg * aN;
+        kD -= lg * aD;
+        kDt -= lg * aDt;
+      }
+    }
+    const double ph[2] = {1.0 - xip, xip}, ps[2] = {1.0 - xir, xir};
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+      const double pp = ph[ab >> 1] * ps[ab & 1], sab = (ab == 0 || ab == 3) ? 1.0 : -1.0;
+      const double c = w * pp, cn = w * sab - kk2h2 * nd * c;
+      v[2 * ab] = fma(c, kS.x, v[2 * ab]);
+      v[2 * ab + 1] = fma(c, kS.y, v[2 * ab + 1]);
+      v[8 + 2 * ab] = fma(c, kD.x, v[8 + 2 * ab]);
+      v[8 + 2 * ab + 1] = fma(c, kD.y, v[8 + 2 * ab + 1]);
+      v[16 + 2 * ab] = fma(c, kDt.x, v[16 + 2 * ab]);
+      v[16 + 2 * ab + 1] = fma(c, kDt.y, v[16 + 2 * ab + 1]);
+      v[24 + 2 * ab] = fma(cn, kN.x, v[24 + 2 * ab]);
+      v[24 + 2 * ab + 1] = fma(cn, kN.y, v[24 + 2 * ab + 1]);
+      if (kind >= 0) {   // uniform over the warp
+        const double cl = lw * pp, cln = lw * (sab - kk2h2 * nd * pp);
+        v[2 * ab] = fma(cl, aS.x, v[2 * ab]);
+        v[2 * ab + 1] = fma(cl, aS.y, v[2 * ab + 1]);
+        v[8 + 2 * ab] = fma(cl, aD.x, v[8 + 2 * ab]);
+        v[8 + 2 * ab + 1] = fma(cl, aD.y, v[8 + 2 * ab + 1]);
+        v[16 + 2 * ab] = fma(cl, aDt.x, v[16 + 2 * ab]);
+        v[16 + 2 * ab + 1] = fma(cl, aDt.y, v[16 + 2 * ab + 1]);
+        v[24 + 2 * ab] = fma(cln, aN.x, v[24 + 2 * ab]);
+        v[24 + 2 * ab + 1] = fma(cln, aN.y, v[24 + 2 * ab + 1]);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  out[pair * 32 + lane] = lane < 24 ? h * h * v[0] : v[0];
+}
+
+int near_band_pairs(const AsmArgs& A, int64_t e0, int64_t ne, double* out, cudaStream_t s) {
+  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
+  const int64_t pairs = ne * (2 * A.near_band + 1);
+  k_near_band<<<(unsigned)((pairs + 3) / 4), 128, 0, s>>>(A, e0, ne, out);
+  note_launch();
+  cudaError_t err = cudaGetLastError();
+  if (err != cudaSuccess) { set_error(std::string("near band: ") + cudaGetErrorString(err)); return 3; }
+  return 0;
+}
+
+// The block of a near-band pair from the table of near_band_pairs
+__device__ __forceinline__ void pair_near(const double* buf, int64_t e0, int64_t ne, int nb, int64_t N, int64_t e,
+                                          int64_t f, PairOut& o) {
+  int64_t off = f - e;
+  if (off > nb) off -= N;
+  else if (off < -nb) off += N;
+  const int64_t u = (e - e0 + N) % N;
+  const zd* b = (const zd*)(buf + ((off + nb) * ne + u) * 32);
+#pragma unroll
+  for (int op = 0; op < 4; ++op)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o.v[op][j] = b[op * 4 + j];
+}
+
+// Element pairs beyond the near band whose point pairs all lie below the table's
+// end (T: the table in shared or global memory): the far rule in FP64, the inner
+// sums over r shared by both target hats, the kernels' constant factors applied
+// to the sums.
+__device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t e, int64_t f, PairOut& o) {
+  const int q = A.q_far;
+  zd v[4][4], vd = mkz(0.0);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[0][j] = v[1][j] = v[2][j] = v[3][j] = mkz(0.0);
+  for (int p = 0; p < q; ++p) {
+    const int64_t ip = e * q + p;
+    const double xt = A.far.x[ip], yt = A.far.y[ip], nxt = A.far.nx[ip], nyt = A.far.ny[ip];
+    zd u[4][2], ud = mkz(0.0);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) u[0][b] = u[1][b] = u[2][b] = u[3][b] = mkz(0.0);
+    for (int r = 0; r < q; ++r) {
+      const int64_t ir = f * q + r;
+      const double dx = xt - A.far.x[ir], dy = yt - A.far.y[ir];
+      const double nxs = A.far.nx[ir], nys = A.far.ny[ir];
+      const double R2 = dx * dx + dy * dy, ri = rsqrt(R2), x = A.k * (R2 * ri);
+      Hankel01 Hk, Ht;
+      if (x >= HT_X0) hankel_tab_poly(T, x, Hk.H0, Hk.H1, Ht.H0, Ht.H1);
+      else hankel_tab_series(T, x, log(0.5 * x), Hk, Ht);
+      const double gg = (dx * nxs + dy * nys) * ri, nd = nxt * nxs + nyt * nys;
+      const zd K[4] = {Ht.H0, gg * Hk.H1, gg * Ht.H1, nd * Hk.H0};
+      const double w1 = c_wf[r] * c_xf[r], w0 = c_wf[r] - w1;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        zfmas(u[i][0], w0, K[i]);
+        zfmas(u[i][1], w1, K[i]);
+      }
+      zfmas(ud, c_wf[r], Hk.H0);
+    }
+    const double w1 = c_wf[p] * c_xf[p], w0 = c_wf[p] - w1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        zfmas(v[i][b], w0, u[i][b]);
+        zfmas(v[i][2 + b], w1, u[i][b]);
+      }
+    zfmas(vd, c_wf[p], ud);
+  }
+  const double h2 = A.h * A.h, kk2h2 = A.k * A.k * h2;
+  const zd fS = mkz(0.0, 0.25 * h2), fD = mkz(0.0, 0.25 * A.k * h2), fDt = mkz(-0.25 * h2 * A.kt.y, 0.25 * h2 * A.kt.x);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    o.v[0][j] = fS * v[0][j];
+    o.v[1][j] = fD * v[1][j];
+    o.v[2][j] = fDt * v[2][j];
+    o.v[3][j] = i4(((j == 0 || j == 3) ? vd : -vd) - kk2h2 * v[3][j]);
+  }
+}
+
+// True when pair_mid's table covers every point pair of (e, f): centres (of the
+// Gauss points) within HT_X1 - 2 k h, points within k h of that (0.9 k h, see pair_integrals).
+__device__ __forceinline__ bool pair_is_mid(const AsmArgs& A, int64_t e, int64_t f) {
+  const int q = A.q_far;
+  const double dx = A.far.x[e * q] - A.far.x[f * q], dy = A.far.y[e * q] - A.far.y[f * q];
+  const double lim = HT_X1 - 2.0 * A.k * A.h;
+  return lim > 0.0 && A.k * A.k * (dx * dx + dy * dy) < lim * lim;
+}
+
 constexpr int TILE = 32;
 constexpr int ASM_THREADS = 256;
 constexpr int FAR_CTAS = 1;
@@ -254,7 +552,7 @@ constexpr int FAR_CTAS = 1;
 // that touch it, accumulated in acc[4][TILE][TILE].  MIXED: pairs far enough for
 // the FP32 route take it.
 template <int MIXED>
-__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc) {
+__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc, const double* T = nullptr) {
   const int64_t N = A.N;
   for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) acc[t] = mkz(0.0);
   __syncthreads();
@@ -272,8 +570,16 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
     if (rowok && colok) {
       const int64_t e = ((i0 - 1 + el) % N + N) % N;
       const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-      if (MIXED && pair_is_far(A, e, f)) pair_far(A, e, f, o);
-      else pair_integrals(A, e, f, o);
+      if (MIXED && T) {
+        if (periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, 0, N, A.near_band, N, e, f, o);
+        else if (pair_is_far(A, e, f)) pair_far(A, e, f, o);
+        else if (pair_is_mid(A, e, f)) pair_mid(A, T, e, f, o);
+        else pair_integrals(A, e, f, o);
+      } else if (MIXED && pair_is_far(A, e, f)) {
+        pair_far(A, e, f, o);
+      } else {
+        pair_integrals(A, e, f, o);
+      }
     }
 #pragma unroll
     for (int ph = 0; ph < 4; ++ph) {
@@ -307,13 +613,18 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A) {
 // Mixed form: the tiles that k_assemble_far listed (those holding an element
 // pair nearer than its route), as split-bf16 planes in both layouts.
 __global__ void __launch_bounds__(ASM_THREADS) k_assemble_near(AsmArgs A, int64_t nt) {
-  extern __shared__ zd acc[];  // [4][TILE][TILE]
+  extern __shared__ zd acc[];  // [4][TILE][TILE], then the Hankel table
   const int64_t N = A.N;
   const int count = A.tile_list[0];
+  double* T = nullptr;
+  if (A.near_buf) {
+    T = (double*)(acc + 4 * TILE * TILE);
+    for (int t = threadIdx.x; t < HT_SIZE; t += blockDim.x) T[t] = A.htab[t];
+  }
   for (int u = blockIdx.x; u < count; u += gridDim.x) {
     const int64_t tile = A.tile_list[1 + u];
     const int64_t i0 = (tile / nt) * TILE, j0 = (tile % nt) * TILE;
-    tile_sums<1>(A, i0, j0, acc);
+    tile_sums<1>(A, i0, j0, acc, T);
     // layout 0: row i0 + li holds (re, im) of column j0 + lj at 2 (j0 + lj);
     // layout 1 (transpose): row j0 + lj holds entry (i0 + li, j0 + lj) at 2 (i0 + li);
     // consecutive threads walk the contiguous index
@@ -351,7 +662,9 @@ __global__ void k_circle_row_part(AsmArgs A, zd* part) {
   const int64_t f = v ? j : (j - 1 + N) % N;
   const int b = v ? 0 : 1;
   PairOut o;
-  pair_integrals(A, e, f, o);
+  if (A.near_buf && periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, N - 1, 2, A.near_band, N, e, f, o);
+  else if (A.near_buf && pair_is_mid(A, e, f)) pair_mid(A, A.htab, e, f, o);
+  else pair_integrals(A, e, f, o);
   for (int op = 0; op < 4; ++op) part[(int64_t)op * 4 * N + t] = o.v[op][a * 2 + b];
 }
 
@@ -551,7 +864,8 @@ __global__ void __launch_bounds__(ASM_THREADS, FAR_CTAS) k_assemble_far(AsmArgs 
 int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t* fp64_tiles, int64_t* tiles) {
   if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const size_t smem = sizeof(zd) * 4 * TILE * TILE;   // float-float and FP64 sums take the same room
-  cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem_near = smem + sizeof(double) * HT_SIZE;
+  cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_near);
   cudaFuncSetAttribute(k_assemble_far<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaFuncSetAttribute(k_assemble_far<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t nt = (A.N + TILE - 1) / TILE;
@@ -561,7 +875,7 @@ int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t*
   else k_assemble_far<0><<<grid, ASM_THREADS, smem, s>>>(A, nt);
   note_launch();
   if (mid) { cudaEventRecord(mid[0], s); cudaEventRecord(mid[1], s); }
-  k_assemble_near<<<(unsigned)std::min<int64_t>(nt * nt, 152 * 3), ASM_THREADS, smem, s>>>(A, nt);
+  k_assemble_near<<<(unsigned)std::min<int64_t>(nt * nt, 152 * 3), ASM_THREADS, smem_near, s>>>(A, nt);
   note_launch();
   if (fp64_tiles) {   // the tiles that took the FP64 kernel (for the work count of each kernel)
     int n = 0;

@@ -106,6 +106,10 @@ struct AsmArgs {
   // FP64 factors of the far pairs' float-float sums, applied once per stored entry (a
   // constant rounded to FP32 would bias every far entry of an operator alike)
   zd fS, fD, fDt, fN;              // S~, D, D~, N (see FarPair)
+  // mixed form: Hankel table of the run (hankeltab.cuh) and the near-band pairs'
+  // blocks (near_band_pairs; null: pair integrals without either)
+  const double* htab = nullptr;
+  const double* near_buf = nullptr;
   int* tile_list = nullptr;        // count, then the tiles that hold a pair nearer than the far route (1 + tiles)
 };
 // Fill kp.asym for kp.t and the term-count thresholds kp.xth for relative
@@ -120,6 +124,12 @@ int assemble_planes(const AsmArgs& a, cudaStream_t s, cudaEvent_t* mid = nullptr
                     int64_t* tiles = nullptr);
 // Tables of the far route: N elements, N q_far points (cen: element centres, xi = 1/2).
 int far_tables(const AsmArgs& a, const Points& cen, FarElem* fe, FarPoint* fp, cudaStream_t s);
+// Hankel table of the run (hankel_table_doubles() of device memory).
+int64_t hankel_table_doubles();
+int hankel_table(double t, double* T, cudaStream_t s);
+// Blocks of the near-band element pairs of elements e0 .. e0 + ne - 1 (mod N):
+// 32 doubles for each of ne (2 near_band + 1) pairs.  Needs a.htab.
+int near_band_pairs(const AsmArgs& a, int64_t e0, int64_t ne, double* out, cudaStream_t s);
 // First row of the four circulant operators on the circle (row 0, N entries each).
 int assemble_circle_row(const AsmArgs& a, cudaStream_t s);
 // Sampled entries (row, col) of the four operators, computed point-wise.

@@ -90,6 +90,7 @@ struct wcs_ctx {
   int64_t ldp = 0;                        // plane leading dimension (bf16 elements)
   DevBuf opplanes;                        // [op][layout][plane] N x ldp bf16
   DevBuf centres, offs;                   // element centres (FP64), tables of the far route
+  DevBuf htab;                            // Hankel table, near-band blocks of gamma and of two elements of gamma_c
   DevBuf tiles;                           // list of the tiles assembled in FP64
   DevBuf stage0, stage1, stage2;          // staged right-hand blocks (bf16 planes)
   int64_t stage_cols = 0;
@@ -843,7 +844,7 @@ static void free_mesh(wcs_ctx* c) {
   cudaFree(c->arc_c.cum); c->arc_c.cum = nullptr;
   c->pts_far.release(); c->pts_near.release(); c->pts_far_c.release(); c->pts_near_c.release();
   c->ops.release(); c->mu.release();
-  c->opplanes.release(); c->centres.release(); c->offs.release(); c->tiles.release();
+  c->opplanes.release(); c->centres.release(); c->offs.release(); c->tiles.release(); c->htab.release();
   c->stage0.release(); c->stage1.release(); c->stage2.release(); c->stage_cols = 0;
   c->gA.release(); c->gB.release(); c->gW.release(); c->qh.release(); c->qt.release();
   c->U.release(); c->Vw.release(); c->Wt.release(); c->Kinv.release(); c->Wa.release();
@@ -1074,6 +1075,7 @@ int wcs_assemble(wcs_ctx* c) {
   if (!c) { set_error("null context"); return WCS_ERR_ARG; }
   if (c->stage < ST_MESH) { set_error("mesh first"); return WCS_ERR_STATE; }
   const int64_t N = c->N, ld = c->ld;
+  bool near_tab = false;
   if (!c->mixed) {
     TRY(c->ops.ensure(sizeof(zd) * 4 * N * ld));
     c->S = c->ops.z(); c->D = c->S + N * ld; c->Dt = c->D + N * ld; c->Nk = c->Dt + N * ld;
@@ -1099,6 +1101,12 @@ int wcs_assemble(wcs_ctx* c) {
     FarPoint* fp = (FarPoint*)(fe + N);
     AsmArgs A = asm_args(c, false);
     TRY(far_tables(A, cp, fe, fp, c->s));
+    // Hankel table and near-band blocks (N (2 near_band + 1) of 256 bytes);
+    // without them (k~ off the table's form, a band of more than 1 GB) the tile
+    // kernel integrates those pairs itself
+    const int64_t band = N * (2 * c->opt.near_band + 1), band_row = 2 * (2 * c->opt.near_band + 1);
+    near_tab = A.kt_pair && 2 * c->opt.near_band + 1 <= N && 256 * band <= ((int64_t)1 << 30);
+    if (near_tab) TRY(c->htab.ensure(sizeof(double) * (hankel_table_doubles() + 32 * (band + band_row))));
     A.planes = c->planes;
     A.ldp = c->ldp;
     for (int op = 0; op < 4; ++op)
@@ -1110,6 +1118,12 @@ int wcs_assemble(wcs_ctx* c) {
     TRY(c->tiles.ensure(sizeof(int) * (1 + nt * nt)));
     A.tile_list = (int*)c->tiles.p;
     set_far_consts(c, A);
+    if (near_tab) {
+      TRY(hankel_table(A.ktp.t, c->htab.d(), c->s));
+      A.htab = c->htab.d();
+      TRY(near_band_pairs(A, 0, N, c->htab.d() + hankel_table_doubles(), c->s));
+      A.near_buf = c->htab.d() + hankel_table_doubles();
+    }
     if (!c->profile) {
       TRY(assemble_planes(A, c->s));
     } else {
@@ -1133,6 +1147,12 @@ int wcs_assemble(wcs_ctx* c) {
   TRY(c->mu.ensure(sizeof(zd) * 6 * N));
   AsmArgs B = asm_args(c, true);
   B.S = mu_ptr(c, MU_S); B.D = mu_ptr(c, MU_D); B.Dt = mu_ptr(c, MU_DT); B.Nk = mu_ptr(c, MU_N);
+  if (near_tab) {   // the same wavenumbers: the table serves the circle as well
+    double* row = c->htab.d() + hankel_table_doubles() + 32 * N * (2 * c->opt.near_band + 1);
+    B.htab = c->htab.d();
+    TRY(near_band_pairs(B, N - 1, 2, row, c->s));
+    B.near_buf = row;
+  }
   TRY(assemble_circle_row(B, c->s));
   // mu_X(m) = sum_j X_0j e^{+2 pi i m j / N}
   TRY(fft_columns(c->fft, mu_ptr(c, MU_S), N, 4, +1, c->s));
