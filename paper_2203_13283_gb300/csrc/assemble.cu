@@ -230,10 +230,10 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
 
 // The four operators of a far pair in FP64 from its float-float sums (farpair.cuh).
 __device__ __noinline__ void pair_far(const AsmArgs& A, int64_t e, int64_t f, PairOut& out) {
-  FarPair o;
+  FarPair<false> o;
   const int q = A.q_far;
-  if (q == 4) far_pair<4>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
-  else far_pair<0>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+  if (q == 4) far_pair<4, false>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+  else far_pair<0, false>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
   const zd fac[4] = {A.fS, A.fD, A.fDt, A.fN};
 #pragma unroll
   for (int op = 0; op < 4; ++op)
@@ -546,7 +546,6 @@ __device__ __forceinline__ bool pair_is_mid(const AsmArgs& A, int64_t e, int64_t
 
 constexpr int TILE = 32;
 constexpr int ASM_THREADS = 256;
-constexpr int FAR_CTAS = 1;
 
 // One tile of node pairs from FP64 pair integrals: the 33 x 33 element pairs
 // that touch it, accumulated in acc[4][TILE][TILE].  MIXED: pairs far enough for
@@ -772,50 +771,62 @@ __device__ __forceinline__ void ff_planes(ff x, uint16_t (&p)[3]) {
   p[1] = __bfloat16_as_ushort(h1);
   p[2] = __bfloat16_as_ushort(__float2bfloat16_rn(r2));
 }
-// (re, im) as adjacent bf16 pairs, one 32-bit store per plane (off even)
-__device__ __forceinline__ void split_store_ff2(ff re, ff im, int planes, uint16_t* const* P, int64_t off) {
-  uint16_t a[3], b[3];
-  ff_planes(re, a);
-  ff_planes(im, b);
-  for (int q = 0; q < planes; ++q) *(uint32_t*)(P[q] + off) = (uint32_t)a[q] | ((uint32_t)b[q] << 16);
-}
-
 // Tiles whose element pairs all take the FP32 route of farpair.cuh; a tile with
-// a nearer pair is put on the list of k_assemble_near instead.  One thread per
-// element pair, the pair's values added into float-float sums per node pair in
-// shared memory in four conflict-free phases, then multiplied by their FP64
-// factors (as float-float) and written as split-bf16 planes in both layouts.
+// a nearer pair is put on the list of k_assemble_near instead.  A CTA owns the
+// tile (ti, tj), ti < tj, and its mirror image (the diagonal tiles are never
+// far): S~ and N are symmetric and every Hankel evaluation serves both.  One
+// thread per element pair, the pair's values added into float-float sums per
+// node pair in shared memory in four conflict-free phases, then multiplied by
+// their FP64 factors (as float-float), split into bf16 planes once and written in
+// both layouts of both tiles.
+// Bound: FP32 issue.  384 threads: three warps per scheduler at 168 registers,
+// and 1089 pairs fill 95% of three rounds (256 threads: 85% of five).
+constexpr int FAR_THREADS = 384, FAR_LD = TILE + 1, FAR_OPS = 6;
+constexpr size_t FAR_SMEM = sizeof(float4) * FAR_OPS * TILE * FAR_LD;
+
 template <int Q>
-__global__ void __launch_bounds__(ASM_THREADS, FAR_CTAS) k_assemble_far(AsmArgs A, int64_t nt) {
-  extern __shared__ float4 facc[];   // [4][TILE][TILE] (re hi, re lo, im hi, im lo)
-  const int64_t ti = blockIdx.y, tj = blockIdx.x;
+__global__ void __launch_bounds__(FAR_THREADS, 1) k_assemble_far(AsmArgs A, int64_t nt) {
+  extern __shared__ float4 facc[];   // [6][TILE][FAR_LD] (re hi, re lo, im hi, im lo), later the planes
+  // blockIdx.x -> (ti, tj), ti < tj: row tj of the lower triangle holds tj tiles
+  const int64_t u0 = blockIdx.x;
+  int64_t tj = (int64_t)((1.0 + sqrt(1.0 + 8.0 * (double)u0)) * 0.5);
+  while (tj * (tj - 1) / 2 > u0) --tj;
+  while ((tj + 1) * tj / 2 <= u0) ++tj;
+  const int64_t ti = u0 - tj * (tj - 1) / 2;
   const int64_t N = A.N;
   const int64_t i0 = ti * TILE, j0 = tj * TILE;
   const int span = TILE + 1;
   const int npairs = span * span;
   int near = 0;
-  for (int u = threadIdx.x; u < npairs; u += blockDim.x) {
+  for (int u = threadIdx.x; u < npairs; u += FAR_THREADS) {
     const int el = u / span, fl = u - (u / span) * span;
-    const int64_t e = ((i0 - 1 + el) % N + N) % N, f = ((j0 - 1 + fl) % N + N) % N;
+    int64_t e = i0 - 1 + el, f = j0 - 1 + fl;
+    if (e < 0) e += N;
+    if (e >= N) e -= N;
+    if (f >= N) f -= N;
     if (!pair_is_far(A, e, f)) near = 1;
   }
-  for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) facc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int t = threadIdx.x; t < FAR_OPS * TILE * FAR_LD; t += FAR_THREADS) facc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (__syncthreads_or(near)) {
-    if (threadIdx.x == 0) A.tile_list[1 + atomicAdd(A.tile_list, 1)] = (int)(ti * nt + tj);
+    if (threadIdx.x == 0) {
+      const int at = 1 + atomicAdd(A.tile_list, 2);
+      A.tile_list[at] = (int)(ti * nt + tj);
+      A.tile_list[at + 1] = (int)(tj * nt + ti);
+    }
     return;
   }
-  for (int base = 0; base < npairs; base += blockDim.x) {
+  for (int base = 0; base < npairs; base += FAR_THREADS) {
     const int idx = base + threadIdx.x;
     const int el = idx / span, fl = idx - (idx / span) * span;
     const bool valid = idx < npairs;
     const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N));
     const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
-    FarPair o;
+    FarPair<true> o;
     if (rowok && colok) {
-      const int64_t e = ((i0 - 1 + el) % N + N) % N;
-      const int64_t f = ((j0 - 1 + fl) % N + N) % N;
+      int64_t e = i0 - 1 + el, f = j0 - 1 + fl;
+      if (e < 0) e += N;
       const int q = Q ? Q : A.q_far;
-      far_pair<Q>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+      far_pair<Q, true>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
     }
 #pragma unroll
     for (int ph = 0; ph < 4; ++ph) {
@@ -824,15 +835,15 @@ __global__ void __launch_bounds__(ASM_THREADS, FAR_CTAS) k_assemble_far(AsmArgs 
         const int li = el - 1 + a, lj = fl - 1 + b;
         if (li >= 0 && li < TILE && lj >= 0 && lj < TILE && i0 + li < N && j0 + lj < N) {
 #pragma unroll
-          for (int op = 0; op < 4; ++op) {
+          for (int op = 0; op < FAR_OPS; ++op) {
             const ffc v = o.value(op, ph);
-            float4 s = facc[(op * TILE + li) * TILE + lj];
+            float4 s = facc[(op * TILE + li) * FAR_LD + lj];
             const ff x = ff_two_sum(s.x, v.x.hi), y = ff_two_sum(s.z, v.y.hi);
             s.x = x.hi;
             s.y += x.lo + v.x.lo;
             s.z = y.hi;
             s.w += y.lo + v.y.lo;
-            facc[(op * TILE + li) * TILE + lj] = s;
+            facc[(op * TILE + li) * FAR_LD + lj] = s;
           }
         }
       }
@@ -840,40 +851,84 @@ __global__ void __launch_bounds__(ASM_THREADS, FAR_CTAS) k_assemble_far(AsmArgs 
     }
   }
   // entries: the FP64 run factors times the tile sums, in float-float on the
-  // FP32 pipe (~44 bits; the FP64 pipe is 64 times slower)
+  // FP32 pipe (~44 bits; the FP64 pipe is 64 times slower), as packed planes
   const ff2 fac[4] = {ff2_of(A.fS), ff2_of(A.fD), ff2_of(A.fDt), ff2_of(A.fN)};
-  for (int lay = 0; lay < 2; ++lay) {
 #pragma unroll
-    for (int op = 0; op < 4; ++op) {
-      for (int u = threadIdx.x; u < TILE * TILE; u += blockDim.x) {
-        const int x = u / TILE, y = u - (u / TILE) * TILE;
-        const int li = lay ? y : x, lj = lay ? x : y;
-        if (i0 + li < N && j0 + lj < N) {
-          const float4 s = facc[(op * TILE + li) * TILE + lj];
-          const ff ar = ff_quick(s.x, s.y), ai = ff_quick(s.z, s.w);
-          const ff re = ff_add(ff_mul(fac[op].r, ar), ff_neg(ff_mul(fac[op].i, ai)));
-          const ff im = ff_add(ff_mul(fac[op].r, ai), ff_mul(fac[op].i, ar));
-          const int64_t off = lay ? (j0 + lj) * A.ldp + 2 * (i0 + li) : (i0 + li) * A.ldp + 2 * (j0 + lj);
-          split_store_ff2(re, im, A.planes, A.P[op][lay], off);
+  for (int op = 0; op < FAR_OPS; ++op) {
+    const ff2 fo = fac[op < 4 ? op : op - 3];
+    for (int u = threadIdx.x; u < TILE * TILE; u += FAR_THREADS) {
+      float4& slot = facc[(op * TILE + u / TILE) * FAR_LD + u % TILE];
+      const float4 s = slot;
+      const ff ar = ff_quick(s.x, s.y), ai = ff_quick(s.z, s.w);
+      uint16_t re[3], im[3];
+      ff_planes(ff_add(ff_mul(fo.r, ar), ff_neg(ff_mul(fo.i, ai))), re);
+      ff_planes(ff_add(ff_mul(fo.r, ai), ff_mul(fo.i, ar)), im);
+      uint4 w;
+      w.x = (uint32_t)re[0] | ((uint32_t)im[0] << 16);
+      w.y = (uint32_t)re[1] | ((uint32_t)im[1] << 16);
+      w.z = (uint32_t)re[2] | ((uint32_t)im[2] << 16);
+      w.w = 0u;
+      *(uint4*)&slot = w;
+    }
+  }
+  __syncthreads();
+  // stored operator x: entry (i, j) from accumulator x; entry (j, i) from x (S~,
+  // N) or from the mirrored accumulator.  "wide" rows run along j for fixed i
+  // (layout 0 of (i, j), layout 1 of (j, i)), "tall" ones along i for fixed j.
+  for (int u = threadIdx.x; u < 4 * TILE * TILE; u += FAR_THREADS) {
+    const int op = u / (TILE * TILE), rem = u - op * TILE * TILE;
+    const int x = rem / TILE, y = rem - (rem / TILE) * TILE;
+    const int mop = (op == 1 || op == 2) ? op + 3 : op;
+    if (i0 + x < N && j0 + y < N) {     // wide: li = x, lj = y
+      const int64_t off = (i0 + x) * A.ldp + 2 * (j0 + y);
+      const uint4 d = *(const uint4*)&facc[(op * TILE + x) * FAR_LD + y];
+      const uint4 m = *(const uint4*)&facc[(mop * TILE + x) * FAR_LD + y];
+      const uint32_t dv[3] = {d.x, d.y, d.z}, mv[3] = {m.x, m.y, m.z};
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (q < A.planes) {
+          *(uint32_t*)(A.P[op][0][q] + off) = dv[q];
+          *(uint32_t*)(A.P[op][1][q] + off) = mv[q];
         }
-      }
+    }
+    if (i0 + y < N && j0 + x < N) {     // tall: li = y, lj = x
+      const int64_t off = (j0 + x) * A.ldp + 2 * (i0 + y);
+      const uint4 d = *(const uint4*)&facc[(op * TILE + y) * FAR_LD + x];
+      const uint4 m = *(const uint4*)&facc[(mop * TILE + y) * FAR_LD + x];
+      const uint32_t dv[3] = {d.x, d.y, d.z}, mv[3] = {m.x, m.y, m.z};
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (q < A.planes) {
+          *(uint32_t*)(A.P[op][1][q] + off) = dv[q];
+          *(uint32_t*)(A.P[op][0][q] + off) = mv[q];
+        }
     }
   }
 }
 
+// the diagonal tiles open the list of the FP64 kernel
+__global__ void k_diag_tiles(int* list, int64_t nt) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t == 0) list[0] = (int)nt;
+  if (t < nt) list[1 + t] = (int)(t * nt + t);
+}
+
 int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t* fp64_tiles, int64_t* tiles) {
   if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
-  const size_t smem = sizeof(zd) * 4 * TILE * TILE;   // float-float and FP64 sums take the same room
+  const size_t smem = sizeof(zd) * 4 * TILE * TILE;
   const size_t smem_near = smem + sizeof(double) * HT_SIZE;
   cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_near);
-  cudaFuncSetAttribute(k_assemble_far<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaFuncSetAttribute(k_assemble_far<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_assemble_far<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FAR_SMEM);
+  cudaFuncSetAttribute(k_assemble_far<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FAR_SMEM);
   const int64_t nt = (A.N + TILE - 1) / TILE;
-  cudaMemsetAsync(A.tile_list, 0, sizeof(int), s);
-  dim3 grid((unsigned)nt, (unsigned)nt);
-  if (A.q_far == 4) k_assemble_far<4><<<grid, ASM_THREADS, smem, s>>>(A, nt);
-  else k_assemble_far<0><<<grid, ASM_THREADS, smem, s>>>(A, nt);
+  k_diag_tiles<<<(unsigned)((nt + 127) / 128), 128, 0, s>>>(A.tile_list, nt);
   note_launch();
+  if (nt > 1) {
+    const unsigned grid = (unsigned)(nt * (nt - 1) / 2);
+    if (A.q_far == 4) k_assemble_far<4><<<grid, FAR_THREADS, FAR_SMEM, s>>>(A, nt);
+    else k_assemble_far<0><<<grid, FAR_THREADS, FAR_SMEM, s>>>(A, nt);
+    note_launch();
+  }
   if (mid) { cudaEventRecord(mid[0], s); cudaEventRecord(mid[1], s); }
   k_assemble_near<<<(unsigned)std::min<int64_t>(nt * nt, 152 * 3), ASM_THREADS, smem_near, s>>>(A, nt);
   note_launch();

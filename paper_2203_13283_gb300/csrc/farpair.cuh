@@ -88,6 +88,14 @@ WCS_HD ff ff_of(double x) {
   const float h = (float)x;
   return ff{h, (float)(x - (double)h)};
 }
+// 1 / x for a factor of the small corrections (2 ulp)
+WCS_HD float far_rcp(float x) {
+#ifdef __CUDA_ARCH__
+  return __fdividef(1.f, x);
+#else
+  return 1.f / x;
+#endif
+}
 // FP32 seeds of the Newton steps below (their error is squared away)
 WCS_HD float ff_seed_rsqrt(float x) {
 #ifdef __CUDA_ARCH__
@@ -163,7 +171,7 @@ struct FarConsts {
   float ikt[2] = {0.f, 0.f};       // 1 / (1 + i t), k~ = k (1 + i t)
   ff kk2h2{0.f, 0.f};              // k^2 h^2 of the Maue form
   float hf = 0.f;                  // h
-  float w[2][FAR_Q] = {}, s[FAR_Q] = {};   // w_p phi_a(xi_p), xi_p - 1/2
+  float w[2][FAR_Q] = {}, w1[FAR_Q] = {}, s[FAR_Q] = {};   // w_p phi_a(xi_p), w_p, xi_p - 1/2
   float pe[FAR_P] = {}, po[FAR_P] = {};    // Re A_0 - 1/2 = sum pe_m alpha^2(m+1); Im A_0 + alpha / 12 = alpha sum po_m alpha^2(m+1)
   float a[2][FAR_M] = {};          // a_m(nu) of the Hankel expansion
 };
@@ -222,6 +230,7 @@ inline void far_consts(FarConsts& F, int q, const double* xi, const double* w, d
     F.s[p] = (float)s;
     F.w[0][p] = (float)(w[p] * (1.0 - xi[p]));
     F.w[1][p] = (float)(w[p] * xi[p]);
+    F.w1[p] = (float)w[p];
     double m = w[p] * (1.0 - xi[p]);
     for (int j = 0; j < 2 * FAR_P + 2; ++j) { me[j] += m; m *= s; }
   }
@@ -247,24 +256,27 @@ struct ffc {
 };
 WCS_HD ffc ffc_mul(ffc a, ff s) { return {ff_mul(a.x, s), ff_mul(a.y, s)}; }
 
-// One element pair: the reference kernels, the exact leading parts and the
-// FP32 corrections of the four operators, [a * 2 + b].  With the factors
-// fS = (i/4) sqrt(2 / (pi k~)) h^2, fD = (i/4) sqrt(2 / (pi k)) k h^2,
-// fDt = fS k~ and fN = (i/4) sqrt(2 / (pi k)) the pair's integral is
-// f (lead + K (i lam + corr)) (see value()).
+// One element pair (e, f): the reference kernels, the exact leading parts and the
+// FP32 corrections of the operators, [a * 2 + b] (a: hat on e, b: hat on f).  With
+// the factors fS = (i/4) sqrt(2 / (pi k~)) h^2, fD = (i/4) sqrt(2 / (pi k)) k h^2,
+// fDt = fS k~ and fN = (i/4) sqrt(2 / (pi k)) an integral is f (lead + K (i lam +
+// corr)) (see value()).  M: also D and D~ of the mirrored pair (f, e) (operators 4
+// and 5); its S~ and N are this pair's, and every Hankel evaluation is shared.
+template <bool M>
 struct FarPair {
-  ffc lead[5];                 // S~, D, D~ (a quarter of the kernel), N for a = b and a != b
-  cf K[3];                     // T0, K1 g, T1 g (heads): factors of the linear phase term
+  static constexpr int OPS = M ? 6 : 4;
+  ffc lead[OPS + 1];           // S~, D, D~ (a quarter of the kernel), N for a = b, [D, D~ mirrored,] N for a != b
+  cf K[OPS];                   // T0, K1 g, T1 g, -, K1 g', T1 g' (heads): factors of the linear phase term
   ff lam[2];                   // (alpha_e - alpha_f) / 24 for a = b = 0, (alpha_e + alpha_f) / 24 for a = 0, b = 1
-  cf corr[4][4];               // K times the corrections
+  cf corr[OPS][4];             // K times the corrections
 
   WCS_HD ffc value(int op, int j) const {
-    const ffc& l = lead[op < 3 ? op : ((j == 0 || j == 3) ? 3 : 4)];
+    const ffc& l = lead[(op == 3 && (j == 1 || j == 2)) ? OPS : op];
     const cf c = corr[op][j];
     ff x = ff_two_sum(l.x.hi, c.x), y = ff_two_sum(l.y.hi, c.y);
     x.lo += l.x.lo;
     y.lo += l.y.lo;
-    if (op < 3) {
+    if (op != 3) {
       // K (i lam): (-K.y lam, K.x lam) with the rounding errors of the products
       const ff la = lam[(j == 1 || j == 2) ? 1 : 0];
       const float sg = (j >= 2) ? -1.f : 1.f;    // j = 2, 3 mirror j = 1, 0
@@ -283,32 +295,46 @@ WCS_HD bool far_ok(const FarConsts& F, const float4& ce, const float4& cg) {
   return F.k.hi * F.k.hi * (dx * dx + dy * dy) >= F.xmin2;
 }
 
-// Hankel series at w = i u (u = 1 / (k R0), or 1 / (k~ R0)): s = sum_{m>=1} a_m w^m,
+// Hankel series at w = i u, u = 1 / (k R0) (or 1 / (k~ R0)): s = sum_{m>=1} a_m w^m,
 // and the coefficients b1, b2 of its change with v = R0 / R - 1 relative to
 // 1 + s: b1 v + b2 v^2.
-WCS_HD void far_series(const float* a, cf w, cf& s, cf& b1, cf& b2) {
+WCS_HD cf far_recip1(cf s) {   // 1 / (1 + s)
+  const float x = 1.f + s.x, iq = 1.f / fmaf(x, x, s.y * s.y);
+  return {x * iq, -s.y * iq};
+}
+WCS_HD void far_series(const float* a, float u, cf& s, cf& b1, cf& b2) {
+  // even and odd powers of w = i u: real polynomials in -u^2
+  const float z = -u * u;
+  float se = a[6], so = a[7], de = 6.f * a[6], od = 7.f * a[7], ee = 15.f * a[6], eo = 10.f * a[5];
+  se = fmaf(se, z, a[4]);
+  so = fmaf(so, z, a[5]);
+  de = fmaf(de, z, 4.f * a[4]);
+  od = fmaf(od, z, 5.f * a[5]);
+  ee = fmaf(ee, z, 6.f * a[4]);
+  eo = fmaf(eo, z, 3.f * a[3]);
+  se = fmaf(se, z, a[2]);
+  so = fmaf(so, z, a[3]);
+  de = fmaf(de, z, 2.f * a[2]);
+  od = fmaf(od, z, 3.f * a[3]);
+  ee = fmaf(ee, z, a[2]);
+  so = fmaf(so, z, a[1]);
+  od = fmaf(od, z, a[1]);
+  s = {se * z, so * u};
+  const cf r = far_recip1(s);
+  b1 = cmul({de * z, od * u}, r);
+  b2 = cmul({ee * z, eo * u * z}, r);
+}
+WCS_HD void far_series_c(const float* a, cf w, cf& s, cf& b1) {
   cf p = {a[FAR_M - 1], 0.f}, d = {(FAR_M - 1) * a[FAR_M - 1], 0.f};
-  cf e = {0.5f * (FAR_M - 1) * (FAR_M - 2) * a[FAR_M - 1], 0.f};
 #pragma unroll
   for (int m = FAR_M - 2; m >= 1; --m) {
     p = cmul(p, w);
     p.x += a[m];
     d = cmul(d, w);
     d.x += m * a[m];
-    if (m >= 2) {
-      e = cmul(e, w);
-      e.x += 0.5f * m * (m - 1) * a[m];
-    }
   }
   s = cmul(p, w);
-  d = cmul(d, w);
-  e = cmul(cmul(e, w), w);
-  // divide by 1 + s
-  const cf q = {1.f + s.x, s.y};
-  const float iq = 1.f / fmaf(q.x, q.x, q.y * q.y);
-  const cf r = {q.x * iq, -q.y * iq};
-  b1 = cmul(d, r);
-  b2 = cmul(e, r);
+  b1 = cmul(cmul(d, w), far_recip1(s));
 }
 
 // e^{i x}, |x| <= 1.2 (k h <= 2.5, |s| < 1/2), to the FP32 accuracy the corrections need
@@ -324,9 +350,9 @@ WCS_HD ffc ffc_grow(const ffc& K, cf s) {
   return {ff_add_f(K.x, px), ff_add_f(K.y, py)};
 }
 
-template <int Q>   // points per element (0: q at run time)
+template <int Q, bool M>   // points per element (0: q at run time); mirrored pair as well
 WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarElem& G, const FarPoint* pe,
-                     const FarPoint* pg, FarPair& o) {
+                     const FarPoint* pg, FarPair<M>& o) {
   const int q = Q ? Q : q_run;
   // ---- geometry of the centres
   const ff dx = ff_add(ff_two_sum(E.c.x, -G.c.x), ff_two_sum(E.c.y, -G.c.y));
@@ -345,6 +371,10 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
   const ff nd0 = ff_add(ff_mul(tex, tgx), ff_mul(tey, tgy));
   const ff sg_ff = ff_add(ff_mul(tex, tgy), ff_neg(ff_mul(tey, tgx)));
   const float sg = sg_ff.hi, ndh = nd0.hi, g0h = g0.hi;
+  // mirrored pair: (c_f - c_e) . n_e / R0 (n_e = (tau_y, -tau_x))
+  ff gm = {0.f, 0.f};
+  if (M) gm = ff_mul(iR0, ff_add(ff_mul(dy, tex), ff_neg(ff_mul(dx, tey))));
+  const float gmh = gm.hi;
   const float dxh = dx.hi, dyh = dy.hi, ux = dxh * ir, uy = dyh * ir;
   // ---- reference kernels
   // k R0 - n 2 pi, 2 pi = 6.28318548 - 1.74845553e-7 - 6.86049999e-15 (n < 2^13), less pi / 4
@@ -359,50 +389,75 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
   const ff damp = ff_exp_neg(ff_mul(F.beta, R0));
   const ffc Et = ffc_mul(E1, damp);
   const float u = 1.f / kr;
-  const cf w = {0.f, u}, wt = {-F.ikt[1] * u, F.ikt[0] * u};
-  cf s0, s1, s0t, s1t, b10, b20, b11, b21, b10t, b20t, b11t, b21t;
-  far_series(F.a[0], w, s0, b10, b20);
-  far_series(F.a[1], w, s1, b11, b21);
-  far_series(F.a[0], wt, s0t, b10t, b20t);
-  far_series(F.a[1], wt, s1t, b11t, b21t);
+  const cf wt = {-F.ikt[1] * u, F.ikt[0] * u};
+  cf s0, s1, s0t, s1t, b10, b20, b11, b21, b10t, b11t;
+  far_series(F.a[0], u, s0, b10, b20);
+  far_series(F.a[1], u, s1, b11, b21);
+  far_series_c(F.a[0], wt, s0t, b10t);
+  far_series_c(F.a[1], wt, s1t, b11t);
+  // the v^2 terms (4e-7 of the kernel at k R0 = 20) follow those of k through their
+  // leading power: b2(k~) = b2(k) (1 + i t)^-2 to ~1e-9 of the kernel
+  const cf ik1 = {F.ikt[0], F.ikt[1]}, ik2 = cmul(ik1, ik1);
+  const cf b20t = cmul(b20, ik2), b21t = cmul(b21, ik2);
   const ffc K0 = ffc_grow(E1, s0), K1r = ffc_grow(E1, s1), T0 = ffc_grow(Et, s0t), T1r = ffc_grow(Et, s1t);
   const ffc K1 = {K1r.y, {-K1r.x.hi, -K1r.x.lo}}, T1 = {T1r.y, {-T1r.x.hi, -T1r.x.lo}};   // times -i
 
-  // ---- corrections: sums over the point pairs
-  cf vS[4], v0[4], v1[4], vt[4], vgk[4], vgt[4], vn[4];
+  // ---- corrections: sums over the point pairs (c0 without hats as well: the
+  // derivative part of N)
+  cf vS[4], vD[4], vt[4], vN[4], vDm[4], vtm[4], v0 = {0.f, 0.f};
 #pragma unroll
-  for (int j = 0; j < 4; ++j) vS[j] = v0[j] = v1[j] = vt[j] = vgk[j] = vgt[j] = vn[j] = cf{0.f, 0.f};
+  for (int j = 0; j < 4; ++j) vS[j] = vD[j] = vt[j] = vN[j] = vDm[j] = vtm[j] = cf{0.f, 0.f};
   const float aef = ae.hi, agf = ag.hi, hir = F.hf * ir;
   const float bR = F.beta.hi * R0.hi;
   const float lte = hir * fmaf(dxh, tex.hi, dyh * tey.hi), ltg = hir * fmaf(dxh, tgx.hi, dyh * tgy.hi);
+  // source points: phase factor, tangential and curved displacement along d0, d0 . nu_r - o_r . n_r
+  constexpr int QR = Q ? Q : 1;
+  cf Zr_[QR];
+  float tr_[QR], er_[QR], Kr_[QR];
+  auto source = [&](int r, cf& Zr, float& tr, float& er, float& Kr) {
+    const float4 ra = pg[r].a;
+    far_cis(agf * F.s[r], Zr);
+    er = fmaf(ux, ra.z, uy * ra.w);
+    tr = fmaf(ltg, F.s[r], er);
+    Kr = fmaf(dxh, pg[r].b.x, dyh * pg[r].b.y) - pg[r].c;
+  };
+  if (Q) {
+#pragma unroll
+    for (int r = 0; r < QR; ++r) source(r, Zr_[r], tr_[r], er_[r], Kr_[r]);
+  }
 #pragma unroll 1
   for (int p = 0; p < q; ++p) {
     const float4 pa = pe[p].a, pb = pe[p].b;
     const float po2 = pe[p].o2;
-    const float xs = aef * F.s[p];
     cf Zp;
-    far_cis(xs, Zp);
+    far_cis(aef * F.s[p], Zp);
     const float ep = fmaf(ux, pa.z, uy * pa.w);        // d0 . (curved part) / R0
     const float tp = fmaf(lte, F.s[p], ep);
     const float Lp = fmaf(pb.z, sg, pb.w * ndh);       // o_p . n_f
     const float np = fmaf(pb.x, tgy.hi, -pb.y * tgx.hi);
-    cf uS[2], u0[2], u1[2], ut[2], ugk[2], ugt[2], un[2];
+    const float Kp = -fmaf(dxh, pb.x, dyh * pb.y) - pe[p].c;   // mirrored: -d0 . nu_p - o_p . n_p
+    cf uS[2], uD[2], ut[2], uN[2], uDm[2], utm[2], u0 = {0.f, 0.f};
 #pragma unroll
-    for (int b = 0; b < 2; ++b) uS[b] = u0[b] = u1[b] = ut[b] = ugk[b] = ugt[b] = un[b] = cf{0.f, 0.f};
+    for (int b = 0; b < 2; ++b) uS[b] = uD[b] = ut[b] = uN[b] = uDm[b] = utm[b] = cf{0.f, 0.f};
 #pragma unroll
     for (int r = 0; r < (Q ? Q : FAR_Q); ++r) {
       if (!Q && r >= q) break;
       const float4 ra = pg[r].a, rb = pg[r].b;
-      const float xr = agf * F.s[r];
       cf Zr;
-      far_cis(xr, Zr);
-      const float er = fmaf(ux, ra.z, uy * ra.w);
-      const float tr = fmaf(ltg, F.s[r], er);
+      float tr, er, Kr;
+      if (Q) {
+        Zr = Zr_[r < QR ? r : 0];
+        tr = tr_[r < QR ? r : 0];
+        er = er_[r < QR ? r : 0];
+        Kr = Kr_[r < QR ? r : 0];
+      } else {
+        source(r, Zr, tr, er, Kr);
+      }
       // rho = R / R0 - 1 = tau + x-terms, tau = d0.D / R0^2, D = o_p - o_r
       const float tau = (tp - tr) * ir;
       const float d2 = (fmaf(-2.f, fmaf(pa.x, ra.x, pa.y * ra.y), po2 + pg[r].o2)) * ir2;
       const float nu = fmaf(-tau, tau, d2);
-      const float o1 = 1.f + tau, io = 1.f / o1;
+      const float o1 = 1.f + tau, io = far_rcp(o1);
       const float x = nu * io * io;
       const float sec = o1 * x * fmaf(x, fmaf(x, 0.0625f, -0.125f), 0.5f);
       const float rho = tau + sec;
@@ -427,28 +482,39 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
       const cf q1 = {v * fmaf(v, b21.x, b11.x), v * fmaf(v, b21.y, b11.y)};
       const cf q0t = {v * fmaf(v, b20t.x, b10t.x), v * fmaf(v, b20t.y, b10t.y)};
       const cf q1t = {v * fmaf(v, b21t.x, b11t.x), v * fmaf(v, b21t.y, b11t.y)};
-      const cf m0 = cmul(q0, Pk), m1 = cmul(q1, Pk), m0t = cmul(q0t, Pt), m1t = cmul(q1t, Pt);
       // (r - r').n' / R = g0 + gd: (d0.nu_r + o_p.n_f + o_p.nu_r - o_r.n_r) / R0 - g0 rho, over 1 + rho
-      const float Kr = fmaf(dxh, rb.x, dyh * rb.y) - pg[r].c;
       const float sr = Kr + fmaf(pa.x, rb.x, fmaf(pa.y, rb.y, Lp));
       const float gd = fmaf(sr, ir, -g0h * rho) * (1.f + v);
       // n_p . n_r = nd0 + nn
       const float nn = np + fmaf(tey.hi, rb.x, fmaf(-tex.hi, rb.y, fmaf(pb.x, rb.x, pb.y * rb.y)));
-      const cf c0 = {Ck.x + m0.x, Ck.y + m0.y}, c1 = {Ck.x + m1.x, Ck.y + m1.y};
-      const cf cS = {Ct.x + m0t.x, Ct.y + m0t.y}, ct = {Ct.x + m1t.x, Ct.y + m1t.y};
-      const cf xk = {gd * (Pk.x + m1.x), gd * (Pk.y + m1.y)}, xt = {gd * (Pt.x + m1t.x), gd * (Pt.y + m1t.y)};
-      const cf xn = {nn * (Pk.x + m0.x), nn * (Pk.y + m0.y)};
+      // per function: c = C + q P (the kernel's deviation), then f0 c + fd (P + q P) = (f0 + fd) c + fd Z with
+      // f0, fd the factor at the centres and its deviation
+      const cf c0 = cfma(q0, Pk, Ck), c1 = cfma(q1, Pk, Ck), cS = cfma(q0t, Pt, Ct), ct = cfma(q1t, Pt, Ct);
+      const float gs = g0h + gd, ns = ndh + nn;
+      const cf yD = {fmaf(gs, c1.x, gd * Z.x), fmaf(gs, c1.y, gd * Z.y)};
+      const cf yt = {fmaf(gs, ct.x, gd * Z.x), fmaf(gs, ct.y, gd * Z.y)};
+      const cf yN = {fmaf(ns, c0.x, nn * Z.x), fmaf(ns, c0.y, nn * Z.y)};
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         const float wr = F.w[b][r];
         caxpy(uS[b], wr, cS);
-        caxpy(u0[b], wr, c0);
-        caxpy(u1[b], wr, c1);
-        caxpy(ut[b], wr, ct);
-        caxpy(ugk[b], wr, xk);
-        caxpy(ugt[b], wr, xt);
-        caxpy(un[b], wr, xn);
+        caxpy(uD[b], wr, yD);
+        caxpy(ut[b], wr, yt);
+        caxpy(uN[b], wr, yN);
       }
+      if (M) {
+        // o_r . n_p = o_r . n_e + o_r . nu_p, tau_f . n_e = -tau_e . n_f
+        const float sm = Kp + fmaf(ra.x, pb.x, fmaf(ra.y, pb.y, fmaf(-rb.z, sg, rb.w * ndh)));
+        const float gdm = fmaf(sm, ir, -gmh * rho) * (1.f + v), gsm = gmh + gdm;
+        const cf ym = {fmaf(gsm, c1.x, gdm * Z.x), fmaf(gsm, c1.y, gdm * Z.y)};
+        const cf yn = {fmaf(gsm, ct.x, gdm * Z.x), fmaf(gsm, ct.y, gdm * Z.y)};
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          caxpy(uDm[b], F.w[b][r], ym);
+          caxpy(utm[b], F.w[b][r], yn);
+        }
+      }
+      caxpy(u0, F.w1[r], c0);
     }
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
@@ -456,14 +522,16 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         caxpy(vS[a * 2 + b], wp, uS[b]);
-        caxpy(v0[a * 2 + b], wp, u0[b]);
-        caxpy(v1[a * 2 + b], wp, u1[b]);
+        caxpy(vD[a * 2 + b], wp, uD[b]);
         caxpy(vt[a * 2 + b], wp, ut[b]);
-        caxpy(vgk[a * 2 + b], wp, ugk[b]);
-        caxpy(vgt[a * 2 + b], wp, ugt[b]);
-        caxpy(vn[a * 2 + b], wp, un[b]);
+        caxpy(vN[a * 2 + b], wp, uN[b]);
+        if (M) {
+          caxpy(vDm[a * 2 + b], wp, uDm[b]);
+          caxpy(vtm[a * 2 + b], wp, utm[b]);
+        }
       }
     }
+    caxpy(v0, F.w1[p], u0);
   }
   // ---- tangential sums: A_0(alpha) = 1/2 + re + i (-alpha / 12 + im), A_1 = conj(A_0)
   float ree = 0.f, ime = 0.f, reg = 0.f, img = 0.f;
@@ -486,7 +554,7 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
   // A_a(alpha_e) conj(A_b(alpha_f)) - 1/4 = i lam_ab + M_ab; lam_ab = (-sa alpha_e + sb alpha_f) / 24 with s_0 = 1, s_1 = -1
   o.lam[0] = ff_mul(ff_add(ae, ff_neg(ag)), ff{0.0416666679f, -1.24176347e-09f});
   o.lam[1] = ff_mul(ff_add(ae, ag), ff{0.0416666679f, -1.24176347e-09f});
-  cf M[4];
+  cf T[4];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -494,7 +562,7 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
       const float sa = a ? -1.f : 1.f, sb = b ? -1.f : 1.f;
       // x = re_e + i sa lie, y = re_g - i sb lig (conjugated)
       const float xi = sa * lie, yi = -sb * lig;
-      M[a * 2 + b] = {fmaf(0.5f, ree + reg, fmaf(ree, reg, -xi * yi)),
+      T[a * 2 + b] = {fmaf(0.5f, ree + reg, fmaf(ree, reg, -xi * yi)),
                       fmaf(0.5f, fmaf(sa, ime, -sb * img), fmaf(ree, yi, reg * xi))};
     }
   // ---- assemble leads and corrections
@@ -507,25 +575,38 @@ WCS_HD void far_pair(const FarConsts& F, int q_run, const FarElem& E, const FarE
   // N: +-1 - k^2 h^2 nd0 / 4
   const ff mq = ff_mul(ff_mul(F.kk2h2, nd0), q4);
   o.lead[3] = ffc_mul(K0, ff_add_f(ff_neg(mq), 1.f));
-  o.lead[4] = ffc_mul(K0, ff_add_f(ff_neg(mq), -1.f));
+  o.lead[FarPair<M>::OPS] = ffc_mul(K0, ff_add_f(ff_neg(mq), -1.f));
   o.K[0] = t0;
   o.K[1] = {k1.x * g0h, k1.y * g0h};
   o.K[2] = {t1.x * g0h, t1.y * g0h};
-  cf sum0 = {0.f, 0.f};
+  o.K[3] = {0.f, 0.f};
+  if (M) {
+    const ff m4 = {0.25f * gm.hi, 0.25f * gm.lo};
+    o.lead[4] = ffc_mul(K1, m4);
+    o.lead[M ? 5 : 0] = ffc_mul(T1, m4);
+    o.K[M ? 4 : 0] = {k1.x * gmh, k1.y * gmh};
+    o.K[M ? 5 : 0] = {t1.x * gmh, t1.y * gmh};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      o.corr[M ? 4 : 0][j] = cmul(k1, {fmaf(gmh, T[j].x, vDm[j].x), fmaf(gmh, T[j].y, vDm[j].y)});
+      o.corr[M ? 5 : 0][j] = cmul(t1, {fmaf(gmh, T[j].x, vtm[j].x), fmaf(gmh, T[j].y, vtm[j].y)});
+    }
+  }
+  cf sum0 = v0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    sum0.x += v0[j].x + M[j].x;
-    sum0.y += v0[j].y + M[j].y;
+    sum0.x += T[j].x;
+    sum0.y += T[j].y;
   }
   const float kk = F.kk2h2.hi;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    o.corr[0][j] = cmul(t0, {vS[j].x + M[j].x, vS[j].y + M[j].y});
-    o.corr[1][j] = cmul(k1, {fmaf(g0h, v1[j].x + M[j].x, vgk[j].x), fmaf(g0h, v1[j].y + M[j].y, vgk[j].y)});
-    o.corr[2][j] = cmul(t1, {fmaf(g0h, vt[j].x + M[j].x, vgt[j].x), fmaf(g0h, vt[j].y + M[j].y, vgt[j].y)});
+    o.corr[0][j] = cmul(t0, {vS[j].x + T[j].x, vS[j].y + T[j].y});
+    o.corr[1][j] = cmul(k1, {fmaf(g0h, T[j].x, vD[j].x), fmaf(g0h, T[j].y, vD[j].y)});
+    o.corr[2][j] = cmul(t1, {fmaf(g0h, T[j].x, vt[j].x), fmaf(g0h, T[j].y, vt[j].y)});
     const float lm = ((j >= 2) ? 1.f : -1.f) * o.lam[(j == 1 || j == 2) ? 1 : 0].hi;
     const float sgn = (j == 0 || j == 3) ? 1.f : -1.f;
-    const cf c0 = {fmaf(ndh, v0[j].x + M[j].x, vn[j].x), fmaf(ndh, v0[j].y + M[j].y + lm, vn[j].y)};
+    const cf c0 = {fmaf(ndh, T[j].x, vN[j].x), fmaf(ndh, T[j].y + lm, vN[j].y)};
     o.corr[3][j] = cmul(k0, {fmaf(-kk, c0.x, sgn * sum0.x), fmaf(-kk, c0.y, sgn * sum0.y)});
   }
 }

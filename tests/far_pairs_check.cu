@@ -7,7 +7,7 @@
 using namespace wcs;
 
 // ce, cg: n x (x, y, nx, ny) centres; pe, pg: n x q x (x, y, nx, ny) points;
-// out: n x 4 operators x 4 (a * 2 + b) x (re, im)
+// out: n x 6 operators (S~, D, D~, N, D and D~ of (f, e)) x 4 (a * 2 + b) x (re, im)
 extern "C" void far_pairs(int q, const double* xi, const double* w, double k, double beta, double h, int n,
                           const double* ce, const double* cg, const double* pe, const double* pg, double* out) {
   FarConsts F;
@@ -21,13 +21,13 @@ extern "C" void far_pairs(int q, const double* xi, const double* w, double k, do
       P[p] = far_point(a[0], a[1], a[2], a[3], u[0], u[1], u[2], u[3], h, xi[p] - 0.5);
       R[p] = far_point(b[0], b[1], b[2], b[3], v[0], v[1], v[2], v[3], h, xi[p] - 0.5);
     }
-    FarPair o;
-    if (q == 4) far_pair<4>(F, q, E, G, P, R, o);
-    else far_pair<0>(F, q, E, G, P, R, o);
-    for (int op = 0; op < 4; ++op)
+    FarPair<true> o;
+    if (q == 4) far_pair<4, true>(F, q, E, G, P, R, o);
+    else far_pair<0, true>(F, q, E, G, P, R, o);
+    for (int op = 0; op < 6; ++op)
       for (int j = 0; j < 4; ++j) {
         const ffc v = o.value(op, j);
-        double* d = out + ((i * 4 + op) * 4 + j) * 2;
+        double* d = out + ((i * 6 + op) * 4 + j) * 2;
         d[0] = (double)v.x.hi + v.x.lo;
         d[1] = (double)v.y.hi + v.y.lo;
       }

@@ -66,7 +66,7 @@ def test_far_pairs_vs_fp64_quadrature(lib, family, N, q, kfac, bits):
     n = len(e)
     assert n > 100
     pe, pg = table(e, xi), table(f, xi)
-    out = np.zeros((n, 4, 4, 2))
+    out = np.zeros((n, 6, 4, 2))
     p = lambda v: v.ctypes.data_as(C.c_void_p)   # noqa: E731
     lib.far_pairs(q, p(xi), p(w), C.c_double(k), C.c_double(beta), C.c_double(h), n, p(ce), p(cg), p(pe), p(pg), p(out))
     got = out[..., 0] + 1j * out[..., 1]
@@ -78,9 +78,11 @@ def test_far_pairs_vs_fp64_quadrature(lib, family, N, q, kfac, bits):
     ck, ak = np.sqrt(2 / (np.pi * kt)), np.sqrt(2 / (np.pi * k))
     H0, H1, T0, T1 = hankel1(0, k * R) / ak, hankel1(1, k * R) / ak, hankel1(0, kt * R) / ck, hankel1(1, kt * R) / ck
     W = [w * (1 - xi), w * xi]
+    gm = -(d * pe[:, :, None, 2:]).sum(-1) / R                  # the mirrored pair's (r' - r).n / R
     amp = [0.25 * np.abs(x).max((1, 2)) for x in (T0, H0, T0)] + [np.abs(H0).max((1, 2))]
+    amp += amp[1:3]
     der = np.einsum("p,npr,r->n", w, H0, w)
-    for i, K in enumerate((T0, H1 * g, T1 * g, nd * H0)):
+    for i, K in enumerate((T0, H1 * g, T1 * g, nd * H0, H1 * gm, T1 * gm)):
         for ab in range(4):
             ref = np.einsum("p,npr,r->n", W[ab // 2], K, W[ab % 2])
             if i == 3:
