@@ -110,20 +110,34 @@ __global__ void k_panel_lengths(Contour c, int P, double* len) {
   len[j] = arc_int(c, j * dth, (j + 1) * dth);
 }
 
-__global__ void k_prefix_kahan(const double* len, int P, double* cum) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0, comp = 0.0;
-  cum[0] = 0.0;
-  for (int j = 0; j < P; ++j) {
-    double y = len[j] - comp;
-    double t = s + y;
-    comp = (t - s) - y;
-    s = t;
-    cum[j + 1] = s;
+// Compensated prefix sum, one after the other (its roundings are part of every
+// mesh point, so the order is kept): one thread walks the chain of four dependent
+// FP64 additions per panel, the block brings the lengths into shared memory and
+// the sums out of it (the same loop on global memory took 1.5 ms for 8192).
+__global__ void __launch_bounds__(512) k_prefix_kahan(const double* len, int P, double* cum) {
+  extern __shared__ double sl[];
+  for (int j = threadIdx.x; j < P; j += blockDim.x) sl[j] = len[j];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0, comp = 0.0;
+#pragma unroll 16
+    for (int j = 0; j < P; ++j) {
+      double y = sl[j] - comp;
+      double t = s + y;
+      comp = (t - s) - y;
+      s = t;
+      sl[j] = s;
+    }
   }
+  __syncthreads();
+  for (int j = threadIdx.x; j < P; j += blockDim.x) cum[j + 1] = sl[j];
+  if (threadIdx.x == 0) cum[0] = 0.0;
 }
 
-__device__ void point_at(const Contour& c, const double* cum, int P, double L, double s,
+// tol: Newton stops once a step is below it; the steps square the error, so 1e-9
+// leaves the root to rounding after two or three of them, and 1e-16 spends all
+// eight on rounding-level corrections.
+__device__ void point_at(const Contour& c, const double* cum, int P, double L, double s, double tol,
                          double& x, double& y, double& nx, double& ny, double& kap) {
   double th;
   if (c.family == FAM_CIRCLE && c.np == 0) {
@@ -144,7 +158,7 @@ __device__ void point_at(const Contour& c, const double* cum, int P, double L, d
       double F = arc_int(c, t0, th) - ds;
       double d = F / speed(c, th);
       th -= d;
-      if (fabs(d) < 1e-16) break;
+      if (fabs(d) < tol) break;
     }
   }
   double r0, r1, r2;
@@ -161,14 +175,14 @@ __device__ void point_at(const Contour& c, const double* cum, int P, double L, d
 }
 
 __global__ void k_points(Contour c, const double* cum, int P, double L, int64_t N, double h,
-                         const double* xi, int nq, Points out) {
+                         const double* xi, int nq, double tol, Points out) {
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= N * nq) return;
   int64_t e = idx / nq;
   int g = (int)(idx - e * nq);
   double s = ((double)e + xi[g]) * h;
   double x, y, nx, ny, kap;
-  point_at(c, cum, P, L, s, x, y, nx, ny, kap);
+  point_at(c, cum, P, L, s, tol, x, y, nx, ny, kap);
   out.x[idx] = x; out.y[idx] = y; out.nx[idx] = nx; out.ny[idx] = ny;
   if (out.kappa) out.kappa[idx] = kap;
 }
@@ -218,7 +232,14 @@ int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s) {
   }
   k_panel_lengths<<<(t.P + 127) / 128, 128, 0, s>>>(c, t.P, len);
   note_launch();
-  k_prefix_kahan<<<1, 32, 0, s>>>(len, t.P, t.cum);
+  static DeviceOnce attr;
+  const int smem = (int)sizeof(double) * t.P;
+  if (attr.need()) {
+    cudaError_t e = cudaFuncSetAttribute(k_prefix_kahan, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) { cudaFree(len); set_error(std::string("arc table: ") + cudaGetErrorString(e)); return 3; }
+    attr.done();
+  }
+  k_prefix_kahan<<<1, 512, smem, s>>>(len, t.P, t.cum);
   note_launch();
   double L = 0.0;
   cudaMemcpyAsync(&L, t.cum + t.P, sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -230,9 +251,9 @@ int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s) {
 }
 
 int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const double* xi_dev,
-                 int nq, Points& out, cudaStream_t s) {
+                 int nq, Points& out, cudaStream_t s, double tol) {
   int64_t n = N * nq;
-  k_points<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(c, t.cum, t.P, t.L, N, h, xi_dev, nq, out);
+  k_points<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(c, t.cum, t.P, t.L, N, h, xi_dev, nq, tol, out);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(cudaGetErrorString(err)); return 3; }

@@ -63,9 +63,10 @@ struct ArcTable {
 };
 
 int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s);
-// Points at arc lengths s_j = (e + xi[g]) * h for e < N, g < nq (index e*nq + g).
+// Points at arc lengths s_j = (e + xi[g]) * h for e < N, g < nq (index e*nq + g); tol: Newton step
+// that ends the inversion of the arc length.
 int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const double* xi_dev,
-                 int nq, Points& out, cudaStream_t s);
+                 int nq, Points& out, cudaStream_t s, double tol = 1e-16);
 // Minimum curvature over a dense sample of the contour (convexity check).
 int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, cudaStream_t s);
 

@@ -925,6 +925,9 @@ int wcs_contour_perturb(wcs_ctx* c, int M, const double* alpha, const double* be
   return set_contour(c, k);
 }
 
+// The mixed form's points need what its 24-bit entries do; the FP64 form keeps every bit.
+static double mesh_tol(const wcs_ctx* c) { return c->mixed ? 1e-9 : 1e-16; }
+
 static int build_points(wcs_ctx* c, const Contour& k, const ArcTable& t, DevBuf& buf, Points& P,
                         const double* xi_dev, int q, bool with_kappa) {
   const int64_t n = c->N * q;
@@ -932,7 +935,7 @@ static int build_points(wcs_ctx* c, const Contour& k, const ArcTable& t, DevBuf&
   double* b = buf.d();
   P.x = b; P.y = b + n; P.nx = b + 2 * n; P.ny = b + 3 * n; P.kappa = with_kappa ? b + 4 * n : nullptr;
   P.n = n;
-  return points_build(k, t, c->N, c->h, xi_dev, q, P, c->s);
+  return points_build(k, t, c->N, c->h, xi_dev, q, P, c->s, mesh_tol(c));
 }
 
 int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
@@ -956,7 +959,7 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   c->circle = Contour{};
   c->circle.family = FAM_CIRCLE;
   c->circle.a = c->a;
-  TRY(arc_table_build(c->circle, c->arc_c, c->s));
+  c->arc_c.L = c->L;   // points of a circle need no arc-length table
   // rules on device
   const int qf = c->opt.q_far, qn = c->opt.q_near;
   TRY(c->xf.ensure(sizeof(double) * 16));
@@ -1095,7 +1098,7 @@ int wcs_assemble(wcs_ctx* c) {
     cudaMemcpyAsync(half, &hv, sizeof(double), cudaMemcpyHostToDevice, c->s);
     Points cp;
     cp.x = c->centres.d(); cp.y = cp.x + N; cp.nx = cp.y + N; cp.ny = cp.nx + N; cp.kappa = nullptr; cp.n = N;
-    TRY(points_build(c->contour, c->arc, N, c->h, half, 1, cp, c->s));
+    TRY(points_build(c->contour, c->arc, N, c->h, half, 1, cp, c->s, mesh_tol(c)));
     TRY(c->offs.ensure(sizeof(FarElem) * N + sizeof(FarPoint) * N * qf));
     FarElem* fe = (FarElem*)c->offs.p;
     FarPoint* fp = (FarPoint*)(fe + N);
