@@ -206,6 +206,7 @@ __global__ void k_splitk_reduce(TcArgs a, int splits) {
     if (t >= plane) return;
     const int row = (int)(t % a.M), col = (int)(t / a.M);
     double sum = 0.0;
+#pragma unroll 8
     for (int z = 0; z < splits; ++z) sum += (double)a.ws[z * plane + t];
     double* o = (double*)a.out + (int64_t)row * a.ldo + col;
     *o = a.alpha.x * sum + ((a.beta.x == 0.0) ? 0.0 : a.beta.x * (*o));
@@ -216,6 +217,7 @@ __global__ void k_splitk_reduce(TcArgs a, int splits) {
   const int row = (int)(t % a.M), j = (int)(t / a.M);
   const float* w = a.ws + (int64_t)(2 * j) * a.M + row;
   double re = 0.0, im = 0.0;
+#pragma unroll 8
   for (int z = 0; z < splits; ++z) {
     re += (double)w[z * plane];
     im += (double)w[z * plane + a.M];
@@ -252,6 +254,26 @@ struct AccSmem {
   static constexpr int TOTAL = STAGES * STAGE_BYTES + 1024 + 256;
 };
 
+// K splits of a launch (the host picks kper so that every split has work)
+static unsigned tc_splits(const TcArgs& a) {
+  const int nk = (a.K + TC_BK - 1) / TC_BK;
+  return a.kper > 0 ? (unsigned)((nk + a.kper - 1) / a.kper) : 1u;
+}
+
+// 32 columns of one row: the epilogue, or the split's FP32 partial, column-major
+// [split][Nc][M] (a warp writes 32 consecutive rows per column)
+__device__ __forceinline__ void tile_store(const TcArgs& a, int row, int col0, const float (&v)[32]) {
+  if (!a.ws) {
+    epilogue_store(a, row, col0, v);
+    return;
+  }
+  if (row >= a.M) return;
+  float* w = a.ws + (int64_t)blockIdx.z * a.Nc * a.M + row;
+#pragma unroll
+  for (int i = 0; i < 32; ++i)
+    if (col0 + i < a.Nc) w[(int64_t)(col0 + i) * a.M] = v[i];
+}
+
 template <int PA, int PB, int STAGES>
 __global__ void __launch_bounds__(ACC_THREADS, 1)
     k_gemm_tc_acc(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
@@ -273,7 +295,9 @@ __global__ void __launch_bounds__(ACC_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * TC_BM;
   const int n0 = blockIdx.x * ACC_NT;
-  const int nk = (args.K + TC_BK - 1) / TC_BK;
+  const int nk_all = (args.K + TC_BK - 1) / TC_BK;
+  const int kb0 = (args.kper > 0) ? (int)blockIdx.z * args.kper : 0;   // split-K: k-blocks [kb0, kb0 + nk)
+  const int nk = (args.kper > 0) ? min(args.kper, nk_all - kb0) : nk_all;
   const int nsteps = nk * (TC_BK / 16);
   // accumulation groups: `drain` consecutive K = 16 steps share one TMEM
   // buffer before it is drained (1: every step)
@@ -316,7 +340,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 1)
         if (*abort_flag) break;
         uint8_t* sp = smem + st * L::STAGE_BYTES;
         mbar_expect_tx(&full[st], L::STAGE_BYTES);
-        const int k0 = kb * TC_BK;
+        const int k0 = (kb0 + kb) * TC_BK;
 #pragma unroll
         for (int p = 0; p < PA; ++p) tma_load_2d(sp + p * L::A_BYTES, mapA[p], &full[st], k0, m0);
 #pragma unroll
@@ -442,10 +466,10 @@ __global__ void __launch_bounds__(ACC_THREADS, 1)
     tmem_ld64(tmem + ((uint32_t)lanebase << 16) + (uint32_t)(ACC_OUTER + colhalf), v);
 #pragma unroll
     for (int i = 0; i < 32; ++i) out[i] = v[i] + inner[i];
-    epilogue_store(args, m0 + lanebase + lane, n0 + colhalf, out);
+    tile_store(args, m0 + lanebase + lane, n0 + colhalf, out);
 #pragma unroll
     for (int i = 0; i < 32; ++i) out[i] = v[32 + i] + inner[32 + i];
-    epilogue_store(args, m0 + lanebase + lane, n0 + colhalf + 32, out);
+    tile_store(args, m0 + lanebase + lane, n0 + colhalf + 32, out);
   }
   tc_fence_before();
   __syncthreads();
@@ -471,7 +495,7 @@ static int launch_tc_acc(const TcOperand& A, const TcOperand& B, TcArgs& args, c
     if (e != cudaSuccess) { set_error(std::string("gemm_tc: shared-memory opt-in: ") + cudaGetErrorString(e)); return 3; }
     attr.done();
   }
-  dim3 grid((unsigned)((args.Nc + ACC_NT - 1) / ACC_NT), (unsigned)((args.M + TC_BM - 1) / TC_BM));
+  dim3 grid((unsigned)((args.Nc + ACC_NT - 1) / ACC_NT), (unsigned)((args.M + TC_BM - 1) / TC_BM), tc_splits(args));
   kern<<<grid, ACC_THREADS, L::TOTAL, s>>>(ma[0], ma[1], ma[2], mb[0], mb[1], mb[2], args);
   note_launch();
   cudaError_t e = cudaGetLastError();
@@ -519,7 +543,9 @@ __global__ void __launch_bounds__(PER_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * TC_BM;
   const int n0 = blockIdx.x * PER_NT;
-  const int nk = (args.K + TC_BK - 1) / TC_BK;
+  const int nk_all = (args.K + TC_BK - 1) / TC_BK;
+  const int kb0 = (args.kper > 0) ? (int)blockIdx.z * args.kper : 0;
+  const int nk = (args.kper > 0) ? min(args.kper, nk_all - kb0) : nk_all;
   const int nsteps = nk * (TC_BK / 16);
   const int drain = args.drain > 1 ? args.drain : 1;
   const int ngroups = (nsteps + drain - 1) / drain;
@@ -558,7 +584,7 @@ __global__ void __launch_bounds__(PER_THREADS, 1)
         if (*abort_flag) break;
         uint8_t* sp = smem + st * L::STAGE_BYTES;
         mbar_expect_tx(&full[st], L::STAGE_BYTES);
-        const int k0 = kb * TC_BK;
+        const int k0 = (kb0 + kb) * TC_BK;
         tma_load_2d(sp, &mA0, &full[st], k0, m0);
         tma_load_2d(sp + L::A_BYTES, &mA1, &full[st], k0, m0);
         tma_load_2d(sp + 2 * L::A_BYTES, &mB0, &full[st], k0, n0);
@@ -647,7 +673,7 @@ __global__ void __launch_bounds__(PER_THREADS, 1)
       float out[32];
 #pragma unroll
       for (int i = 0; i < 32; ++i) out[i] = sum[32 * c4 + i];
-      epilogue_store(args, m0 + lanebase + lane, n0 + colbase + 32 * c4, out);
+      tile_store(args, m0 + lanebase + lane, n0 + colbase + 32 * c4, out);
     }
   }
   tc_fence_before();
@@ -672,12 +698,44 @@ static int launch_tc_per(const TcOperand& A, const TcOperand& B, TcArgs& args, c
     if (e != cudaSuccess) { set_error(std::string("gemm_tc: shared-memory opt-in: ") + cudaGetErrorString(e)); return 3; }
     attr.done();
   }
-  dim3 grid((unsigned)((args.Nc + PER_NT - 1) / PER_NT), (unsigned)((args.M + TC_BM - 1) / TC_BM));
+  dim3 grid((unsigned)((args.Nc + PER_NT - 1) / PER_NT), (unsigned)((args.M + TC_BM - 1) / TC_BM), tc_splits(args));
   kern<<<grid, PER_THREADS, L::TOTAL, s>>>(ma[0], ma[1], mb[0], mb[1], args);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error(std::string("gemm_tc_per launch: ") + cudaGetErrorString(e)); return 3; }
   return 0;
+}
+
+static int launch_splitk_reduce(const TcArgs& args, int splits, cudaStream_t s) {
+  const int64_t n = (int64_t)args.M * ((args.epi == EPI_RAW_F64) ? args.Nc : args.Nc / 2);
+  k_splitk_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(args, splits);
+  note_launch();
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { set_error(std::string("split-K reduce: ") + cudaGetErrorString(e)); return 3; }
+  return 0;
+}
+
+// k-blocks per split of a drained product (0: no split).  A launch takes whole
+// waves of 152 CTAs, so a grid of 24 or 192 tiles leaves most of the chip idle in
+// its only or last wave; splitting K evens it out at the price of the partials
+// (written and read once, FP32, summed in FP64) and of a prologue and epilogue per
+// CTA.  Microseconds: a K = 64 block of a 128 x 128 tile is 0.8 with three planes
+// (24 MMAs of 64 clocks) and 0.4 with two, of a 128 x 256 tile with two 0.8; about
+// 4 per CTA; 8 bytes per partial at 5 TB/s and a 4 us reduction launch.
+static int acc_kper(const TcArgs& a, int nt, int planes) {
+  if (!a.ws || !(a.epi == EPI_RAW_F64 || (a.epi == EPI_CPLX_F64 && (a.Nc % 2) == 0))) return 0;
+  const int nk = (a.K + TC_BK - 1) / TC_BK;
+  const int64_t tiles = (int64_t)((a.Nc + nt - 1) / nt) * ((a.M + TC_BM - 1) / TC_BM);
+  const double block = (planes == 3 || nt == PER_NT) ? 0.8 : 0.4, part = 8.0e-6 / 5.0 * (double)a.M * a.Nc;
+  double best = 1e300;
+  int kper = 0;
+  for (int sp = 1; sp <= std::min(64, nk / 4 > 0 ? nk / 4 : 1); ++sp) {
+    if (sp > 1 && (int64_t)sp * a.Nc * a.M > a.ws_elems) break;
+    const int per = (nk + sp - 1) / sp;
+    const double t = (double)((tiles * sp + 151) / 152) * (per * block + 4.0) + (sp > 1 ? sp * part + 4.0 : 0.0);
+    if (t < best) { best = t; kper = sp > 1 ? per : 0; }
+  }
+  return kper;
 }
 
 int gemm_tc_accurate(const TcOperand& A, const TcOperand& B, TcArgs args, cudaStream_t s) {
@@ -694,13 +752,19 @@ int gemm_tc_accurate(const TcOperand& A, const TcOperand& B, TcArgs args, cudaSt
     for (int p = 0; same && p < ref.nprod; ++p) same = (args.ia[p] == ref.ia[p] && args.ib[p] == ref.ib[p]);
     if (!same) { set_error("gemm_tc_accurate: needs the full product list of tc_products"); return 1; }
   }
-  if (A.planes == 3 && B.planes == 3) return launch_tc_acc<3, 3, 2>(A, B, args, s);
   // two planes drained every 16 or more steps on a grid of more than one
   // column tile: the wide-tile kernel
-  if (A.planes == 2 && B.planes == 2 && args.drain >= 16 && args.Nc > 128) return launch_tc_per<2>(A, B, args, s);
-  if (A.planes == 2 && B.planes == 2) return launch_tc_acc<2, 2, 3>(A, B, args, s);
-  set_error("gemm_tc_accurate: plane combination not built");
-  return 1;
+  const bool wide = A.planes == 2 && B.planes == 2 && args.drain >= 16 && args.Nc > 128;
+  args.kper = acc_kper(args, wide ? PER_NT : ACC_NT, A.planes);
+  if (args.kper == 0) args.ws = nullptr;
+  const int splits = (int)tc_splits(args);
+  int r = 1;
+  if (A.planes == 3 && B.planes == 3) r = launch_tc_acc<3, 3, 2>(A, B, args, s);
+  else if (wide) r = launch_tc_per<2>(A, B, args, s);
+  else if (A.planes == 2 && B.planes == 2) r = launch_tc_acc<2, 2, 3>(A, B, args, s);
+  else set_error("gemm_tc_accurate: plane combination not built");
+  if (r || splits == 1) return r;
+  return launch_splitk_reduce(args, splits, s);
 }
 
 int gemm_tc_split_plan(int M, int Nc, int K, int planesA, int planesB, int epi, int64_t* ws_elems) {
@@ -762,12 +826,7 @@ int gemm_tc(const TcOperand& A, const TcOperand& B, TcArgs args, cudaStream_t s)
     default: set_error("gemm_tc: plane combination not built"); return 1;
   }
   if (r || args.no_reduce || splits == 1) return r;
-  const int64_t n = (int64_t)args.M * ((args.epi == EPI_RAW_F64) ? args.Nc : args.Nc / 2);
-  k_splitk_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(args, splits);
-  note_launch();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) { set_error(std::string("split-K reduce: ") + cudaGetErrorString(e)); return 3; }
-  return 0;
+  return launch_splitk_reduce(args, splits, s);
 }
 
 }  // namespace wcs
