@@ -159,6 +159,32 @@ int split_complex_rows(const zd* X, int64_t rows, int64_t cols, int64_t ld, int 
 int stage_rhs(const zd* X, int64_t n, int64_t B, int64_t ldx, int conj_in, int planes, uint16_t* const* P,
               int64_t ldp, cudaStream_t s);
 
+// The vector algebra between two operator products of the mixed form, fused with
+// the staging of the second: y = G^-1 (x + ca add) + cz z for each column, as the
+// planes of stage_rhs and, when y is given, in FP64.  y must not overlap x, add
+// or z.
+struct GramStage {
+  int64_t n = 0;
+  const zd* x = nullptr;
+  int64_t ldx = 0;
+  const zd* add = nullptr;
+  int64_t ld_add = 0;
+  zd ca = {0.0, 0.0};
+  const zd* z = nullptr;
+  int64_t ldz = 0;
+  double cz = 0.0;
+  zd* y = nullptr;
+  int64_t ldy = 0;
+  int conj = 0, planes = 0;
+  uint16_t* P[3] = {nullptr, nullptr, nullptr};
+  int64_t ldp = 0;
+  double rho = 0.0, scale = 0.0;   // set by gram_stage
+};
+int gram_stage(GramStage g, int64_t cols, double h, cudaStream_t s);
+// out = cb b + c1 (p + g G t) (b optional; out may be p or b)
+int gram_combine(const zd* p, int64_t ldp, const zd* t, int64_t ldt, double g, double c1, const zd* b, int64_t ldb,
+                 double cb, zd* out, int64_t ldo, int64_t n, int64_t cols, double h, cudaStream_t s);
+
 // Stage a strided complex matrix view (element (i, j) at X[i*rs + j*cs],
 // optionally conjugated) as real rows x 2cols bf16 planes (K-major A operand).
 int stage_view(const zd* X, int64_t rows, int64_t cols, int64_t rs, int64_t cs, int conj, int planes,

@@ -479,38 +479,65 @@ static int apply_C_exact(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ld
   return 0;
 }
 
+// What becomes of a product P = C X (or C^H X) of the mixed form: out = cb b + c1 P,
+// formed in the kernel that adds its Gram term.
+struct Finish {
+  const zd* b = nullptr;
+  int64_t ldb = 0;
+  double cb = 0.0, c1 = 1.0;
+  zd* out = nullptr;
+  int64_t ldo = 0;
+};
+
+// G^-1 (X + ca add) + cz Z staged into buf, and in FP64 into Y when given
+static int ginv_stage(wcs_ctx* c, DevBuf& buf, const zd* X, int64_t ldx, const zd* add, int64_t ld_add, zd ca,
+                      const zd* Z, int64_t ldz, double cz, zd* Y, int64_t ldy, int64_t cols, int conj) {
+  GramStage g;
+  g.n = c->N;
+  g.x = X; g.ldx = ldx;
+  g.add = add; g.ld_add = ld_add; g.ca = ca;
+  g.z = Z; g.ldz = ldz; g.cz = cz;
+  g.y = Y; g.ldy = ldy;
+  g.conj = conj;
+  g.planes = c->rhs_planes;
+  for (int p = 0; p < c->rhs_planes; ++p) g.P[p] = (uint16_t*)buf.p + p * 2 * c->stage_cols * c->ldp;
+  g.ldp = c->ldp;
+  return gram_stage(g, cols, c->h, c->s);
+}
+
+// C X (adj: C^H X) in the given precision; Y receives the operator products, fin
+// says where the result goes (null: Y).  Uses w1, w2; G^-1 (T + G X / 2) is
+// formed as G^-1 T + X / 2.
 static int apply_C_mixed(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t cols, bool adj,
-                         int acc) {
-  if (acc == PREC_EXACT && !adj) return apply_C_exact(c, X, ldx, Y, ldy, cols);
+                         int acc, const Finish* fin = nullptr) {
+  Finish own;
+  own.out = Y;
+  own.ldo = ldy;
+  const Finish& F = fin ? *fin : own;
+  if (acc == PREC_EXACT && !adj) {
+    TRY(apply_C_exact(c, X, ldx, Y, ldy, cols));
+    if (!fin) return 0;
+    if (F.out == Y) return axpby(c->N, cols, mkz(F.cb), F.b, F.ldb, mkz(F.c1), Y, ldy, c->s);
+    return axpby(c->N, cols, mkz(F.c1), Y, ldy, mkz(F.cb), F.out, F.ldo, c->s);   // b is out
+  }
   if (acc == PREC_EXACT) acc = PREC_ACCURATE;   // adjoint products: the drained split-bf16 product
   const int64_t N = c->N;
   zd* T1 = c->w1.z();
   zd* T2 = c->w2.z();
   const zd one = mkz(1.0), zero = mkz(0.0), mone = mkz(-1.0);
   TRY(ensure_stage(c, cols));
+  TRY(c->gwork.ensure(sizeof(zd) * N * cols));
+  zd* V1 = c->gwork.z();
   const int cj = adj ? 1 : 0;
   TRY(stage(c, c->stage0, X, ldx, cols, cj));
-  if (!adj) {
-    TRY(tc_apply(c, 1, false, c->stage0, cols, mone, zero, T1, N, acc));   // -D X
-    TRY(tc_apply(c, 3, false, c->stage0, cols, one, zero, T2, N, acc));    // N X
-  } else {
-    TRY(tc_apply(c, 2, true, c->stage0, cols, one, zero, T1, N, acc));     // D~^H X
-    TRY(tc_apply(c, 0, true, c->stage0, cols, one, zero, T2, N, acc));     // S~^H X
-  }
-  TRY(gram_apply(X, ldx, T1, N, N, cols, c->h, 0.5, 1.0, c->s));
-  TRY(ginv(c, T1, N, T1, N, cols));
-  TRY(ginv(c, T2, N, T2, N, cols));
-  TRY(stage(c, c->stage1, T1, N, cols, cj));
-  TRY(stage(c, c->stage2, T2, N, cols, cj));
-  if (!adj) {
-    TRY(tc_apply(c, 2, false, c->stage1, cols, one, zero, Y, ldy, acc));   // D~ T1
-    TRY(tc_apply(c, 0, false, c->stage2, cols, one, one, Y, ldy, acc));    // + S~ T2
-  } else {
-    TRY(tc_apply(c, 1, true, c->stage1, cols, mone, zero, Y, ldy, acc));   // -D^H T1
-    TRY(tc_apply(c, 3, true, c->stage2, cols, one, one, Y, ldy, acc));     // + N^H T2
-  }
-  TRY(gram_apply(T1, N, Y, ldy, N, cols, c->h, 0.5, 1.0, c->s));
-  return 0;
+  // forward: -D X, N X, then D~ and S~; adjoint: D~^H X, S~^H X, then -D^H and N^H
+  TRY(tc_apply(c, adj ? 2 : 1, adj, c->stage0, cols, adj ? one : mone, zero, T1, N, acc));
+  TRY(tc_apply(c, adj ? 0 : 3, adj, c->stage0, cols, one, zero, T2, N, acc));
+  TRY(ginv_stage(c, c->stage1, T1, N, nullptr, 0, zero, X, ldx, 0.5, V1, N, cols, cj));
+  TRY(ginv_stage(c, c->stage2, T2, N, nullptr, 0, zero, nullptr, 0, 0.0, nullptr, 0, cols, cj));
+  TRY(tc_apply(c, adj ? 1 : 2, adj, c->stage1, cols, adj ? mone : one, zero, Y, ldy, acc));
+  TRY(tc_apply(c, adj ? 3 : 0, adj, c->stage2, cols, one, one, Y, ldy, acc));
+  return gram_combine(Y, ldy, V1, N, 0.5, F.c1, F.b, F.ldb, F.cb, F.out, F.ldo, N, cols, c->h, c->s);
 }
 
 // Y = C X (adjoint: C^H X); uses w1, w2 as temporaries.  Y must not alias X.
@@ -573,9 +600,18 @@ static int apply_Cc(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ldy, in
 // Y = (C - C_c) X or its adjoint; uses w1, w2, w3.
 static int apply_remainder(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t cols,
                            bool adj, int mode = PREC_FAST) {
-  TRY(apply_C(c, X, ldx, Y, ldy, cols, adj, mode));
   zd* T3 = c->w3.z();
   TRY(apply_Cc(c, X, ldx, T3, c->N, cols, adj ? 1 : 0));
+  if (c->mixed) {
+    Finish f;
+    f.b = T3;
+    f.ldb = c->N;
+    f.cb = -1.0;
+    f.out = Y;
+    f.ldo = ldy;
+    return apply_C_mixed(c, X, ldx, Y, ldy, cols, adj, mode, &f);
+  }
+  TRY(apply_C(c, X, ldx, Y, ldy, cols, adj, mode));
   TRY(axpby(c->N, cols, mkz(-1.0), T3, c->N, mkz(1.0), Y, ldy, c->s));
   return 0;
 }
@@ -1914,18 +1950,19 @@ static int precondition(wcs_ctx* c, const zd* e, const zd* hv, int64_t ld, zd* b
   const int64_t N = c->N;
   zd* T1 = c->w1.z();
   zd* T2 = c->w2.z();
-  TRY(ginv(c, e, ld, T1, N, cc));
-  TRY(ginv(c, hv, ld, T2, N, cc));
   if (c->mixed) {
     TRY(ensure_stage(c, cc));
-    TRY(stage(c, c->stage1, T1, N, cc, 0));
-    TRY(stage(c, c->stage2, T2, N, cc, 0));
-    TRY(tc_apply(c, 0, false, c->stage1, cc, mkz(0.0, -c->k), mkz(0.0), b, ldb, mode));
+    const zd zero = mkz(0.0);
+    TRY(ginv_stage(c, c->stage1, e, ld, nullptr, 0, zero, nullptr, 0, 0.0, nullptr, 0, cc, 0));
+    TRY(ginv_stage(c, c->stage2, hv, ld, nullptr, 0, zero, nullptr, 0, 0.0, T2, N, cc, 0));
+    TRY(tc_apply(c, 0, false, c->stage1, cc, mkz(0.0, -c->k), zero, b, ldb, mode));
     TRY(tc_apply(c, 2, false, c->stage2, cc, mkz(-1.0), mkz(1.0), b, ldb, mode));
-  } else {
-    TRY(cz(c, N, cc, N, mkz(0.0, -c->k), op_view(c->S, c->ld, false), blk(T1, N), mkz(0.0), b, ldb));
-    TRY(cz(c, N, cc, N, mkz(-1.0), op_view(c->Dt, c->ld, false), blk(T2, N), mkz(1.0), b, ldb));
+    return gram_combine(b, ldb, T2, N, -0.5, 1.0, nullptr, 0, 0.0, b, ldb, N, cc, c->h, c->s);
   }
+  TRY(ginv(c, e, ld, T1, N, cc));
+  TRY(ginv(c, hv, ld, T2, N, cc));
+  TRY(cz(c, N, cc, N, mkz(0.0, -c->k), op_view(c->S, c->ld, false), blk(T1, N), mkz(0.0), b, ldb));
+  TRY(cz(c, N, cc, N, mkz(-1.0), op_view(c->Dt, c->ld, false), blk(T2, N), mkz(1.0), b, ldb));
   TRY(gram_apply(T2, N, b, ldb, N, cc, c->h, -0.5, 1.0, c->s));
   return 0;
 }
@@ -1953,20 +1990,16 @@ static int residual_rhs_mixed(wcs_ctx* c, const zd* e, const zd* hv, int64_t ld,
     return 0;
   }
   TRY(ensure_stage(c, cc));
+  TRY(c->gwork.ensure(sizeof(zd) * N * cc));
+  zd* V1 = c->gwork.z();
   TRY(stage(c, c->stage0, x, ldx, cc, 0));
   TRY(tc_apply(c, 1, false, c->stage0, cc, mone, zero, T1, N, mode));   // -D x
   TRY(tc_apply(c, 3, false, c->stage0, cc, one, zero, T2, N, mode));    // N x
-  TRY(gram_apply(x, ldx, T1, N, N, cc, c->h, 0.5, 1.0, c->s));          // + G x / 2
-  TRY(axpby(N, cc, one, hv, ld, one, T1, N, c->s));                     // + h
-  TRY(axpby(N, cc, mkz(0.0, c->k), e, ld, one, T2, N, c->s));           // + i k e
-  TRY(ginv(c, T1, N, T1, N, cc));
-  TRY(ginv(c, T2, N, T2, N, cc));
-  TRY(stage(c, c->stage1, T1, N, cc, 0));
-  TRY(stage(c, c->stage2, T2, N, cc, 0));
-  TRY(tc_apply(c, 2, false, c->stage1, cc, mone, zero, R, N, mode));    // -D~ T1
-  TRY(tc_apply(c, 0, false, c->stage2, cc, mone, one, R, N, mode));     // - S~ T2
-  TRY(gram_apply(T1, N, R, N, N, cc, c->h, -0.5, 1.0, c->s));           // - G T1 / 2
-  return 0;
+  TRY(ginv_stage(c, c->stage1, T1, N, hv, ld, one, x, ldx, 0.5, V1, N, cc, 0));                       // G^-1 (T1 + h) + x / 2
+  TRY(ginv_stage(c, c->stage2, T2, N, e, ld, mkz(0.0, c->k), nullptr, 0, 0.0, nullptr, 0, cc, 0));    // G^-1 (T2 + i k e)
+  TRY(tc_apply(c, 2, false, c->stage1, cc, mone, zero, R, N, mode));    // -D~ V1
+  TRY(tc_apply(c, 0, false, c->stage2, cc, mone, one, R, N, mode));     // - S~ V2
+  return gram_combine(R, N, V1, N, -0.5, 1.0, nullptr, 0, 0.0, R, N, N, cc, c->h, c->s);   // - G V1 / 2
 }
 
 // x = C^{-1} b with Woodbury + iterative refinement on the exact operator.
@@ -2033,13 +2066,28 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
     }
     return 0;
   };
+  // R = v - (C X), the finish of a mixed product
+  Finish fin;
+  auto minus = [&](const zd* v, int64_t ldv) -> const Finish& {
+    fin.b = v;
+    fin.ldb = ldv;
+    fin.cb = 1.0;
+    fin.c1 = -1.0;
+    fin.out = R;
+    fin.ldo = N;
+    return fin;
+  };
   // R = b - C x with the given precision
   auto residual = [&](int mode, double& worst) -> int {
     if (c->mixed && e && hv && !adj) {
       TRY(residual_rhs_mixed(c, e, hv, ld_eh, x, ldx, R, cc, mode));
     } else {
-      TRY(apply_C(c, x, ldx, R, N, cc, adj, mode));
-      TRY(axpby(N, cc, mkz(1.0), b, ldb, mkz(-1.0), R, N, c->s));
+      if (c->mixed) {
+        TRY(apply_C_mixed(c, x, ldx, R, N, cc, adj, mode, &minus(b, ldb)));
+      } else {
+        TRY(apply_C(c, x, ldx, R, N, cc, adj, mode));
+        TRY(axpby(N, cc, mkz(1.0), b, ldb, mkz(-1.0), R, N, c->s));
+      }
     }
     return worst_of(worst);
   };
@@ -2086,8 +2134,7 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
         ++it;
         if (ends_round(upd, prev_upd)) break;
         const int m = (upd > 5e-5) ? PREC_EXACT : (upd > 5e-7 ? PREC_ACCURATE : PREC_PERIODIC);
-        TRY(apply_C(c, dx, N, T, N, cc, adj, m));
-        TRY(axpby(N, cc, mkz(-1.0), T, N, mkz(1.0), R, N, c->s));
+        TRY(apply_C_mixed(c, dx, N, T, N, cc, adj, m, &minus(R, N)));
         prev_upd = upd;
         TRY(worst_of(upd));
       }
@@ -2120,8 +2167,7 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
         // (~2e-7) carries it instead, so the carried residual does not drift
         // from the true one
         const int m = (2e-5 * upd <= 0.1 * c->opt.refine_tol) ? PREC_PERIODIC : PREC_ACCURATE;
-        TRY(apply_C(c, dx, N, T, N, cc, adj, m));
-        TRY(axpby(N, cc, mkz(-1.0), T, N, mkz(1.0), R, N, c->s));
+        TRY(apply_C_mixed(c, dx, N, T, N, cc, adj, m, &minus(R, N)));
         prev_upd = upd;
         TRY(worst_of(upd));
       }
