@@ -24,19 +24,6 @@ struct ExactOperand {
 // exponent table for `rows` rows of K values.
 int exact_operand_alloc_bytes(int64_t rows, int64_t K, int64_t* ld, int64_t* nchunks, size_t* slice_bytes,
                               size_t* expo_bytes);
-// Slices of an operator held as split-bf16 planes (row-major, ld_planes).
-int exact_slice_planes(const uint16_t* const* planes, int nplanes, int64_t rows, int64_t K, int64_t ld_planes,
-                       const ExactOperand& out, cudaStream_t s);
-// Slices of a right-hand block X (n x cols complex, column-major ldx) in the
-// real K-major layout of the complex product (see stage_rhs).
-int exact_slice_rhs(const zd* X, int64_t n, int64_t cols, int64_t ldx, int conj_in, const ExactOperand& out,
-                    cudaStream_t s);
-// out = beta * out + alpha * (A x) for the ncols complex columns of B, exact
-// up to the FP64 sums of the scaled integer partials.  ws: FP32 workspace of
-// nchunks * 2 ncols * M values.
-int exact_product(const ExactOperand& A, int M, const ExactOperand& B, int ncols, int K, zd alpha, zd beta,
-                  int conj_out, zd* out, int64_t ldo, float* ws, int64_t ws_elems, int* err, cudaStream_t s);
-
 // Real rows (rows x K, row-major FP64, ld) as slices; and the exact real
 // product D (M x Nc, row-major FP64, ldd) = A B^T (ws: nchunks * Nc * M floats).
 int exact_slice_real(const double* X, int64_t rows, int64_t K, int64_t ld, const ExactOperand& out, cudaStream_t s);

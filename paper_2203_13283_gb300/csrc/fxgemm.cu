@@ -39,15 +39,19 @@
 
 namespace wcs {
 
-constexpr int FX_BM = 128, FX_BN = 64, FX_BK = 32, FX_CHUNK = 4, FX_STAGES = 2, FX_THREADS = 320;
+constexpr int FX_BM = 128, FX_BN = 64, FX_BK = 32, FX_CHUNK = 4, FX_THREADS = 320;
 constexpr int FX_BAD = 1 << 20;                       // row exponent of a row that is not finite
-constexpr int FX_TOP = 8 * (FX_SLICES - 1) + 6;       // fixed-point position: |v| 2^(FX_TOP - E) < 2^FX_TOP
-constexpr int FX_ROW = FX_SLICES * FX_BK;             // bf16 values of one row and stage
-constexpr int FX_A_BYTES = FX_BM * FX_ROW * 2, FX_B_BYTES = FX_BN * FX_ROW * 2;
-constexpr int FX_STAGE_BYTES = FX_A_BYTES + FX_B_BYTES;
-constexpr int FX_SMEM = FX_STAGES * FX_STAGE_BYTES + 1024 + 512;
-static_assert(FX_SLICES * FX_BN <= 512, "one TMEM accumulator per level");
-static_assert((int64_t)FX_SLICES * FX_CHUNK * FX_BK * (1 << 14) <= (1 << 24), "level sums stay exact in FP32");
+template <int NS>
+struct Fx {
+  static constexpr int TOP = 8 * (NS - 1) + 6;        // fixed-point position: |v| 2^(TOP - E) < 2^TOP
+  static constexpr int ROW = NS * FX_BK;              // bf16 values of one row and stage
+  static constexpr int A_BYTES = FX_BM * ROW * 2, B_BYTES = FX_BN * ROW * 2;
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = NS == 8 ? 2 : 3;
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 512;
+  static_assert(NS % 2 == 0 && NS * FX_BN <= 512, "two slices per TMA row, one TMEM accumulator per level");
+  static_assert((int64_t)NS * FX_CHUNK * FX_BK * (1 << 14) <= (1 << 24), "level sums stay exact in FP32");
+};
 
 // ----------------------------------------------------------------------------- slices
 // Operand view: row i, complex K index t at p[i * si + t * sk].  dup: the B'
@@ -66,19 +70,20 @@ struct FxSrc {
 // The digits of v in a row of exponent E (|v| < 2^E), by integer operations on
 // its bits (the FP64 pipe would take ~20 operations per value): rounded to the
 // last digit, balanced digits -128..127 from the low end.
-__device__ __forceinline__ void fx_digits(double v, int E, int (&d)[FX_SLICES]) {
+template <int NS>
+__device__ __forceinline__ void fx_digits(double v, int E, int (&d)[NS]) {
   const long long u = __double_as_longlong(v);
   const int be = (int)((u >> 52) & 0x7FF);
   long long x = 0;
   if (be > 0) {
     const long long mant = (u & 0xFFFFFFFFFFFFFll) | (1ll << 52);
-    const int sh = be - 1075 + FX_TOP - E;    // v 2^(FX_TOP - E) = mant 2^sh
-    if (sh >= 0) x = mant << sh;              // below 2^FX_TOP by the choice of E
+    const int sh = be - 1075 + Fx<NS>::TOP - E;    // v 2^(TOP - E) = mant 2^sh
+    if (sh >= 0) x = mant << sh;              // below 2^TOP by the choice of E
     else if (sh >= -54) x = (mant + (1ll << (-sh - 1))) >> -sh;
     if (u < 0) x = -x;
   }
 #pragma unroll
-  for (int s = FX_SLICES - 1; s > 0; --s) {
+  for (int s = NS - 1; s > 0; --s) {
     d[s] = (int)(signed char)(x & 255);
     x = (x - d[s]) >> 8;
   }
@@ -102,22 +107,23 @@ __device__ __forceinline__ int fx_exp(unsigned hi) {
   return be == 0x7FF ? FX_BAD : (be == 0 ? 0 : be - 1022);
 }
 
+template <int NS>
 __device__ __forceinline__ void fx_write(const FxSrc& S, int64_t row, int64_t t, zd v, int E) {
-  int re[FX_SLICES], im[FX_SLICES];
+  int re[NS], im[NS];
   if (E == FX_BAD) v = mkz(0.0);
   if (S.conj) v.y = -v.y;
-  fx_digits(v.x, E, re);
-  fx_digits(v.y, E, im);
-  const int64_t in = (t >> 4) * FX_ROW + 2 * (t & 15);
+  fx_digits<NS>(v.x, E, re);
+  fx_digits<NS>(v.y, E, im);
+  const int64_t in = (t >> 4) * Fx<NS>::ROW + 2 * (t & 15);
   if (!S.dup) {
-    uint16_t* o = S.d + row * S.kb * FX_ROW + in;
+    uint16_t* o = S.d + row * S.kb * Fx<NS>::ROW + in;
 #pragma unroll
-    for (int s = 0; s < FX_SLICES; ++s) *(uint32_t*)(o + s * FX_BK) = fx_pack(re[s], im[s]);
+    for (int s = 0; s < NS; ++s) *(uint32_t*)(o + s * FX_BK) = fx_pack(re[s], im[s]);
   } else {
-    uint16_t* o = S.d + 2 * row * S.kb * FX_ROW + in;
-    uint16_t* o1 = o + S.kb * FX_ROW;
+    uint16_t* o = S.d + 2 * row * S.kb * Fx<NS>::ROW + in;
+    uint16_t* o1 = o + S.kb * Fx<NS>::ROW;
 #pragma unroll
-    for (int s = 0; s < FX_SLICES; ++s) {
+    for (int s = 0; s < NS; ++s) {
       *(uint32_t*)(o + s * FX_BK) = fx_pack(re[s], -im[s]);
       *(uint32_t*)(o1 + s * FX_BK) = fx_pack(im[s], re[s]);
     }
@@ -127,6 +133,7 @@ __device__ __forceinline__ void fx_write(const FxSrc& S, int64_t row, int64_t t,
 // Both operands of a product in one launch: blocks [0, a.blocks) slice a, the
 // rest b.  A block reads its row(s) once for the largest magnitude and again
 // (from L1 or L2) for the digits of its segment of K.
+template <int NS>
 __global__ void __launch_bounds__(256) k_fx_slice(FxSrc a, FxSrc b) {
   const bool first = (int64_t)blockIdx.x < a.blocks;
   const FxSrc& S = first ? a : b;
@@ -151,7 +158,7 @@ __global__ void __launch_bounds__(256) k_fx_slice(FxSrc a, FxSrc b) {
     for (int w = 1; w < 8; ++w) m = max(m, red[w]);
     const int E = fx_exp(m);
     if (tid == 0 && seg == 0) S.e[group] = E;
-    for (int64_t t = t0 + tid; t < t1; t += 256) fx_write(S, group, t, t < S.K ? p[t] : mkz(0.0), E);
+    for (int64_t t = t0 + tid; t < t1; t += 256) fx_write<NS>(S, group, t, t < S.K ? p[t] : mkz(0.0), E);
   } else {
     // 16 rows, contiguous (or strided) across the low thread index; tiles of 16 x 16 turned in shared memory
     __shared__ zd tile[16][17];
@@ -171,8 +178,53 @@ __global__ void __launch_bounds__(256) k_fx_slice(FxSrc a, FxSrc b) {
       __syncthreads();
       tile[r][kk] = (row < S.rows && t + kk < S.K) ? S.p[row * S.si + (t + kk) * S.sk] : mkz(0.0);
       __syncthreads();
-      if (wrow < S.rows) fx_write(S, wrow, t + r, tile[kk][r], E);
+      if (wrow < S.rows) fx_write<NS>(S, wrow, t + r, tile[kk][r], E);
     }
+  }
+}
+
+// Rows of an operand held as split-bf16 planes (row-major, ld values, K of them
+// valid): value = sum of its planes.  One block per row; the leading plane alone
+// fixes the exponent (the rest is below half a unit of its last place).
+template <int NS>
+__global__ void __launch_bounds__(256) k_fx_slice_planes(const uint16_t* p0, const uint16_t* p1, const uint16_t* p2,
+                                                         int64_t K, int64_t ld, int64_t kb, uint16_t* d, int* e) {
+  __shared__ unsigned red[8];
+  const int64_t row = blockIdx.x;
+  const int tid = threadIdx.x;
+  const uint32_t* a0 = (const uint32_t*)(p0 + row * ld);
+  const uint32_t* a1 = p1 ? (const uint32_t*)(p1 + row * ld) : nullptr;
+  const uint32_t* a2 = p2 ? (const uint32_t*)(p2 + row * ld) : nullptr;
+  const int64_t K2 = (K + 1) / 2;
+  unsigned m = 0;
+  for (int64_t t = tid; t < K2; t += 256) {
+    const uint32_t w = a0[t];
+    m = max(m, max(w & 0x7FFFu, (w >> 16) & 0x7FFFu));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((tid & 31) == 0) red[tid >> 5] = m;
+  __syncthreads();
+  m = red[0];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+  const int be = (int)(m >> 7);
+  const int E = be == 255 ? FX_BAD : (be == 0 ? 0 : be - 126);   // |x| < 2^(be - 126)
+  if (tid == 0) e[row] = E;
+  uint16_t* o = d + row * kb * Fx<NS>::ROW;
+  for (int64_t t = tid; t < kb * 16; t += 256) {
+    const uint32_t w0 = t < K2 ? a0[t] : 0u, w1 = (a1 && t < K2) ? a1[t] : 0u, w2 = (a2 && t < K2) ? a2[t] : 0u;
+    int u[NS], v[NS];
+    double x = 0.0, y = 0.0;
+    if (E != FX_BAD) {
+      x = (double)__uint_as_float(w0 << 16) + (double)__uint_as_float(w1 << 16) + (double)__uint_as_float(w2 << 16);
+      y = (double)__uint_as_float(w0 & 0xFFFF0000u) + (double)__uint_as_float(w1 & 0xFFFF0000u) +
+          (double)__uint_as_float(w2 & 0xFFFF0000u);
+    }
+    fx_digits<NS>(x, E, u);
+    fx_digits<NS>(y, E, v);
+    uint16_t* q = o + (t >> 4) * Fx<NS>::ROW + 2 * (t & 15);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) *(uint32_t*)(q + s * FX_BK) = fx_pack(u[s], v[s]);
   }
 }
 
@@ -195,16 +247,18 @@ __device__ __forceinline__ void fx_store(const FxArgs& a, int64_t i, int64_t j, 
   *o = p;
 }
 
+template <int NS>
 __global__ void __launch_bounds__(FX_THREADS, 1)
     k_gemm_fx(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, FxArgs args) {
+  using L = Fx<NS>;
   extern __shared__ uint8_t smem_raw[];
   if (*(volatile int*)args.err != 0) return;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(smem + FX_STAGES * FX_STAGE_BYTES);
-  uint64_t* empty = full + FX_STAGES;
-  uint64_t* tfull = empty + FX_STAGES;        // [level] MMA -> drain
-  uint64_t* tempty = tfull + FX_SLICES;       // [level] drain -> MMA
-  uint32_t* tslot = (uint32_t*)(tempty + FX_SLICES);
+  uint64_t* full = (uint64_t*)(smem + L::STAGES * L::STAGE_BYTES);
+  uint64_t* empty = full + L::STAGES;
+  uint64_t* tfull = empty + L::STAGES;        // [level] MMA -> drain
+  uint64_t* tempty = tfull + NS;       // [level] drain -> MMA
+  uint32_t* tslot = (uint32_t*)(tempty + NS);
   volatile int* abort_flag = (volatile int*)(tslot + 1);
   volatile int* issued = (volatile int*)(tslot + 2);
   volatile int* consumed = (volatile int*)(tslot + 3);
@@ -216,8 +270,8 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
   const int nchunks = (nk + FX_CHUNK - 1) / FX_CHUNK;
 
   if (threadIdx.x == 0) {
-    for (int q = 0; q < FX_STAGES; ++q) { mbar_init(&full[q], 1); mbar_init(&empty[q], 1); }
-    for (int q = 0; q < FX_SLICES; ++q) { mbar_init(&tfull[q], 1); mbar_init(&tempty[q], 8); }
+    for (int q = 0; q < L::STAGES; ++q) { mbar_init(&full[q], 1); mbar_init(&empty[q], 1); }
+    for (int q = 0; q < NS; ++q) { mbar_init(&tfull[q], 1); mbar_init(&tempty[q], 8); }
     *abort_flag = 0;
     *issued = 0;
     *consumed = 0;
@@ -246,19 +300,19 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
   if (warp == 8) {
     if (lane == 0) {
       for (int kb = 0; kb < nk; ++kb) {
-        const int st = kb % FX_STAGES;
-        if (kb >= FX_STAGES) {
-          if (!mbar_wait(&empty[st], ((kb / FX_STAGES) + 1) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 41; break; }
+        const int st = kb % L::STAGES;
+        if (kb >= L::STAGES) {
+          if (!mbar_wait(&empty[st], ((kb / L::STAGES) + 1) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 41; break; }
         }
         if (*abort_flag) break;
-        uint8_t* sp = smem + st * FX_STAGE_BYTES;
-        mbar_expect_tx(&full[st], FX_STAGE_BYTES);
-        const int x = (kb0 + kb) * FX_ROW;
+        uint8_t* sp = smem + st * L::STAGE_BYTES;
+        mbar_expect_tx(&full[st], L::STAGE_BYTES);
+        const int x = (kb0 + kb) * L::ROW;
 #pragma unroll
-        for (int q = 0; q < FX_SLICES / 2; ++q) tma_load_2d(sp + q * (FX_BM * 128), &mA, &full[st], x + 64 * q, m0);
+        for (int q = 0; q < NS / 2; ++q) tma_load_2d(sp + q * (FX_BM * 128), &mA, &full[st], x + 64 * q, m0);
 #pragma unroll
-        for (int q = 0; q < FX_SLICES / 2; ++q)
-          tma_load_2d(sp + FX_A_BYTES + q * (FX_BN * 128), &mB, &full[st], x + 64 * q, n0);
+        for (int q = 0; q < NS / 2; ++q)
+          tma_load_2d(sp + L::A_BYTES + q * (FX_BN * 128), &mB, &full[st], x + 64 * q, n0);
         *issued = kb + 1;
       }
     }
@@ -266,31 +320,31 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
     if (lane == 0) {
       bool ok = true;
       for (int kb = 0; kb < nk && ok; ++kb) {
-        const int st = kb % FX_STAGES, ch = kb / FX_CHUNK, in = kb % FX_CHUNK;
-        if (!mbar_wait(&full[st], (kb / FX_STAGES) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 42; break; }
+        const int st = kb % L::STAGES, ch = kb / FX_CHUNK, in = kb % FX_CHUNK;
+        if (!mbar_wait(&full[st], (kb / L::STAGES) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 42; break; }
         *consumed = kb + 1;
         if (*abort_flag) break;
         tc_fence_after();
-        const uint8_t* sp = smem + st * FX_STAGE_BYTES;
-        const uint64_t da = sw128_desc(sp), db = sw128_desc(sp + FX_A_BYTES);
+        const uint8_t* sp = smem + st * L::STAGE_BYTES;
+        const uint64_t da = sw128_desc(sp), db = sw128_desc(sp + L::A_BYTES);
         const bool last = (in == FX_CHUNK - 1) || (kb == nk - 1);
 #pragma unroll
-        for (int L = FX_SLICES - 1; L >= 0; --L) {
+        for (int lev = NS - 1; lev >= 0; --lev) {
           if (in == 0 && ch > 0) {
-            if (!mbar_wait(&tempty[L], (ch - 1) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 45; ok = false; break; }
+            if (!mbar_wait(&tempty[lev], (ch - 1) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 45; ok = false; break; }
             tc_fence_after();
           }
-          const uint32_t dt = tmem + (uint32_t)(L * FX_BN);
+          const uint32_t dt = tmem + (uint32_t)(lev * FX_BN);
 #pragma unroll
-          for (int s = 0; s <= L; ++s) {
+          for (int s = 0; s <= lev; ++s) {
             // slice s of a tile: box s / 2, 64 bytes into the 128-byte rows when odd (descriptors count 16 bytes)
-            const int t = L - s;
+            const int t = lev - s;
             const uint64_t a = da + (uint64_t)(((s >> 1) * (FX_BM * 128) + (s & 1) * 64) >> 4);
             const uint64_t b = db + (uint64_t)(((t >> 1) * (FX_BN * 128) + (t & 1) * 64) >> 4);
             mma_bf16(dt, a, b, idesc, (in > 0 || s > 0) ? 1u : 0u);
             mma_bf16(dt, a + 2, b + 2, idesc, 1u);
           }
-          if (last) mma_commit(&tfull[L]);
+          if (last) mma_commit(&tfull[lev]);
         }
         mma_commit(&empty[st]);
       }
@@ -300,20 +354,20 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
     bool ok = true;
     for (int ch = 0; ch < nchunks && ok; ++ch) {
 #pragma unroll
-      for (int L = FX_SLICES - 1; L >= 0; --L) {
-        bool got = mbar_wait_sleep(&tfull[L], ch & 1, WAIT_LIMIT, args.err, 64u);
+      for (int lev = NS - 1; lev >= 0; --lev) {
+        bool got = mbar_wait_sleep(&tfull[lev], ch & 1, WAIT_LIMIT, args.err, 64u);
         got = __all_sync(0xffffffffu, got) && (__shfl_sync(0xffffffffu, *abort_flag, 0) == 0);
         if (!got) { if (lane == 0) atomicCAS((int*)abort_flag, 0, 44); ok = false; break; }
         tc_fence_after();
         float v[32];
-        tmem_ld32(tmem + ((uint32_t)lanebase << 16) + (uint32_t)(L * FX_BN + colhalf), v);
+        tmem_ld32(tmem + ((uint32_t)lanebase << 16) + (uint32_t)(lev * FX_BN + colhalf), v);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[L])) : "memory");
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[lev])) : "memory");
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
-          if (L > 4) lo[i] = fmaf(v[i], 1.f / (float)(1 << (8 * (L > 4 ? L - 4 : 0))), lo[i]);
-          else hi[i] += (long long)__float2int_rn(v[i]) << (8 * (L > 4 ? 0 : 4 - L));
+          if (lev > 4) lo[i] = fmaf(v[i], 1.f / (float)(1 << (8 * (lev > 4 ? lev - 4 : 0))), lo[i]);
+          else hi[i] += (long long)__float2int_rn(v[i]) << (8 * (lev > 4 ? 0 : 4 - lev));
         }
       }
     }
@@ -325,7 +379,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
       const int zero_flag = 0;
       atomicExch(args.err, 1000 * (*abort_flag) + (int)(blockIdx.x % 1000));
       for (int kb = *consumed; kb < *issued; ++kb)
-        (void)mbar_wait(&full[kb % FX_STAGES], (kb / FX_STAGES) & 1, WAIT_LIMIT, &zero_flag);
+        (void)mbar_wait(&full[kb % L::STAGES], (kb / L::STAGES) & 1, WAIT_LIMIT, &zero_flag);
     }
   } else if (warp < 8) {
     const int row = m0 + 32 * (warp & 3) + lane, j0 = (n0 + 32 * (warp >> 2)) >> 1;
@@ -375,6 +429,12 @@ bool zgemm_fx_wanted(int64_t m, int64_t n, int64_t k) {
          m <= ((int64_t)1 << 30) && n <= ((int64_t)1 << 30);
 }
 
+#define TRY_FX(x)          \
+  do {                     \
+    int _r = (x);          \
+    if (_r) return _r;     \
+  } while (0)
+
 struct FxPlan {
   int64_t kb, mp, np;        // stages; rows and complex columns of a panel
   size_t a_bytes, b_bytes, e_bytes, ws_bytes;
@@ -386,7 +446,7 @@ static size_t fx_up(size_t b) { return (b + 255) & ~(size_t)255; }
 static FxPlan fx_plan(int64_t m, int64_t n, int64_t k) {
   FxPlan p;
   p.kb = (2 * k + FX_BK - 1) / FX_BK;
-  const size_t row = (size_t)p.kb * FX_ROW * 2;
+  const size_t row = (size_t)p.kb * Fx<FX_SLICES>::ROW * 2;
   p.mp = std::max<int64_t>(FX_BM, (int64_t)(FX_PANEL / row) / FX_BM * FX_BM);
   p.mp = std::min(p.mp, std::min<int64_t>(m, 65535 * FX_BM));
   p.np = std::max<int64_t>(FX_BN / 2, (int64_t)(FX_PANEL / (2 * row)) / (FX_BN / 2) * (FX_BN / 2));
@@ -434,15 +494,44 @@ static int fx_splits(int64_t tiles, int64_t kb, int64_t elems) {
   return best;
 }
 
+template <int NS>
+static int fx_attributes() {
+  static DeviceOnce attr;   // one instance per template instantiation
+  if (!attr.need()) return 0;
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_fx<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fx<NS>::SMEM);
+  if (e != cudaSuccess) { set_error(std::string("zgemm_fx: shared-memory opt-in: ") + cudaGetErrorString(e)); return 3; }
+  attr.done();
+  return 0;
+}
+
+// One panel: sliced operands (a.m rows of A, 2 a.n rows of B'), kb stages; part:
+// FX_PARTIALS bytes.
+template <int NS>
+static int fx_panel(const uint16_t* da, const uint16_t* db, FxArgs a, zd* part, cudaStream_t s) {
+  TRY_FX(fx_attributes<NS>());
+  const int64_t ld = (int64_t)a.kb * Fx<NS>::ROW;
+  CUtensorMap mA, mB;
+  TRY_FX(make_map(&mA, da, a.m, ld, ld, FX_BM));
+  TRY_FX(make_map(&mB, db, 2 * (int64_t)a.n, ld, ld, FX_BN));
+  const int64_t mt = (a.m + FX_BM - 1) / FX_BM, nt = (2 * (int64_t)a.n + FX_BN - 1) / FX_BN;
+  int sp = fx_splits(mt * nt, a.kb, (int64_t)a.m * a.n);
+  const int64_t chunks = (a.kb + FX_CHUNK - 1) / FX_CHUNK, per = (chunks + sp - 1) / sp;
+  sp = (int)((chunks + per - 1) / per);   // every split has work
+  a.kb_split = (int)(per * FX_CHUNK);
+  a.ws = sp > 1 ? part : nullptr;
+  dim3 grid((unsigned)nt, (unsigned)mt, (unsigned)sp);
+  k_gemm_fx<NS><<<grid, FX_THREADS, Fx<NS>::SMEM, s>>>(mA, mB, a);
+  note_launch();
+  if (sp > 1) {
+    k_fx_reduce<<<(unsigned)(((int64_t)a.m * a.n + 255) / 256), 256, 0, s>>>(a, sp);
+    note_launch();
+  }
+  return 0;
+}
+
 int zgemm_fx(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc, void* ws,
              int* err, cudaStream_t s) {
   if (m <= 0 || n <= 0 || k <= 0) return 0;
-  static DeviceOnce attr;
-  if (attr.need()) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_SMEM);
-    if (e != cudaSuccess) { set_error(std::string("zgemm_fx: shared-memory opt-in: ") + cudaGetErrorString(e)); return 3; }
-    attr.done();
-  }
   const FxPlan P = fx_plan(m, n, k);
   char* base = (char*)ws;
   uint16_t* da = (uint16_t*)base;
@@ -450,7 +539,6 @@ int zgemm_fx(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd bet
   int* ea = (int*)(base + P.a_bytes + P.b_bytes);
   int* eb = ea + P.mp;
   zd* part = (zd*)(base + P.a_bytes + P.b_bytes + P.e_bytes);
-  const int64_t ld = P.kb * FX_ROW;
   for (int64_t j0 = 0; j0 < n; j0 += P.np) {
     const int64_t nn = std::min(P.np, n - j0);
     for (int64_t i0 = 0; i0 < m; i0 += P.mp) {
@@ -458,12 +546,8 @@ int zgemm_fx(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd bet
       FxSrc sa = fx_src(A.p + i0 * A.rs, A.rs, A.cs, A.conj, false, mm, k, P.kb, da, ea);
       FxSrc sb = fx_src(B.p + j0 * B.cs, B.cs, B.rs, B.conj, true, nn, k, P.kb, db, eb);
       if (i0 > 0) sb.blocks = 0;   // B' of this column panel is in place
-      k_fx_slice<<<(unsigned)(sa.blocks + sb.blocks), 256, 0, s>>>(sa, sb);
+      k_fx_slice<FX_SLICES><<<(unsigned)(sa.blocks + sb.blocks), 256, 0, s>>>(sa, sb);
       note_launch();
-      CUtensorMap mA, mB;
-      int r = make_map(&mA, da, mm, ld, ld, FX_BM);
-      if (!r) r = make_map(&mB, db, 2 * nn, ld, ld, FX_BN);
-      if (r) return r;
       FxArgs a;
       a.m = (int)mm; a.n = (int)nn;
       a.kb = (int)P.kb;
@@ -472,23 +556,62 @@ int zgemm_fx(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd bet
       a.out = C + j0 * ldc + i0;
       a.ldo = ldc;
       a.err = err;
-      const int64_t mt = (mm + FX_BM - 1) / FX_BM, nt = (2 * nn + FX_BN - 1) / FX_BN;
-      int sp = fx_splits(mt * nt, P.kb, mm * nn);
-      const int64_t chunks = (P.kb + FX_CHUNK - 1) / FX_CHUNK, per = (chunks + sp - 1) / sp;
-      sp = (int)((chunks + per - 1) / per);   // every split has work
-      a.kb_split = (int)(per * FX_CHUNK);
-      a.ws = sp > 1 ? part : nullptr;
-      dim3 grid((unsigned)nt, (unsigned)mt, (unsigned)sp);
-      k_gemm_fx<<<grid, FX_THREADS, FX_SMEM, s>>>(mA, mB, a);
-      note_launch();
-      if (sp > 1) {
-        k_fx_reduce<<<(unsigned)((mm * nn + 255) / 256), 256, 0, s>>>(a, sp);
-        note_launch();
-      }
+      TRY_FX(fx_panel<FX_SLICES>(da, db, a, part, s));
     }
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error(std::string("zgemm_fx: ") + cudaGetErrorString(e)); return 3; }
+  return 0;
+}
+
+// ----------------------------------------------------------------------------- operators kept as slices
+void fx_operand_bytes(int64_t rows, int64_t K, int64_t* kb, size_t* digits, size_t* exps) {
+  *kb = (K + FX_BK - 1) / FX_BK;
+  *digits = fx_up((size_t)rows * (size_t)(*kb) * Fx<FX_OP_SLICES>::ROW * 2);
+  *exps = fx_up(sizeof(int) * (size_t)rows);
+}
+
+int fx_slice_planes(const uint16_t* const* planes, int nplanes, int64_t rows, int64_t K, int64_t ld,
+                    const FxOperand& out, cudaStream_t s) {
+  k_fx_slice_planes<FX_OP_SLICES><<<(unsigned)rows, 256, 0, s>>>(planes[0], nplanes > 1 ? planes[1] : nullptr,
+                                                                 nplanes > 2 ? planes[2] : nullptr, K, ld, out.kb, out.d,
+                                                                 out.e);
+  note_launch();
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { set_error(std::string("fx_slice_planes: ") + cudaGetErrorString(e)); return 3; }
+  return 0;
+}
+
+size_t fx_apply_bytes(int64_t n, int64_t K) {
+  int64_t kb;
+  size_t d, e;
+  fx_operand_bytes(2 * n, K, &kb, &d, &e);
+  return d + e + FX_PARTIALS;
+}
+
+int fx_apply(const FxOperand& A, int64_t m, int64_t n, int64_t k, zd alpha, const zd* X, int64_t ldx, zd beta, zd* Y,
+             int64_t ldy, void* ws, int* err, cudaStream_t s) {
+  if (m <= 0 || n <= 0) return 0;
+  int64_t kb;
+  size_t db, eb;
+  fx_operand_bytes(2 * n, 2 * k, &kb, &db, &eb);
+  uint16_t* d = (uint16_t*)ws;
+  int* e = (int*)((char*)ws + db);
+  FxSrc none{};
+  FxSrc sb = fx_src(X, ldx, 1, false, true, n, k, kb, d, e);
+  k_fx_slice<FX_OP_SLICES><<<(unsigned)sb.blocks, 256, 0, s>>>(none, sb);
+  note_launch();
+  FxArgs a;
+  a.m = (int)m; a.n = (int)n;
+  a.kb = (int)kb;
+  a.EA = A.e; a.EB = e;
+  a.alpha = alpha; a.beta = beta;
+  a.out = Y;
+  a.ldo = ldy;
+  a.err = err;
+  TRY_FX(fx_panel<FX_OP_SLICES>(A.d, d, a, (zd*)((char*)ws + db + eb), s));
+  cudaError_t er = cudaGetLastError();
+  if (er != cudaSuccess) { set_error(std::string("fx_apply: ") + cudaGetErrorString(er)); return 3; }
   return 0;
 }
 

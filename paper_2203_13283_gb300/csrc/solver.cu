@@ -104,10 +104,10 @@ struct wcs_ctx {
   // the factors of Eq. (9) as two split-bf16 planes each (row-major real view),
   // staged at the first solve that multiplies by them
   struct Planes { DevBuf b; int64_t ld = 0; bool ready = false; } pVwH, pWt, pUH, pKinvH, pWa;
-  // exact residuals (mixed form, exact_residual = 1): fixed-point slices of
+  // exact residuals (mixed form, exact_residual = 1): fixed-point digits of
   // the four operators (layout 0), built at the first solve that needs them
-  DevBuf exops, exrhs, exws;
-  ExactOperand exA[4];
+  DevBuf exops, exws;
+  FxOperand exA[4];
   bool exact_ready = false;
   // optional per-kernel timing: CUDA events on the context stream
   bool profile = false;
@@ -410,55 +410,38 @@ static int cgemm_planes(wcs_ctx* c, int64_t m, int64_t n, int64_t k, zd alpha, c
   return 0;
 }
 
-// The operators' exact slices (from their layout-0 split-bf16 planes), once per assembly.
+// The operators' digits (from their layout-0 split-bf16 planes), once per assembly.
 static int ensure_exact_ops(wcs_ctx* c) {
   if (c->exact_ready) return 0;
-  int64_t ld = 0, nch = 0;
-  size_t sb = 0, eb = 0;
-  exact_operand_alloc_bytes(c->N, 2 * c->N, &ld, &nch, &sb, &eb);
-  const size_t per_op = ((EX_SLICES * sb + eb + 255) / 256) * 256;   // keeps every slice 256-byte aligned
-  TRY(c->exops.ensure(4 * per_op));
-  char* base = (char*)c->exops.p;
+  int64_t kb = 0;
+  size_t db = 0, eb = 0;
+  fx_operand_bytes(c->N, 2 * c->N, &kb, &db, &eb);
+  TRY(c->exops.ensure(4 * (db + eb)));
   for (int op = 0; op < 4; ++op) {
-    ExactOperand& o = c->exA[op];
-    o.ld = ld;
-    o.nchunks = nch;
-    for (int q = 0; q < EX_SLICES; ++q) o.slice[q] = (uint16_t*)(base + op * per_op + q * sb);
-    o.expo = (int16_t*)(base + op * per_op + EX_SLICES * sb);
+    FxOperand& o = c->exA[op];
+    o.kb = kb;
+    o.d = (uint16_t*)((char*)c->exops.p + op * (db + eb));
+    o.e = (int*)((char*)o.d + db);
     const uint16_t* P[3] = {plane_ptr(c, op, 0, 0), c->planes > 1 ? plane_ptr(c, op, 0, 1) : nullptr,
                             c->planes > 2 ? plane_ptr(c, op, 0, 2) : nullptr};
-    TRY(exact_slice_planes(P, c->planes, c->N, 2 * c->N, c->ldp, o, c->s));
+    TRY(fx_slice_planes(P, c->planes, c->N, 2 * c->N, c->ldp, o, c->s));
   }
   c->exact_ready = true;
   return 0;
 }
 
-// Y = alpha * op X + beta * Y, exactly up to FP64 sums (op 0 S~, 1 D, 2 D~, 3 N).
+// Y = alpha * op X + beta * Y, exactly up to FP64 rounding of the result (op 0 S~, 1 D, 2 D~, 3 N).
 static int ex_apply(wcs_ctx* c, int op, const zd* X, int64_t ldx, int64_t cols, zd alpha, zd beta, zd* Y,
                     int64_t ldy) {
   if (cols <= 0) return 0;
   TRY(ensure_exact_ops(c));
   TRY(ensure_tcerr(c));
-  const int64_t N = c->N, G = 256;   // right-hand sides per pass: bounds the split-K workspace
-  int64_t ld = 0, nch = 0;
-  size_t sb = 0, eb = 0;
-  exact_operand_alloc_bytes(2 * G, 2 * N, &ld, &nch, &sb, &eb);
-  const size_t sbr = ((sb + 255) / 256) * 256;
-  TRY(c->exrhs.ensure(EX_SLICES * sbr + sizeof(int16_t) * (size_t)G * nch + 256));
-  const int64_t ws_elems = nch * 2 * G * N;
-  TRY(c->exws.ensure(sizeof(float) * (size_t)ws_elems));
-  ExactOperand B;
-  B.ld = ld;
-  B.nchunks = nch;
-  for (int q = 0; q < EX_SLICES; ++q) B.slice[q] = (uint16_t*)((char*)c->exrhs.p + q * sbr);
-  B.expo = (int16_t*)((char*)c->exrhs.p + EX_SLICES * sbr);
+  const int64_t N = c->N, G = std::min<int64_t>(256, cols);   // right-hand sides per pass: bounds their digits
+  TRY(c->exws.ensure(fx_apply_bytes(G, 2 * N)));
   ProfScope ps(c, CAT_GEMM_EXACT, 2.0 * N * (2.0 * cols) * (2.0 * N), 0.0);
-  for (int64_t c0 = 0; c0 < cols; c0 += G) {
-    const int64_t cc = std::min(G, cols - c0);
-    TRY(exact_slice_rhs(X + c0 * ldx, N, cc, ldx, 0, B, c->s));
-    TRY(exact_product(c->exA[op], (int)N, B, (int)cc, (int)(2 * N), alpha, beta, 0, Y + c0 * ldy, ldy,
-                      (float*)c->exws.p, ws_elems, (int*)c->tcerr.p, c->s));
-  }
+  for (int64_t c0 = 0; c0 < cols; c0 += G)
+    TRY(fx_apply(c->exA[op], N, std::min(G, cols - c0), N, alpha, X + c0 * ldx, ldx, beta, Y + c0 * ldy, ldy, c->exws.p,
+                 (int*)c->tcerr.p, c->s));
   return 0;
 }
 
@@ -790,14 +773,6 @@ __global__ void k_two_minus(zd* T, int64_t r) {
   T[t] = v;
 }
 
-// At = A^T for an r x r complex column-major A (At row-major A)
-__global__ void k_transpose_z(const zd* __restrict__ A, int64_t r, zd* __restrict__ At) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= r * r) return;
-  const int64_t i = t / r, j = t % r;   // At row i, column j (coalesced writes)
-  At[t] = A[i + j * r];
-}
-
 // ||I - T||_F^2 partial sums (one block)
 // ||T - I||_F in two deterministic stages: per-block partial sums, then one block
 constexpr int EYE_BLOCKS = 304;
@@ -926,7 +901,7 @@ static void free_mesh(wcs_ctx* c) {
   c->U.release(); c->Vw.release(); c->Wt.release(); c->Kinv.release(); c->Wa.release();
   for (wcs_ctx::Planes* p : {&c->pVwH, &c->pWt, &c->pUH, &c->pKinvH, &c->pWa}) { p->b.release(); p->ready = false; }
   c->sol_e.release(); c->sol_h.release(); c->sol_b.release(); c->sol_ang.release(); c->sol_j.release();
-  c->exops.release(); c->exrhs.release(); c->exws.release(); c->exact_ready = false;
+  c->exops.release(); c->exws.release(); c->exact_ready = false;
   if (c->fft_ready) { fft_plan_destroy(c->fft); c->fft_ready = false; }
   circ32_release(c->circ);
   c->kinv_res = -1.0;
@@ -1504,47 +1479,13 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   return status;
 }
 
-// Y = A X for r x r complex A and r x cols complex X (column-major, ld r),
-// exact up to the FP64 sums of the scaled integer partials (exact.cu): the
-// rows of A as fixed-point slices, X as slices of a right-hand block.
+// Y = A X for r x r complex A and r x cols complex X (column-major, ld r) with
+// FP64 accuracy on the tensor cores (fxgemm.cu).
 static int exact_square(wcs_ctx* c, const zd* A, int64_t r, const zd* X, int64_t cols, zd* Y) {
   TRY(ensure_tcerr(c));
-  DevBuf At, pa, pb, ws;
-  TRY(At.ensure(sizeof(zd) * r * r));
-  k_transpose_z<<<(unsigned)((r * r + 255) / 256), 256, 0, c->s>>>(A, r, At.z());
-  note_launch();
-  int64_t lda = 0, ncha = 0, ldb = 0, nchb = 0;
-  size_t sa = 0, ea = 0, sb = 0, eb = 0;
-  // columns per pass: wide passes keep the 21 slice-pair launches large
-  // (the FP32 partials take nchunks x 2G x r floats, 268 MB at r = 4096)
-  const int64_t G = std::min<int64_t>(1024, std::max<int64_t>(cols, 1));
-  exact_operand_alloc_bytes(r, 2 * r, &lda, &ncha, &sa, &ea);
-  exact_operand_alloc_bytes(2 * G, 2 * r, &ldb, &nchb, &sb, &eb);
-  const size_t sa2 = ((sa + 255) / 256) * 256, sb2 = ((sb + 255) / 256) * 256;
-  TRY(pa.ensure(EX_SLICES * sa2 + ea + 256));
-  TRY(pb.ensure(EX_SLICES * sb2 + eb + 256));
-  const int64_t ws_elems = nchb * 2 * G * r;
-  TRY(ws.ensure(sizeof(float) * (size_t)ws_elems));
-  ExactOperand oa, ob;
-  oa.ld = lda;
-  oa.nchunks = ncha;
-  ob.ld = ldb;
-  ob.nchunks = nchb;
-  for (int q = 0; q < EX_SLICES; ++q) {
-    oa.slice[q] = (uint16_t*)((char*)pa.p + q * sa2);
-    ob.slice[q] = (uint16_t*)((char*)pb.p + q * sb2);
-  }
-  oa.expo = (int16_t*)((char*)pa.p + EX_SLICES * sa2);
-  ob.expo = (int16_t*)((char*)pb.p + EX_SLICES * sb2);
-  TRY(exact_slice_real((const double*)At.p, r, 2 * r, 2 * r, oa, c->s));
+  TRY(c->fx.ensure(zgemm_fx_bytes(r, cols, r)));
   ProfScope ps(c, CAT_GEMM_EXACT, 2.0 * r * (2.0 * cols) * (2.0 * r), 0.0);
-  for (int64_t c0 = 0; c0 < cols; c0 += G) {
-    const int64_t cc = std::min(G, cols - c0);
-    TRY(exact_slice_rhs(X + c0 * r, r, cc, r, 0, ob, c->s));
-    TRY(exact_product(oa, (int)r, ob, (int)cc, (int)(2 * r), mkz(1.0), mkz(0.0), 0, Y + c0 * r, r,
-                      (float*)ws.p, ws_elems, (int*)c->tcerr.p, c->s));
-  }
-  return check_tc(c);
+  return zgemm_fx(r, cols, r, mkz(1.0), blk(A, r), blk(X, r), mkz(0.0), Y, r, c->fx.p, (int*)c->tcerr.p, c->s);
 }
 
 int wcs_factor(wcs_ctx* c) {
