@@ -549,9 +549,10 @@ constexpr int ASM_THREADS = 256;
 
 // One tile of node pairs from FP64 pair integrals: the 33 x 33 element pairs
 // that touch it, accumulated in acc[4][TILE][TILE].  MIXED: pairs far enough for
-// the FP32 route take it.
+// the FP32 route take it.  pre: the pairs' blocks, already integrated.
 template <int MIXED>
-__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc, const double* T = nullptr) {
+__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc, const double* T = nullptr,
+                                          const zd* pre = nullptr) {
   const int64_t N = A.N;
   for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) acc[t] = mkz(0.0);
   __syncthreads();
@@ -569,7 +570,12 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
     if (rowok && colok) {
       const int64_t e = ((i0 - 1 + el) % N + N) % N;
       const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-      if (MIXED && T) {
+      if (!MIXED && pre) {
+#pragma unroll
+        for (int op = 0; op < 4; ++op)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) o.v[op][j] = pre[(int64_t)idx * 16 + op * 4 + j];
+      } else if (MIXED && T) {
         if (periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, 0, N, A.near_band, N, e, f, o);
         else if (pair_is_far(A, e, f)) pair_far(A, e, f, o);
         else if (pair_is_mid(A, e, f)) pair_mid(A, T, e, f, o);
@@ -595,12 +601,61 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
   }
 }
 
-// FP64 form: every tile, dense complex output
-__global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A) {
+// FP64 form.  The tiles around the diagonal hold the near band (144 singular
+// points a pair) and the pairs below the expansion range: a CTA of eight warps
+// that walks such a tile takes 40 ms while the others take one.  Their pairs are
+// integrated by one warp per CTA first (k_assemble_pairs; the 32 pairs of a warp
+// are those of the tile kernel, whose recurrences start at the warp's largest
+// index), so that the work spreads over the chip; the tile kernel then only sums.
+constexpr int PRE_OFF = 3, PRE_SLOTS = 2 * PRE_OFF + 1, PRE_PAIRS = (TILE + 1) * (TILE + 1);
+
+// Slot of tile (ti, tj) in its row's integrated tiles, -1 for the others: tile
+// offsets up to PRE_OFF (cyclic) whose element ranges come within 34 elements.
+__device__ __forceinline__ int pre_slot(int64_t ti, int64_t tj, int64_t nt, int64_t N) {
+  int64_t off = tj - ti;
+  if (nt <= PRE_SLOTS) return (int)(off < 0 ? off + nt : off);   // few tiles: all of them
+  if (off > PRE_OFF) off -= nt;
+  if (off < -PRE_OFF) off += nt;
+  if (off < -PRE_OFF || off > PRE_OFF) return -1;
+  const int64_t a0 = ti * TILE - 1, a1 = min(N - 1, ti * TILE + TILE - 1), b0 = tj * TILE - 1, b1 = min(N - 1, tj * TILE + TILE - 1);
+  const int64_t g1 = ((b0 - a1) % N + N) % N, g2 = ((a0 - b1) % N + N) % N;
+  return (off == 0 || min(g1, g2) <= 34) ? (int)(off + PRE_OFF) : -1;
+}
+
+__global__ void __launch_bounds__(32) k_assemble_pairs(AsmArgs A, int64_t nt, int64_t row0, zd* pre) {
+  const int64_t N = A.N, ti = row0 + blockIdx.z;
+  const int64_t slot = blockIdx.y;
+  int64_t tj = nt <= PRE_SLOTS ? ti + slot : ti + slot - PRE_OFF;
+  tj = ((tj % nt) + nt) % nt;
+  if (slot >= nt || pre_slot(ti, tj, nt, N) != slot) return;
+  const int64_t i0 = ti * TILE, j0 = tj * TILE;
+  const int span = TILE + 1;
+  const int idx = blockIdx.x * 32 + threadIdx.x;
+  const int el = idx / span, fl = idx - (idx / span) * span;
+  const bool valid = idx < PRE_PAIRS;
+  const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N));
+  const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
+  if (rowok && colok) {
+    const int64_t e = ((i0 - 1 + el) % N + N) % N;
+    const int64_t f = ((j0 - 1 + fl) % N + N) % N;
+    PairOut o;
+    pair_integrals(A, e, f, o);
+    zd* out = pre + ((int64_t)blockIdx.z * PRE_SLOTS + slot) * PRE_PAIRS * 16 + (int64_t)idx * 16;
+#pragma unroll
+    for (int op = 0; op < 4; ++op)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) out[op * 4 + j] = o.v[op][j];
+  }
+}
+
+// every tile of the rows from row0 on, dense complex output
+__global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A, int64_t nt, int64_t row0, const zd* pre) {
   extern __shared__ zd acc[];  // [4][TILE][TILE]
-  const int64_t N = A.N;
-  const int64_t i0 = (int64_t)blockIdx.y * TILE, j0 = (int64_t)blockIdx.x * TILE;
-  tile_sums<0>(A, i0, j0, acc);
+  const int64_t N = A.N, ti = row0 + blockIdx.y, tj = blockIdx.x;
+  const int64_t i0 = ti * TILE, j0 = tj * TILE;
+  const int slot = pre ? pre_slot(ti, tj, nt, N) : -1;
+  tile_sums<0>(A, i0, j0, acc, nullptr,
+               slot < 0 ? nullptr : pre + ((int64_t)blockIdx.y * PRE_SLOTS + slot) * PRE_PAIRS * 16);
   zd* outs[4] = {A.S, A.D, A.Dt, A.Nk};
   for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) {
     const int op = t / (TILE * TILE), rem = t - op * TILE * TILE;
@@ -742,14 +797,26 @@ static int upload_rules(const AsmArgs& A) {
   return 0;
 }
 
-int assemble_dense(const AsmArgs& A, cudaStream_t s) {
+size_t assemble_dense_bytes(int64_t N) {
+  const int64_t rows = std::min<int64_t>((N + TILE - 1) / TILE, 128);
+  return sizeof(zd) * 16 * PRE_PAIRS * PRE_SLOTS * (size_t)rows;
+}
+
+int assemble_dense(const AsmArgs& A, void* ws, cudaStream_t s) {
   if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const size_t smem = sizeof(zd) * 4 * TILE * TILE;
   cudaFuncSetAttribute(k_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t nt = (A.N + TILE - 1) / TILE;
-  dim3 grid((unsigned)nt, (unsigned)nt);
-  k_assemble<<<grid, ASM_THREADS, smem, s>>>(A);
-  note_launch();
+  // 128 rows of tiles at a time bound the blocks kept (250 MB)
+  for (int64_t r0 = 0; r0 < nt; r0 += 128) {
+    const unsigned rows = (unsigned)std::min<int64_t>(128, nt - r0);
+    if (ws) {
+      k_assemble_pairs<<<dim3((PRE_PAIRS + 31) / 32, PRE_SLOTS, rows), 32, 0, s>>>(A, nt, r0, (zd*)ws);
+      note_launch();
+    }
+    k_assemble<<<dim3((unsigned)nt, rows), ASM_THREADS, smem, s>>>(A, nt, r0, (const zd*)ws);
+    note_launch();
+  }
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("assemble: ") + cudaGetErrorString(err)); return 3; }
   return 0;

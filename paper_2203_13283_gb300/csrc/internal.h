@@ -116,7 +116,9 @@ struct AsmArgs {
 // Fill kp.asym for kp.t and the term-count thresholds kp.xth for relative
 // tolerance tol (host).
 void fill_asymptotic(KtPair& kp, double tol);
-int assemble_dense(const AsmArgs& a, cudaStream_t s);
+// FP64 form; ws: assemble_dense_bytes(N) of device memory, or null (slower).
+size_t assemble_dense_bytes(int64_t N);
+int assemble_dense(const AsmArgs& a, void* ws, cudaStream_t s);
 // Mixed form: the same operators written as split-bf16 planes (see AsmArgs):
 // the far-pair kernel over the tiles it can take, then the FP64 kernel
 // over the rest.  mid (optional, two events) is recorded between the two;
@@ -242,8 +244,9 @@ int lu_inverse(zd* A, int64_t n, zd* Ainv, int* piv, int* info_dev, double* minp
 int planewave_rhs(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                   double h, double k, const double* angles, int B, zd* e, zd* hv, int64_t ld,
                   cudaStream_t s, bool split_phase = false);
+// differenced: the map of a central difference (one evaluation on every route)
 int farfield_matrix(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                     double h, double k, const double* phi, int nphi, zd* E, int64_t lde,
-                    cudaStream_t s);
+                    cudaStream_t s, bool differenced);
 
 }  // namespace wcs

@@ -1137,7 +1137,10 @@ int wcs_assemble(wcs_ctx* c) {
     AsmArgs A = asm_args(c, false);
     A.S = c->S; A.D = c->D; A.Dt = c->Dt; A.Nk = c->Nk;
     ProfScope ps(c, CAT_ASSEMBLY, (double)N * N * c->opt.q_far * c->opt.q_far, 0.0);
-    TRY(assemble_dense(A, c->s));
+    DevBuf pre;
+    if (pre.ensure(assemble_dense_bytes(N))) (void)cudaGetLastError();   // no room: without it
+    TRY(assemble_dense(A, pre.p, c->s));
+    TRY(sync(c));
   } else {
     c->ldp = ((2 * N + 63) / 64) * 64;
     TRY(c->opplanes.ensure(sizeof(uint16_t) * (size_t)8 * c->planes * N * c->ldp));
@@ -2369,7 +2372,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
   if (r == WCS_ERR_NOT_CONVERGED) status = r;
   else if (r) return r;
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, N, c->h, c->k, phd.d(), nphi, E.z(),
-                      nphi, c->s));
+                      nphi, c->s, true));
   TRY(cz(c, nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), F.z(), nphi));
   std::vector<zd> hd(4 * B);
   TRY(column_dotc(F.z(), nphi, F.z(), nphi, nphi, B, dots.z(), c->s));
@@ -2444,7 +2447,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
     for (int sgn = 0; sgn < 2; ++sgn) {
       wcs_ctx* t = sgn == 0 ? tp.t : tm.t;
       TRY(farfield_matrix(t->near, t->quad.wn, t->quad.xn, t->opt.q_near, N, t->h, t->k, phd.d(), nphi, E.z(),
-                          nphi, c->s));
+                          nphi, c->s, true));
       TRY(cz(c, nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), Wf.z(), nphi));
       TRY(column_dotc(F.z(), nphi, Wf.z(), nphi, nphi, B, dots.z(), c->s));
       cudaMemcpyAsync(hd.data(), dots.p, sizeof(zd) * B, cudaMemcpyDeviceToHost, c->s);
@@ -2565,7 +2568,7 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
   TRY(ang.ensure(sizeof(double) * nphi));
   cudaMemcpyAsync(ang.p, phi, sizeof(double) * nphi, cudaMemcpyHostToDevice, c->s);
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, c->N, c->h, c->k, ang.d(),
-                      nphi, E.z(), nphi, c->s));
+                      nphi, E.z(), nphi, c->s, false));
   TRY(cz(c, nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
          (zd*)F, ldf));
   int r = check_tc(c);
