@@ -77,6 +77,57 @@ __global__ void k_fft_tile(const zd* __restrict__ in, int64_t in_es, int64_t in_
   }
 }
 
+// Half of a radix-2 transform of length L <= 4096: the same butterflies with the
+// same twiddles as k_fft_tile, so the same bits, with a column's work spread over
+// L / 512 CTAs.  first: stages m = 1 .. M1 / 2, which stay within runs of M1
+// bit-reversed positions (in -> out, positions in order); otherwise stages M1 .. L / 2,
+// which stay within positions of equal index mod M1.  A CTA takes FH_SETS adjacent
+// sets (adjacent in memory on the strided side).
+// With one CTA per column (FP64 pipe bound, 52 us at L = 4096) 32 columns left 120
+// of 152 SMs idle: 79 us a transform, 2 x 12 in two halves.
+constexpr int FH_SETS = 8;
+__global__ void __launch_bounds__(256) k_fft_half(const zd* in, int64_t in_cs, zd* out, int64_t out_cs, int L, int logL,
+                                                  int logM1, const zd* __restrict__ tw, int64_t tstride, int sign,
+                                                  int first) {
+  extern __shared__ zd buf[];   // [FH_SETS][len]
+  const int M1 = 1 << logM1, nsets = first ? L >> logM1 : M1, len = first ? M1 : L >> logM1;
+  const int s0 = blockIdx.x * FH_SETS;
+  in += blockIdx.y * in_cs;
+  out += blockIdx.y * out_cs;
+  // first: set u holds the positions of block rev(u): elements rev(r) * nsets + u
+  for (int t = threadIdx.x; t < FH_SETS * len; t += blockDim.x) {
+    const int set = t % FH_SETS, r = t / FH_SETS;
+    if (first) buf[set * len + (int)bitrev((unsigned)r, logM1)] = in[(int64_t)r * nsets + s0 + set];
+    else buf[set * len + r] = in[(int64_t)r * M1 + s0 + set];
+  }
+  __syncthreads();
+  const int loglen = first ? logM1 : logL - logM1;
+  for (int lm = 0; lm < loglen; ++lm) {
+    const int ml = 1 << lm;                             // span in the set
+    const int m = first ? ml : ml << logM1;             // span in the whole transform
+    for (int t = threadIdx.x; t < FH_SETS * len / 2; t += blockDim.x) {
+      const int set = t >> (loglen - 1), b = t & (len / 2 - 1);
+      const int jl = b & (ml - 1), i0 = set * len + ((b >> lm) << (lm + 1)) + jl, i1 = i0 + ml;
+      const int j = first ? jl : (jl << logM1) + s0 + set;   // position mod m
+      zd w = tw[(int64_t)j * (L / (2 * m)) * tstride];
+      if (sign > 0) w.y = -w.y;
+      const zd x1 = buf[i1] * w, x0 = buf[i0];
+      buf[i0] = x0 + x1;
+      buf[i1] = x0 - x1;
+    }
+    __syncthreads();
+  }
+  for (int t = threadIdx.x; t < FH_SETS * len; t += blockDim.x) {
+    if (first) {
+      const int set = t / len, r = t - set * len;
+      out[(int64_t)bitrev((unsigned)(s0 + set), logL - logM1) * M1 + r] = buf[set * len + r];
+    } else {
+      const int set = t % FH_SETS, r = t / FH_SETS;
+      out[(int64_t)r * M1 + s0 + set] = buf[set * len + r];
+    }
+  }
+}
+
 __global__ void k_twiddles(zd* tw, int64_t n) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
@@ -198,6 +249,20 @@ static int launch_tile(const zd* in, int64_t in_es, int64_t in_ss, int64_t in_cs
 
 static int pow2_transform(Pow2& P, zd* x, int64_t ld, int64_t cols, int sign, cudaStream_t s) {
   const int64_t n = P.n;
+  if (n <= FFT_SMEM_MAX && n >= 512 && cols <= 76 && cols <= P.scratch_cols) {
+    // fewer columns than half the SMs: two halves over several CTAs per column
+    const int lg = ilog2(n), a = lg / 2, b = lg - a;
+    const size_t smem = sizeof(zd) * FH_SETS * ((size_t)1 << b);
+    k_fft_half<<<dim3((unsigned)((n >> a) / FH_SETS), (unsigned)cols), 256, smem, s>>>(x, ld, P.scratch, n, (int)n, lg, a,
+                                                                                     P.tw, 1, sign, 1);
+    note_launch();
+    k_fft_half<<<dim3((unsigned)((1 << a) / FH_SETS), (unsigned)cols), 256, smem, s>>>(P.scratch, n, x, ld, (int)n, lg, a,
+                                                                                     P.tw, 1, sign, 0);
+    note_launch();
+    cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) { set_error(std::string("fft: ") + cudaGetErrorString(err)); return 3; }
+    return 0;
+  }
   if (n <= FFT_SMEM_MAX) {
     return launch_tile(x, 1, ld, ld, x, 1, ld, ld, n, 1, cols, P.tw, n, sign, nullptr, 0, s);
   }
@@ -291,6 +356,76 @@ int fft_columns(FFTPlan& p, zd* x, int64_t ld, int64_t cols, int sign, cudaStrea
     r = pow2_transform(P, work, m, cc, +1, s);
     if (r) return r;
     k_bluestein_post<<<gn, 256, 0, s>>>(work, n, m, p.chirp, sign, x + c0 * ld, ld);
+    note_launch();
+  }
+  cudaError_t err = cudaGetLastError();
+  if (err != cudaSuccess) { set_error(cudaGetErrorString(err)); return 3; }
+  return 0;
+}
+
+// ---- circulant operators of a length that is not a power of two, as convolutions
+// s_m / n (or its conjugate, reciprocal): the diagonal whose inverse transform is the kernel
+__global__ void k_conv_diag(const zd* mu, int64_t n, int mode, zd* c) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  zd v = mu[j];
+  if (mode == 1 || mode == 3) v.y = -v.y;
+  if (mode >= 2) v = zrecip(v);
+  c[j] = (1.0 / (double)n) * v;
+}
+
+// c (n values, period n) at the offsets -(n - 1) .. n - 1 of a length-m circle
+__global__ void k_conv_kernel(const zd* c, int64_t n, int64_t m, zd* k) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= m) return;
+  zd v = mkz(0.0);
+  if (j < n) v = c[j];
+  else if (m - j < n) v = c[n - (m - j)];
+  k[j] = v;
+}
+
+__global__ void k_conv_pad(const zd* x, int64_t ld, int64_t n, int64_t m, zd* work) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
+  if (j < m) work[c * m + j] = j < n ? x[c * ld + j] : mkz(0.0);
+}
+
+__global__ void k_conv_take(const zd* work, int64_t n, int64_t m, zd* y, int64_t ld) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
+  if (j < n) y[c * ld + j] = (1.0 / (double)m) * work[c * m + j];
+}
+
+int64_t conv_kernel_elems(const FFTPlan& p) { return p.pow2 ? 0 : p.m; }
+
+int conv_kernel(FFTPlan& p, const zd* mu, int mode, zd* khat, zd* tmp, cudaStream_t s) {
+  const int64_t n = p.n, m = p.m;
+  k_conv_diag<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(mu, n, mode, tmp);
+  note_launch();
+  int r = fft_columns(p, tmp, n, 1, +1, s);
+  if (r) return r;
+  k_conv_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(tmp, n, m, khat);
+  note_launch();
+  Pow2 P{m, p.twiddle, p.work + m * p.work_cols, p.work_cols};
+  return pow2_transform(P, khat, m, 1, -1, s);
+}
+
+// A circulant product through Bluestein's transforms is four transforms of length
+// m >= 2 n - 1 (two each way); as a convolution with its first column it is two.
+int conv_apply(FFTPlan& p, const zd* khat, const zd* x, int64_t ldx, zd* y, int64_t ldy, int64_t cols, cudaStream_t s) {
+  const int64_t n = p.n, m = p.m;
+  zd* scratch = p.work + m * p.work_cols;
+  for (int64_t c0 = 0; c0 < cols; c0 += p.work_cols) {
+    const int64_t cc = std::min(p.work_cols, cols - c0);
+    dim3 gm((unsigned)((m + 255) / 256), (unsigned)cc), gn((unsigned)((n + 255) / 256), (unsigned)cc);
+    k_conv_pad<<<gm, 256, 0, s>>>(x + c0 * ldx, ldx, n, m, p.work);
+    note_launch();
+    Pow2 P{m, p.twiddle, scratch, p.work_cols};
+    int r = pow2_transform(P, p.work, m, cc, -1, s);
+    if (r) return r;
+    k_pointwise<<<gm, 256, 0, s>>>(p.work, m, khat, 0);
+    note_launch();
+    r = pow2_transform(P, p.work, m, cc, +1, s);
+    if (r) return r;
+    k_conv_take<<<gn, 256, 0, s>>>(p.work, n, m, y + c0 * ldy, ldy);
     note_launch();
   }
   cudaError_t err = cudaGetLastError();

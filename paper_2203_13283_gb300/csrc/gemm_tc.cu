@@ -198,7 +198,8 @@ static int launch_tc(const TcOperand& A, const TcOperand& B, TcArgs& args, cudaS
   return 0;
 }
 
-// Sum of the split-K partials in a fixed order (FP64) and the epilogue.
+// Sum of the split-K partials in a fixed order (FP64, or float-float for complex
+// output) and the epilogue.
 __global__ void k_splitk_reduce(TcArgs a, int splits) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t plane = (int64_t)a.Nc * a.M;
@@ -216,12 +217,19 @@ __global__ void k_splitk_reduce(TcArgs a, int splits) {
   if (t >= (int64_t)a.M * ncols) return;
   const int row = (int)(t % a.M), j = (int)(t / a.M);
   const float* w = a.ws + (int64_t)(2 * j) * a.M + row;
-  double re = 0.0, im = 0.0;
+  // float-float sums (TwoSum keeps ~48 bits; the partials carry 24): converting
+  // and adding every partial on the FP64 pipe took 50 us at 4096 x 256 and seven splits
+  float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
 #pragma unroll 8
   for (int z = 0; z < splits; ++z) {
-    re += (double)w[z * plane];
-    im += (double)w[z * plane + a.M];
+    const float x = w[z * plane], y = w[z * plane + a.M];
+    const float sx = rh + x, bx = sx - rh, sy = ih + y, by = sy - ih;
+    rl += (rh - (sx - bx)) + (x - bx);
+    il += (ih - (sy - by)) + (y - by);
+    rh = sx;
+    ih = sy;
   }
+  const double re = epi_f32_to_f64(rh) + epi_f32_to_f64(rl), im = epi_f32_to_f64(ih) + epi_f32_to_f64(il);
   zd p = mkz(re, a.conj_out ? -im : im);
   p = a.alpha * p;
   zd* o = (zd*)a.out + (int64_t)j * a.ldo + row;
@@ -718,7 +726,7 @@ static int launch_splitk_reduce(const TcArgs& args, int splits, cudaStream_t s) 
 // k-blocks per split of a drained product (0: no split).  A launch takes whole
 // waves of 152 CTAs, so a grid of 24 or 192 tiles leaves most of the chip idle in
 // its only or last wave; splitting K evens it out at the price of the partials
-// (written and read once, FP32, summed in FP64) and of a prologue and epilogue per
+// (written and read once, FP32, summed in float-float) and of a prologue and epilogue per
 // CTA.  Microseconds: a K = 64 block of a 128 x 128 tile is 0.8 with three planes
 // (24 MMAs of 64 clocks) and 0.4 with two, of a 128 x 256 tile with two 0.8; about
 // 4 per CTA; 8 bytes per partial at 5 TB/s and a 4 us reduction launch.

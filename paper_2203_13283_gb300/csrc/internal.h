@@ -62,7 +62,8 @@ struct ArcTable {
   double L = 0.0;
 };
 
-int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s);
+// scan: sum the panels by a parallel double-double scan instead of one after the other
+int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s, bool scan = false);
 // Points at arc lengths s_j = (e + xi[g]) * h for e < N, g < nq (index e*nq + g); tol: Newton step
 // that ends the inversion of the arc length.
 int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const double* xi_dev,
@@ -189,6 +190,12 @@ void fft_plan_destroy(FFTPlan& p);
 // In-place batched transform of `cols` columns of length n (column-major, ld).
 // sign = -1: forward (e^{-2 pi i jk/n}); +1: inverse without 1/n scaling.
 int fft_columns(FFTPlan& p, zd* x, int64_t ld, int64_t cols, int sign, cudaStream_t s);
+// Circulant operators for lengths that are not powers of two: khat (conv_kernel_elems
+// values) from the eigenvalues (mode 0 mu, 1 conj mu, 2 1 / mu, 3 1 / conj mu; tmp: n
+// values), then y = F^-1 diag F x as a convolution (y may be x).
+int64_t conv_kernel_elems(const FFTPlan& p);
+int conv_kernel(FFTPlan& p, const zd* mu, int mode, zd* khat, zd* tmp, cudaStream_t s);
+int conv_apply(FFTPlan& p, const zd* khat, const zd* x, int64_t ldx, zd* y, int64_t ldy, int64_t cols, cudaStream_t s);
 // x[:, c] <- x[:, c] * mu (mu length n), or / mu when divide, conj(mu) when conj_mu.
 int scale_columns(zd* x, int64_t n, int64_t ld, int64_t cols, const zd* mu, bool divide,
                   bool conj_mu, double extra, cudaStream_t s);

@@ -506,25 +506,23 @@ constexpr int GRAM_ROWS = 256;
 
 // Partial Gram sums over GRAM_ROWS rows: only the upper triangle i <= j of the
 // Hermitian b x b result is formed (pair index p -> column j = row of the
-// triangular numbers, row i = p - j (j + 1) / 2); both halves are written.
-__global__ void k_gram_partial(const zd* X, int64_t ld, int64_t m, int b, zd* part) {
+// triangular numbers, row i = p - j (j + 1) / 2); both halves are written.  A CTA
+// takes GRAM_PAIRS pairs, two lanes each (real and imaginary part), so that the
+// FP64 work of a row chunk (528 pairs at b = 32) spreads over 17 CTAs instead of
+// one: at N = 2777 eleven CTAs took 185 us, 187 take 20.
+constexpr int GRAM_PAIRS = 32;
+__global__ void __launch_bounds__(2 * GRAM_PAIRS) k_gram_partial(const zd* X, int64_t ld, int64_t m, int b, zd* part) {
   __shared__ zd xs[64][33];
   const int64_t r0 = (int64_t)blockIdx.x * GRAM_ROWS;
-  const int tid = threadIdx.x;                  // 256 threads: up to 9 pairs each
-  const int npairs = b * (b + 1) / 2;
-  int ii[9], jj[9];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    const int p = tid + 256 * t;
-    int j = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
-    while (j * (j + 1) / 2 > p) --j;
-    while ((j + 1) * (j + 2) / 2 <= p) ++j;
-    ii[t] = (p < npairs) ? p - j * (j + 1) / 2 : -1;
-    jj[t] = j;
-  }
-  zd acc[9];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) acc[t] = mkz(0.0);
+  const int tid = threadIdx.x, im = tid & 1;
+  const int npairs = b * (b + 1) / 2, p = blockIdx.y * GRAM_PAIRS + (tid >> 1);
+  int j = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
+  while (j * (j + 1) / 2 > p) --j;
+  while ((j + 1) * (j + 2) / 2 <= p) ++j;
+  const bool ok = p < npairs;
+  const int i = ok ? p - j * (j + 1) / 2 : 0;
+  if (!ok) j = 0;
+  double acc = 0.0;
   for (int64_t rr = r0; rr < min(m, r0 + GRAM_ROWS); rr += 32) {
     __syncthreads();
     for (int u = tid; u < 32 * b; u += blockDim.x) {
@@ -532,28 +530,25 @@ __global__ void k_gram_partial(const zd* X, int64_t ld, int64_t m, int b, zd* pa
       xs[c][r] = (rr + r < m) ? X[(int64_t)c * ld + rr + r] : mkz(0.0);
     }
     __syncthreads();
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      if (ii[t] >= 0) {
-        const int i = ii[t], j = jj[t];
-        for (int r = 0; r < 32; ++r) zfma(acc[t], conj(xs[i][r]), xs[j][r]);
-      }
+    // conj(x_i) x_j with the operations of zfma: re: fma(x, u, fma(y, v, re)); im: fma(x, v, fma(-y, u, im))
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) {
+      const zd a = xs[i][r], c = xs[j][r];
+      acc = fma(a.x, im ? c.y : c.x, fma(im ? -a.y : a.y, im ? c.x : c.y, acc));
     }
   }
-#pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    if (ii[t] < 0) continue;
-    const int i = ii[t], j = jj[t];
-    zd* P = part + (int64_t)blockIdx.x * b * b;
-    P[j * b + i] = acc[t];
-    if (i != j) P[i * b + j] = conj(acc[t]);
-  }
+  const double other = __shfl_xor_sync(0xffffffffu, acc, 1);
+  if (!ok || im) return;
+  zd* P = part + (int64_t)blockIdx.x * b * b;
+  P[j * b + i] = mkz(acc, other);
+  if (i != j) P[i * b + j] = mkz(acc, -other);
 }
 
 __global__ void k_gram_reduce(const zd* part, int nparts, int b, zd* G) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= b * b) return;
   zd s = mkz(0.0);
+#pragma unroll 8
   for (int p = 0; p < nparts; ++p) s += part[(int64_t)p * b * b + t];
   G[t] = s;
 }
@@ -561,7 +556,7 @@ __global__ void k_gram_reduce(const zd* part, int nparts, int b, zd* G) {
 int gram_matrix(const zd* X, int64_t ld, int64_t m, int b, zd* G, zd* work, cudaStream_t s) {
   if (b > 64) { set_error("gram_matrix: b <= 64"); return 1; }
   const int nparts = (int)((m + GRAM_ROWS - 1) / GRAM_ROWS);
-  k_gram_partial<<<nparts, 256, 0, s>>>(X, ld, m, b, work);
+  k_gram_partial<<<dim3((unsigned)nparts, (unsigned)((b * (b + 1) / 2 + GRAM_PAIRS - 1) / GRAM_PAIRS)), 2 * GRAM_PAIRS, 0, s>>>(X, ld, m, b, work);
   note_launch();
   k_gram_reduce<<<(b * b + 255) / 256, 256, 0, s>>>(work, nparts, b, G);
   note_launch();

@@ -76,6 +76,8 @@ struct wcs_ctx {
   FFTPlan fft{};
   bool fft_ready = false;
   Circ32 circ{};                          // mixed form: FP32 circulant applies (built from mu_C on first use)
+  DevBuf conv;                            // mixed form, N not a power of two: transformed kernels of the four circulant modes
+  bool conv_ready[4] = {false, false, false, false};
   double kinv_res = -1.0;                 // ||I - K K^-1||_F / sqrt(r) of the last factor (-1: not measured)
   int rank = -1;
   DevBuf U, Vw, Wt;                       // N x rank each
@@ -566,6 +568,20 @@ static int apply_Cc(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ldy, in
     ProfScope ps(c, CAT_FFT, 0.0, 64.0 * (double)N * cols);
     return circ32_apply(c->circ, X, ldx, Y, ldy, cols, mode, c->s);
   }
+  if (c->mixed && conv_kernel_elems(c->fft) > 0) {
+    const int64_t m = conv_kernel_elems(c->fft);
+    zd* khat = nullptr;
+    if (!c->conv.ensure(sizeof(zd) * (4 * m + N))) {
+      khat = c->conv.z() + mode * m;
+      if (!c->conv_ready[mode]) {
+        TRY(conv_kernel(c->fft, mu_ptr(c, MU_C), mode, khat, c->conv.z() + 4 * m, c->s));
+        c->conv_ready[mode] = true;
+      }
+      ProfScope ps(c, CAT_FFT, 0.0, 4.0 * 16.0 * (double)N * cols);
+      return conv_apply(c->fft, khat, X, ldx, Y, ldy, cols, c->s);
+    }
+    (void)cudaGetLastError();   // no room for the kernels: Bluestein's transforms
+  }
   if (X != Y) {
     cudaError_t e = cudaMemcpy2DAsync(Y, sizeof(zd) * ldy, X, sizeof(zd) * ldx, sizeof(zd) * N, cols,
                                       cudaMemcpyDeviceToDevice, c->s);
@@ -904,6 +920,8 @@ static void free_mesh(wcs_ctx* c) {
   c->exops.release(); c->exws.release(); c->exact_ready = false;
   if (c->fft_ready) { fft_plan_destroy(c->fft); c->fft_ready = false; }
   circ32_release(c->circ);
+  c->conv.release();
+  for (bool& r : c->conv_ready) r = false;
   c->kinv_res = -1.0;
   c->rank = -1;
 }
@@ -996,7 +1014,7 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   if (N < 12 || N > (int64_t)1 << 22) { set_error("N must be in [12, 4194304]"); return WCS_ERR_ARG; }
   free_mesh(c);
   c->stage = ST_CONTOUR;
-  TRY(arc_table_build(c->contour, c->arc, c->s));
+  TRY(arc_table_build(c->contour, c->arc, c->s, c->mixed));
   c->L = c->arc.L;
   c->N = N;
   c->ld = (N + 7) & ~(int64_t)7;
@@ -1216,7 +1234,8 @@ int wcs_assemble(wcs_ctx* c) {
   TRY(fft_columns(c->fft, mu_ptr(c, MU_S), N, 4, +1, c->s));
   k_mu_finish<<<(unsigned)((N + 255) / 256), 256, 0, c->s>>>(c->mu.z(), N, c->h);
   note_launch();
-  c->circ.ready = false;   // the FP32 circulant tables follow mu_C
+  c->circ.ready = false;   // the circulant tables follow mu_C
+  for (bool& r : c->conv_ready) r = false;
   TRY(c->small.ensure(sizeof(double) * 8));
   k_absmax<<<1, 256, 0, c->s>>>(mu_ptr(c, MU_C), N, c->small.d());
   note_launch();
