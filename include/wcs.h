@@ -151,7 +151,9 @@ int wcs_default_options(wcs_options* opt);
  * be NULL for defaults. */
 int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream);
 
-/* Free every device buffer of ctx and the context itself (NULL is a no-op). */
+/* Free every device buffer of ctx and the context itself (NULL is a no-op).
+ * Until then a context keeps its buffers from one contour and mesh to the next
+ * (growing them as needed; large ones shrink when a quarter would do). */
 int wcs_destroy(wcs_ctx* ctx);
 
 /* --- contour gamma (Sec. II: a convex 2D contour), as r(theta) = rho(theta) (cos, sin) --- */

@@ -31,8 +31,6 @@
 
 namespace wcs {
 
-__constant__ double c_xf[16], c_wf[16], c_xn[16], c_wn[16];
-static int upload_rules(const AsmArgs& A);
 
 struct PairOut {
   zd v[4][4];  // [operator S~, D, D~, N][a * 2 + b]
@@ -98,7 +96,7 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
     for (int p = 0; p < q; ++p) {
       const int64_t ip = e * q + p;
       const double xt = A.far.x[ip], yt = A.far.y[ip], nxt = A.far.nx[ip], nyt = A.far.ny[ip];
-      const double xip = c_xf[p], wp = c_wf[p];
+      const double xip = A.xf[p], wp = A.wf[p];
       for (int r = 0; r < q; ++r) {
         const int64_t ir = f * q + r;
         const double dx = xt - A.far.x[ir], dy = yt - A.far.y[ir];
@@ -123,8 +121,8 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
         const zd gt = i4(Ht.H0);
         const zd dgk = (k * gg) * i4(Hk.H1);
         const zd dgt = gg * (kt * i4(Ht.H1));
-        const double w = wp * c_wf[r];
-        const double xir = c_xf[r];
+        const double w = wp * A.wf[r];
+        const double xir = A.xf[r];
         const double ph[2] = {1.0 - xip, xip}, ps[2] = {1.0 - xir, xir};
 #pragma unroll
         for (int a = 0; a < 2; ++a)
@@ -152,14 +150,14 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
       const int64_t ip = e * q + p;
       const double xt = A.near.x[ip], yt = A.near.y[ip], nxt = A.near.nx[ip], nyt = A.near.ny[ip];
       const double kap = A.near.kappa[ip];
-      const double xip = c_xn[p], wp = c_wn[p];
+      const double xip = A.xn[p], wp = A.wn[p];
       for (int r = 0; r < q; ++r) {
         const int64_t ir = f * q + r;
-        const double xir = c_xn[r];
+        const double xir = A.xn[r];
         const double dx = xt - A.near.x[ir], dy = yt - A.near.y[ir];
         const double nxs = A.near.nx[ir], nys = A.near.ny[ir];
         const double nd = nxt * nxs + nyt * nys;
-        const double w = wp * c_wn[r];
+        const double w = wp * A.wn[r];
         zd kS, kD, kDt, kN;       // smooth parts (full kernels for regular pairs)
         zd aS = mkz(0.0), aD = mkz(0.0), aDt = mkz(0.0), aN = mkz(0.0);  // log coefficients
         double lw = 0.0;          // weight of the log part
@@ -376,7 +374,7 @@ __global__ void __launch_bounds__(128) k_near_band(AsmArgs A, int64_t e0, int64_
   for (int pt = lane; pt < q * q; pt += 32) {
     const int p = pt / q, r = pt - p * q;
     const int64_t ip = e * q + p, ir = f * q + r;
-    const double xip = c_xn[p], xir = c_xn[r], w = c_wn[p] * c_wn[r];
+    const double xip = A.xn[p], xir = A.xn[r], w = A.wn[p] * A.wn[r];
     const double dx = A.near.x[ip] - A.near.x[ir], dy = A.near.y[ip] - A.near.y[ir];
     const double nxs = A.near.nx[ir], nys = A.near.ny[ir];
     const double nd = A.near.nx[ip] * nxs + A.near.ny[ip] * nys;
@@ -458,7 +456,6 @@ __global__ void __launch_bounds__(128) k_near_band(AsmArgs A, int64_t e0, int64_
 }
 
 int near_band_pairs(const AsmArgs& A, int64_t e0, int64_t ne, double* out, cudaStream_t s) {
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const int64_t pairs = ne * (2 * A.near_band + 1);
   k_near_band<<<(unsigned)((pairs + 3) / 4), 128, 0, s>>>(A, e0, ne, out);
   note_launch();
@@ -506,15 +503,15 @@ __device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t
       else hankel_tab_series(T, x, log(0.5 * x), Hk, Ht);
       const double gg = (dx * nxs + dy * nys) * ri, nd = nxt * nxs + nyt * nys;
       const zd K[4] = {Ht.H0, gg * Hk.H1, gg * Ht.H1, nd * Hk.H0};
-      const double w1 = c_wf[r] * c_xf[r], w0 = c_wf[r] - w1;
+      const double w1 = A.wf[r] * A.xf[r], w0 = A.wf[r] - w1;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         zfmas(u[i][0], w0, K[i]);
         zfmas(u[i][1], w1, K[i]);
       }
-      zfmas(ud, c_wf[r], Hk.H0);
+      zfmas(ud, A.wf[r], Hk.H0);
     }
-    const double w1 = c_wf[p] * c_xf[p], w0 = c_wf[p] - w1;
+    const double w1 = A.wf[p] * A.xf[p], w0 = A.wf[p] - w1;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -522,7 +519,7 @@ __device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t
         zfmas(v[i][b], w0, u[i][b]);
         zfmas(v[i][2 + b], w1, u[i][b]);
       }
-    zfmas(vd, c_wf[p], ud);
+    zfmas(vd, A.wf[p], ud);
   }
   const double h2 = A.h * A.h, kk2h2 = A.k * A.k * h2;
   const zd fS = mkz(0.0, 0.25 * h2), fD = mkz(0.0, 0.25 * A.k * h2), fDt = mkz(-0.25 * h2 * A.kt.y, 0.25 * h2 * A.kt.x);
@@ -786,24 +783,12 @@ void fill_asymptotic(KtPair& kp, double tol) {
   }
 }
 
-static int upload_rules(const AsmArgs& A) {
-  double xf[16], wf[16], xn[16], wn[16];
-  gauss_legendre01(A.q_far, xf, wf);
-  gauss_legendre01(A.q_near, xn, wn);
-  if (cudaMemcpyToSymbol(c_xf, xf, sizeof(double) * A.q_far) != cudaSuccess) return 3;
-  if (cudaMemcpyToSymbol(c_wf, wf, sizeof(double) * A.q_far) != cudaSuccess) return 3;
-  if (cudaMemcpyToSymbol(c_xn, xn, sizeof(double) * A.q_near) != cudaSuccess) return 3;
-  if (cudaMemcpyToSymbol(c_wn, wn, sizeof(double) * A.q_near) != cudaSuccess) return 3;
-  return 0;
-}
-
 size_t assemble_dense_bytes(int64_t N) {
   const int64_t rows = std::min<int64_t>((N + TILE - 1) / TILE, 128);
   return sizeof(zd) * 16 * PRE_PAIRS * PRE_SLOTS * (size_t)rows;
 }
 
 int assemble_dense(const AsmArgs& A, void* ws, cudaStream_t s) {
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const size_t smem = sizeof(zd) * 4 * TILE * TILE;
   cudaFuncSetAttribute(k_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t nt = (A.N + TILE - 1) / TILE;
@@ -981,7 +966,6 @@ __global__ void k_diag_tiles(int* list, int64_t nt) {
 }
 
 int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t* fp64_tiles, int64_t* tiles) {
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const size_t smem = sizeof(zd) * 4 * TILE * TILE;
   const size_t smem_near = smem + sizeof(double) * HT_SIZE;
   cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_near);
@@ -1011,35 +995,32 @@ int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t*
   return 0;
 }
 
-__global__ void k_far_tables(Points far, Points cen, int64_t N, int q, double h, FarElem* fe, FarPoint* fp) {
+__global__ void k_far_tables(AsmArgs A, Points cen, FarElem* fe, FarPoint* fp) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= N * q) return;
+  const int q = A.q_far;
+  const Points& far = A.far;
+  const double h = A.h;
+  if (t >= A.N * q) return;
   const int64_t e = t / q;
   const int p = (int)(t - e * q);
   fp[t] = far_point(cen.x[e], cen.y[e], cen.nx[e], cen.ny[e], far.x[t], far.y[t], far.nx[t], far.ny[t], h,
-                    c_xf[p] - 0.5);
+                    A.xf[p] - 0.5);
   if (p == 0) fe[e] = far_elem(cen.x[e], cen.y[e], cen.nx[e], cen.ny[e]);
 }
 
 int far_tables(const AsmArgs& A, const Points& cen, FarElem* fe, FarPoint* fp, cudaStream_t s) {
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const int64_t n = A.N * A.q_far;
-  k_far_tables<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(A.far, cen, A.N, A.q_far, A.h, fe, fp);
+  k_far_tables<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(A, cen, fe, fp);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("far tables: ") + cudaGetErrorString(err)); return 3; }
   return 0;
 }
 
-int assemble_circle_row(const AsmArgs& A, cudaStream_t s) {
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
-  zd* part = nullptr;
-  if (cudaMalloc(&part, sizeof(zd) * 16 * A.N) != cudaSuccess) { set_error("oom (circle row)"); return 4; }
+int assemble_circle_row(const AsmArgs& A, zd* part, cudaStream_t s) {
   k_circle_row_part<<<(unsigned)((4 * A.N + 63) / 64), 64, 0, s>>>(A, part);
   note_launch();
   k_circle_row_sum<<<(unsigned)((A.N + 127) / 128), 128, 0, s>>>(A, part);
-  cudaStreamSynchronize(s);
-  cudaFree(part);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("circle row: ") + cudaGetErrorString(err)); return 3; }
@@ -1049,7 +1030,6 @@ int assemble_circle_row(const AsmArgs& A, cudaStream_t s) {
 int assemble_entries(const AsmArgs& A, int64_t count, const int64_t* rows, const int64_t* cols,
                      zd* out4, cudaStream_t s) {
   if (count <= 0) return 0;
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   k_entries<<<(unsigned)((count + 63) / 64), 64, 0, s>>>(A, count, rows, cols, out4);
   note_launch();
   cudaError_t err = cudaGetLastError();
@@ -1105,7 +1085,7 @@ __global__ void __launch_bounds__(256) k_shape_far(ShapeArgs S) {
     double col[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     const int64_t iq = fvalid ? f * q + r : 0;
     const double xq = A.far.x[iq], yq = A.far.y[iq], nxq = A.far.nx[iq], nyq = A.far.ny[iq];
-    const double eta = c_xf[r], wr = c_wf[r];
+    const double eta = A.xf[r], wr = A.wf[r];
     const double pb0 = 1.0 - eta, pb1 = eta;
     for (int el = 0; el < SH_E; ++el) {
       const int64_t e = e0 + el;
@@ -1133,7 +1113,7 @@ __global__ void __launch_bounds__(256) k_shape_far(ShapeArgs S) {
         if (ok) {
           const int64_t ip = e * q + p;
           const double xp = A.far.x[ip], yp = A.far.y[ip], nxp = A.far.nx[ip], nyp = A.far.ny[ip];
-          const double xi = c_xf[p], ww = c_wf[p] * wr;
+          const double xi = A.xf[p], ww = A.wf[p] * wr;
           const double pa0 = 1.0 - xi, pa1 = xi;
           // point-pair coefficients of the four operators
           const zd cS = (h2 * ww) * (pa0 * cw[0][0] + pa1 * cw[0][1]);
@@ -1254,7 +1234,6 @@ __global__ void __launch_bounds__(128) k_shape_near(AsmArgs A, const zd* W0, con
 
 int shape_far_forms(const ShapeArgs& a, cudaStream_t s) {
   if (a.A.q_far > 16) { set_error("shape derivative: q_far <= 16"); return 1; }
-  if (upload_rules(a.A)) { set_error("uploading quadrature rules failed"); return 3; }
   dim3 grid((unsigned)((a.A.N + SH_F - 1) / SH_F), (unsigned)((a.A.N + SH_E - 1) / SH_E));
   k_shape_far<<<grid, 256, 0, s>>>(a);
   note_launch();
@@ -1264,7 +1243,6 @@ int shape_far_forms(const ShapeArgs& a, cudaStream_t s) {
 }
 
 int shape_near_forms(const AsmArgs& A, const zd* const* W, double* part, int* nparts, cudaStream_t s) {
-  if (upload_rules(A)) { set_error("uploading quadrature rules failed"); return 3; }
   const int64_t n = A.N * (2 * A.near_band + 1);
   const unsigned blocks = (unsigned)((n + 127) / 128);
   k_shape_near<<<blocks, 128, 0, s>>>(A, W[0], W[1], W[2], W[3], part);

@@ -256,22 +256,21 @@ static int ensure_gl16() {
   return 0;
 }
 
-int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s, bool scan) {
+constexpr int ARC_P = 8192;
+int64_t arc_table_doubles() { return 2 * ARC_P + 1; }
+
+int arc_table_build(const Contour& c, ArcTable& t, double* buf, cudaStream_t s, bool scan) {
   if (ensure_gl16()) { set_error("uploading Gauss-Legendre table failed"); return 3; }
-  t.P = 8192;
-  double* len = nullptr;
-  if (cudaMalloc(&len, sizeof(double) * t.P) != cudaSuccess ||
-      cudaMalloc(&t.cum, sizeof(double) * (t.P + 1)) != cudaSuccess) {
-    set_error("out of device memory (arc table)");
-    return 4;
-  }
+  t.P = ARC_P;
+  t.cum = buf;
+  double* len = buf + ARC_P + 1;
   k_panel_lengths<<<(t.P + 127) / 128, 128, 0, s>>>(c, t.P, len);
   note_launch();
   static DeviceOnce attr;
   const int smem = (int)sizeof(double) * t.P;
   if (attr.need()) {
     cudaError_t e = cudaFuncSetAttribute(k_prefix_kahan, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) { cudaFree(len); set_error(std::string("arc table: ") + cudaGetErrorString(e)); return 3; }
+    if (e != cudaSuccess) { set_error(std::string("arc table: ") + cudaGetErrorString(e)); return 3; }
     attr.done();
   }
   if (scan) k_prefix_scan<<<1, 1024, 0, s>>>(len, t.P, t.cum);
@@ -280,7 +279,6 @@ int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s, bool scan) {
   double L = 0.0;
   cudaMemcpyAsync(&L, t.cum + t.P, sizeof(double), cudaMemcpyDeviceToHost, s);
   cudaError_t err = cudaStreamSynchronize(s);
-  cudaFree(len);
   if (err != cudaSuccess) { set_error(cudaGetErrorString(err)); return 3; }
   t.L = L;
   return 0;
@@ -296,17 +294,14 @@ int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const
   return 0;
 }
 
-int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin,
+int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, double* d,
                   cudaStream_t s) {
   const int blocks = 304;
-  double* d = nullptr;
-  if (cudaMalloc(&d, sizeof(double) * blocks) != cudaSuccess) { set_error("oom"); return 4; }
   k_min_curv<<<blocks, 256, 0, s>>>(c, t.cum, t.P, t.L, samples, d);
   note_launch();
   double h[blocks];
   cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t err = cudaStreamSynchronize(s);
-  cudaFree(d);
   if (err != cudaSuccess) { set_error(cudaGetErrorString(err)); return 3; }
   double m = 1e300;
   for (int i = 0; i < blocks; ++i) m = fmin(m, h[i]);

@@ -63,13 +63,16 @@ struct ArcTable {
 };
 
 // scan: sum the panels by a parallel double-double scan instead of one after the other
-int arc_table_build(const Contour& c, ArcTable& t, cudaStream_t s, bool scan = false);
+// buf: arc_table_doubles() of device memory, which the table keeps using.
+int64_t arc_table_doubles();
+int arc_table_build(const Contour& c, ArcTable& t, double* buf, cudaStream_t s, bool scan = false);
 // Points at arc lengths s_j = (e + xi[g]) * h for e < N, g < nq (index e*nq + g); tol: Newton step
 // that ends the inversion of the arc length.
 int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const double* xi_dev,
                  int nq, Points& out, cudaStream_t s, double tol = 1e-16);
 // Minimum curvature over a dense sample of the contour (convexity check).
-int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, cudaStream_t s);
+// (work: 304 doubles of device memory)
+int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, double* work, cudaStream_t s);
 
 // ---------------------------------------------------------------- quadrature
 struct QuadTables {
@@ -92,6 +95,7 @@ struct AsmArgs {
   int rot_ok = 0;                  // 1: far element pairs may share a reference phase (k h <= 1.2, t <= 0.019)
   KtPair ktp;
   int q_far, q_near, near_band;
+  double xf[16], wf[16], xn[16], wn[16];   // Gauss rules on [0, 1] (by value: contexts with other rules may run at the same time)
   Points far, near;                // point tables (far: q_far per element, near: q_near)
   const double* wlog;              // 3 * q_near^2 product weights (device)
   zd *S, *D, *Dt, *Nk;             // outputs
@@ -135,7 +139,8 @@ int hankel_table(double t, double* T, cudaStream_t s);
 // 32 doubles for each of ne (2 near_band + 1) pairs.  Needs a.htab.
 int near_band_pairs(const AsmArgs& a, int64_t e0, int64_t ne, double* out, cudaStream_t s);
 // First row of the four circulant operators on the circle (row 0, N entries each).
-int assemble_circle_row(const AsmArgs& a, cudaStream_t s);
+// (part: 16 N values of scratch).
+int assemble_circle_row(const AsmArgs& a, zd* part, cudaStream_t s);
 // Sampled entries (row, col) of the four operators, computed point-wise.
 int assemble_entries(const AsmArgs& a, int64_t count, const int64_t* rows, const int64_t* cols,
                      zd* out4, cudaStream_t s);
@@ -242,9 +247,9 @@ int pivoted_cholesky(zd* Gm, int b, double rel_tol, int* perm, int* rank_dev, cu
 // R^{-1}; Y must not alias X)
 int trsm_right_upper(const zd* X, int64_t ldx, int64_t m, const zd* R, int b, const int* perm,
                      const int* rank_dev, int rank_host, zd* Y, int64_t ldy, zd* work, cudaStream_t s);
-// LU with partial pivoting of an n x n column-major matrix (in place) and explicit inverse.
-int lu_inverse(zd* A, int64_t n, zd* Ainv, int* piv, int* info_dev, double* minpiv_dev,
-               cudaStream_t s);
+// Explicit inverse of an n x n column-major matrix (Gauss-Jordan, partial pivoting);
+// work: 2 n^2 + 3 n values.
+int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minpiv_dev, cudaStream_t s);
 
 // ---------------------------------------------------------------- right-hand sides / far field
 // split_phase: FP64 phase at one point per hat and FP32 offsets (~1e-7; mixed form)

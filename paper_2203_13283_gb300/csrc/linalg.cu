@@ -813,17 +813,8 @@ __global__ void k_identity(zd* M, int64_t n) {
   if (i < n) M[i * n + i] = mkz(1.0);
 }
 
-int lu_inverse(zd* A, int64_t n, zd* Ainv, int* piv, int* info_dev, double* minpiv_dev,
-               cudaStream_t s) {
-  (void)piv;
-  zd *M = nullptr, *colj = nullptr, *rowj = nullptr;
-  if (cudaMalloc(&M, sizeof(zd) * n * 2 * n) != cudaSuccess ||
-      cudaMalloc(&colj, sizeof(zd) * n) != cudaSuccess ||
-      cudaMalloc(&rowj, sizeof(zd) * 2 * n) != cudaSuccess) {
-    cudaFree(M); cudaFree(colj); cudaFree(rowj);
-    set_error("oom (capacitance inverse)");
-    return 4;
-  }
+int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minpiv_dev, cudaStream_t s) {
+  zd *M = work, *colj = M + 2 * n * n, *rowj = colj + n;
   cudaMemcpy2DAsync(M, sizeof(zd) * n, A, sizeof(zd) * n, sizeof(zd) * n, n, cudaMemcpyDeviceToDevice, s);
   cudaMemsetAsync(M + n * n, 0, sizeof(zd) * n * n, s);
   k_identity<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(M + n * n, n);
@@ -844,7 +835,6 @@ int lu_inverse(zd* A, int64_t n, zd* Ainv, int* piv, int* info_dev, double* minp
   cudaMemcpy2DAsync(Ainv, sizeof(zd) * n, M + n * n, sizeof(zd) * n, sizeof(zd) * n, n,
                     cudaMemcpyDeviceToDevice, s);
   cudaError_t err = cudaStreamSynchronize(s);
-  cudaFree(M); cudaFree(colj); cudaFree(rowj);
   if (err != cudaSuccess) { set_error(std::string("inverse: ") + cudaGetErrorString(err)); return 3; }
   return 0;
 }

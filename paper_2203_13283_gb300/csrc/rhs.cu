@@ -11,9 +11,13 @@
 
 namespace wcs {
 
-__constant__ double c_rx[16], c_rw[16];
+// Gauss rule on [0, 1], passed by value (no table shared between contexts, no
+// synchronising upload per call)
+struct Rule {
+  double x[16], w[16];
+};
 
-__global__ void k_planewave(Points P, int q, int64_t N, double h, double k, const double* angles,
+__global__ void k_planewave(Rule R, Points P, int q, int64_t N, double h, double k, const double* angles,
                             int B, zd* e, zd* hv, int64_t ld) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
@@ -25,8 +29,8 @@ __global__ void k_planewave(Points P, int q, int64_t N, double h, double k, cons
     const int64_t el = (a == 1) ? (i - 1 + N) % N : i;  // a = 1: hat i is xi on element i-1
     for (int g = 0; g < q; ++g) {
       const int64_t ip = el * q + g;
-      const double phi = (a == 1) ? c_rx[g] : 1.0 - c_rx[g];
-      const double w = h * c_rw[g] * phi;
+      const double phi = (a == 1) ? R.x[g] : 1.0 - R.x[g];
+      const double w = h * R.w[g] * phi;
       double s, c;
       sincos(k * (dc * P.x[ip] + ds * P.y[ip]), &s, &c);
       const double dn = dc * P.nx[ip] + ds * P.ny[ip];
@@ -44,7 +48,7 @@ __global__ void k_planewave(Points P, int q, int64_t N, double h, double k, cons
 // (~1e-7 absolute error).  A thread walks the 2q points of its hat once for
 // PW_ANGLES angles.
 constexpr int PW_ANGLES = 8;
-__global__ void k_planewave_split(Points P, int q, int64_t N, double h, double k, const double* angles,
+__global__ void k_planewave_split(Rule R, Points P, int q, int64_t N, double h, double k, const double* angles,
                                   int B, zd* e, zd* hv, int64_t ld) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int b0 = blockIdx.y * PW_ANGLES;
@@ -68,8 +72,8 @@ __global__ void k_planewave_split(Points P, int q, int64_t N, double h, double k
       const int64_t ip = el * q + g;
       const float dx = (float)(P.x[ip] - x0), dy = (float)(P.y[ip] - y0);
       const float nx = (float)P.nx[ip], ny = (float)P.ny[ip];
-      const float lam = (side == 1) ? (float)c_rx[g] : (float)(1.0 - c_rx[g]);
-      const float w = (float)(h * c_rw[g]) * lam;
+      const float lam = (side == 1) ? (float)R.x[g] : (float)(1.0 - R.x[g]);
+      const float w = (float)(h * R.w[g]) * lam;
 #pragma unroll
       for (int a = 0; a < PW_ANGLES; ++a) {
         float sn, cs;
@@ -95,7 +99,7 @@ __global__ void k_planewave_split(Points P, int q, int64_t N, double h, double k
   }
 }
 
-__global__ void k_farfield_matrix(Points P, int q, int64_t N, double h, double k, const double* phi,
+__global__ void k_farfield_matrix(Rule R, Points P, int q, int64_t N, double h, double k, const double* phi,
                                   int nphi, zd* E, int64_t lde) {
   const int o = blockIdx.y;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -107,8 +111,8 @@ __global__ void k_farfield_matrix(Points P, int q, int64_t N, double h, double k
     const int64_t el = (a == 1) ? (i - 1 + N) % N : i;
     for (int g = 0; g < q; ++g) {
       const int64_t ip = el * q + g;
-      const double lam = (a == 1) ? c_rx[g] : 1.0 - c_rx[g];
-      const double w = h * c_rw[g] * lam * (oc * P.nx[ip] + os * P.ny[ip]);
+      const double lam = (a == 1) ? R.x[g] : 1.0 - R.x[g];
+      const double w = h * R.w[g] * lam * (oc * P.nx[ip] + os * P.ny[ip]);
       double s, c;
       sincos(-k * (oc * P.x[ip] + os * P.y[ip]), &s, &c);
       acc += mkz(w * c, w * s);
@@ -152,7 +156,7 @@ __device__ __forceinline__ void cis_small(double d, double& s, double& c) {
   s = fma(s * z, d, d);
 }
 
-__global__ void __launch_bounds__(128) k_farfield_map(Points P, int q, int64_t N, double h, double k, const double* phi,
+__global__ void __launch_bounds__(128) k_farfield_map(Rule R, Points P, int q, int64_t N, double h, double k, const double* phi,
                                                       int nphi, zd* E, int64_t lde) {
   const int o = blockIdx.x * 32 + (threadIdx.x & 31);
   const int64_t i0 = ((int64_t)blockIdx.y * 4 + (threadIdx.x >> 5)) * FM_NODES;
@@ -173,8 +177,8 @@ __global__ void __launch_bounds__(128) k_farfield_map(Points P, int q, int64_t N
       const double d = -k * fma(oc, px[g] - x0, os * (py[g] - y0));
       double sn, cs;
       cis_small(d, sn, cs);
-      const double w = h * c_rw[g] * fma(oc, P.nx[e * q + g], os * P.ny[e * q + g]);
-      const double wr = c_rx[g] * w, wl = w - wr;
+      const double w = h * R.w[g] * fma(oc, P.nx[e * q + g], os * P.ny[e * q + g]);
+      const double wr = R.x[g] * w, wl = w - wr;
       l.x = fma(wl, cs, l.x);
       l.y = fma(wl, sn, l.y);
       r.x = fma(wr, cs, r.x);
@@ -188,21 +192,24 @@ __global__ void __launch_bounds__(128) k_farfield_map(Points P, int q, int64_t N
   }
 }
 
-static int upload(const double* xn, const double* wn, int q) {
-  if (cudaMemcpyToSymbol(c_rx, xn, sizeof(double) * q) != cudaSuccess) return 3;
-  if (cudaMemcpyToSymbol(c_rw, wn, sizeof(double) * q) != cudaSuccess) return 3;
-  return 0;
+static Rule rule(const double* xn, const double* wn, int q) {
+  Rule R{};
+  for (int i = 0; i < q; ++i) {
+    R.x[i] = xn[i];
+    R.w[i] = wn[i];
+  }
+  return R;
 }
 
 int planewave_rhs(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                   double h, double k, const double* angles, int B, zd* e, zd* hv, int64_t ld,
                   cudaStream_t s, bool split_phase) {
-  if (upload(xn, wn, q)) { set_error("upload rule"); return 3; }
+  const Rule R = rule(xn, wn, q);
   if (split_phase) {
     for (int b0 = 0; b0 < B; b0 += 65535 * PW_ANGLES) {
       const int bb = std::min(65535 * PW_ANGLES, B - b0);
       dim3 g((unsigned)((N + 127) / 128), (unsigned)((bb + PW_ANGLES - 1) / PW_ANGLES));
-      k_planewave_split<<<g, 128, 0, s>>>(near, q, N, h, k, angles + b0, bb, e + (int64_t)b0 * ld,
+      k_planewave_split<<<g, 128, 0, s>>>(R, near, q, N, h, k, angles + b0, bb, e + (int64_t)b0 * ld,
                                           hv + (int64_t)b0 * ld, ld);
       note_launch();
     }
@@ -213,7 +220,7 @@ int planewave_rhs(const Points& near, const double* wn, const double* xn, int q,
   for (int b0 = 0; b0 < B; b0 += 65535) {
     int bb = std::min(65535, B - b0);
     dim3 g((unsigned)((N + 127) / 128), (unsigned)bb);
-    k_planewave<<<g, 128, 0, s>>>(near, q, N, h, k, angles + b0, bb, e + (int64_t)b0 * ld,
+    k_planewave<<<g, 128, 0, s>>>(R, near, q, N, h, k, angles + b0, bb, e + (int64_t)b0 * ld,
                                   hv + (int64_t)b0 * ld, ld);
     note_launch();
   }
@@ -225,10 +232,10 @@ int planewave_rhs(const Points& near, const double* wn, const double* xn, int q,
 int farfield_matrix(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                     double h, double k, const double* phi, int nphi, zd* E, int64_t lde,
                     cudaStream_t s, bool differenced) {
-  if (upload(xn, wn, q)) { set_error("upload rule"); return 3; }
+  const Rule R = rule(xn, wn, q);
   const int64_t segs = (N + 4 * FM_NODES - 1) / (4 * FM_NODES);
   if (!differenced && k * h <= 0.9 && segs <= 65535) {
-    k_farfield_map<<<dim3((unsigned)((nphi + 31) / 32), (unsigned)segs), 128, 0, s>>>(near, q, N, h, k, phi, nphi, E, lde);
+    k_farfield_map<<<dim3((unsigned)((nphi + 31) / 32), (unsigned)segs), 128, 0, s>>>(R, near, q, N, h, k, phi, nphi, E, lde);
     note_launch();
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) { set_error(std::string("farfield: ") + cudaGetErrorString(err)); return 3; }
@@ -237,7 +244,7 @@ int farfield_matrix(const Points& near, const double* wn, const double* xn, int 
   for (int o0 = 0; o0 < nphi; o0 += 65535) {
     int oo = std::min(65535, nphi - o0);
     dim3 g((unsigned)((N + 127) / 128), (unsigned)oo);
-    k_farfield_matrix<<<g, 128, 0, s>>>(near, q, N, h, k, phi + o0, oo, E + o0, lde);
+    k_farfield_matrix<<<g, 128, 0, s>>>(R, near, q, N, h, k, phi + o0, oo, E + o0, lde);
     note_launch();
   }
   cudaError_t err = cudaGetLastError();

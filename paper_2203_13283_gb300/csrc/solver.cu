@@ -51,6 +51,11 @@ struct DevBuf {
     bytes = b;
     return 0;
   }
+  // ensure, giving a large buffer back first when less than a quarter of it is asked for
+  int fit(size_t b) {
+    if (bytes > ((size_t)256 << 20) && b < bytes / 4) release();
+    return ensure(b);
+  }
   void release() { cudaFree(p); p = nullptr; bytes = 0; }
   zd* z() { return (zd*)p; }
   double* d() { return (double*)p; }
@@ -80,7 +85,10 @@ struct wcs_ctx {
   bool conv_ready[4] = {false, false, false, false};
   double kinv_res = -1.0;                 // ||I - K K^-1||_F / sqrt(r) of the last factor (-1: not measured)
   int rank = -1;
+  DevBuf arcbuf;                          // arc-length table
   DevBuf U, Vw, Wt;                       // N x rank each
+  DevBuf tmp[7];                          // scratch of the skeleton (0-4) and of the factorisation (0-6), kept across calls
+  DevBuf norms, far_map;                  // column norms of a solve; far-field map
   DevBuf w1, w2, w3, w4, w5;              // N x chunk scratch
   DevBuf small;                           // small scratch
   DevBuf gwork;                           // work of the Gram inverse (N x cols)
@@ -92,7 +100,8 @@ struct wcs_ctx {
   int64_t ldp = 0;                        // plane leading dimension (bf16 elements)
   DevBuf opplanes;                        // [op][layout][plane] N x ldp bf16
   DevBuf centres, offs;                   // element centres (FP64), tables of the far route
-  DevBuf htab;                            // Hankel table, near-band blocks of gamma and of two elements of gamma_c
+  DevBuf htab;                            // mixed form: Hankel table, near-band blocks of gamma and of two elements of gamma_c;
+                                          // FP64 form: the diagonal tiles' pairs
   DevBuf tiles;                           // list of the tiles assembled in FP64
   DevBuf stage0, stage1, stage2;          // staged right-hand blocks (bf16 planes)
   int64_t stage_cols = 0;
@@ -906,21 +915,16 @@ int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream) {
   return WCS_OK;
 }
 
+// A new contour or mesh invalidates everything built on the old one.  The device
+// buffers stay with the context for the next mesh (an allocation of gigabytes and
+// its release cost milliseconds); fit() gives them back when that is much smaller.
 static void free_mesh(wcs_ctx* c) {
-  cudaFree(c->arc.cum); c->arc.cum = nullptr;
-  cudaFree(c->arc_c.cum); c->arc_c.cum = nullptr;
-  c->pts_far.release(); c->pts_near.release(); c->pts_far_c.release(); c->pts_near_c.release();
-  c->ops.release(); c->mu.release();
-  c->opplanes.release(); c->centres.release(); c->offs.release(); c->tiles.release(); c->htab.release();
-  c->stage0.release(); c->stage1.release(); c->stage2.release(); c->stage_cols = 0;
-  c->gA.release(); c->gB.release(); c->gW.release(); c->qh.release(); c->qt.release();
-  c->U.release(); c->Vw.release(); c->Wt.release(); c->Kinv.release(); c->Wa.release();
-  for (wcs_ctx::Planes* p : {&c->pVwH, &c->pWt, &c->pUH, &c->pKinvH, &c->pWa}) { p->b.release(); p->ready = false; }
-  c->sol_e.release(); c->sol_h.release(); c->sol_b.release(); c->sol_ang.release(); c->sol_j.release();
+  c->arc.cum = nullptr;
+  c->stage_cols = 0;
+  c->Kinv.release(); c->Wa.release();
+  for (wcs_ctx::Planes* p : {&c->pVwH, &c->pWt, &c->pUH, &c->pKinvH, &c->pWa}) p->ready = false;
   c->exops.release(); c->exws.release(); c->exact_ready = false;
-  if (c->fft_ready) { fft_plan_destroy(c->fft); c->fft_ready = false; }
-  circ32_release(c->circ);
-  c->conv.release();
+  c->circ.ready = false;
   for (bool& r : c->conv_ready) r = false;
   c->kinv_res = -1.0;
   c->rank = -1;
@@ -928,10 +932,8 @@ static void free_mesh(wcs_ctx* c) {
 
 int wcs_destroy(wcs_ctx* c) {
   if (!c) return WCS_OK;
-  free_mesh(c);
-  c->xf.release(); c->xn.release(); c->wn.release(); c->wlog.release();
-  c->w1.release(); c->w2.release(); c->w3.release(); c->w4.release(); c->w5.release();
-  c->small.release(); c->tcerr.release(); c->gwork.release(); c->fx.release();
+  if (c->fft_ready) fft_plan_destroy(c->fft);
+  circ32_release(c->circ);
   delete c;
   return WCS_OK;
 }
@@ -1014,7 +1016,8 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   if (N < 12 || N > (int64_t)1 << 22) { set_error("N must be in [12, 4194304]"); return WCS_ERR_ARG; }
   free_mesh(c);
   c->stage = ST_CONTOUR;
-  TRY(arc_table_build(c->contour, c->arc, c->s, c->mixed));
+  TRY(c->arcbuf.ensure(sizeof(double) * arc_table_doubles()));
+  TRY(arc_table_build(c->contour, c->arc, c->arcbuf.d(), c->s, c->mixed));
   c->L = c->arc.L;
   c->N = N;
   c->ld = (N + 7) & ~(int64_t)7;
@@ -1023,7 +1026,8 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   c->k = (k > 0) ? k : 2.0 * WCS_PI * ((double)N / 10.0) / c->L;
   if (c->k * c->h > 2.5) { set_error("k h > 2.5: mesh too coarse for the wavenumber"); return WCS_ERR_ARG; }
   c->kt = mkz(c->k, 0.4 * cbrt(c->k) * pow(c->a, -2.0 / 3.0));
-  TRY(min_curvature(c->contour, c->arc, std::max<int64_t>(16 * N, 65536), &c->kmin, c->s));
+  TRY(c->small.ensure(sizeof(double) * 304));
+  TRY(min_curvature(c->contour, c->arc, std::max<int64_t>(16 * N, 65536), &c->kmin, c->small.d(), c->s));
   if (c->kmin < -1e-9) { set_error("contour is not convex (negative curvature)"); return WCS_ERR_NOT_CONVEX; }
   // equivalent circle
   c->circle = Contour{};
@@ -1046,8 +1050,13 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   TRY(build_points(c, c->contour, c->arc, c->pts_near, c->near, c->xn.d(), qn, true));
   TRY(build_points(c, c->circle, c->arc_c, c->pts_far_c, c->far_c, c->xf.d(), qf, false));
   TRY(build_points(c, c->circle, c->arc_c, c->pts_near_c, c->near_c, c->xn.d(), qn, true));
-  TRY(fft_plan_create(c->fft, N, c->s));
-  c->fft_ready = true;
+  if (!c->fft_ready || c->fft.n != N) {   // the plan depends on N alone
+    if (c->fft_ready) fft_plan_destroy(c->fft);
+    c->fft_ready = false;
+    const int r = fft_plan_create(c->fft, N, c->s);
+    if (r) { fft_plan_destroy(c->fft); return r; }
+    c->fft_ready = true;
+  }
   TRY(sync(c));
   c->stage = ST_MESH;
   return WCS_OK;
@@ -1070,6 +1079,10 @@ static AsmArgs asm_args(wcs_ctx* c, bool circle) {
   AsmArgs A{};
   A.N = c->N; A.h = c->h; A.k = c->k; A.kt = c->kt;
   A.q_far = c->opt.q_far; A.q_near = c->opt.q_near; A.near_band = c->opt.near_band;
+  std::copy(c->quad.xf, c->quad.xf + 16, A.xf);
+  std::copy(c->quad.wf, c->quad.wf + 16, A.wf);
+  std::copy(c->quad.xn, c->quad.xn + 16, A.xn);
+  std::copy(c->quad.wn, c->quad.wn + 16, A.wn);
   A.far = circle ? c->far_c : c->far;
   A.near = circle ? c->near_c : c->near;
   A.wlog = c->wlog.d();
@@ -1150,19 +1163,18 @@ int wcs_assemble(wcs_ctx* c) {
   const int64_t N = c->N, ld = c->ld;
   bool near_tab = false;
   if (!c->mixed) {
-    TRY(c->ops.ensure(sizeof(zd) * 4 * N * ld));
+    TRY(c->ops.fit(sizeof(zd) * 4 * N * ld));
     c->S = c->ops.z(); c->D = c->S + N * ld; c->Dt = c->D + N * ld; c->Nk = c->Dt + N * ld;
     AsmArgs A = asm_args(c, false);
     A.S = c->S; A.D = c->D; A.Dt = c->Dt; A.Nk = c->Nk;
     ProfScope ps(c, CAT_ASSEMBLY, (double)N * N * c->opt.q_far * c->opt.q_far, 0.0);
-    DevBuf pre;
-    if (pre.ensure(assemble_dense_bytes(N))) (void)cudaGetLastError();   // no room: without it
-    TRY(assemble_dense(A, pre.p, c->s));
-    TRY(sync(c));
+    if (c->htab.ensure(assemble_dense_bytes(N))) (void)cudaGetLastError();   // no room: without it
+    TRY(assemble_dense(A, c->htab.bytes >= assemble_dense_bytes(N) ? c->htab.p : nullptr, c->s));
   } else {
     c->ldp = ((2 * N + 63) / 64) * 64;
-    TRY(c->opplanes.ensure(sizeof(uint16_t) * (size_t)8 * c->planes * N * c->ldp));
-    if (c->ldp != 2 * N) cudaMemsetAsync(c->opplanes.p, 0, c->opplanes.bytes, c->s);   // zero the padding columns
+    const size_t plane_bytes = sizeof(uint16_t) * (size_t)8 * c->planes * N * c->ldp;
+    TRY(c->opplanes.fit(plane_bytes));
+    if (c->ldp != 2 * N) cudaMemsetAsync(c->opplanes.p, 0, plane_bytes, c->s);   // zero the padding columns
     // element centres (xi = 1/2) and the far points relative to them
     const int qf = c->opt.q_far;
     TRY(c->centres.ensure(sizeof(double) * 6 * N));
@@ -1229,7 +1241,8 @@ int wcs_assemble(wcs_ctx* c) {
     TRY(near_band_pairs(B, N - 1, 2, row, c->s));
     B.near_buf = row;
   }
-  TRY(assemble_circle_row(B, c->s));
+  TRY(c->gwork.ensure(sizeof(zd) * 16 * N));
+  TRY(assemble_circle_row(B, c->gwork.z(), c->s));
   // mu_X(m) = sum_j X_0j e^{+2 pi i m j / N}
   TRY(fft_columns(c->fft, mu_ptr(c, MU_S), N, 4, +1, c->s));
   k_mu_finish<<<(unsigned)((N + 255) / 256), 256, 0, c->s>>>(c->mu.z(), N, c->h);
@@ -1241,7 +1254,7 @@ int wcs_assemble(wcs_ctx* c) {
   note_launch();
   cudaMemcpyAsync(&c->norm_cc, c->small.p, sizeof(double), cudaMemcpyDeviceToHost, c->s);
   TRY(sync(c));
-  c->U.release(); c->Vw.release(); c->Wt.release(); c->Kinv.release(); c->Wa.release();
+  c->Kinv.release(); c->Wa.release();
   drop_planes(c);
   c->rank = -1;
   c->stage = ST_ASSEMBLED;
@@ -1382,7 +1395,7 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   zd* Q = c->U.z();
   const double thr = tol * c->norm_cc / (10.0 * std::sqrt(2.0 / WCS_PI));
   // small scratch: Z (cap x b), Gram (b x b), perm, rank, norms
-  DevBuf Zb, Gb, Ib, Nb, GW;
+  DevBuf &GW = c->tmp[0], &Zb = c->tmp[1], &Gb = c->tmp[2], &Ib = c->tmp[3], &Nb = c->tmp[4];
   TRY(GW.ensure(sizeof(zd) * ((N + 255) / 256) * b * b));
   TRY(Zb.ensure(sizeof(zd) * (cap + b) * b));
   TRY(Gb.ensure(sizeof(zd) * 2 * b * b));   // Gram / Cholesky factor, then R^{-1}
@@ -1481,8 +1494,8 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
     ell += rk;
     if (ell > cap) ell = cap;
   }
-  c->qh.release();
-  c->qt.release();
+  for (DevBuf* q : {&c->qh, &c->qt})
+    if (q->bytes > ((size_t)256 << 20)) q->release();
   c->rank = (int)ell;
   // V^T = Q^H (C - C_c)  <=>  Vw = (C - C_c)^H Q  (V = conj(Vw))
   TRY(c->Vw.ensure(sizeof(zd) * N * std::max<int64_t>(ell, 1)));
@@ -1495,7 +1508,7 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   }
   TRY(check_tc(c));
   if (rank_out) *rank_out = (int)ell;
-  c->Wt.release(); c->Kinv.release(); c->Wa.release();
+  c->Kinv.release(); c->Wa.release();
   drop_planes(c);
   c->stage = ST_SKELETON;
   return status;
@@ -1521,7 +1534,7 @@ int wcs_factor(wcs_ctx* c) {
   if (r > 0) {
     TRY(c->Wt.ensure(sizeof(zd) * N * r));
     // W = C_c^{-1} U  (held in Wt until the inverse is applied)
-    DevBuf Wb, Kb, info;
+    DevBuf &Wb = c->tmp[0], &Kb = c->tmp[1], &info = c->tmp[2];
     DevBuf& Kinv = c->Kinv;   // kept for adjoint solves
     c->Wa.release();
     TRY(Wb.ensure(sizeof(zd) * N * r));
@@ -1537,7 +1550,8 @@ int wcs_factor(wcs_ctx* c) {
     double* minpiv = (double*)((char*)info.p + 8);
     if (!c->mixed || r < 256) {
       ProfScope ps(c, CAT_INVERSE, 8.0 * r * (double)r * r, 0.0);
-      TRY(lu_inverse(Kb.z(), r, Kinv.z(), nullptr, infod, minpiv, c->s));
+      TRY(c->tmp[3].ensure(sizeof(zd) * (2 * r * r + 3 * r)));
+      TRY(lu_inverse(Kb.z(), r, Kinv.z(), c->tmp[3].z(), infod, minpiv, c->s));
       int infoh = 0;
       double mp = 0;
       cudaMemcpyAsync(&infoh, infod, sizeof(int), cudaMemcpyDeviceToHost, c->s);
@@ -1552,7 +1566,7 @@ int wcs_factor(wcs_ctx* c) {
       // Newton-Schulz: X <- X (2I - K X) from X0 = K^H / (||K||_1 ||K||_inf),
       // which converges for any nonsingular K; products on the tensor cores
       ProfScope ps(c, CAT_INVERSE, 16.0 * r * (double)r * r, 0.0);
-      DevBuf T, sums;
+      DevBuf &T = c->tmp[4], &sums = c->tmp[5];
       TRY(T.ensure(sizeof(zd) * r * r));
       TRY(sums.ensure(sizeof(double) * (3 * r + 2 + EYE_BLOCKS)));
       double* cs = sums.d();
@@ -1562,7 +1576,7 @@ int wcs_factor(wcs_ctx* c) {
       note_launch();
       k_scaled_adjoint<<<1024, 256, 0, c->s>>>(Kb.z(), r, cs, cs + r, Kinv.z());
       note_launch();
-      DevBuf X2;
+      DevBuf& X2 = c->tmp[6];
       TRY(X2.ensure(sizeof(zd) * r * r));
       zd* X = Kinv.z();
       zd* Xn = X2.z();
@@ -1897,13 +1911,12 @@ int wcs_planewave_rhs(wcs_ctx* c, int64_t B, const double* angles, double* e, do
   TRY(check_block(c, B, hv, ld));
   if (B == 0) return WCS_OK;
   TRY(check_angles(B, angles, "planewave_rhs"));
-  DevBuf ang;
+  DevBuf& ang = c->sol_ang;
   TRY(ang.ensure(sizeof(double) * B));
   cudaMemcpyAsync(ang.p, angles, sizeof(double) * B, cudaMemcpyHostToDevice, c->s);
   int r = planewave_rhs(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, c->N, c->h, c->k, ang.d(),
                         (int)B, (zd*)e, (zd*)hv, ld, c->s);
   if (!r) r = sync(c);
-  ang.release();
   return r;
 }
 
@@ -1979,7 +1992,7 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
     return adj ? woodbury_adj(c, B, ldb_, X, ldx_, cc) : woodbury(c, B, ldb_, X, ldx_, cc);
   };
   TRY(approx_inverse(b, ldb, x, ldx));
-  DevBuf nb;
+  DevBuf& nb = c->norms;
   TRY(nb.ensure(sizeof(double) * 2 * cc));
   std::vector<double> bn(cc), rn(cc);
   TRY(column_norms(b, ldb, N, cc, nb.d(), c->s));
@@ -2140,7 +2153,6 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
       floor = worst > 10.0 * upd;
     }
   }
-  nb.release();
   TRY(check_tc(c));
   finish(worst);
   return (worst <= c->opt.refine_tol) ? 0 : WCS_ERR_NOT_CONVERGED;
@@ -2155,7 +2167,7 @@ int wcs_solve_rhs(wcs_ctx* c, int64_t B, const double* e, const double* hv, int6
   TRY(check_block(c, B, j, ldj));
   const int64_t chunk = c->opt.rhs_chunk, N = c->N;
   TRY(ensure_work(c, std::min(B, chunk)));
-  DevBuf bb;
+  DevBuf& bb = c->sol_b;
   TRY(bb.ensure(sizeof(zd) * N * std::min(B, chunk)));
   int status = WCS_OK;
   wcs_solve_info acc{};
@@ -2169,7 +2181,6 @@ int wcs_solve_rhs(wcs_ctx* c, int64_t B, const double* e, const double* hv, int6
     if (r == WCS_ERR_NOT_CONVERGED) status = r;
     else if (r) return r;
   }
-  bb.release();
   if (info) *info = acc;
   if (status) set_error("iterative refinement did not reach refine_tol");
   return status;
@@ -2582,18 +2593,15 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
   TRY(check_block(c, B, j, ldj));
   if (B == 0 || nphi == 0) return WCS_OK;
   TRY(check_angles(nphi, phi, "farfield"));
-  DevBuf E, ang;
-  TRY(E.ensure(sizeof(zd) * (int64_t)nphi * c->N));
+  DevBuf &E = c->far_map, &ang = c->sol_ang;
+  TRY(E.fit(sizeof(zd) * (int64_t)nphi * c->N));
   TRY(ang.ensure(sizeof(double) * nphi));
   cudaMemcpyAsync(ang.p, phi, sizeof(double) * nphi, cudaMemcpyHostToDevice, c->s);
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, c->N, c->h, c->k, ang.d(),
                       nphi, E.z(), nphi, c->s, false));
   TRY(cz(c, nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
          (zd*)F, ldf));
-  int r = check_tc(c);
-  E.release();
-  ang.release();
-  return r;
+  return check_tc(c);
 }
 
 static int gemm_split_impl(int64_t M, int64_t Nc, int64_t K, const double* A, int64_t lda, const double* B,
