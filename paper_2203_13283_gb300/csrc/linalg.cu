@@ -335,11 +335,107 @@ __global__ void k_gram_bwd(const zd* __restrict__ U, zd* __restrict__ Y, int64_t
   }
 }
 
+// Both filters in one kernel, the same values.  The kernels above walk a chunk with one
+// thread, every sample a load from memory behind the last (45 us for one column of 256,
+// where the two chains of 104 dependent FMA take 7).  Here a CTA keeps up to GI_SLOTS
+// chunks of one column in shared memory, each with its own GI_WARM samples before it, and
+// two lanes (real and imaginary part) filter each chunk in place.  A chunk's backward
+// filter starts in the next one, behind a short last chunk in the one after it: with more
+// than GI_SLOTS chunks a CTA also runs the forward filter of the two that follow its own.
+constexpr int GI_SLOTS = 32, GI_LD = GI_CH + GI_WARM + 1;   // odd stride: no bank conflicts
+
+__global__ void __launch_bounds__(2 * GI_SLOTS) k_gram_inverse(const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t n,
+                                                               int per, double rho, double scale) {
+  extern __shared__ zd gi[];
+  const int64_t chunks = (n + GI_CH - 1) / GI_CH, c0 = (int64_t)blockIdx.y * per;
+  const int own = (int)min((int64_t)per, chunks - c0);
+  const bool ring = chunks <= GI_SLOTS;
+  const int slots = ring ? own : own + 2;
+  const int last = (int)(n - (chunks - 1) * GI_CH);   // samples of the last chunk
+  const zd* x = X + (int64_t)blockIdx.x * ldx;
+  auto chunk = [&](int q) { return c0 + q < chunks ? c0 + q : c0 + q - chunks; };
+  auto len = [&](int q) { return chunk(q) == chunks - 1 ? last : GI_CH; };
+  for (int u = threadIdx.x; u < slots * (GI_CH + GI_WARM); u += blockDim.x) {
+    const int q = u / (GI_CH + GI_WARM), t = u - q * (GI_CH + GI_WARM);
+    if (t >= GI_WARM + len(q)) continue;
+    int64_t ii = chunk(q) * GI_CH + t - GI_WARM;
+    while (ii < 0) ii += n;
+    gi[q * GI_LD + t] = x[ii];
+  }
+  __syncthreads();
+  const int q = threadIdx.x >> 1;
+  double* g = (double*)gi + (threadIdx.x & 1);
+  if (q < slots) {
+    double acc = 0.0, *p = g + 2 * q * GI_LD;
+    const int m = len(q);
+#pragma unroll 8
+    for (int t = 0; t < GI_WARM; ++t) acc = fma(rho, acc, p[2 * t]);
+    p += 2 * GI_WARM;
+#pragma unroll 8
+    for (int t = 0; t < m; ++t) {
+      acc = fma(rho, acc, p[2 * t]);
+      p[2 * t] = acc;
+    }
+  }
+  __syncthreads();
+  double acc = 0.0;
+  if (q < own) {
+    int cur = q, off = len(q) - 1 + GI_WARM;
+    while (off >= len(cur)) {
+      off -= len(cur);
+      cur = (ring && cur + 1 == own) ? 0 : cur + 1;
+    }
+#pragma unroll 4
+    for (int t = 0; t < GI_WARM; ++t) {
+      acc = fma(rho, acc, g[2 * (cur * GI_LD + GI_WARM + off)]);
+      if (--off < 0) {
+        cur = (ring && cur == 0) ? own - 1 : cur - 1;
+        off = len(cur) - 1;
+      }
+    }
+  }
+  __syncthreads();   // the filters write in place from here on
+  if (q < own) {
+    double* p = g + 2 * (q * GI_LD + GI_WARM);
+#pragma unroll 8
+    for (int t = len(q) - 1; t >= 0; --t) {
+      acc = fma(rho, acc, p[2 * t]);
+      p[2 * t] = scale * acc;
+    }
+  }
+  __syncthreads();
+  zd* y = Y + (int64_t)blockIdx.x * ldy + c0 * GI_CH;
+  for (int u = threadIdx.x; u < own * GI_CH; u += blockDim.x) {
+    const int b = u / GI_CH, t = u - b * GI_CH;
+    if (t < len(b)) y[u] = gi[b * GI_LD + GI_WARM + t];
+  }
+}
+
 int gram_inverse(const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t n, int64_t cols, double h,
                  zd* work, cudaStream_t s) {
   if (cols <= 0) return 0;
   if (!work) { set_error("gram: no work buffer"); return 1; }
   const double rho = sqrt(3.0) - 2.0;
+  const int64_t chunks = (n + GI_CH - 1) / GI_CH;
+  const bool apart = Y + (cols - 1) * ldy + n <= X || X + (cols - 1) * ldx + n <= Y;
+  // in place only where one CTA holds the whole column
+  if (chunks <= GI_SLOTS || apart) {
+    const int per = chunks <= GI_SLOTS ? (int)chunks : GI_SLOTS - 2;
+    const size_t smem = sizeof(zd) * GI_LD * (chunks <= GI_SLOTS ? chunks : GI_SLOTS);
+    static DeviceOnce attr;
+    if (attr.need()) {
+      cudaError_t e = cudaFuncSetAttribute(k_gram_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(sizeof(zd) * GI_LD * GI_SLOTS));
+      if (e != cudaSuccess) { set_error(std::string("gram: ") + cudaGetErrorString(e)); return 3; }
+      attr.done();
+    }
+    k_gram_inverse<<<dim3((unsigned)cols, (unsigned)((chunks + per - 1) / per)), 2 * GI_SLOTS, smem, s>>>(
+        X, ldx, Y, ldy, n, per, rho, -rho * 6.0 / h);
+    note_launch();
+    cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) { set_error(std::string("gram: ") + cudaGetErrorString(err)); return 3; }
+    return 0;
+  }
   const int64_t tasks = ((n + GI_CH - 1) / GI_CH) * cols;
   const unsigned blocks = (unsigned)((tasks + 127) / 128);
   k_gram_fwd<<<blocks, 128, 0, s>>>(X, ldx, work, n, cols, rho);
@@ -509,11 +605,13 @@ constexpr int GRAM_ROWS = 256;
 // triangular numbers, row i = p - j (j + 1) / 2); both halves are written.  A CTA
 // takes GRAM_PAIRS pairs, two lanes each (real and imaginary part), so that the
 // FP64 work of a row chunk (528 pairs at b = 32) spreads over 17 CTAs instead of
-// one: at N = 2777 eleven CTAs took 185 us, 187 take 20.
-constexpr int GRAM_PAIRS = 32;
+// one: at N = 2777 eleven CTAs took 185 us.  With plain loads between the tiles'
+// barriers 187 CTAs took 91 us, most of it the loads' latency: GRAM_STAGES tiles are
+// in flight (cp.async), and what is left is the chain of 512 dependent FMA (17 us).
+constexpr int GRAM_PAIRS = 32, GRAM_TILE = 32, GRAM_STAGES = 4;
 __global__ void __launch_bounds__(2 * GRAM_PAIRS) k_gram_partial(const zd* X, int64_t ld, int64_t m, int b, zd* part) {
-  __shared__ zd xs[64][33];
-  const int64_t r0 = (int64_t)blockIdx.x * GRAM_ROWS;
+  extern __shared__ zd gram_s[];   // [stage][column][GRAM_TILE + 1]
+  const int64_t r0 = (int64_t)blockIdx.x * GRAM_ROWS, r1 = min(m, r0 + GRAM_ROWS);
   const int tid = threadIdx.x, im = tid & 1;
   const int npairs = b * (b + 1) / 2, p = blockIdx.y * GRAM_PAIRS + (tid >> 1);
   int j = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
@@ -522,18 +620,38 @@ __global__ void __launch_bounds__(2 * GRAM_PAIRS) k_gram_partial(const zd* X, in
   const bool ok = p < npairs;
   const int i = ok ? p - j * (j + 1) / 2 : 0;
   if (!ok) j = 0;
-  double acc = 0.0;
-  for (int64_t rr = r0; rr < min(m, r0 + GRAM_ROWS); rr += 32) {
-    __syncthreads();
-    for (int u = tid; u < 32 * b; u += blockDim.x) {
-      const int c = u / 32, r = u % 32;
-      xs[c][r] = (rr + r < m) ? X[(int64_t)c * ld + rr + r] : mkz(0.0);
+  __shared__ int jmax;             // the columns past the CTA's last pair are not read
+  if (tid == 0) jmax = 0;
+  __syncthreads();
+  if (ok) atomicMax(&jmax, j);
+  __syncthreads();
+  const int nc = jmax + 1;
+  const int tiles = (int)((r1 - r0 + GRAM_TILE - 1) / GRAM_TILE);
+  auto fetch = [&](int t) {
+    if (t < tiles) {
+      zd* dst = gram_s + (size_t)(t % GRAM_STAGES) * b * (GRAM_TILE + 1);
+      for (int u = tid; u < GRAM_TILE * nc; u += blockDim.x) {
+        const int c = u / GRAM_TILE, r = u % GRAM_TILE;
+        const int64_t row = r0 + (int64_t)t * GRAM_TILE + r;
+        const unsigned d = (unsigned)__cvta_generic_to_shared(dst + c * (GRAM_TILE + 1) + r);
+        const zd* src = X + (int64_t)c * ld + (row < m ? row : 0);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(row < m ? 16 : 0) : "memory");
+      }
     }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;" ::: "memory");   // one group per tile, also past the last
+  };
+  for (int t = 0; t < GRAM_STAGES - 1; ++t) fetch(t);
+  double acc = 0.0;
+  for (int t = 0; t < tiles; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(GRAM_STAGES - 2) : "memory");
+    __syncthreads();               // tile t is there; tile t - 1's stage is free
+    fetch(t + GRAM_STAGES - 1);
+    const zd* xi = gram_s + ((size_t)(t % GRAM_STAGES) * b + i) * (GRAM_TILE + 1);
+    const zd* xj = gram_s + ((size_t)(t % GRAM_STAGES) * b + j) * (GRAM_TILE + 1);
     // conj(x_i) x_j with the operations of zfma: re: fma(x, u, fma(y, v, re)); im: fma(x, v, fma(-y, u, im))
 #pragma unroll 8
-    for (int r = 0; r < 32; ++r) {
-      const zd a = xs[i][r], c = xs[j][r];
+    for (int r = 0; r < GRAM_TILE; ++r) {
+      const zd a = xi[r], c = xj[r];
       acc = fma(a.x, im ? c.y : c.x, fma(im ? -a.y : a.y, im ? c.x : c.y, acc));
     }
   }
@@ -556,7 +674,15 @@ __global__ void k_gram_reduce(const zd* part, int nparts, int b, zd* G) {
 int gram_matrix(const zd* X, int64_t ld, int64_t m, int b, zd* G, zd* work, cudaStream_t s) {
   if (b > 64) { set_error("gram_matrix: b <= 64"); return 1; }
   const int nparts = (int)((m + GRAM_ROWS - 1) / GRAM_ROWS);
-  k_gram_partial<<<dim3((unsigned)nparts, (unsigned)((b * (b + 1) / 2 + GRAM_PAIRS - 1) / GRAM_PAIRS)), 2 * GRAM_PAIRS, 0, s>>>(X, ld, m, b, work);
+  static DeviceOnce attr;
+  if (attr.need()) {
+    cudaError_t e = cudaFuncSetAttribute(k_gram_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(zd) * GRAM_STAGES * 64 * (GRAM_TILE + 1));
+    if (e != cudaSuccess) { set_error(std::string("gram: ") + cudaGetErrorString(e)); return 3; }
+    attr.done();
+  }
+  k_gram_partial<<<dim3((unsigned)nparts, (unsigned)((b * (b + 1) / 2 + GRAM_PAIRS - 1) / GRAM_PAIRS)), 2 * GRAM_PAIRS,
+                   sizeof(zd) * GRAM_STAGES * b * (GRAM_TILE + 1), s>>>(X, ld, m, b, work);
   note_launch();
   k_gram_reduce<<<(b * b + 255) / 256, 256, 0, s>>>(work, nparts, b, G);
   note_launch();
@@ -571,9 +697,15 @@ int gram_matrix(const zd* X, int64_t ld, int64_t m, int b, zd* G, zd* work, cuda
 // (upper, row j holds R[j, j..b-1] in permuted order) in Gm's upper triangle.
 // Pivot: the largest remaining diagonal entry, the first of equal ones; the
 // factorisation stops when it is <= rel_tol^2 times the first pivot (or <= 0).
-__global__ void k_pchol(zd* Gm, int b, double rel_tol, int* perm, int* rank_out) {
+// Bound: the chain of b steps (110 us at b = 32 with six barriers a step).  The pivot
+// search compares bit patterns (non-negative doubles order like integers), warp 0 takes
+// the pivot's root and reciprocal with it, the swap and the scaling of row j touch
+// disjoint elements per thread and share a phase, and the Schur update packs the
+// triangle's elements into full warps (an FP64 instruction costs its warp the same with
+// one lane or 32).
+__global__ void __launch_bounds__(512) k_pchol(zd* Gm, int b, double rel_tol, int* perm, int* rank_out) {
   extern __shared__ zd G[];
-  __shared__ double best_s, dmax_s, rjj_s, rinv_s;
+  __shared__ double dmax_s, rjj_s, rinv_s;
   __shared__ int piv_s, perm_s[64];
   const int tid = threadIdx.x;
   for (int u = tid; u < b * b; u += blockDim.x) G[u] = Gm[u];
@@ -582,67 +714,74 @@ __global__ void k_pchol(zd* Gm, int b, double rel_tol, int* perm, int* rank_out)
   int rank = b;
   for (int j = 0; j < b; ++j) {
     if (tid < 32) {
-      // warp argmax over the remaining diagonal; ties go to the lower index
-      double v = -1.0;
+      // warp argmax over the remaining diagonal; ties go to the lower index, NaN and
+      // entries below zero are never taken
+      long long v = -1;
       int p = INT_MAX;
       for (int i = j + tid; i < b; i += 32) {
-        const double d = G[i * b + i].x;
-        if (d > v) { v = d; p = i; }
+        const long long d = __double_as_longlong(G[i * b + i].x);
+        if (d > v && d <= 0x7ff0000000000000ll) { v = d; p = i; }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double v2 = __shfl_down_sync(0xffffffffu, v, o);
-        const int p2 = __shfl_down_sync(0xffffffffu, p, o);
+        const long long v2 = __shfl_xor_sync(0xffffffffu, v, o);
+        const int p2 = __shfl_xor_sync(0xffffffffu, p, o);
         if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
       }
+      const double best = v < 0 ? -1.0 : __longlong_as_double(v);
+      if (j == 0 && tid == 0) dmax_s = best;
+      __syncwarp();
+      const bool stop = best <= rel_tol * rel_tol * dmax_s || best <= 0.0;
+      const double rjj = sqrt(best), rinv = 1.0 / rjj;
       if (tid == 0) {
-        if (p == INT_MAX) { p = j; v = -1.0; }
-        if (j == 0) dmax_s = v;
-        piv_s = p;
-        best_s = v;
+        piv_s = stop ? -1 : p;
+        rjj_s = rjj;
+        rinv_s = rinv;
       }
     }
     __syncthreads();
-    const double best = best_s;
-    if (best <= rel_tol * rel_tol * dmax_s || best <= 0.0) { rank = j; break; }
     const int p = piv_s;
-    if (p != j) {
-      // symmetric swap of rows/columns j and p
-      for (int i = tid; i < b; i += blockDim.x) {
-        zd t = G[j * b + i]; G[j * b + i] = G[p * b + i]; G[p * b + i] = t;  // columns
-      }
-      __syncthreads();
-      for (int i = tid; i < b; i += blockDim.x) {
-        zd t = G[i * b + j]; G[i * b + j] = G[i * b + p]; G[i * b + p] = t;  // rows
-      }
-      if (tid == 0) { int t = perm_s[j]; perm_s[j] = perm_s[p]; perm_s[p] = t; }
-      __syncthreads();
-    }
-    // sqrt and reciprocal once: on the FP64 pipe of one SM, 512 copies of
-    // them would cost more than the whole Schur update of the step
-    if (tid == 0) {
-      rjj_s = sqrt(G[j * b + j].x);
-      rinv_s = 1.0 / rjj_s;
-    }
-    __syncthreads();
-    const double rjj = rjj_s, rinv = rinv_s;
-    // row j of R: R[j, i] = G[j, i] / rjj  (G[j, i] at column i, row j)
+    if (p < 0) { rank = j; break; }
+    // symmetric swap of rows and columns j and p, then row j of R:
+    // R[j, i] = G[j, i] / rjj (G[j, i] at column i, row j), R[j, j] = rjj.  Thread i
+    // touches G[j, i], G[p, i], G[i, j], G[i, p]; thread p the four corners.
     for (int i = tid; i < b; i += blockDim.x) {
-      if (i > j) G[i * b + j] = rinv * G[i * b + j];
-      if (i == j) G[j * b + j] = mkz(rjj);
+      if (i == j) continue;
+      zd rji = G[i * b + j];
+      if (p != j) {
+        if (i == p) {
+          const zd cpj = G[j * b + p];
+          G[p * b + p] = G[j * b + j];
+          G[j * b + p] = rji;
+          rji = cpj;
+          const int t = perm_s[j];
+          perm_s[j] = perm_s[p];
+          perm_s[p] = t;
+        } else {
+          const zd t = G[j * b + i];
+          G[j * b + i] = G[p * b + i];
+          G[p * b + i] = t;
+          const zd u = G[i * b + p];
+          G[i * b + p] = rji;
+          rji = u;
+        }
+      }
+      G[i * b + j] = i > j ? rinv_s * rji : rji;
     }
     __syncthreads();
-    // Schur complement: G[l, i] -= conj(R[j, l]) R[j, i] for j < l <= i
-    // (warp w: columns i = j + 1 + w + 16 t; lanes: rows l), mirrored into
+    if (tid == 0) G[j * b + j] = mkz(rjj_s);   // read by nobody before the next barrier
+    // Schur complement: G[l, i] -= conj(R[j, l]) R[j, i] for j < l <= i, mirrored into
     // the lower triangle, which the pivot swaps read
-    const int warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-    for (int i = j + 1 + warp; i < b; i += nw) {
+    const int w = b - 1 - j;
+    for (int u = tid; u < w * (w + 1) / 2; u += blockDim.x) {
+      int di = (int)((sqrtf(8.f * (float)u + 1.f) - 1.f) * 0.5f);
+      while (di * (di + 1) / 2 > u) --di;
+      while ((di + 1) * (di + 2) / 2 <= u) ++di;
+      const int i = j + 1 + di, l = j + 1 + u - di * (di + 1) / 2;
       const zd rji = G[i * b + j];
-      for (int l = j + 1 + lane; l <= i; l += 32) {
-        const zd v = G[i * b + l] - conj(G[l * b + j]) * rji;
-        G[i * b + l] = v;
-        if (l < i) G[l * b + i] = conj(v);
-      }
+      const zd v = G[i * b + l] - conj(G[l * b + j]) * rji;
+      G[i * b + l] = v;
+      if (l < i) G[l * b + i] = conj(v);
     }
     __syncthreads();
   }
@@ -764,48 +903,53 @@ int trsm_right_upper(const zd* X, int64_t ldx, int64_t m, const zd* R, int b, co
 // =========================================================================== Gauss-Jordan inverse
 // M = [A | I] (n x 2n, column-major, ld = n).  Step j: pick the pivot row in
 // column j, swap, scale the pivot row, eliminate column j from every other row.
-__global__ void k_gj_pivot(zd* M, int64_t n, int64_t j, zd* colj, zd* rowj, int* info,
-                           double* minpiv) {
-  __shared__ double best[512];
-  __shared__ int bidx[512];
+//
+// One launch a step: CTA c owns a column right of j (the columns up to j are not read
+// again, so column j itself stays as it is while all CTAs read it).  Each finds the pivot
+// for itself, so no step waits for a kernel that runs on one SM: pivot and update kernels
+// took 11 + 4 us a step at n = 90.
+__global__ void __launch_bounds__(256) k_gj_step(zd* M, int64_t n, int64_t j, int* info, double* minpiv) {
+  __shared__ long long key_s[8];
+  __shared__ int idx_s[8];
+  __shared__ zd inv_s;
   const int tid = threadIdx.x;
-  double b = -1.0;
-  int bi = (int)j;
+  const zd* cj = M + j * n;
+  zd* col = M + (j + 1 + blockIdx.x) * n;
+  // largest |entry|^2 of column j from row j on, the first of equal ones; squares compare
+  // like their bit patterns, NaN is never taken
+  long long key = -1;
+  int p = INT_MAX;
   for (int64_t i = j + tid; i < n; i += blockDim.x) {
-    double v = abs2(M[j * n + i]);
-    if (v > b) { b = v; bi = (int)i; }
+    const long long v = __double_as_longlong(abs2(cj[i]));
+    if (v > key && v <= 0x7ff0000000000000ll) { key = v; p = (int)i; }
   }
-  best[tid] = b;
-  bidx[tid] = bi;
+  auto take = [&](long long k2, int p2) {
+    if (k2 > key || (k2 == key && p2 < p)) { key = k2; p = p2; }
+  };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    take(__shfl_xor_sync(0xffffffffu, key, o), __shfl_xor_sync(0xffffffffu, p, o));
+  if ((tid & 31) == 0) { key_s[tid >> 5] = key; idx_s[tid >> 5] = p; }
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (tid < o && best[tid + o] > best[tid]) { best[tid] = best[tid + o]; bidx[tid] = bidx[tid + o]; }
-    __syncthreads();
-  }
-  const int64_t p = bidx[0];
-  const double pv = sqrt(best[0]);
+  for (int w = 0; w < 8; ++w) take(key_s[w], idx_s[w]);
+  if (key < 0) p = (int)j;
   if (tid == 0) {
-    if (pv < *minpiv) *minpiv = pv;
-    if (!(pv > 0.0)) *info = (int)j + 1;
-  }
-  // swap rows j and p over all 2n columns
-  if (p != j)
-    for (int64_t c = tid; c < 2 * n; c += blockDim.x) {
-      zd t = M[c * n + j]; M[c * n + j] = M[c * n + p]; M[c * n + p] = t;
+    inv_s = key > 0 ? zrecip(cj[p]) : mkz(0.0);
+    if (blockIdx.x == 0) {
+      const double pv = sqrt(key < 0 ? -1.0 : __longlong_as_double(key));
+      if (pv < *minpiv) *minpiv = pv;
+      if (!(pv > 0.0)) *info = (int)j + 1;
     }
-  __syncthreads();
-  const zd inv = (pv > 0.0) ? zrecip(M[j * n + j]) : mkz(0.0);
-  for (int64_t i = tid; i < n; i += blockDim.x) colj[i] = M[j * n + i];
-  for (int64_t c = tid; c < 2 * n; c += blockDim.x) rowj[c] = M[c * n + j] * inv;
-}
-
-__global__ void k_gj_update(zd* M, int64_t n, int64_t j, int64_t cbase, const zd* colj,
-                            const zd* rowj) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t c = cbase + blockIdx.y;
-  if (i >= n || c >= 2 * n) return;
-  if (i == j) M[c * n + i] = rowj[c];
-  else M[c * n + i] -= colj[i] * rowj[c];
+  }
+  const zd mj = col[j], mp = col[p];
+  __syncthreads();   // row j and the pivot's row of this column are read
+  const zd rowj = mp * inv_s;
+  for (int64_t i = tid; i < n; i += blockDim.x) {
+    if (i == j) { col[i] = rowj; continue; }
+    zd v = i == p ? mj : col[i];
+    v -= (i == p ? cj[j] : cj[i]) * rowj;
+    col[i] = v;
+  }
 }
 
 __global__ void k_identity(zd* M, int64_t n) {
@@ -814,7 +958,7 @@ __global__ void k_identity(zd* M, int64_t n) {
 }
 
 int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minpiv_dev, cudaStream_t s) {
-  zd *M = work, *colj = M + 2 * n * n, *rowj = colj + n;
+  zd* M = work;
   cudaMemcpy2DAsync(M, sizeof(zd) * n, A, sizeof(zd) * n, sizeof(zd) * n, n, cudaMemcpyDeviceToDevice, s);
   cudaMemsetAsync(M + n * n, 0, sizeof(zd) * n * n, s);
   k_identity<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(M + n * n, n);
@@ -823,14 +967,8 @@ int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minp
   cudaMemcpyAsync(minpiv_dev, &big, sizeof(double), cudaMemcpyHostToDevice, s);
   cudaMemsetAsync(info_dev, 0, sizeof(int), s);
   for (int64_t j = 0; j < n; ++j) {
-    k_gj_pivot<<<1, 512, 0, s>>>(M, n, j, colj, rowj, info_dev, minpiv_dev);
+    k_gj_step<<<(unsigned)(2 * n - 1 - j), 256, 0, s>>>(M, n, j, info_dev, minpiv_dev);
     note_launch();
-    const int64_t ncols = 2 * n - j;
-    for (int64_t c0 = 0; c0 < ncols; c0 += 65535) {
-      dim3 g((unsigned)((n + 255) / 256), (unsigned)std::min<int64_t>(65535, ncols - c0));
-      k_gj_update<<<g, 256, 0, s>>>(M, n, j, j + c0, colj, rowj);
-      note_launch();
-    }
   }
   cudaMemcpy2DAsync(Ainv, sizeof(zd) * n, M + n * n, sizeof(zd) * n, sizeof(zd) * n, n,
                     cudaMemcpyDeviceToDevice, s);
