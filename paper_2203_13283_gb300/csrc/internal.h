@@ -248,7 +248,7 @@ int pivoted_cholesky(zd* Gm, int b, double rel_tol, int* perm, int* rank_dev, cu
 int trsm_right_upper(const zd* X, int64_t ldx, int64_t m, const zd* R, int b, const int* perm,
                      const int* rank_dev, int rank_host, zd* Y, int64_t ldy, zd* work, cudaStream_t s);
 // Explicit inverse of an n x n column-major matrix (Gauss-Jordan, partial pivoting);
-// work: 2 n^2 + 3 n values.
+// work: 2 n^2 values.
 int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minpiv_dev, cudaStream_t s);
 
 // ---------------------------------------------------------------- right-hand sides / far field
@@ -256,9 +256,11 @@ int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minp
 int planewave_rhs(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                   double h, double k, const double* angles, int B, zd* e, zd* hv, int64_t ld,
                   cudaStream_t s, bool split_phase = false);
-// differenced: the map of a central difference (one evaluation on every route)
+// mom: farfield_moments(N) values of scratch; without it (the map of a central
+// difference) every k h takes one evaluation
 int farfield_matrix(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                     double h, double k, const double* phi, int nphi, zd* E, int64_t lde,
-                    cudaStream_t s, bool differenced);
+                    cudaStream_t s, zd* mom);
+int64_t farfield_moments(int64_t N);
 
 }  // namespace wcs

@@ -124,73 +124,125 @@ __global__ void k_farfield_matrix(Rule R, Points P, int q, int64_t N, double h, 
   E[i * lde + o] = pre * acc;
 }
 
-// The same map for the far field alone (k h <= 0.9; the shape gradient differences
-// the map and keeps the kernel above).  There every node walks the 2 q points of
-// its two elements, a full-range FP64 sincos each, and stores 16 bytes to a row of
-// the column-major map.  Here lanes run over the observation angles (contiguous in
-// the map), a thread walks FM_NODES elements and splits each element's integral
-// between the hats of its two nodes as it goes; the phase is a sincos at the
-// element's middle point and a Taylor polynomial of the difference, |d| <= k h < 0.9
-// (to d^17 / d^16: omitted terms below 2e-17 / 1e-17 of 1 at 0.9, 1e-21 at 0.5).
-// Bound: FP64 pipe, ~26 operations a point instead of ~80 twice.
+// The same map for the far field alone (k h <= 0.9; the shape gradient differences the
+// map and keeps the kernel above).  There every node walks the 2 q points of its two
+// elements, a full-range FP64 sincos each.  An element is short against the wavelength, so
+// its part of the integral, as a function of the observation angle phi, is a short
+// trigonometric polynomial: with d = k (y - y0) = r e^{i theta} from the element's middle
+// point y0 (|r| < 0.55),
+//   cos(r cos(phi - theta)) = J_0(r) + 2 sum_{even m} (-1)^(m/2) J_m(r) cos m(phi - theta),
+//   sin(r cos(phi - theta)) = 2 sum_{odd m} (-1)^((m-1)/2) J_m(r) cos m(phi - theta)
+// (Jacobi-Anger; terms above FM_M = 12 are below 4e-17), and the normal's factor moves
+// each term by one harmonic.  k_farfield_moments sums the coefficients over the
+// element's points once for all angles, one set for each of the element's two hats;
+// k_farfield_map evaluates them: 56 FMA and one sincos per element and angle, whatever
+// q, where walking the points with a Taylor polynomial each took 700 (5.6 ms at
+// N = 16384, 360 angles).  Bound: FP64 pipe.
+constexpr int FM_M = 12, FM_H = FM_M + 2;   // harmonics 0 .. FM_M + 1
 constexpr int FM_NODES = 16;
-__device__ __forceinline__ void cis_small(double d, double& s, double& c) {
-  const double z = d * d;
-  c = 4.779477332387385e-14;                     // 1 / 16!
-  c = fma(c, z, -1.1470745597729725e-11);
-  c = fma(c, z, 2.08767569878681e-09);
-  c = fma(c, z, -2.755731922398589e-07);
-  c = fma(c, z, 2.48015873015873e-05);
-  c = fma(c, z, -0.001388888888888889);
-  c = fma(c, z, 0.041666666666666664);
-  c = fma(c, z, -0.5);
-  c = fma(c, z, 1.0);
-  s = 2.8114572543455206e-15;                    // 1 / 17!
-  s = fma(s, z, -7.647163731819816e-13);
-  s = fma(s, z, 1.6059043836821613e-10);
-  s = fma(s, z, -2.505210838544172e-08);
-  s = fma(s, z, 2.7557319223985893e-06);
-  s = fma(s, z, -0.0001984126984126984);
-  s = fma(s, z, 0.008333333333333333);
-  s = fma(s, z, -0.16666666666666666);
-  s = fma(s * z, d, d);
+
+// mom[(2 e + hat) FM_H + j] = H_j: the integral's cos part (odd j) and sin part (even j)
+// are sums of Re(e^{i j phi} H_j).  Four lanes share the points of an element and hat.
+__global__ void __launch_bounds__(128) k_farfield_moments(Rule R, Points P, int q, int64_t N, double h, double k, zd* mom) {
+  const int64_t t = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const int part = (int)(t & 3), hat = (int)((t >> 2) & 1);
+  const bool ok = (t >> 3) < N;
+  const int64_t e = ok ? t >> 3 : N - 1;
+  const double* px = P.x + e * q;
+  const double* py = P.y + e * q;
+  const double x0 = px[q / 2], y0 = py[q / 2];
+  zd H[FM_H];
+#pragma unroll
+  for (int j = 0; j < FM_H; ++j) H[j] = mkz(0.0);
+  for (int g = part; g < q; g += 4) {
+    const double w = h * R.w[g] * (hat ? R.x[g] : 1.0 - R.x[g]);
+    const zd n = mkz(w * P.nx[e * q + g], w * P.ny[e * q + g]);
+    const zd zeta = mkz(0.5 * k * (px[g] - x0), -0.5 * k * (py[g] - y0));
+    const double s = abs2(zeta);
+    // J_m(r) e^{-i m theta} = zeta^m / m! f_m, f_m = sum_i (-s)^i m! / (i! (m + i)!); the two
+    // last by their series, the others by f_{m-1} = f_m - s f_{m+1} / (m (m + 1))
+    double f[FM_M + 1], up = 1.0, fm = 1.0;
+#pragma unroll
+    for (int i = 7; i >= 1; --i) {
+      up = fma(-s / (double)(i * (FM_M + 1 + i)), up, 1.0);
+      fm = fma(-s / (double)(i * (FM_M + i)), fm, 1.0);
+    }
+    f[FM_M] = fm;
+#pragma unroll
+    for (int m = FM_M; m >= 1; --m) {
+      const double lo = fma(-s * (1.0 / (double)(m * (m + 1))), up, f[m]);
+      up = f[m];
+      f[m - 1] = lo;
+    }
+    zd pw = mkz(1.0);
+#pragma unroll
+    for (int m = 0; m <= FM_M; ++m) {
+      // half of the series' coefficient: cos m(phi - theta) times the normal's factor
+      const double c = m == 0 ? f[0] : ((m / 2) % 2 ? -f[m] : f[m]);
+      const zd G = c * pw;
+      zfma(H[m + 1], conj(n), G);
+      if (m >= 2) zfma(H[m - 1], n, G);
+      if (m == 1) H[0].x += n.x * G.x - n.y * G.y;
+      pw = (1.0 / (double)(m + 1)) * (pw * zeta);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < FM_H; ++j)
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+      H[j].x += __shfl_xor_sync(0xffffffffu, H[j].x, o);
+      H[j].y += __shfl_xor_sync(0xffffffffu, H[j].y, o);
+    }
+  if (!ok || part) return;
+#pragma unroll
+  for (int j = 0; j < FM_H; ++j) mom[(2 * e + hat) * FM_H + j] = H[j];
 }
 
-__global__ void __launch_bounds__(128) k_farfield_map(Rule R, Points P, int q, int64_t N, double h, double k, const double* phi,
-                                                      int nphi, zd* E, int64_t lde) {
+// Lanes run over the observation angles (contiguous in the map); a thread walks FM_NODES
+// elements and splits each element's integral between the hats of its two nodes.
+__global__ void __launch_bounds__(128) k_farfield_map(const zd* __restrict__ mom, Points P, int q, int64_t N, double k,
+                                                      const double* phi, int nphi, zd* E, int64_t lde) {
   const int o = blockIdx.x * 32 + (threadIdx.x & 31);
   const int64_t i0 = ((int64_t)blockIdx.y * 4 + (threadIdx.x >> 5)) * FM_NODES;
   if (o >= nphi || i0 >= N) return;
   double os, oc;
   sincos(phi[o], &os, &oc);
+  double cj[FM_H], sj[FM_H];
+  cj[0] = 1.0;
+  sj[0] = 0.0;
+#pragma unroll
+  for (int j = 1; j < FM_H; ++j) {
+    cj[j] = cj[j - 1] * oc - sj[j - 1] * os;
+    sj[j] = cj[j - 1] * os + sj[j - 1] * oc;
+  }
   const double amp = k / sqrt(8.0 * WCS_PI * k);
   const zd pre = mkz(-amp * sqrt(0.5), amp * sqrt(0.5));   // i k e^{i pi/4} / sqrt(8 pi k)
   const int64_t i1 = min(N, i0 + FM_NODES);
   zd right = mkz(0.0);   // of the element before the node: its share for the hat that rises on it
   for (int64_t i = i0 - 1; i < i1; ++i) {
     const int64_t e = i < 0 ? N - 1 : i;
-    const double* px = P.x + e * q;
-    const double* py = P.y + e * q;
-    const double x0 = px[q / 2], y0 = py[q / 2];
-    zd l = mkz(0.0), r = mkz(0.0);
-    for (int g = 0; g < q; ++g) {
-      const double d = -k * fma(oc, px[g] - x0, os * (py[g] - y0));
-      double sn, cs;
-      cis_small(d, sn, cs);
-      const double w = h * R.w[g] * fma(oc, P.nx[e * q + g], os * P.ny[e * q + g]);
-      const double wr = R.x[g] * w, wl = w - wr;
-      l.x = fma(wl, cs, l.x);
-      l.y = fma(wl, sn, l.y);
-      r.x = fma(wr, cs, r.x);
-      r.y = fma(wr, sn, r.y);
+    const zd* H = mom + 2 * e * FM_H;
+    zd v[2];
+#pragma unroll
+    for (int hat = 0; hat < 2; ++hat) {
+      double a = 0.0, b = H[hat * FM_H].x;
+#pragma unroll
+      for (int j = 1; j < FM_H; ++j) {
+        const zd c = H[hat * FM_H + j];
+        if (j & 1) a = fma(cj[j], c.x, fma(-sj[j], c.y, a));
+        else b = fma(cj[j], c.x, fma(-sj[j], c.y, b));
+      }
+      v[hat] = mkz(a, -b);
     }
     double s0, c0;
-    sincos(-k * fma(oc, x0, os * y0), &s0, &c0);
+    sincos(-k * fma(oc, P.x[e * q + q / 2], os * P.y[e * q + q / 2]), &s0, &c0);
     const zd ph = pre * mkz(c0, s0);
-    if (i >= i0) E[i * lde + o] = ph * l + right;
-    right = ph * r;
+    if (i >= i0) E[i * lde + o] = ph * v[0] + right;
+    right = ph * v[1];
   }
 }
+
+int64_t farfield_moments(int64_t N) { return 2 * N * FM_H; }
 
 static Rule rule(const double* xn, const double* wn, int q) {
   Rule R{};
@@ -231,11 +283,13 @@ int planewave_rhs(const Points& near, const double* wn, const double* xn, int q,
 
 int farfield_matrix(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                     double h, double k, const double* phi, int nphi, zd* E, int64_t lde,
-                    cudaStream_t s, bool differenced) {
+                    cudaStream_t s, zd* mom) {
   const Rule R = rule(xn, wn, q);
   const int64_t segs = (N + 4 * FM_NODES - 1) / (4 * FM_NODES);
-  if (!differenced && k * h <= 0.9 && segs <= 65535) {
-    k_farfield_map<<<dim3((unsigned)((nphi + 31) / 32), (unsigned)segs), 128, 0, s>>>(R, near, q, N, h, k, phi, nphi, E, lde);
+  if (mom && k * h <= 0.9 && segs <= 65535) {
+    k_farfield_moments<<<(unsigned)((8 * N + 127) / 128), 128, 0, s>>>(R, near, q, N, h, k, mom);
+    note_launch();
+    k_farfield_map<<<dim3((unsigned)((nphi + 31) / 32), (unsigned)segs), 128, 0, s>>>(mom, near, q, N, k, phi, nphi, E, lde);
     note_launch();
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) { set_error(std::string("farfield: ") + cudaGetErrorString(err)); return 3; }

@@ -1550,7 +1550,7 @@ int wcs_factor(wcs_ctx* c) {
     double* minpiv = (double*)((char*)info.p + 8);
     if (!c->mixed || r < 256) {
       ProfScope ps(c, CAT_INVERSE, 8.0 * r * (double)r * r, 0.0);
-      TRY(c->tmp[3].ensure(sizeof(zd) * (2 * r * r + 3 * r)));
+      TRY(c->tmp[3].ensure(sizeof(zd) * 2 * r * r));
       TRY(lu_inverse(Kb.z(), r, Kinv.z(), c->tmp[3].z(), infod, minpiv, c->s));
       int infoh = 0;
       double mp = 0;
@@ -2402,7 +2402,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
   if (r == WCS_ERR_NOT_CONVERGED) status = r;
   else if (r) return r;
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, N, c->h, c->k, phd.d(), nphi, E.z(),
-                      nphi, c->s, true));
+                      nphi, c->s, nullptr));
   TRY(cz(c, nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), F.z(), nphi));
   std::vector<zd> hd(4 * B);
   TRY(column_dotc(F.z(), nphi, F.z(), nphi, nphi, B, dots.z(), c->s));
@@ -2477,7 +2477,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
     for (int sgn = 0; sgn < 2; ++sgn) {
       wcs_ctx* t = sgn == 0 ? tp.t : tm.t;
       TRY(farfield_matrix(t->near, t->quad.wn, t->quad.xn, t->opt.q_near, N, t->h, t->k, phd.d(), nphi, E.z(),
-                          nphi, c->s, true));
+                          nphi, c->s, nullptr));
       TRY(cz(c, nphi, B, N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk(j.z(), N), mkz(0.0), Wf.z(), nphi));
       TRY(column_dotc(F.z(), nphi, Wf.z(), nphi, nphi, B, dots.z(), c->s));
       cudaMemcpyAsync(hd.data(), dots.p, sizeof(zd) * B, cudaMemcpyDeviceToHost, c->s);
@@ -2594,11 +2594,11 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
   if (B == 0 || nphi == 0) return WCS_OK;
   TRY(check_angles(nphi, phi, "farfield"));
   DevBuf &E = c->far_map, &ang = c->sol_ang;
-  TRY(E.fit(sizeof(zd) * (int64_t)nphi * c->N));
+  TRY(E.fit(sizeof(zd) * ((int64_t)nphi * c->N + farfield_moments(c->N))));
   TRY(ang.ensure(sizeof(double) * nphi));
   cudaMemcpyAsync(ang.p, phi, sizeof(double) * nphi, cudaMemcpyHostToDevice, c->s);
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, c->N, c->h, c->k, ang.d(),
-                      nphi, E.z(), nphi, c->s, false));
+                      nphi, E.z(), nphi, c->s, E.z() + (int64_t)nphi * c->N));
   TRY(cz(c, nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
          (zd*)F, ldf));
   return check_tc(c);
