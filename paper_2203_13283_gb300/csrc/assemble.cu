@@ -32,9 +32,11 @@
 namespace wcs {
 
 
-struct PairOut {
-  zd v[4][4];  // [operator S~, D, D~, N][a * 2 + b]
+template <int OPS>
+struct PairSums {
+  zd v[OPS][4];  // [operator S~, D, D~, N, D and D~ of the swapped pair][a * 2 + b]
 };
+using PairOut = PairSums<4>;
 
 __device__ __forceinline__ int periodic_dist(int64_t e, int64_t f, int64_t N) {
   int64_t d = e - f;
@@ -226,15 +228,15 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
 }
 
 
-// The four operators of a far pair in FP64 from its float-float sums (farpair.cuh).
-__device__ __noinline__ void pair_far(const AsmArgs& A, int64_t e, int64_t f, PairOut& out) {
-  FarPair<false> o;
+// The operators of a far pair in FP64 from its float-float sums (farpair.cuh).
+__device__ __noinline__ void pair_far(const AsmArgs& A, int64_t e, int64_t f, PairSums<6>& out) {
+  FarPair<true> o;
   const int q = A.q_far;
-  if (q == 4) far_pair<4, false>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
-  else far_pair<0, false>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
-  const zd fac[4] = {A.fS, A.fD, A.fDt, A.fN};
+  if (q == 4) far_pair<4, true>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+  else far_pair<0, true>(A.fc, q, A.fe[e], A.fe[f], A.fp + e * q, A.fp + f * q, o);
+  const zd fac[6] = {A.fS, A.fD, A.fDt, A.fN, A.fD, A.fDt};
 #pragma unroll
-  for (int op = 0; op < 4; ++op)
+  for (int op = 0; op < 6; ++op)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const ffc v = o.value(op, j);
@@ -481,18 +483,22 @@ __device__ __forceinline__ void pair_near(const double* buf, int64_t e0, int64_t
 // Element pairs beyond the near band whose point pairs all lie below the table's
 // end (T: the table in shared or global memory): the far rule in FP64, the inner
 // sums over r shared by both target hats, the kernels' constant factors applied
-// to the sums.
-__device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t e, int64_t f, PairOut& o) {
+// to the sums.  OPS = 6 adds D and D~ of the pair (f, e), indexed by (e, f)'s hats:
+// the same Hankel values with the other element's normal.
+template <int OPS>
+__device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t e, int64_t f, PairSums<OPS>& o) {
   const int q = A.q_far;
-  zd v[4][4], vd = mkz(0.0);
+  zd v[OPS][4], vd = mkz(0.0);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) v[0][j] = v[1][j] = v[2][j] = v[3][j] = mkz(0.0);
+  for (int i = 0; i < OPS; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[i][j] = mkz(0.0);
   for (int p = 0; p < q; ++p) {
     const int64_t ip = e * q + p;
     const double xt = A.far.x[ip], yt = A.far.y[ip], nxt = A.far.nx[ip], nyt = A.far.ny[ip];
-    zd u[4][2], ud = mkz(0.0);
+    zd u[OPS][2], ud = mkz(0.0);
 #pragma unroll
-    for (int b = 0; b < 2; ++b) u[0][b] = u[1][b] = u[2][b] = u[3][b] = mkz(0.0);
+    for (int i = 0; i < OPS; ++i) u[i][0] = u[i][1] = mkz(0.0);
     for (int r = 0; r < q; ++r) {
       const int64_t ir = f * q + r;
       const double dx = xt - A.far.x[ir], dy = yt - A.far.y[ir];
@@ -502,10 +508,19 @@ __device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t
       if (x >= HT_X0) hankel_tab_poly(T, x, Hk.H0, Hk.H1, Ht.H0, Ht.H1);
       else hankel_tab_series(T, x, log(0.5 * x), Hk, Ht);
       const double gg = (dx * nxs + dy * nys) * ri, nd = nxt * nxs + nyt * nys;
-      const zd K[4] = {Ht.H0, gg * Hk.H1, gg * Ht.H1, nd * Hk.H0};
+      zd K[OPS];
+      K[0] = Ht.H0;
+      K[1] = gg * Hk.H1;
+      K[2] = gg * Ht.H1;
+      K[3] = nd * Hk.H0;
+      if constexpr (OPS == 6) {
+        const double gm = -(dx * nxt + dy * nyt) * ri;
+        K[4] = gm * Hk.H1;
+        K[5] = gm * Ht.H1;
+      }
       const double w1 = A.wf[r] * A.xf[r], w0 = A.wf[r] - w1;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < OPS; ++i) {
         zfmas(u[i][0], w0, K[i]);
         zfmas(u[i][1], w1, K[i]);
       }
@@ -513,7 +528,7 @@ __device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t
     }
     const double w1 = A.wf[p] * A.xf[p], w0 = A.wf[p] - w1;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < OPS; ++i)
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         zfmas(v[i][b], w0, u[i][b]);
@@ -529,6 +544,10 @@ __device__ __noinline__ void pair_mid(const AsmArgs& A, const double* T, int64_t
     o.v[1][j] = fD * v[1][j];
     o.v[2][j] = fDt * v[2][j];
     o.v[3][j] = i4(((j == 0 || j == 3) ? vd : -vd) - kk2h2 * v[3][j]);
+    if constexpr (OPS == 6) {
+      o.v[4][j] = fD * v[4][j];
+      o.v[5][j] = fDt * v[5][j];
+    }
   }
 }
 
@@ -545,11 +564,9 @@ constexpr int TILE = 32;
 constexpr int ASM_THREADS = 256;
 
 // One tile of node pairs from FP64 pair integrals: the 33 x 33 element pairs
-// that touch it, accumulated in acc[4][TILE][TILE].  MIXED: pairs far enough for
-// the FP32 route take it.  pre: the pairs' blocks, already integrated.
-template <int MIXED>
-__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc, const double* T = nullptr,
-                                          const zd* pre = nullptr) {
+// that touch it, accumulated in acc[4][TILE][TILE].  pre: the pairs' blocks, already
+// integrated.
+__device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t j0, zd* acc, const zd* pre) {
   const int64_t N = A.N;
   for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) acc[t] = mkz(0.0);
   __syncthreads();
@@ -567,18 +584,11 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
     if (rowok && colok) {
       const int64_t e = ((i0 - 1 + el) % N + N) % N;
       const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-      if (!MIXED && pre) {
+      if (pre) {
 #pragma unroll
         for (int op = 0; op < 4; ++op)
 #pragma unroll
           for (int j = 0; j < 4; ++j) o.v[op][j] = pre[(int64_t)idx * 16 + op * 4 + j];
-      } else if (MIXED && T) {
-        if (periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, 0, N, A.near_band, N, e, f, o);
-        else if (pair_is_far(A, e, f)) pair_far(A, e, f, o);
-        else if (pair_is_mid(A, e, f)) pair_mid(A, T, e, f, o);
-        else pair_integrals(A, e, f, o);
-      } else if (MIXED && pair_is_far(A, e, f)) {
-        pair_far(A, e, f, o);
       } else {
         pair_integrals(A, e, f, o);
       }
@@ -651,8 +661,8 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A, int64_t nt,
   const int64_t N = A.N, ti = row0 + blockIdx.y, tj = blockIdx.x;
   const int64_t i0 = ti * TILE, j0 = tj * TILE;
   const int slot = pre ? pre_slot(ti, tj, nt, N) : -1;
-  tile_sums<0>(A, i0, j0, acc, nullptr,
-               slot < 0 ? nullptr : pre + ((int64_t)blockIdx.y * PRE_SLOTS + slot) * PRE_PAIRS * 16);
+  tile_sums(A, i0, j0, acc,
+            slot < 0 ? nullptr : pre + ((int64_t)blockIdx.y * PRE_SLOTS + slot) * PRE_PAIRS * 16);
   zd* outs[4] = {A.S, A.D, A.Dt, A.Nk};
   for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) {
     const int op = t / (TILE * TILE), rem = t - op * TILE * TILE;
@@ -661,37 +671,151 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A, int64_t nt,
   }
 }
 
-// Mixed form: the tiles that k_assemble_far listed (those holding an element
-// pair nearer than its route), as split-bf16 planes in both layouts.
-__global__ void __launch_bounds__(ASM_THREADS) k_assemble_near(AsmArgs A, int64_t nt) {
-  extern __shared__ zd acc[];  // [4][TILE][TILE], then the Hankel table
+// Mixed form: the diagonal tiles and the tiles (ti, tj), ti < tj, that k_assemble_far
+// listed (those holding an element pair nearer than its route) with their mirror
+// images, as split-bf16 planes in both layouts.  S~ and N are symmetric and the Hankel
+// values of a pair (e, f) serve (f, e) too, so a listed tile and its mirror are one pass
+// (six sums per node pair) and a diagonal tile walks the pairs el <= fl only: that is 5%
+// more work a pair on half the pairs (3.1 -> 2.2 ms at N = 2777).  The sums of a diagonal
+// tile's lower half are those of its upper half, as of a tile and its mirror.
+// Bound: FP64 pipe.  A listed tile is two jobs of 16 rows, 561 pairs like a diagonal
+// tile's, so that a few hundred equal jobs spread evenly over the GPU; 192 threads fill
+// 97% of their three rounds, two CTAs a SM, the Hankel table from L1.
+constexpr int NEAR_THREADS = 192, NEAR_LD = TILE + 1, NEAR_OPS = 6;
+constexpr size_t NEAR_SMEM = sizeof(zd) * NEAR_OPS * TILE * NEAR_LD;
+
+__device__ __forceinline__ void pair_both(const AsmArgs& A, int64_t e, int64_t f, PairSums<6>& o) {
   const int64_t N = A.N;
-  const int count = A.tile_list[0];
-  double* T = nullptr;
-  if (A.near_buf) {
-    T = (double*)(acc + 4 * TILE * TILE);
-    for (int t = threadIdx.x; t < HT_SIZE; t += blockDim.x) T[t] = A.htab[t];
+  const bool band = A.near_buf && periodic_dist(e, f, N) <= A.near_band;
+  if (!band && pair_is_far(A, e, f)) { pair_far(A, e, f, o); return; }
+  if (!band && A.near_buf && pair_is_mid(A, e, f)) { pair_mid<6>(A, A.htab, e, f, o); return; }
+  PairOut p;
+  for (int m = 0; m < 2; ++m) {
+    const int64_t x = m ? f : e, y = m ? e : f;
+    if (band) pair_near(A.near_buf, 0, N, A.near_band, N, x, y, p);
+    else pair_integrals(A, x, y, p);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (m) {
+        o.v[4][j] = p.v[1][(j & 1) * 2 + (j >> 1)];
+        o.v[5][j] = p.v[2][(j & 1) * 2 + (j >> 1)];
+      } else {
+#pragma unroll
+        for (int op = 0; op < 4; ++op) o.v[op][j] = p.v[op][j];
+      }
+    }
   }
-  for (int u = blockIdx.x; u < count; u += gridDim.x) {
-    const int64_t tile = A.tile_list[1 + u];
-    const int64_t i0 = (tile / nt) * TILE, j0 = (tile % nt) * TILE;
-    tile_sums<1>(A, i0, j0, acc, T);
-    // layout 0: row i0 + li holds (re, im) of column j0 + lj at 2 (j0 + lj);
-    // layout 1 (transpose): row j0 + lj holds entry (i0 + li, j0 + lj) at 2 (i0 + li);
-    // consecutive threads walk the contiguous index
-    for (int lay = 0; lay < 2; ++lay) {
-      for (int t = threadIdx.x; t < 4 * TILE * TILE; t += blockDim.x) {
-        const int op = t / (TILE * TILE), rem = t - op * TILE * TILE;
-        const int x = rem / TILE, y = rem - (rem / TILE) * TILE;
-        const int li = lay ? y : x, lj = lay ? x : y;
+}
+
+__global__ void __launch_bounds__(NEAR_THREADS, 2) k_assemble_near(AsmArgs A, int64_t nt) {
+  extern __shared__ zd acc[];  // [6][TILE][NEAR_LD], later the packed planes
+  const int64_t N = A.N;
+  const int64_t jobs = nt + 2 * ((int64_t)A.tile_list[0] - nt);
+  const int span = TILE + 1;
+  for (int64_t u = blockIdx.x; u < jobs; u += gridDim.x) {
+    const bool diag = u < nt;
+    const int64_t tile = diag ? u * nt + u : A.tile_list[1 + nt + ((u - nt) >> 1)];
+    const int rows = diag ? TILE : TILE / 2;
+    const int64_t i0 = (tile / nt) * TILE + (diag ? 0 : ((u - nt) & 1) * rows), j0 = (tile % nt) * TILE;
+    if (i0 >= N) continue;
+    const int npairs = diag ? span * (span + 1) / 2 : (rows + 1) * span;
+    for (int t = threadIdx.x; t < NEAR_OPS * TILE * NEAR_LD; t += NEAR_THREADS) acc[t] = mkz(0.0);
+    __syncthreads();
+    for (int base = 0; base < npairs; base += NEAR_THREADS) {
+      const int idx = base + threadIdx.x;
+      int el, fl;
+      if (diag) {
+        fl = (int)((sqrtf(8.f * (float)idx + 1.f) - 1.f) * 0.5f);
+        while (fl * (fl + 1) / 2 > idx) --fl;
+        while ((fl + 1) * (fl + 2) / 2 <= idx) ++fl;
+        el = idx - fl * (fl + 1) / 2;
+      } else {
+        el = idx / span;
+        fl = idx - el * span;
+      }
+      // element row e = i0 - 1 + el feeds tile rows el - 1 (a = 1) and el (a = 0)
+      const bool valid = idx < npairs;
+      const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < rows && i0 + el < N));
+      const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
+      PairSums<6> o;
+      if (rowok && colok) {
+        const int64_t e = ((i0 - 1 + el) % N + N) % N;
+        const int64_t f = ((j0 - 1 + fl) % N + N) % N;
+        pair_both(A, e, f, o);
+      }
+#pragma unroll
+      for (int ph = 0; ph < 4; ++ph) {
+        const int a = ph >> 1, b = ph & 1;
+        const int li = el - 1 + a, lj = fl - 1 + b;
+        // a diagonal tile's sums live on and above its diagonal: a pair el < fl adds its
+        // swapped pair's share on the diagonal, a pair el = fl leaves out its lower corner
+        const bool ok = rowok && colok && li >= 0 && li < rows && lj >= 0 && lj < TILE && i0 + li < N && j0 + lj < N &&
+                        !(diag && li > lj);
+        if (ok) {
+          zd* c = acc + li * NEAR_LD + lj;
+          const bool twice = diag && li == lj && el < fl;
+#pragma unroll
+          for (int op = 0; op < 4; ++op) {
+            zd v = o.v[op][ph];
+            if (twice) v += (op == 1 || op == 2) ? o.v[op + 3][ph] : v;
+            c[op * TILE * NEAR_LD] += v;
+          }
+#pragma unroll
+          for (int op = 4; op < 6; ++op) c[op * TILE * NEAR_LD] += o.v[op][ph];
+        }
+        __syncthreads();
+      }
+    }
+    // entries as packed planes, in place
+    for (int t = threadIdx.x; t < NEAR_OPS * rows * TILE; t += NEAR_THREADS) {
+      zd* slot = acc + (t / (rows * TILE) * TILE + t / TILE % rows) * NEAR_LD + t % TILE;
+      const zd v = *slot;
+      uint16_t re[3] = {0, 0, 0}, im[3] = {0, 0, 0};
+      split3_bits(v.x, A.planes, &re[0], &re[1], &re[2]);
+      split3_bits(v.y, A.planes, &im[0], &im[1], &im[2]);
+      uint4 w;
+      w.x = (uint32_t)re[0] | ((uint32_t)im[0] << 16);
+      w.y = (uint32_t)re[1] | ((uint32_t)im[1] << 16);
+      w.z = (uint32_t)re[2] | ((uint32_t)im[2] << 16);
+      w.w = 0u;
+      *(uint4*)slot = w;
+    }
+    __syncthreads();
+    // layout 0: row i holds (re, im) of column j at 2 j; layout 1 (transpose): row j
+    // holds entry (i, j) at 2 i; consecutive threads walk the contiguous index.  Entry
+    // (j, i) of operator x comes from x (S~, N) or from the swapped pair's sums.
+    auto at = [&](int op, int li, int lj) {
+      return *(const uint4*)(acc + ((size_t)op * TILE + li) * NEAR_LD + lj);
+    };
+    auto put = [&](int op, int lay, int64_t off, const uint4& w) {
+      const uint32_t p[3] = {w.x, w.y, w.z};
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (q < A.planes) *(uint32_t*)(A.P[op][lay][q] + off) = p[q];
+    };
+    for (int t = threadIdx.x; t < 4 * rows * TILE; t += NEAR_THREADS) {
+      const int op = t / (rows * TILE), rem = t - op * rows * TILE;
+      const int mop = (op == 1 || op == 2) ? op + 3 : op;
+      if (diag) {
+        const int x = rem / TILE, y = rem % TILE;
+        if (i0 + x < N && j0 + y < N) {
+          const int64_t off = (i0 + x) * A.ldp + 2 * (j0 + y);
+          put(op, 0, off, x <= y ? at(op, x, y) : at(mop, y, x));    // entry (x, y)
+          put(op, 1, off, y <= x ? at(op, y, x) : at(mop, x, y));    // entry (y, x)
+        }
+      } else {
+        int li = rem / TILE, lj = rem % TILE;   // along j for fixed i
         if (i0 + li < N && j0 + lj < N) {
-          const zd v = acc[(op * TILE + li) * TILE + lj];
-          uint16_t re[3] = {0, 0, 0}, im[3] = {0, 0, 0};
-          split3_bits(v.x, A.planes, &re[0], &re[1], &re[2]);
-          split3_bits(v.y, A.planes, &im[0], &im[1], &im[2]);
-          const int64_t off = lay ? (j0 + lj) * A.ldp + 2 * (i0 + li) : (i0 + li) * A.ldp + 2 * (j0 + lj);
-          for (int q = 0; q < A.planes; ++q)
-            *(uint32_t*)(A.P[op][lay][q] + off) = (uint32_t)re[q] | ((uint32_t)im[q] << 16);
+          const int64_t off = (i0 + li) * A.ldp + 2 * (j0 + lj);
+          put(op, 0, off, at(op, li, lj));
+          put(op, 1, off, at(mop, li, lj));
+        }
+        lj = rem / rows;                        // along i for fixed j
+        li = rem % rows;
+        if (i0 + li < N && j0 + lj < N) {
+          const int64_t off = (j0 + lj) * A.ldp + 2 * (i0 + li);
+          put(op, 1, off, at(op, li, lj));
+          put(op, 0, off, at(mop, li, lj));
         }
       }
     }
@@ -714,7 +838,7 @@ __global__ void k_circle_row_part(AsmArgs A, zd* part) {
   const int b = v ? 0 : 1;
   PairOut o;
   if (A.near_buf && periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, N - 1, 2, A.near_band, N, e, f, o);
-  else if (A.near_buf && pair_is_mid(A, e, f)) pair_mid(A, A.htab, e, f, o);
+  else if (A.near_buf && pair_is_mid(A, e, f)) pair_mid<4>(A, A.htab, e, f, o);
   else pair_integrals(A, e, f, o);
   for (int op = 0; op < 4; ++op) part[(int64_t)op * 4 * N + t] = o.v[op][a * 2 + b];
 }
@@ -861,9 +985,7 @@ __global__ void __launch_bounds__(FAR_THREADS, 1) k_assemble_far(AsmArgs A, int6
   for (int t = threadIdx.x; t < FAR_OPS * TILE * FAR_LD; t += FAR_THREADS) facc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (__syncthreads_or(near)) {
     if (threadIdx.x == 0) {
-      const int at = 1 + atomicAdd(A.tile_list, 2);
-      A.tile_list[at] = (int)(ti * nt + tj);
-      A.tile_list[at + 1] = (int)(tj * nt + ti);
+      A.tile_list[1 + atomicAdd(A.tile_list, 1)] = (int)(ti * nt + tj);
     }
     return;
   }
@@ -966,9 +1088,7 @@ __global__ void k_diag_tiles(int* list, int64_t nt) {
 }
 
 int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t* fp64_tiles, int64_t* tiles) {
-  const size_t smem = sizeof(zd) * 4 * TILE * TILE;
-  const size_t smem_near = smem + sizeof(double) * HT_SIZE;
-  cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_near);
+  cudaFuncSetAttribute(k_assemble_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
   cudaFuncSetAttribute(k_assemble_far<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FAR_SMEM);
   cudaFuncSetAttribute(k_assemble_far<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FAR_SMEM);
   const int64_t nt = (A.N + TILE - 1) / TILE;
@@ -981,13 +1101,13 @@ int assemble_planes(const AsmArgs& A, cudaStream_t s, cudaEvent_t* mid, int64_t*
     note_launch();
   }
   if (mid) { cudaEventRecord(mid[0], s); cudaEventRecord(mid[1], s); }
-  k_assemble_near<<<(unsigned)std::min<int64_t>(nt * nt, 152 * 3), ASM_THREADS, smem_near, s>>>(A, nt);
+  k_assemble_near<<<(unsigned)std::min<int64_t>(nt * nt, 152 * 2), NEAR_THREADS, NEAR_SMEM, s>>>(A, nt);
   note_launch();
   if (fp64_tiles) {   // the tiles that took the FP64 kernel (for the work count of each kernel)
     int n = 0;
     cudaMemcpyAsync(&n, A.tile_list, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
-    *fp64_tiles = n;
+    *fp64_tiles = 2 * (int64_t)n - nt;   // the list holds one of a tile and its mirror
     *tiles = nt * nt;
   }
   cudaError_t err = cudaGetLastError();

@@ -116,7 +116,7 @@ struct AsmArgs {
   // blocks (near_band_pairs; null: pair integrals without either)
   const double* htab = nullptr;
   const double* near_buf = nullptr;
-  int* tile_list = nullptr;        // count, then the tiles that hold a pair nearer than the far route (1 + tiles)
+  int* tile_list = nullptr;        // count, then the diagonal tiles and the tiles above them that hold a pair nearer than the far route
 };
 // Fill kp.asym for kp.t and the term-count thresholds kp.xth for relative
 // tolerance tol (host).
