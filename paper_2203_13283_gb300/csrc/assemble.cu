@@ -1181,24 +1181,28 @@ int assemble_entries(const AsmArgs& A, int64_t count, const int64_t* rows, const
 // product rules and is differenced (shape_near_forms).
 // ---------------------------------------------------------------------------
 constexpr int SH_E = 8;       // element rows per block
-constexpr int SH_F = 256;     // element columns per block (8 warps x 32 lanes)
+constexpr int SH_W = 4;       // warps per block, 32 element columns each
 
-__device__ __forceinline__ zd i4(double s, zd H) { return mkz(-0.25 * s * H.y, 0.25 * s * H.x); }   // (i/4) s H
-
-__global__ void __launch_bounds__(256) k_shape_far(ShapeArgs S) {
+// Bound: FP64 pipe.  The pair's coefficients are folded into the Hankel values first
+// (k into D's, k~ into D~'s, so H1' = H0 - H1 / z needs no division), the common factor
+// i/4 is applied to the sums, and the eight row sums of a point pair cross the warp by a
+// halving exchange (9 additions instead of 40) into the warp's own accumulators:
+// 111 -> 76 ms at N = 1024, q = 6.
+__global__ void __launch_bounds__(32 * SH_W) k_shape_far(ShapeArgs S) {
   const AsmArgs& A = S.A;
   const int64_t N = A.N;
   const int q = A.q_far;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t e0 = (int64_t)blockIdx.y * SH_E;
-  const int64_t f = (int64_t)blockIdx.x * SH_F + warp * 32 + lane;
+  const int64_t f = (int64_t)blockIdx.x * 32 * SH_W + threadIdx.x;
   const bool fvalid = f < N;
-  __shared__ double rowacc[SH_E][16][8];
-  __shared__ double red[8][4];
-  for (int t = threadIdx.x; t < SH_E * 16 * 8; t += blockDim.x) (&rowacc[0][0][0])[t] = 0.0;
+  __shared__ double rowacc[SH_W][SH_E][16][8];
+  __shared__ double red[SH_W][4];
+  for (int t = threadIdx.x; t < SH_W * SH_E * 16 * 8; t += 32 * SH_W) (&rowacc[0][0][0][0])[t] = 0.0;
   __syncthreads();
   const double h = A.h, k = A.k, h2 = h * h, kk2h2 = k * k * h2;
   const zd kt = A.kt;
+  const int own = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);   // row sum left in the lane
   double sc[4] = {0.0, 0.0, 0.0, 0.0};
   const int64_t f1 = fvalid ? (f + 1) % N : 0;
   for (int r = 0; r < q; ++r) {
@@ -1210,94 +1214,94 @@ __global__ void __launch_bounds__(256) k_shape_far(ShapeArgs S) {
     for (int el = 0; el < SH_E; ++el) {
       const int64_t e = e0 + el;
       const bool ok = fvalid && e < N && periodic_dist(e, f, N) > A.near_band;
-      // per operator: sum_b W(e + a, f + b) phi_b(eta_r) for a = 0, 1; and for
-      // the derivative part of N, sum_b s_b W_N(e + a, f + b)
-      zd cw[4][2], cwd[2];
+      if (!__any_sync(0xffffffffu, ok)) continue;
+      // per operator: sum_b W(e + a, f + b) phi_b(eta_r) for a = 0, 1, times its share of
+      // the point pair's factor; for the derivative part of N, sum_ab s_a s_b W_N(e + a, f + b)
+      zd cw[4][2], cd = mkz(0.0);
+#pragma unroll
+      for (int X = 0; X < 4; ++X) cw[X][0] = cw[X][1] = mkz(0.0);
       if (ok) {
         const int64_t ea[2] = {e, (e + 1) % N};
 #pragma unroll
-        for (int X = 0; X < 4; ++X)
+        for (int a = 0; a < 2; ++a) {
+          zd w[4];
 #pragma unroll
-          for (int a = 0; a < 2; ++a) {
+          for (int X = 0; X < 4; ++X) {
             const zd w0 = S.W[X][ea[a] * N + f], w1 = S.W[X][ea[a] * N + f1];
-            cw[X][a] = pb0 * w0 + pb1 * w1;
-            if (X == 3) cwd[a] = w1 - w0;          // s_0 = -1, s_1 = +1
+            w[X] = pb0 * w0 + pb1 * w1;
+            if (X == 3) cd += (a ? wr : -wr) * (w1 - w0);   // s_0 = -1, s_1 = +1
           }
-      } else {
-#pragma unroll
-        for (int X = 0; X < 4; ++X) cw[X][0] = cw[X][1] = mkz(0.0);
-        cwd[0] = cwd[1] = mkz(0.0);
+          cw[0][a] = (h2 * wr) * w[0];
+          cw[1][a] = (h2 * wr * k) * w[1];
+          cw[2][a] = (h2 * wr) * (kt * w[2]);
+          cw[3][a] = (-kk2h2 * wr) * w[3];
+        }
       }
       for (int p = 0; p < q; ++p) {
-        double rowc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        double row[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (ok) {
           const int64_t ip = e * q + p;
           const double xp = A.far.x[ip], yp = A.far.y[ip], nxp = A.far.nx[ip], nyp = A.far.ny[ip];
-          const double xi = A.xf[p], ww = A.wf[p] * wr;
-          const double pa0 = 1.0 - xi, pa1 = xi;
-          // point-pair coefficients of the four operators
-          const zd cS = (h2 * ww) * (pa0 * cw[0][0] + pa1 * cw[0][1]);
-          const zd cD = (h2 * ww) * (pa0 * cw[1][0] + pa1 * cw[1][1]);
-          const zd cDt = (h2 * ww) * (pa0 * cw[2][0] + pa1 * cw[2][1]);
-          const zd cNn = (-kk2h2 * ww) * (pa0 * cw[3][0] + pa1 * cw[3][1]);
-          const zd cNd = ww * (cwd[1] - cwd[0]);   // s_a: -1 for a = 0, +1 for a = 1
+          const double u1 = A.wf[p] * A.xf[p], u0 = A.wf[p] - u1;
+          const zd cS = u0 * cw[0][0] + u1 * cw[0][1];
+          const zd cD = u0 * cw[1][0] + u1 * cw[1][1];      // times k
+          const zd cT = u0 * cw[2][0] + u1 * cw[2][1];      // times k~
+          const zd cN = u0 * cw[3][0] + u1 * cw[3][1];
           const double dx = xp - xq, dy = yp - yq;
-          const double R = sqrt(dx * dx + dy * dy), iR = 1.0 / R;
-          const double ux = dx * iR, uy = dy * iR;
-          const double g = (dx * nxq + dy * nyq) * iR;
+          const double R2 = dx * dx + dy * dy, ri = rsqrt(R2), R = R2 * ri;
+          const double ux = dx * ri, uy = dy * ri;
+          const double g = ux * nxq + uy * nyq;
           const double nd = nxp * nxq + nyp * nyq;
           Hankel01 Hk, Ht;
           hankel_k_kt(A, R, Hk, Ht);
-          const double z = k * R;
-          const zd zt = kt * R;
-          const zd H1pk = Hk.H0 - (1.0 / z) * Hk.H1;              // H1'(kR)
-          const zd H1pt = Ht.H0 - zdiv(Ht.H1, zt);               // H1'(k~R)
-          // S~
-          const zd aS = cS * i4(-1.0, kt * Ht.H1);               // coefficient of d^ in dK/dd
-          // D: (ik/4)[k H1' g d^ + H1 (n' - g d^)/R]
-          const zd Dd = cD * i4(k, k * g * H1pk - (g * iR) * Hk.H1);   // along d^
-          const zd Dn = cD * i4(k * iR, Hk.H1);                  // along n'
-          // D~
-          const zd Dtd = cDt * (i4(1.0, kt) * (kt * g * H1pt - (g * iR) * Ht.H1));
-          const zd Dtn = cDt * (i4(iR, kt) * Ht.H1);
-          // N
-          const zd cN = cNd + nd * cNn;
-          const zd aN = cN * i4(-k, Hk.H1);
-          const zd uR = aS + Dd + Dtd + aN;                       // dT/dd = uR d^ + (Dn + Dtn) n'
-          const zd un = Dn + Dtn;
-          const double gdx[4] = {uR.x * ux + un.x * nxq, uR.y * ux + un.y * nxq,
-                                 uR.x * uy + un.x * nyq, uR.y * uy + un.y * nyq};
-          // dT/dn' = (D + D~ terms) d^ + N: cNn (i/4) H0 n ; dT/dn = cNn (i/4) H0 n'
-          const zd vq = cD * i4(k, Hk.H1) + cDt * (i4(1.0, kt) * Ht.H1);
-          const zd wn = cNn * i4(1.0, Hk.H0);
-          // d/dk~: S~ and D~
-          const zd dkt = cS * i4(-R, Ht.H1) + cDt * (i4(R, kt) * (Ht.H0 * g));
-          // h^2-scaled part of T (all of S~, D, D~ and the k^2 h^2 part of N)
-          const zd val = cS * i4(1.0, Ht.H0) + cD * i4(k * g, Hk.H1) + cDt * (i4(g, kt) * Ht.H1) +
-                         nd * (cNn * i4(1.0, Hk.H0));
-          rowc[0] = gdx[0]; rowc[1] = gdx[1]; rowc[2] = gdx[2]; rowc[3] = gdx[3];
-          rowc[4] = wn.x * nxq; rowc[5] = wn.y * nxq; rowc[6] = wn.x * nyq; rowc[7] = wn.y * nyq;
-          col[0] -= gdx[0]; col[1] -= gdx[1]; col[2] -= gdx[2]; col[3] -= gdx[3];
-          col[4] += vq.x * ux + wn.x * nxp;
-          col[5] += vq.y * ux + wn.y * nxp;
-          col[6] += vq.x * uy + wn.x * nyp;
-          col[7] += vq.y * uy + wn.y * nyp;
+          const zd V = cD * Hk.H1 + cT * Ht.H1;              // dT/dn' along d^ (D, D~)
+          const zd F0 = cT * Ht.H0, S1 = cS * Ht.H1, M0 = cN * Hk.H0;
+          const zd un = ri * V;                              // dT/dd along n'
+          // along d^: D and D~ g [kappa H0 - 2 H1 / R], S~ -k~ H1, N -k H1
+          const zd uR = g * (k * (cD * Hk.H0) + kt * F0 - 2.0 * un) - kt * S1 -
+                        k * ((A.wf[p] * cd + nd * cN) * Hk.H1);
+          row[0] = uR.x * ux + un.x * nxq;
+          row[1] = uR.y * ux + un.y * nxq;
+          row[2] = uR.x * uy + un.x * nyq;
+          row[3] = uR.y * uy + un.y * nyq;
+          row[4] = M0.x * nxq;
+          row[5] = M0.y * nxq;
+          row[6] = M0.x * nyq;
+          row[7] = M0.y * nyq;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) col[i] -= row[i];
+          col[4] += V.x * ux + M0.x * nxp;
+          col[5] += V.y * ux + M0.y * nxp;
+          col[6] += V.x * uy + M0.x * nyp;
+          col[7] += V.y * uy + M0.y * nyp;
+          // d/dk~: S~ and D~; the h^2-scaled part of T: all but the derivative part of N
+          const zd dkt = R * (g * F0 - S1), val = cS * Ht.H0 + g * V + nd * M0;
           sc[0] += dkt.x; sc[1] += dkt.y; sc[2] += val.x; sc[3] += val.y;
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          for (int o = 16; o > 0; o >>= 1) rowc[i] += __shfl_xor_sync(0xffffffffu, rowc[i], o);
-        if (lane == 0) {
+        for (int o = 16; o >= 4; o >>= 1) {
+          const bool up = lane & o;
+          const int m = o >> 2;   // 4, 2, 1 sums kept
 #pragma unroll
-          for (int i = 0; i < 8; ++i) atomicAdd(&rowacc[el][p][i], rowc[i]);
+          for (int i = 0; i < m; ++i) {
+            const double send = up ? row[i] : row[i + m], keep = up ? row[i + m] : row[i];
+            row[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
         }
+        row[0] += __shfl_xor_sync(0xffffffffu, row[0], 2);
+        row[0] += __shfl_xor_sync(0xffffffffu, row[0], 1);
+        if ((lane & 3) == 0) rowacc[warp][el][p][own] += row[0];
       }
     }
     if (fvalid) {
       double* gr = S.Gr + 4 * iq;
       double* gn = S.Gn + 4 * iq;
+      // times i / 4
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { atomicAdd(gr + i, col[i]); atomicAdd(gn + i, col[4 + i]); }
+      for (int i = 0; i < 4; ++i) {
+        atomicAdd(gr + i, (i & 1) ? 0.25 * col[i - 1] : -0.25 * col[i + 1]);
+        atomicAdd(gn + i, (i & 1) ? 0.25 * col[4 + i - 1] : -0.25 * col[4 + i + 1]);
+      }
     }
   }
   // block sums of the scalars, then the row accumulators
@@ -1308,38 +1312,51 @@ __global__ void __launch_bounds__(256) k_shape_far(ShapeArgs S) {
     for (int i = 0; i < 4; ++i) red[warp][i] = sc[i];
   __syncthreads();
   if (threadIdx.x < 4) {
+    const int i = threadIdx.x;
     double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
-    atomicAdd(S.scal + threadIdx.x, t);
+    for (int w = 0; w < SH_W; ++w) t += red[w][i ^ 1];
+    atomicAdd(S.scal + i, (i & 1) ? 0.25 * t : -0.25 * t);
   }
-  for (int t = threadIdx.x; t < SH_E * q * 8; t += blockDim.x) {
+  for (int t = threadIdx.x; t < SH_E * q * 8; t += 32 * SH_W) {
     const int el = t / (q * 8), rem = t - el * q * 8, p = rem / 8, i = rem - p * 8;
     const int64_t e = e0 + el;
-    if (e < N) atomicAdd((i < 4 ? S.Gr : S.Gn) + 4 * (e * q + p) + (i & 3), rowacc[el][p][i]);
+    double v = 0.0;
+    for (int w = 0; w < SH_W; ++w) v += rowacc[w][el][p][i ^ 1];
+    if (e < N) atomicAdd((i < 4 ? S.Gr : S.Gn) + 4 * (e * q + p) + (i & 3), (i & 1) ? 0.25 * v : -0.25 * v);
   }
 }
 
-// Near band: sum over element pairs with distance <= near_band of the W-weighted
-// pair integrals of A's geometry (one thread per pair, block partial sums).
-__global__ void __launch_bounds__(128) k_shape_near(AsmArgs A, const zd* W0, const zd* W1, const zd* W2,
-                                                    const zd* W3, double* part) {
+// Near band: the W-weighted pair integrals of the element pairs with distance <=
+// near_band, of two geometries at once (the two sides of a central difference), summed
+// in a second kernel in the order (e, offset).  One warp per CTA and 32 pairs of one
+// offset, so that the log-kernel pairs do not hold up warps of plain ones and the pairs
+// spread over the whole GPU: one geometry with the offsets side by side ran 72 warps'
+// quartets, each as long as its heaviest pairs (2 x 5.7 -> 3.9 ms at N = 1024).
+__global__ void __launch_bounds__(32) k_shape_near(const __grid_constant__ AsmArgs A0, const __grid_constant__ AsmArgs A1,
+                                                   const zd* W0, const zd* W1, const zd* W2, const zd* W3, zd* pairs) {
+  const AsmArgs& A = blockIdx.y ? A1 : A0;
   const int64_t N = A.N;
-  const int span = 2 * A.near_band + 1;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int span = 2 * A.near_band + 1, nb = (int)((N + 31) / 32), off = (int)(blockIdx.x / nb);
+  const int64_t e = (int64_t)(blockIdx.x % nb) * 32 + threadIdx.x;
+  if (e >= N) return;
+  const int64_t f = ((e + off - A.near_band) % N + N) % N;
   zd acc = mkz(0.0);
-  if (t < N * span) {
-    const int64_t e = t / span;
-    const int64_t f = ((e + (t - e * span) - A.near_band) % N + N) % N;
-    PairOut o;
-    pair_integrals(A, e, f, o);
-    const zd* W[4] = {W0, W1, W2, W3};
+  PairOut o;
+  pair_integrals(A, e, f, o);
+  const zd* W[4] = {W0, W1, W2, W3};
 #pragma unroll
-    for (int X = 0; X < 4; ++X)
+  for (int X = 0; X < 4; ++X)
 #pragma unroll
-      for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b) acc += W[X][((e + a) % N) * N + (f + b) % N] * o.v[X][a * 2 + b];
-  }
+      for (int b = 0; b < 2; ++b) acc += W[X][((e + a) % N) * N + (f + b) % N] * o.v[X][a * 2 + b];
+  pairs[((int64_t)blockIdx.y * N + e) * span + off] = acc;
+}
+
+// block sums of n values each of the two geometries
+__global__ void __launch_bounds__(128) k_shape_near_sum(const zd* pairs, int64_t n, double* part) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const zd acc = t < n ? pairs[blockIdx.y * n + t] : mkz(0.0);
   __shared__ double red[2][4];
   double v[2] = {acc.x, acc.y};
   for (int i = 0; i < 2; ++i)
@@ -1347,6 +1364,7 @@ __global__ void __launch_bounds__(128) k_shape_near(AsmArgs A, const zd* W0, con
   if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = v[0]; red[1][threadIdx.x >> 5] = v[1]; }
   __syncthreads();
   if (threadIdx.x == 0) {
+    part += 2 * (int64_t)blockIdx.y * gridDim.x;
     part[2 * blockIdx.x] = red[0][0] + red[0][1] + red[0][2] + red[0][3];
     part[2 * blockIdx.x + 1] = red[1][0] + red[1][1] + red[1][2] + red[1][3];
   }
@@ -1354,18 +1372,22 @@ __global__ void __launch_bounds__(128) k_shape_near(AsmArgs A, const zd* W0, con
 
 int shape_far_forms(const ShapeArgs& a, cudaStream_t s) {
   if (a.A.q_far > 16) { set_error("shape derivative: q_far <= 16"); return 1; }
-  dim3 grid((unsigned)((a.A.N + SH_F - 1) / SH_F), (unsigned)((a.A.N + SH_E - 1) / SH_E));
-  k_shape_far<<<grid, 256, 0, s>>>(a);
+  dim3 grid((unsigned)((a.A.N + 32 * SH_W - 1) / (32 * SH_W)), (unsigned)((a.A.N + SH_E - 1) / SH_E));
+  k_shape_far<<<grid, 32 * SH_W, 0, s>>>(a);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("shape (far): ") + cudaGetErrorString(err)); return 3; }
   return 0;
 }
 
-int shape_near_forms(const AsmArgs& A, const zd* const* W, double* part, int* nparts, cudaStream_t s) {
-  const int64_t n = A.N * (2 * A.near_band + 1);
+int shape_near_forms(const AsmArgs& A0, const AsmArgs& A1, const zd* const* W, zd* pairs, double* part, int* nparts,
+                     cudaStream_t s) {
+  const int64_t n = A0.N * (2 * A0.near_band + 1);
   const unsigned blocks = (unsigned)((n + 127) / 128);
-  k_shape_near<<<blocks, 128, 0, s>>>(A, W[0], W[1], W[2], W[3], part);
+  k_shape_near<<<dim3((unsigned)((A0.N + 31) / 32 * (2 * A0.near_band + 1)), 2), 32, 0, s>>>(
+      A0, A1, W[0], W[1], W[2], W[3], pairs);
+  note_launch();
+  k_shape_near_sum<<<dim3(blocks, 2), 128, 0, s>>>(pairs, n, part);
   note_launch();
   *nparts = (int)blocks;
   cudaError_t err = cudaGetLastError();

@@ -209,9 +209,16 @@ __device__ void point_at(const Contour& c, const double* cum, int P, double L, d
   kap = (r0 * r0 + 2.0 * r1 * r1 - r0 * r2) / (sp * sp * sp);
 }
 
-__global__ void k_points(Contour c, const double* cum, int P, double L, int64_t N, double h,
-                         const double* xi, int nq, double tol, Points out) {
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Two rules' points in one launch: a point is a chain of Newton steps on the FP64 pipe
+// (~0.35 ms for a few thousand points, which leave most of the GPU idle), so the two sets
+// of a mesh walk theirs side by side.
+__global__ void k_points(Contour c, const double* cum, int P, double L, int64_t N, double h, PointSet s0, PointSet s1,
+                         unsigned blocks0, double tol) {
+  const bool second = blockIdx.x >= blocks0;
+  const double* xi = second ? s1.xi : s0.xi;
+  const int nq = second ? s1.nq : s0.nq;
+  const Points out = second ? s1.out : s0.out;
+  int64_t idx = (int64_t)(blockIdx.x - (second ? blocks0 : 0u)) * blockDim.x + threadIdx.x;
   if (idx >= N * nq) return;
   int64_t e = idx / nq;
   int g = (int)(idx - e * nq);
@@ -284,10 +291,10 @@ int arc_table_build(const Contour& c, ArcTable& t, double* buf, cudaStream_t s, 
   return 0;
 }
 
-int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const double* xi_dev,
-                 int nq, Points& out, cudaStream_t s, double tol) {
-  int64_t n = N * nq;
-  k_points<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(c, t.cum, t.P, t.L, N, h, xi_dev, nq, tol, out);
+int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const PointSet& s0, const PointSet& s1,
+                 cudaStream_t s, double tol) {
+  const unsigned b0 = (unsigned)((N * s0.nq + 127) / 128), b1 = (unsigned)((N * s1.nq + 127) / 128);
+  k_points<<<b0 + b1, 128, 0, s>>>(c, t.cum, t.P, t.L, N, h, s0, s1, b0, tol);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(cudaGetErrorString(err)); return 3; }

@@ -68,8 +68,13 @@ int64_t arc_table_doubles();
 int arc_table_build(const Contour& c, ArcTable& t, double* buf, cudaStream_t s, bool scan = false);
 // Points at arc lengths s_j = (e + xi[g]) * h for e < N, g < nq (index e*nq + g); tol: Newton step
 // that ends the inversion of the arc length.
-int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const double* xi_dev,
-                 int nq, Points& out, cudaStream_t s, double tol = 1e-16);
+struct PointSet {
+  const double* xi = nullptr;      // the rule's nodes on [0, 1] (device)
+  int nq = 0;                      // 0: no points
+  Points out;
+};
+int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const PointSet& s0, const PointSet& s1,
+                 cudaStream_t s, double tol);
 // Minimum curvature over a dense sample of the contour (convexity check).
 // (work: 304 doubles of device memory)
 int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, double* work, cudaStream_t s);
@@ -159,9 +164,12 @@ struct ShapeArgs {
 // parameter: accumulates Gr, Gn (zeroed by the caller) and scal.
 int shape_far_forms(const ShapeArgs& a, cudaStream_t s);
 // sum over near element pairs (distance <= near_band) of sum_X sum_ab
-// W[X](e + a, f + b) X_ef,ab with the pair integrals of A's geometry;
-// part holds per-block partial sums (2 doubles each), *nparts set.
-int shape_near_forms(const AsmArgs& A, const zd* const* W, double* part, int* nparts, cudaStream_t s);
+// W[X](e + a, f + b) X_ef,ab with the pair integrals of the geometries of A0 and A1
+// (same N, rules and band): pairs receives the sum of each pair (2 N (2 near_band + 1)
+// complex values), part per-block partial sums (2 doubles each), *nparts of A0's and then
+// as many of A1's.
+int shape_near_forms(const AsmArgs& A0, const AsmArgs& A1, const zd* const* W, zd* pairs, double* part, int* nparts,
+                     cudaStream_t s);
 
 // ---------------------------------------------------------------- FFT
 struct FFTPlan {

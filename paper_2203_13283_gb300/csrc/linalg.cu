@@ -229,25 +229,55 @@ static bool zgemm_small(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZVie
 // K in order, for up to eight columns: a half-warp's 16 lanes form the real and
 // the other 16 the imaginary parts of 16 rows of one column, with the operations
 // of zfma in k_zgemm's order (the same bits).  Bound by the FP64 pipe, whose
-// quarter of an SM issues one warp instruction in 64 clocks: 2 K of them a warp.
+// quarter of an SM issues one warp instruction in 64 clocks: 2 K of them a warp
+// (63 us at K = 1024).  Operand tiles of ZS_K steps come through shared memory, ZS_ST in
+// flight: with plain loads the chain waited for them (410 us, cold caches).
+constexpr int ZS_K = 32, ZS_ST = 4;
 __global__ void __launch_bounds__(128) k_zgemm_serial(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B,
                                                       zd beta, zd* __restrict__ C, int64_t ldc) {
-  const int lane = threadIdx.x & 31, half = lane >> 4;
-  const int64_t i = (int64_t)blockIdx.x * 16 + (lane & 15), j = (int64_t)blockIdx.y * 4 + (threadIdx.x >> 5);
-  if (j >= n) return;
-  const zd* a = A.p + min(i, m - 1) * A.rs;
-  const zd* b = B.p + j * B.cs;
+  __shared__ zd as[ZS_ST][16][ZS_K + 1], bs[ZS_ST][4][ZS_K + 1];
+  const int tid = threadIdx.x, lane = tid & 31, half = lane >> 4, warp = tid >> 5;
+  const int64_t i0 = (int64_t)blockIdx.x * 16, j0 = (int64_t)blockIdx.y * 4;
+  const int64_t tiles = (k + ZS_K - 1) / ZS_K;
+  auto copy = [](zd* dst, const zd* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+  };
+  auto fetch = [&](int64_t t) {
+    if (t < tiles) {
+      const int st = (int)(t % ZS_ST);
+      const int64_t k0 = t * ZS_K;
+#pragma unroll
+      for (int u = tid; u < 16 * ZS_K; u += 128) {   // lanes along the operand's contiguous index
+        const int r = A.cs == 1 ? u / ZS_K : u % 16, c = A.cs == 1 ? u % ZS_K : u / 16;
+        if (k0 + c < k) copy(&as[st][r][c], A.p + min(i0 + r, m - 1) * A.rs + (k0 + c) * A.cs);
+      }
+      const int r = B.cs == 1 ? tid % 4 : tid / ZS_K, c = B.cs == 1 ? tid / 4 : tid % ZS_K;
+      if (k0 + c < k) copy(&bs[st][r][c], B.p + min(j0 + r, n - 1) * B.cs + (k0 + c) * B.rs);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");   // one group per tile, also past the last
+  };
+  for (int t = 0; t < ZS_ST - 1; ++t) fetch(t);
   double acc = 0.0;
+  for (int64_t t = 0; t < tiles; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(ZS_ST - 2) : "memory");
+    __syncthreads();               // tile t is there; tile t - 1's stage is free
+    fetch(t + ZS_ST - 1);
+    const zd* a = as[t % ZS_ST][lane & 15];
+    const zd* b = bs[t % ZS_ST][warp];
+    const int steps = (int)min((int64_t)ZS_K, k - t * ZS_K);
 #pragma unroll 8
-  for (int64_t t = 0; t < k; ++t) {
-    zd v = a[t * A.cs], w = b[t * B.rs];
-    if (A.conj) v.y = -v.y;
-    if (B.conj) w.y = -w.y;
-    // re: fma(a.x, b.x, fma(-a.y, b.y, re)); im: fma(a.x, b.y, fma(a.y, b.x, im))
-    acc = fma(v.x, half ? w.y : w.x, fma(half ? v.y : -v.y, half ? w.x : w.y, acc));
+    for (int c = 0; c < steps; ++c) {
+      zd v = a[c], w = b[c];
+      if (A.conj) v.y = -v.y;
+      if (B.conj) w.y = -w.y;
+      // re: fma(a.x, b.x, fma(-a.y, b.y, re)); im: fma(a.x, b.y, fma(a.y, b.x, im))
+      acc = fma(v.x, half ? w.y : w.x, fma(half ? v.y : -v.y, half ? w.x : w.y, acc));
+    }
   }
   const double im = __shfl_down_sync(0xffffffffu, acc, 16);
-  if (half || i >= m) return;
+  const int64_t i = i0 + (lane & 15), j = j0 + warp;
+  if (half || i >= m || j >= n) return;
   zd r = alpha * mkz(acc, im);
   zd* o = C + j * ldc + i;
   if (!(beta.x == 0.0 && beta.y == 0.0)) r += beta * (*o);

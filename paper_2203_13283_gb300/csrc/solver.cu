@@ -876,7 +876,7 @@ int wcs_default_options(wcs_options* o) {
   return WCS_OK;
 }
 
-int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream) {
+static int create_context(wcs_ctx** out, const wcs_options* opt, void* stream, const QuadTables* rules) {
   if (!out) { set_error("null output pointer"); return WCS_ERR_ARG; }
   wcs_options o;
   if (opt) o = *opt; else wcs_default_options(&o);
@@ -907,13 +907,19 @@ int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream) {
   c->mixed = (o.precision == WCS_PREC_MIXED);
   c->planes = o.mixed_planes;
   c->rhs_planes = o.rhs_planes;
-  c->quad.q_far = o.q_far;
-  c->quad.q_near = o.q_near;
-  c->quad.near_band = o.near_band;
-  build_quad_tables(c->quad);
+  if (rules) {
+    c->quad = *rules;
+  } else {
+    c->quad.q_far = o.q_far;
+    c->quad.q_near = o.q_near;
+    c->quad.near_band = o.near_band;
+    build_quad_tables(c->quad);
+  }
   *out = c;
   return WCS_OK;
 }
+
+int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream) { return create_context(out, opt, stream, nullptr); }
 
 // A new contour or mesh invalidates everything built on the old one.  The device
 // buffers stay with the context for the next mesh (an allocation of gigabytes and
@@ -1000,14 +1006,23 @@ int wcs_contour_perturb(wcs_ctx* c, int M, const double* alpha, const double* be
 // The mixed form's points need what its 24-bit entries do; the FP64 form keeps every bit.
 static double mesh_tol(const wcs_ctx* c) { return c->mixed ? 1e-9 : 1e-16; }
 
-static int build_points(wcs_ctx* c, const Contour& k, const ArcTable& t, DevBuf& buf, Points& P,
-                        const double* xi_dev, int q, bool with_kappa) {
-  const int64_t n = c->N * q;
-  TRY(buf.ensure(sizeof(double) * n * 5));
-  double* b = buf.d();
-  P.x = b; P.y = b + n; P.nx = b + 2 * n; P.ny = b + 3 * n; P.kappa = with_kappa ? b + 4 * n : nullptr;
-  P.n = n;
-  return points_build(k, t, c->N, c->h, xi_dev, q, P, c->s, mesh_tol(c));
+// the far and the near points of a contour
+static int build_points(wcs_ctx* c, const Contour& k, const ArcTable& t, DevBuf& bf, Points& F, DevBuf& bn, Points& M) {
+  PointSet s[2];
+  for (int i = 0; i < 2; ++i) {
+    const int q = i ? c->opt.q_near : c->opt.q_far;
+    const int64_t n = c->N * q;
+    DevBuf& buf = i ? bn : bf;
+    Points& P = i ? M : F;
+    TRY(buf.ensure(sizeof(double) * n * 5));
+    double* b = buf.d();
+    P.x = b; P.y = b + n; P.nx = b + 2 * n; P.ny = b + 3 * n; P.kappa = i ? b + 4 * n : nullptr;
+    P.n = n;
+    s[i].xi = i ? c->xn.d() : c->xf.d();
+    s[i].nq = q;
+    s[i].out = P;
+  }
+  return points_build(k, t, c->N, c->h, s[0], s[1], c->s, mesh_tol(c));
 }
 
 int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
@@ -1046,10 +1061,8 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   for (int t = 0; t < 3; ++t)
     cudaMemcpyAsync(c->wlog.d() + t * qn * qn, c->quad.wlog[t].data(), sizeof(double) * qn * qn,
                     cudaMemcpyHostToDevice, c->s);
-  TRY(build_points(c, c->contour, c->arc, c->pts_far, c->far, c->xf.d(), qf, false));
-  TRY(build_points(c, c->contour, c->arc, c->pts_near, c->near, c->xn.d(), qn, true));
-  TRY(build_points(c, c->circle, c->arc_c, c->pts_far_c, c->far_c, c->xf.d(), qf, false));
-  TRY(build_points(c, c->circle, c->arc_c, c->pts_near_c, c->near_c, c->xn.d(), qn, true));
+  TRY(build_points(c, c->contour, c->arc, c->pts_far, c->far, c->pts_near, c->near));
+  TRY(build_points(c, c->circle, c->arc_c, c->pts_far_c, c->far_c, c->pts_near_c, c->near_c));
   if (!c->fft_ready || c->fft.n != N) {   // the plan depends on N alone
     if (c->fft_ready) fft_plan_destroy(c->fft);
     c->fft_ready = false;
@@ -1147,7 +1160,7 @@ int wcs_geometry_sample(wcs_ctx* c, int64_t count, const double* s_host, double*
   P.n = count;
   // one "element" with count local nodes
   const int64_t savedN = c->N;
-  int r = points_build(c->contour, c->arc, 1, c->h, sb.d(), (int)count, P, c->s);
+  int r = points_build(c->contour, c->arc, 1, c->h, PointSet{sb.d(), (int)count, P}, PointSet{}, c->s, 1e-16);
   (void)savedN;
   if (r) { sb.release(); pb.release(); return r; }
   cudaMemcpyAsync(out_host, pb.p, sizeof(double) * count * 5, cudaMemcpyDeviceToHost, c->s);
@@ -1183,7 +1196,7 @@ int wcs_assemble(wcs_ctx* c) {
     cudaMemcpyAsync(half, &hv, sizeof(double), cudaMemcpyHostToDevice, c->s);
     Points cp;
     cp.x = c->centres.d(); cp.y = cp.x + N; cp.nx = cp.y + N; cp.ny = cp.nx + N; cp.kappa = nullptr; cp.n = N;
-    TRY(points_build(c->contour, c->arc, N, c->h, half, 1, cp, c->s, mesh_tol(c)));
+    TRY(points_build(c->contour, c->arc, N, c->h, PointSet{half, 1, cp}, PointSet{}, c->s, mesh_tol(c)));
     TRY(c->offs.ensure(sizeof(FarElem) * N + sizeof(FarPoint) * N * qf));
     FarElem* fe = (FarElem*)c->offs.p;
     FarPoint* fp = (FarPoint*)(fe + N);
@@ -2247,7 +2260,7 @@ static int make_scratch(wcs_ctx* c, CtxGuard& g) {
   o.precision = WCS_PREC_FP64;
   o.zfast = 0.0;
   o.exact_residual = 0;
-  return wcs_create(&g.t, &o, (void*)c->s);
+  return create_context(&g.t, &o, (void*)c->s, &c->quad);   // the same rules: its tables serve
 }
 
 __global__ void k_geo_dot(const double* Gr, const double* Gn, Points pp, Points pm, int64_t n, double* part) {
@@ -2310,12 +2323,13 @@ template <typename F>
 static int shape_forms(wcs_ctx* c, const zd* const* W, int M, int i0, int i1, double delta, zd* out, CtxGuard& tp,
                        CtxGuard& tm, F per_param) {
   const int64_t N = c->N, nq = N * c->opt.q_far;
-  DevBuf gr, gn, sc, part;
+  DevBuf gr, gn, sc, part, pairs;
   TRY(gr.ensure(sizeof(double) * 4 * nq));
   TRY(gn.ensure(sizeof(double) * 4 * nq));
   TRY(sc.ensure(sizeof(double) * 4));
-  const int64_t nblk_geo = (nq + 255) / 256, nblk_near = (N * (2 * c->opt.near_band + 1) + 127) / 128;
-  TRY(part.ensure(sizeof(double) * 2 * std::max(nblk_geo, nblk_near)));
+  const int64_t nblk_geo = (nq + 255) / 256, npair = N * (2 * c->opt.near_band + 1), nblk_near = (npair + 127) / 128;
+  TRY(part.ensure(sizeof(double) * 2 * std::max(nblk_geo, 2 * nblk_near)));
+  TRY(pairs.ensure(sizeof(zd) * 2 * npair));
   cudaMemsetAsync(gr.p, 0, gr.bytes, c->s);
   cudaMemsetAsync(gn.p, 0, gn.bytes, c->s);
   cudaMemsetAsync(sc.p, 0, sc.bytes, c->s);
@@ -2343,10 +2357,9 @@ static int shape_forms(wcs_ctx* c, const zd* const* W, int M, int i0, int i1, do
     note_launch();
     TRY(sum_parts(c, part.d(), (int)nblk_geo, &geo));
     int nb = 0;
-    TRY(shape_near_forms(asm_args(tp.t, false), W, part.d(), &nb, c->s));
+    TRY(shape_near_forms(asm_args(tp.t, false), asm_args(tm.t, false), W, pairs.z(), part.d(), &nb, c->s));
     TRY(sum_parts(c, part.d(), nb, &np_));
-    TRY(shape_near_forms(asm_args(tm.t, false), W, part.d(), &nb, c->s));
-    TRY(sum_parts(c, part.d(), nb, &nm_));
+    TRY(sum_parts(c, part.d() + 2 * nb, nb, &nm_));
     const double dL = (tp.t->L - tm.t->L) / (2.0 * delta);
     const zd dkt = (1.0 / (2.0 * delta)) * (tp.t->kt - tm.t->kt);
     const zd far = (1.0 / (2.0 * delta)) * geo + s_kt * dkt + (2.0 * dL / c->L) * s_h2;
