@@ -584,7 +584,9 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
     if (rowok && colok) {
       const int64_t e = ((i0 - 1 + el) % N + N) % N;
       const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-      if (pre) {
+      if (A.near_buf && periodic_dist(e, f, N) <= A.near_band) {
+        pair_near(A.near_buf, 0, N, A.near_band, N, e, f, o);
+      } else if (pre) {
 #pragma unroll
         for (int op = 0; op < 4; ++op)
 #pragma unroll
@@ -611,9 +613,14 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
 // FP64 form.  The tiles around the diagonal hold the near band (144 singular
 // points a pair) and the pairs below the expansion range: a CTA of eight warps
 // that walks such a tile takes 40 ms while the others take one.  Their pairs are
-// integrated by one warp per CTA first (k_assemble_pairs; the 32 pairs of a warp
-// are those of the tile kernel, whose recurrences start at the warp's largest
-// index), so that the work spreads over the chip; the tile kernel then only sums.
+// integrated by one warp per CTA first (k_assemble_pairs), so that the work spreads
+// over the chip; the tile kernel then only sums.  The far pairs of a warp are those of
+// the tile kernel's warp, whose recurrences start at the warp's largest index.  Near-band
+// pairs are taken out of these warps (in a diagonal tile every warp had some, and its 23
+// far lanes waited for them: 54 ms at N = 1024, 34 apart): a table with 32
+// pairs of one offset to a warp, as long as every point below x = 4 starts its
+// recurrence at the same index (28) whatever the warp.  The circle's row, a chain of one
+// near-band pair's length on a few warps (5.9 ms on its own), runs beside them.
 constexpr int PRE_OFF = 3, PRE_SLOTS = 2 * PRE_OFF + 1, PRE_PAIRS = (TILE + 1) * (TILE + 1);
 
 // Slot of tile (ti, tj) in its row's integrated tiles, -1 for the others: tile
@@ -629,30 +636,83 @@ __device__ __forceinline__ int pre_slot(int64_t ti, int64_t tj, int64_t nt, int6
   return (off == 0 || min(g1, g2) <= 34) ? (int)(off + PRE_OFF) : -1;
 }
 
-__global__ void __launch_bounds__(32) k_assemble_pairs(AsmArgs A, int64_t nt, int64_t row0, zd* pre) {
-  const int64_t N = A.N, ti = row0 + blockIdx.z;
-  const int64_t slot = blockIdx.y;
-  int64_t tj = nt <= PRE_SLOTS ? ti + slot : ti + slot - PRE_OFF;
-  tj = ((tj % nt) + nt) % nt;
-  if (slot >= nt || pre_slot(ti, tj, nt, N) != slot) return;
-  const int64_t i0 = ti * TILE, j0 = tj * TILE;
-  const int span = TILE + 1;
-  const int idx = blockIdx.x * 32 + threadIdx.x;
-  const int el = idx / span, fl = idx - (idx / span) * span;
-  const bool valid = idx < PRE_PAIRS;
-  const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N));
-  const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
-  if (rowok && colok) {
-    const int64_t e = ((i0 - 1 + el) % N + N) % N;
-    const int64_t f = ((j0 - 1 + fl) % N + N) % N;
-    PairOut o;
-    pair_integrals(A, e, f, o);
-    zd* out = pre + ((int64_t)blockIdx.z * PRE_SLOTS + slot) * PRE_PAIRS * 16 + (int64_t)idx * 16;
+// Row 0 of the circle's four operators: node 0 gets element N-1 (a = 1) and element 0
+// (a = 0); column j gets elements j-1 (b = 1) and j (b = 0).  One thread per
+// (column, element pair); the four partial values are summed in fixed order.
+__device__ __forceinline__ void circle_pair(int64_t t, int64_t N, int64_t& e, int64_t& f) {
+  const int64_t j = t >> 2;
+  e = ((t >> 1) & 1) ? 0 : N - 1;
+  f = (t & 1) ? j : (j - 1 + N) % N;
+}
+__device__ __forceinline__ void circle_store(const PairOut& o, int64_t t, int64_t N, zd* part) {
+  const int a = ((t >> 1) & 1) ? 0 : 1, b = (t & 1) ? 0 : 1;
 #pragma unroll
-    for (int op = 0; op < 4; ++op)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) out[op * 4 + j] = o.v[op][j];
+  for (int op = 0; op < 4; ++op) {
+    const zd v = a ? (b ? o.v[op][3] : o.v[op][2]) : (b ? o.v[op][1] : o.v[op][0]);
+    part[(int64_t)op * 4 * N + t] = v;
   }
+}
+
+// k R of a near-band point pair is below k h (near_band + 1), its elements' span
+__host__ __device__ __forceinline__ bool band_sorts(const AsmArgs& A) {
+  return A.kt_pair && A.k * A.h * (A.near_band + 1) < 3.9 && 2 * A.near_band + 1 <= A.N;
+}
+
+// CTAs: ncirc of the circle B's row (part: 16 N values), nband of the table band, then
+// the tiles' far pairs (and, without the table, their near ones)
+__global__ void __launch_bounds__(32) k_assemble_pairs(const __grid_constant__ AsmArgs A, const __grid_constant__ AsmArgs B,
+                                                       int64_t nt, int64_t row0, zd* pre, unsigned ncirc, zd* part,
+                                                       unsigned nband, zd* band) {
+  const int64_t N = A.N;
+  const int span = TILE + 1;
+  unsigned id = blockIdx.x;
+  int64_t e = 0, f = 0;
+  zd* out = nullptr;               // the pair's block; null: nothing to do
+  bool circle = false;
+  int64_t t = 0;
+  if (id < ncirc) {
+    t = (int64_t)id * 32 + threadIdx.x;
+    circle = t < 4 * N;
+    if (circle) circle_pair(t, N, e, f);
+  } else if ((id -= ncirc) < nband) {
+    const unsigned nb = (unsigned)((N + 31) / 32);
+    const int64_t off = id / nb, u = (int64_t)(id % nb) * 32 + threadIdx.x;
+    if (u < N) {
+      e = u;
+      f = ((e + off - A.near_band) % N + N) % N;
+      out = band + (off * N + e) * 16;
+    }
+  } else {
+    id -= nband;
+    constexpr unsigned CHUNKS = (PRE_PAIRS + 31) / 32;
+    const int64_t row = id / (CHUNKS * PRE_SLOTS), ti = row0 + row, slot = id / CHUNKS % PRE_SLOTS;
+    int64_t tj = nt <= PRE_SLOTS ? ti + slot : ti + slot - PRE_OFF;
+    tj = ((tj % nt) + nt) % nt;
+    if (slot >= nt || pre_slot(ti, tj, nt, N) != slot) return;
+    const int64_t i0 = ti * TILE, j0 = tj * TILE;
+    const int idx = (int)(id % CHUNKS) * 32 + threadIdx.x;
+    const int el = idx / span, fl = idx - (idx / span) * span;
+    const bool valid = idx < PRE_PAIRS;
+    const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N));
+    const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
+    if (rowok && colok) {
+      e = ((i0 - 1 + el) % N + N) % N;
+      f = ((j0 - 1 + fl) % N + N) % N;
+      if (!A.near_buf || periodic_dist(e, f, N) > A.near_band)
+        out = pre + (row * PRE_SLOTS + slot) * PRE_PAIRS * 16 + (int64_t)idx * 16;
+    }
+  }
+  if (!circle && !out) return;
+  PairOut o;
+  pair_integrals(circle ? B : A, e, f, o);
+  if (circle) {
+    circle_store(o, t, N, part);
+    return;
+  }
+#pragma unroll
+  for (int op = 0; op < 4; ++op)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[op * 4 + j] = o.v[op][j];
 }
 
 // every tile of the rows from row0 on, dense complex output
@@ -823,24 +883,17 @@ __global__ void __launch_bounds__(NEAR_THREADS, 2) k_assemble_near(AsmArgs A, in
   }
 }
 
-// Row 0 of the four operators: node 0 gets element N-1 (a = 1) and element 0
-// (a = 0); column j gets elements j-1 (b = 1) and j (b = 0).  One thread per
-// (column, element pair); the four partial values are summed in fixed order.
 __global__ void k_circle_row_part(AsmArgs A, zd* part) {
   const int64_t N = A.N;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * N) return;
-  const int64_t j = t >> 2;
-  const int u = (int)((t >> 1) & 1), v = (int)(t & 1);
-  const int64_t e = u ? 0 : N - 1;
-  const int a = u ? 0 : 1;
-  const int64_t f = v ? j : (j - 1 + N) % N;
-  const int b = v ? 0 : 1;
+  int64_t e, f;
+  circle_pair(t, N, e, f);
   PairOut o;
   if (A.near_buf && periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, N - 1, 2, A.near_band, N, e, f, o);
   else if (A.near_buf && pair_is_mid(A, e, f)) pair_mid<4>(A, A.htab, e, f, o);
   else pair_integrals(A, e, f, o);
-  for (int op = 0; op < 4; ++op) part[(int64_t)op * 4 * N + t] = o.v[op][a * 2 + b];
+  circle_store(o, t, N, part);
 }
 
 __global__ void k_circle_row_sum(AsmArgs A, const zd* part) {
@@ -907,25 +960,46 @@ void fill_asymptotic(KtPair& kp, double tol) {
   }
 }
 
-size_t assemble_dense_bytes(int64_t N) {
+static size_t pre_bytes(int64_t N) {
   const int64_t rows = std::min<int64_t>((N + TILE - 1) / TILE, 128);
   return sizeof(zd) * 16 * PRE_PAIRS * PRE_SLOTS * (size_t)rows;
 }
 
-int assemble_dense(const AsmArgs& A, void* ws, cudaStream_t s) {
+size_t assemble_dense_bytes(const AsmArgs& A) {
+  const size_t band = sizeof(zd) * 16 * (size_t)A.N * (size_t)(2 * A.near_band + 1);
+  return pre_bytes(A.N) + (band_sorts(A) && band <= ((size_t)1 << 30) ? band : 0);
+}
+
+int assemble_dense(AsmArgs A, const AsmArgs& B, zd* part, void* ws, cudaStream_t s) {
   const size_t smem = sizeof(zd) * 4 * TILE * TILE;
   cudaFuncSetAttribute(k_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t nt = (A.N + TILE - 1) / TILE;
+  zd* pre = (zd*)ws;
+  unsigned ncirc = 0, nband = 0;
+  if (ws) {
+    ncirc = (unsigned)((4 * A.N + 31) / 32);
+    if (assemble_dense_bytes(A) > pre_bytes(A.N)) {
+      A.near_buf = (const double*)((char*)ws + pre_bytes(A.N));
+      nband = (unsigned)((A.N + 31) / 32 * (2 * A.near_band + 1));
+    }
+  } else {
+    k_circle_row_part<<<(unsigned)((4 * A.N + 63) / 64), 64, 0, s>>>(B, part);
+    note_launch();
+  }
   // 128 rows of tiles at a time bound the blocks kept (250 MB)
   for (int64_t r0 = 0; r0 < nt; r0 += 128) {
     const unsigned rows = (unsigned)std::min<int64_t>(128, nt - r0);
     if (ws) {
-      k_assemble_pairs<<<dim3((PRE_PAIRS + 31) / 32, PRE_SLOTS, rows), 32, 0, s>>>(A, nt, r0, (zd*)ws);
+      if (r0 > 0) ncirc = nband = 0;
+      k_assemble_pairs<<<ncirc + nband + (PRE_PAIRS + 31) / 32 * PRE_SLOTS * rows, 32, 0, s>>>(
+          A, B, nt, r0, pre, ncirc, part, nband, (zd*)A.near_buf);
       note_launch();
     }
-    k_assemble<<<dim3((unsigned)nt, rows), ASM_THREADS, smem, s>>>(A, nt, r0, (const zd*)ws);
+    k_assemble<<<dim3((unsigned)nt, rows), ASM_THREADS, smem, s>>>(A, nt, r0, pre);
     note_launch();
   }
+  k_circle_row_sum<<<(unsigned)((A.N + 127) / 128), 128, 0, s>>>(B, part);
+  note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("assemble: ") + cudaGetErrorString(err)); return 3; }
   return 0;
@@ -1332,12 +1406,23 @@ __global__ void __launch_bounds__(32 * SH_W) k_shape_far(ShapeArgs S) {
 // offset, so that the log-kernel pairs do not hold up warps of plain ones and the pairs
 // spread over the whole GPU: one geometry with the offsets side by side ran 72 warps'
 // quartets, each as long as its heaviest pairs (2 x 5.7 -> 3.9 ms at N = 1024).
+// Where the recurrences' start depends on the warp (see band_sorts) the offsets stay
+// side by side, whose grouping the FP64 values then follow.
 __global__ void __launch_bounds__(32) k_shape_near(const __grid_constant__ AsmArgs A0, const __grid_constant__ AsmArgs A1,
-                                                   const zd* W0, const zd* W1, const zd* W2, const zd* W3, zd* pairs) {
+                                                   const zd* W0, const zd* W1, const zd* W2, const zd* W3, zd* pairs,
+                                                   int sorted) {
   const AsmArgs& A = blockIdx.y ? A1 : A0;
-  const int64_t N = A.N;
-  const int span = 2 * A.near_band + 1, nb = (int)((N + 31) / 32), off = (int)(blockIdx.x / nb);
-  const int64_t e = (int64_t)(blockIdx.x % nb) * 32 + threadIdx.x;
+  const int64_t N = A.N, u = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  const int span = 2 * A.near_band + 1;
+  int64_t e, off;
+  if (sorted) {
+    const int64_t nb = (N + 31) / 32;
+    off = blockIdx.x / nb;
+    e = u - off * nb * 32;
+  } else {
+    e = u / span;
+    off = u - e * span;
+  }
   if (e >= N) return;
   const int64_t f = ((e + off - A.near_band) % N + N) % N;
   zd acc = mkz(0.0);
@@ -1384,8 +1469,9 @@ int shape_near_forms(const AsmArgs& A0, const AsmArgs& A1, const zd* const* W, z
                      cudaStream_t s) {
   const int64_t n = A0.N * (2 * A0.near_band + 1);
   const unsigned blocks = (unsigned)((n + 127) / 128);
-  k_shape_near<<<dim3((unsigned)((A0.N + 31) / 32 * (2 * A0.near_band + 1)), 2), 32, 0, s>>>(
-      A0, A1, W[0], W[1], W[2], W[3], pairs);
+  const bool sorted = band_sorts(A0) && band_sorts(A1);
+  k_shape_near<<<dim3((unsigned)(sorted ? (A0.N + 31) / 32 * (2 * A0.near_band + 1) : (n + 31) / 32), 2), 32, 0, s>>>(
+      A0, A1, W[0], W[1], W[2], W[3], pairs, sorted);
   note_launch();
   k_shape_near_sum<<<dim3(blocks, 2), 128, 0, s>>>(pairs, n, part);
   note_launch();

@@ -126,9 +126,11 @@ struct AsmArgs {
 // Fill kp.asym for kp.t and the term-count thresholds kp.xth for relative
 // tolerance tol (host).
 void fill_asymptotic(KtPair& kp, double tol);
-// FP64 form; ws: assemble_dense_bytes(N) of device memory, or null (slower).
-size_t assemble_dense_bytes(int64_t N);
-int assemble_dense(const AsmArgs& a, void* ws, cudaStream_t s);
+// FP64 form: the operators of a and, in the outputs of the circle's args, row 0 of each of
+// its operators; part: 16 N values of scratch; ws: assemble_dense_bytes(a) of device
+// memory, or null (slower).
+size_t assemble_dense_bytes(const AsmArgs& a);
+int assemble_dense(AsmArgs a, const AsmArgs& circle, zd* part, void* ws, cudaStream_t s);
 // Mixed form: the same operators written as split-bf16 planes (see AsmArgs):
 // the far-pair kernel over the tiles it can take, then the FP64 kernel
 // over the rest.  mid (optional, two events) is recorded between the two;

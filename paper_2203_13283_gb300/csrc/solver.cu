@@ -1175,14 +1175,18 @@ int wcs_assemble(wcs_ctx* c) {
   if (c->stage < ST_MESH) { set_error("mesh first"); return WCS_ERR_STATE; }
   const int64_t N = c->N, ld = c->ld;
   bool near_tab = false;
+  TRY(c->mu.ensure(sizeof(zd) * 6 * N));
+  TRY(c->gwork.ensure(sizeof(zd) * 16 * N));
+  AsmArgs B = asm_args(c, true);
+  B.S = mu_ptr(c, MU_S); B.D = mu_ptr(c, MU_D); B.Dt = mu_ptr(c, MU_DT); B.Nk = mu_ptr(c, MU_N);
   if (!c->mixed) {
     TRY(c->ops.fit(sizeof(zd) * 4 * N * ld));
     c->S = c->ops.z(); c->D = c->S + N * ld; c->Dt = c->D + N * ld; c->Nk = c->Dt + N * ld;
     AsmArgs A = asm_args(c, false);
     A.S = c->S; A.D = c->D; A.Dt = c->Dt; A.Nk = c->Nk;
     ProfScope ps(c, CAT_ASSEMBLY, (double)N * N * c->opt.q_far * c->opt.q_far, 0.0);
-    if (c->htab.ensure(assemble_dense_bytes(N))) (void)cudaGetLastError();   // no room: without it
-    TRY(assemble_dense(A, c->htab.bytes >= assemble_dense_bytes(N) ? c->htab.p : nullptr, c->s));
+    if (c->htab.ensure(assemble_dense_bytes(A))) (void)cudaGetLastError();   // no room: without it
+    TRY(assemble_dense(A, B, c->gwork.z(), c->htab.bytes >= assemble_dense_bytes(A) ? c->htab.p : nullptr, c->s));
   } else {
     c->ldp = ((2 * N + 63) / 64) * 64;
     const size_t plane_bytes = sizeof(uint16_t) * (size_t)8 * c->planes * N * c->ldp;
@@ -1245,17 +1249,13 @@ int wcs_assemble(wcs_ctx* c) {
     }
   }
   // circle: first rows -> eigenvalues
-  TRY(c->mu.ensure(sizeof(zd) * 6 * N));
-  AsmArgs B = asm_args(c, true);
-  B.S = mu_ptr(c, MU_S); B.D = mu_ptr(c, MU_D); B.Dt = mu_ptr(c, MU_DT); B.Nk = mu_ptr(c, MU_N);
   if (near_tab) {   // the same wavenumbers: the table serves the circle as well
     double* row = c->htab.d() + hankel_table_doubles() + 32 * N * (2 * c->opt.near_band + 1);
     B.htab = c->htab.d();
     TRY(near_band_pairs(B, N - 1, 2, row, c->s));
     B.near_buf = row;
   }
-  TRY(c->gwork.ensure(sizeof(zd) * 16 * N));
-  TRY(assemble_circle_row(B, c->gwork.z(), c->s));
+  if (c->mixed) TRY(assemble_circle_row(B, c->gwork.z(), c->s));
   // mu_X(m) = sum_j X_0j e^{+2 pi i m j / N}
   TRY(fft_columns(c->fft, mu_ptr(c, MU_S), N, 4, +1, c->s));
   k_mu_finish<<<(unsigned)((N + 255) / 256), 256, 0, c->s>>>(c->mu.z(), N, c->h);
