@@ -49,16 +49,19 @@ __device__ __forceinline__ int periodic_dist(int64_t e, int64_t f, int64_t N) {
 __device__ __forceinline__ zd i4(zd H) { return mkz(-0.25 * H.y, 0.25 * H.x); }
 
 // Hankel functions at k R and k~ R
-__device__ __forceinline__ void hankel_k_kt(const AsmArgs& A, double R, Hankel01& Hk, Hankel01& Ht) {
+template <bool FROM = false>
+__device__ __forceinline__ void hankel_k_kt(const AsmArgs& A, double R, Hankel01& Hk, Hankel01& Ht, int start = 0) {
   if (A.kt_pair) {
-    hankel01_pair(A.k * R, A.ktp, Hk, Ht);
+    hankel01_pair<FROM>(A.k * R, A.ktp, Hk, Ht, start);
   } else {
     Hk = hankel01(mkz(A.k * R));
     Ht = hankel01(A.kt * R);
   }
 }
 
-__device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& o) {
+// FROM (far pairs): the start of the recurrence of each point pair is given (q_far^2 bytes)
+template <bool FROM = false>
+__device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& o, const uint8_t* starts = nullptr) {
 #pragma unroll
   for (int op = 0; op < 4; ++op)
 #pragma unroll
@@ -117,7 +120,7 @@ __device__ void pair_integrals(const AsmArgs& A, int64_t e, int64_t f, PairOut& 
         } else {
           R = sqrt(dx * dx + dy * dy);
           gg = (dx * nxs + dy * nys) / R;
-          hankel_k_kt(A, R, Hk, Ht);
+          hankel_k_kt<FROM>(A, R, Hk, Ht, FROM ? starts[p * q + r] : 0);
         }
         const zd gk = i4(Hk.H0);
         const zd gt = i4(Ht.H0);
@@ -614,13 +617,15 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
 // points a pair) and the pairs below the expansion range: a CTA of eight warps
 // that walks such a tile takes 40 ms while the others take one.  Their pairs are
 // integrated by one warp per CTA first (k_assemble_pairs), so that the work spreads
-// over the chip; the tile kernel then only sums.  The far pairs of a warp are those of
-// the tile kernel's warp, whose recurrences start at the warp's largest index.  Near-band
-// pairs are taken out of these warps (in a diagonal tile every warp had some, and its 23
-// far lanes waited for them: 54 ms at N = 1024, 34 apart): a table with 32
-// pairs of one offset to a warp, as long as every point below x = 4 starts its
-// recurrence at the same index (28) whatever the warp.  The circle's row, a chain of one
-// near-band pair's length on a few warps (5.9 ms on its own), runs beside them.
+// over the chip; the tile kernel then only sums.  FP64 pipe bound, and a warp pays for
+// every branch that one of its lanes takes: near-band rule, recurrence, two expansions.
+// So the lanes of a warp hold pairs of one element offset: the near band as a table of
+// its own, the tile's far pairs sorted by offset (54 ms at N = 1024 with the pairs in
+// tile order, 14 sorted).  The values stay those of the tile order, whose
+// recurrences start at the largest index of 32 consecutive pairs: k_pair_starts tables
+// these, and in the near band every point below x = 4 starts at 28 in any company
+// (band_sorts; otherwise the tile order stays).  The circle's row, a chain of one near-band
+// pair's length on a few warps (5.9 ms on its own), runs beside them.
 constexpr int PRE_OFF = 3, PRE_SLOTS = 2 * PRE_OFF + 1, PRE_PAIRS = (TILE + 1) * (TILE + 1);
 
 // Slot of tile (ti, tj) in its row's integrated tiles, -1 for the others: tile
@@ -658,12 +663,52 @@ __host__ __device__ __forceinline__ bool band_sorts(const AsmArgs& A) {
   return A.kt_pair && A.k * A.h * (A.near_band + 1) < 3.9 && 2 * A.near_band + 1 <= A.N;
 }
 
+constexpr unsigned PRE_CHUNKS = (PRE_PAIRS + 31) / 32;
+
+// Column tile of a row's slot, -1 when the slot holds none
+__device__ __forceinline__ int64_t pre_tile(int64_t ti, int64_t slot, int64_t nt, int64_t N) {
+  int64_t tj = nt <= PRE_SLOTS ? ti + slot : ti + slot - PRE_OFF;
+  tj = ((tj % nt) + nt) % nt;
+  return slot < nt && pre_slot(ti, tj, nt, N) == slot ? tj : -1;
+}
+
+// Element pair (el, fl) of the tile at (i0, j0): false when it touches no node of it
+__device__ __forceinline__ bool pre_pair(int64_t i0, int64_t j0, int el, int fl, int64_t N, int64_t& e, int64_t& f) {
+  e = ((i0 - 1 + el) % N + N) % N;
+  f = ((j0 - 1 + fl) % N + N) % N;
+  return ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N)) &&
+         ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
+}
+
+// First index of the recurrence at every far point pair of 32 consecutive pairs of a tile
+__global__ void __launch_bounds__(32) k_pair_starts(const __grid_constant__ AsmArgs A, int64_t nt, int64_t row0,
+                                                    uint8_t* starts) {
+  const int64_t N = A.N;
+  const unsigned id = blockIdx.x, chunk = id % PRE_CHUNKS;
+  const int64_t ti = row0 + id / (PRE_CHUNKS * PRE_SLOTS), tj = pre_tile(ti, id / PRE_CHUNKS % PRE_SLOTS, nt, N);
+  if (tj < 0) return;
+  const int idx = (int)chunk * 32 + threadIdx.x, span = TILE + 1, q = A.q_far;
+  int64_t e = 0, f = 0;
+  const bool ok = idx < PRE_PAIRS && pre_pair(ti * TILE, tj * TILE, idx / span, idx % span, N, e, f) &&
+                  periodic_dist(e, f, N) > A.near_band;
+  for (int u = 0; u < q * q; ++u) {
+    const int64_t ip = e * q + u / q, ir = f * q + u % q;
+    const double dx = A.far.x[ip] - A.far.x[ir], dy = A.far.y[ip] - A.far.y[ir];
+    const double x = A.k * sqrt(dx * dx + dy * dy);
+    const int n0 = __reduce_max_sync(0xffffffffu, ok && x > 2.0 && x <= 17.0 ? miller_start(x) : 0);
+    if (threadIdx.x == 0) starts[(int64_t)id * q * q + u] = (uint8_t)n0;
+  }
+}
+
 // CTAs: ncirc of the circle B's row (part: 16 N values), nband of the table band, then
-// the tiles' far pairs (and, without the table, their near ones)
+// the tiles' far pairs, sorted by offset with the table (starts: k_pair_starts), otherwise
+// all pairs in tile order
+template <bool SORTED>
 __global__ void __launch_bounds__(32) k_assemble_pairs(const __grid_constant__ AsmArgs A, const __grid_constant__ AsmArgs B,
                                                        int64_t nt, int64_t row0, zd* pre, unsigned ncirc, zd* part,
-                                                       unsigned nband, zd* band) {
+                                                       unsigned nband, zd* band, const uint8_t* starts) {
   const int64_t N = A.N;
+  const uint8_t* first = nullptr;
   const int span = TILE + 1;
   unsigned id = blockIdx.x;
   int64_t e = 0, f = 0;
@@ -684,27 +729,32 @@ __global__ void __launch_bounds__(32) k_assemble_pairs(const __grid_constant__ A
     }
   } else {
     id -= nband;
-    constexpr unsigned CHUNKS = (PRE_PAIRS + 31) / 32;
-    const int64_t row = id / (CHUNKS * PRE_SLOTS), ti = row0 + row, slot = id / CHUNKS % PRE_SLOTS;
-    int64_t tj = nt <= PRE_SLOTS ? ti + slot : ti + slot - PRE_OFF;
-    tj = ((tj % nt) + nt) % nt;
-    if (slot >= nt || pre_slot(ti, tj, nt, N) != slot) return;
-    const int64_t i0 = ti * TILE, j0 = tj * TILE;
-    const int idx = (int)(id % CHUNKS) * 32 + threadIdx.x;
-    const int el = idx / span, fl = idx - (idx / span) * span;
-    const bool valid = idx < PRE_PAIRS;
-    const bool rowok = valid && ((el >= 1 && i0 + el - 1 < N) || (el < TILE && i0 + el < N));
-    const bool colok = valid && ((fl >= 1 && j0 + fl - 1 < N) || (fl < TILE && j0 + fl < N));
-    if (rowok && colok) {
-      e = ((i0 - 1 + el) % N + N) % N;
-      f = ((j0 - 1 + fl) % N + N) % N;
-      if (!A.near_buf || periodic_dist(e, f, N) > A.near_band)
+    const int64_t row = id / (PRE_CHUNKS * PRE_SLOTS), ti = row0 + row, slot = id / PRE_CHUNKS % PRE_SLOTS;
+    const int64_t tj = pre_tile(ti, slot, nt, N);
+    if (tj < 0) return;
+    int idx = (int)(id % PRE_CHUNKS) * 32 + threadIdx.x;
+    if (idx < PRE_PAIRS) {
+      int el = idx / span, fl = idx % span;
+      if (SORTED) {   // by fl - el: offsets -32 .. 0 hold 1 .. 33 pairs, their mirror 32 .. 1
+        const bool up = idx >= span * (span + 1) / 2;
+        const int u = up ? PRE_PAIRS - 1 - idx : idx;
+        int d = (int)((sqrtf(8.f * (float)u + 1.f) - 1.f) * 0.5f);
+        while (d * (d + 1) / 2 > u) --d;
+        while ((d + 1) * (d + 2) / 2 <= u) ++d;
+        const int at = u - d * (d + 1) / 2;
+        el = up ? at : at + TILE - d;
+        fl = up ? at + TILE - d : at;
+        idx = el * span + fl;
+        first = starts + ((row * PRE_SLOTS + slot) * PRE_CHUNKS + idx / 32) * A.q_far * A.q_far;
+      }
+      if (pre_pair(ti * TILE, tj * TILE, el, fl, N, e, f) && (!SORTED || periodic_dist(e, f, N) > A.near_band))
         out = pre + (row * PRE_SLOTS + slot) * PRE_PAIRS * 16 + (int64_t)idx * 16;
     }
   }
   if (!circle && !out) return;
   PairOut o;
-  pair_integrals(circle ? B : A, e, f, o);
+  if (SORTED && first) pair_integrals<true>(A, e, f, o, first);
+  else pair_integrals(circle ? B : A, e, f, o);
   if (circle) {
     circle_store(o, t, N, part);
     return;
@@ -965,9 +1015,15 @@ static size_t pre_bytes(int64_t N) {
   return sizeof(zd) * 16 * PRE_PAIRS * PRE_SLOTS * (size_t)rows;
 }
 
-size_t assemble_dense_bytes(const AsmArgs& A) {
+static size_t band_bytes(const AsmArgs& A) {
   const size_t band = sizeof(zd) * 16 * (size_t)A.N * (size_t)(2 * A.near_band + 1);
-  return pre_bytes(A.N) + (band_sorts(A) && band <= ((size_t)1 << 30) ? band : 0);
+  return band_sorts(A) && band <= ((size_t)1 << 30) ? band : 0;
+}
+
+size_t assemble_dense_bytes(const AsmArgs& A) {
+  const int64_t rows = std::min<int64_t>((A.N + TILE - 1) / TILE, 128);
+  const size_t starts = (size_t)rows * PRE_SLOTS * PRE_CHUNKS * A.q_far * A.q_far;
+  return pre_bytes(A.N) + (band_bytes(A) > 0 ? band_bytes(A) + starts : 0);
 }
 
 int assemble_dense(AsmArgs A, const AsmArgs& B, zd* part, void* ws, cudaStream_t s) {
@@ -976,10 +1032,12 @@ int assemble_dense(AsmArgs A, const AsmArgs& B, zd* part, void* ws, cudaStream_t
   const int64_t nt = (A.N + TILE - 1) / TILE;
   zd* pre = (zd*)ws;
   unsigned ncirc = 0, nband = 0;
+  uint8_t* starts = nullptr;
   if (ws) {
     ncirc = (unsigned)((4 * A.N + 31) / 32);
-    if (assemble_dense_bytes(A) > pre_bytes(A.N)) {
+    if (band_bytes(A) > 0) {
       A.near_buf = (const double*)((char*)ws + pre_bytes(A.N));
+      starts = (uint8_t*)A.near_buf + band_bytes(A);
       nband = (unsigned)((A.N + 31) / 32 * (2 * A.near_band + 1));
     }
   } else {
@@ -988,11 +1046,16 @@ int assemble_dense(AsmArgs A, const AsmArgs& B, zd* part, void* ws, cudaStream_t
   }
   // 128 rows of tiles at a time bound the blocks kept (250 MB)
   for (int64_t r0 = 0; r0 < nt; r0 += 128) {
-    const unsigned rows = (unsigned)std::min<int64_t>(128, nt - r0);
+    const unsigned rows = (unsigned)std::min<int64_t>(128, nt - r0), far = PRE_CHUNKS * PRE_SLOTS * rows;
     if (ws) {
       if (r0 > 0) ncirc = nband = 0;
-      k_assemble_pairs<<<ncirc + nband + (PRE_PAIRS + 31) / 32 * PRE_SLOTS * rows, 32, 0, s>>>(
-          A, B, nt, r0, pre, ncirc, part, nband, (zd*)A.near_buf);
+      if (starts) {
+        k_pair_starts<<<far, 32, 0, s>>>(A, nt, r0, starts);
+        note_launch();
+        k_assemble_pairs<true><<<ncirc + nband + far, 32, 0, s>>>(A, B, nt, r0, pre, ncirc, part, nband, (zd*)A.near_buf, starts);
+      } else {
+        k_assemble_pairs<false><<<ncirc + far, 32, 0, s>>>(A, B, nt, r0, pre, ncirc, part, 0, nullptr, nullptr);
+      }
       note_launch();
     }
     k_assemble<<<dim3((unsigned)nt, rows), ASM_THREADS, smem, s>>>(A, nt, r0, pre);

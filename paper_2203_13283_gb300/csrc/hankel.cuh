@@ -199,16 +199,22 @@ __device__ inline Bessel01 bessel01_series_real(double x) {
   return b;
 }
 
-__device__ inline Bessel01 bessel01_miller_real(double x) {
-  // the backward recurrence of hankel01_miller for real x; the threads that
-  // run this branch together start at their largest index, which keeps the
-  // loop (and the reciprocal-table reads) uniform across the warp
-  int n0 = (int)(x + (x < 12.0 ? 25.0 : 45.0));
-  n0 += (n0 & 1);
-  n0 = __reduce_max_sync(__activemask(), n0);
+__device__ __forceinline__ int miller_start(double x) {
+  const int n0 = (int)(x + (x < 12.0 ? 25.0 : 45.0));
+  return n0 + (n0 & 1);
+}
+
+// The backward recurrence of hankel01_miller for real x; the threads that
+// run this branch together start at their largest index, which keeps the
+// loop (and the reciprocal-table reads) uniform across the warp.  FROM: each
+// thread's recurrence starts at its own `start` (zeros before it).
+template <bool FROM = false>
+__device__ inline Bessel01 bessel01_miller_real(double x, int start = 0) {
+  const int n0 = __reduce_max_sync(__activemask(), FROM ? start : miller_start(x));
   const double iz2 = 2.0 / x;
-  double jp1 = 0.0, j = 1e-30, norm = 0.0, s0 = 0.0, s1 = 0.0, J1 = 0.0;
+  double jp1 = 0.0, j = FROM ? 0.0 : 1e-30, norm = 0.0, s0 = 0.0, s1 = 0.0, J1 = 0.0;
   for (int n = n0; n > 0; --n) {
+    if (FROM && n == start) j = 1e-30;
     if ((n & 1) == 0) {
       const int k = n >> 1;
       const double r = (k & 1) ? -c_recip[k] : c_recip[k];
@@ -427,10 +433,11 @@ __device__ inline void hankel01_asymptotic_rot(double x, double rs, double x0, z
 }
 
 // H0, H1 (and J0, J1 below the expansion range) at k R = x and at k~ R
-__device__ inline void hankel01_pair(double x, const KtPair& kp, Hankel01& hk, Hankel01& ht) {
+template <bool FROM = false>
+__device__ inline void hankel01_pair(double x, const KtPair& kp, Hankel01& hk, Hankel01& ht, int start = 0) {
   if (x >= 20.0) { hankel01_asymptotic_fixed(x, kp, hk, ht); return; }
   if (x > 17.0) { hankel01_asymptotic_pair(x, kp, hk, ht); return; }
-  const Bessel01 b = (x <= 2.0) ? bessel01_series_real(x) : bessel01_miller_real(x);
+  const Bessel01 b = (x <= 2.0) ? bessel01_series_real(x) : bessel01_miller_real<FROM>(x, start);
   hk.J0 = mkz(b.J0);
   hk.J1 = mkz(b.J1);
   hk.H0 = mkz(b.J0, b.Y0);
