@@ -313,6 +313,15 @@ int fft_plan_create(FFTPlan& p, int64_t n, cudaStream_t s) {
       set_error("oom (bluestein)");
       return 4;
     }
+    // linear convolution of n values needs 2 n - 1: three quarters of m where that is enough
+    p.conv_r = 3 * (m / 4) >= 2 * n - 1 ? 3 : 2;
+    p.conv_m = p.conv_r == 3 ? m / 4 : m / 2;
+    const int64_t c = p.conv_r * p.conv_m;
+    if (cudaMalloc(&p.conv_tw, sizeof(zd) * (c + p.conv_m)) != cudaSuccess) { set_error("oom (convolution)"); return 4; }
+    k_twiddles<<<(unsigned)((c + 255) / 256), 256, 0, s>>>(p.conv_tw, c);
+    note_launch();
+    k_twiddles<<<(unsigned)((p.conv_m + 255) / 256), 256, 0, s>>>(p.conv_tw + c, p.conv_m);
+    note_launch();
     k_chirp<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p.chirp, n);
     note_launch();
     k_bluestein_filter<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(p.chirp, n, m, p.chirp_hat);
@@ -330,6 +339,7 @@ void fft_plan_destroy(FFTPlan& p) {
   cudaFree(p.twiddle);
   cudaFree(p.chirp);
   cudaFree(p.chirp_hat);
+  cudaFree(p.conv_tw);
   cudaFree(p.work);
   p = FFTPlan();
 }
@@ -384,48 +394,96 @@ __global__ void k_conv_kernel(const zd* c, int64_t n, int64_t m, zd* k) {
   k[j] = v;
 }
 
-__global__ void k_conv_pad(const zd* x, int64_t ld, int64_t n, int64_t m, zd* work) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
-  if (j < m) work[c * m + j] = j < n ? x[c * ld + j] : mkz(0.0);
+// A transform of length R M is R of length M: x_s[j] = x[j + s M] give
+// y_r[j] = W^(r j) sum_s w^(r s) x_s[j], W = e^{-2 pi i / (R M)}, w = W^M, whose transforms
+// are the entries R k + r.  The convolution never needs them in order.  With R = 3 a
+// convolution of n <= 1.5 * 2^a values takes 3 * 2^a points instead of 4 * 2^a, and M
+// fits one CTA's shared memory up to n = 6144 (R = 2: 4096), where a power of two
+// twice as long went through memory a second time: at n = 2777 (3 x 2048 for 8192 points)
+// 256 columns took 4 x 143 us of transforms, 2 x 185 now.
+template <int R>
+__device__ __forceinline__ void conv_mix(const zd (&x)[3], double dir, zd (&y)[3]) {
+  if (R == 2) {
+    y[0] = x[0] + x[1];
+    y[1] = x[0] - x[1];
+    return;
+  }
+  const double c = dir * 0.86602540378443864676;   // sin(2 pi / 3)
+  const zd t = x[1] + x[2], d = x[1] - x[2], a = x[0] - 0.5 * t, b = mkz(-c * d.y, c * d.x);
+  y[0] = x[0] + t;
+  y[1] = a + b;
+  y[2] = a - b;
 }
 
-__global__ void k_conv_take(const zd* work, int64_t n, int64_t m, zd* y, int64_t ld) {
+template <int R>
+__global__ void k_conv_split(const zd* x, int64_t ld, int64_t n, int64_t M, const zd* __restrict__ tw, zd* out) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
-  if (j < n) y[c * ld + j] = (1.0 / (double)m) * work[c * m + j];
+  if (j >= M) return;
+  zd v[3], y[3];
+#pragma unroll
+  for (int s = 0; s < R; ++s) v[s] = j + s * M < n ? x[c * ld + j + s * M] : mkz(0.0);
+  conv_mix<R>(v, -1.0, y);
+#pragma unroll
+  for (int r = 0; r < R; ++r) out[(c * R + r) * M + j] = r == 0 ? y[0] : y[r] * tw[r * j];
 }
 
-int64_t conv_kernel_elems(const FFTPlan& p) { return p.pow2 ? 0 : p.m; }
+template <int R>
+__global__ void k_conv_join(const zd* work, int64_t n, int64_t M, const zd* __restrict__ tw, zd* y, int64_t ld) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
+  if (j >= M) return;
+  zd v[3], o[3];
+#pragma unroll
+  for (int r = 0; r < R; ++r) v[r] = r == 0 ? work[c * R * M + j] : work[(c * R + r) * M + j] * conj(tw[r * j]);
+  conv_mix<R>(v, 1.0, o);
+  const double sc = 1.0 / (double)(R * M);
+#pragma unroll
+  for (int s = 0; s < R; ++s)
+    if (j + s * M < n) y[c * ld + j + s * M] = sc * o[s];
+}
+
+static void conv_split(const FFTPlan& p, const zd* x, int64_t ld, int64_t n, int64_t cols, zd* out, cudaStream_t s) {
+  const dim3 g((unsigned)((p.conv_m + 255) / 256), (unsigned)cols);
+  if (p.conv_r == 3) k_conv_split<3><<<g, 256, 0, s>>>(x, ld, n, p.conv_m, p.conv_tw, out);
+  else k_conv_split<2><<<g, 256, 0, s>>>(x, ld, n, p.conv_m, p.conv_tw, out);
+  note_launch();
+}
+
+int64_t conv_kernel_elems(const FFTPlan& p) { return p.pow2 ? 0 : p.conv_r * p.conv_m; }
+
+static Pow2 conv_pow2(const FFTPlan& p) {
+  return Pow2{p.conv_m, p.conv_tw + p.conv_r * p.conv_m, p.work + p.m * p.work_cols, p.work_cols * (p.m / p.conv_m)};
+}
 
 int conv_kernel(FFTPlan& p, const zd* mu, int mode, zd* khat, zd* tmp, cudaStream_t s) {
-  const int64_t n = p.n, m = p.m;
+  const int64_t n = p.n, m = p.conv_r * p.conv_m;
   k_conv_diag<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(mu, n, mode, tmp);
   note_launch();
   int r = fft_columns(p, tmp, n, 1, +1, s);
   if (r) return r;
-  k_conv_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(tmp, n, m, khat);
+  k_conv_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(tmp, n, m, p.work);
   note_launch();
-  Pow2 P{m, p.twiddle, p.work + m * p.work_cols, p.work_cols};
-  return pow2_transform(P, khat, m, 1, -1, s);
+  conv_split(p, p.work, m, m, 1, khat, s);
+  Pow2 P = conv_pow2(p);
+  return pow2_transform(P, khat, p.conv_m, p.conv_r, -1, s);
 }
 
 // A circulant product through Bluestein's transforms is four transforms of length
 // m >= 2 n - 1 (two each way); as a convolution with its first column it is two.
 int conv_apply(FFTPlan& p, const zd* khat, const zd* x, int64_t ldx, zd* y, int64_t ldy, int64_t cols, cudaStream_t s) {
-  const int64_t n = p.n, m = p.m;
-  zd* scratch = p.work + m * p.work_cols;
+  const int64_t n = p.n, M = p.conv_m, m = p.conv_r * M;
   for (int64_t c0 = 0; c0 < cols; c0 += p.work_cols) {
     const int64_t cc = std::min(p.work_cols, cols - c0);
-    dim3 gm((unsigned)((m + 255) / 256), (unsigned)cc), gn((unsigned)((n + 255) / 256), (unsigned)cc);
-    k_conv_pad<<<gm, 256, 0, s>>>(x + c0 * ldx, ldx, n, m, p.work);
-    note_launch();
-    Pow2 P{m, p.twiddle, scratch, p.work_cols};
-    int r = pow2_transform(P, p.work, m, cc, -1, s);
+    const dim3 gm((unsigned)((m + 255) / 256), (unsigned)cc), gj((unsigned)((M + 255) / 256), (unsigned)cc);
+    conv_split(p, x + c0 * ldx, ldx, n, cc, p.work, s);
+    Pow2 P = conv_pow2(p);
+    int r = pow2_transform(P, p.work, M, cc * p.conv_r, -1, s);
     if (r) return r;
     k_pointwise<<<gm, 256, 0, s>>>(p.work, m, khat, 0);
     note_launch();
-    r = pow2_transform(P, p.work, m, cc, +1, s);
+    r = pow2_transform(P, p.work, M, cc * p.conv_r, +1, s);
     if (r) return r;
-    k_conv_take<<<gn, 256, 0, s>>>(p.work, n, m, y + c0 * ldy, ldy);
+    if (p.conv_r == 3) k_conv_join<3><<<gj, 256, 0, s>>>(p.work, n, M, p.conv_tw, y + c0 * ldy, ldy);
+    else k_conv_join<2><<<gj, 256, 0, s>>>(p.work, n, M, p.conv_tw, y + c0 * ldy, ldy);
     note_launch();
   }
   cudaError_t err = cudaGetLastError();

@@ -183,6 +183,10 @@ struct FFTPlan {
   zd* chirp_hat = nullptr;         // FFT of the Bluestein filter (m)
   zd* work = nullptr;              // Bluestein work (m * batch_cap)
   int64_t work_cols = 0;
+  // convolutions (lengths that are not a power of two): conv_r transforms of conv_m
+  int conv_r = 0;
+  int64_t conv_m = 0;
+  zd* conv_tw = nullptr;           // e^{-2 pi i j / (conv_r conv_m)}, then e^{-2 pi i j / conv_m}
 };
 // FP32 circulant applies of the mixed form (circ32.cu): y = F^-1 diag(s) F x
 // with s = mu, conj(mu), 1/mu, 1/conj(mu) (mode 0..3) for power-of-two
