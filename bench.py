@@ -236,14 +236,14 @@ def roofline_entry(cat, prof, hbm, bf16s, fma):
     if cat in ("assembly", "assembly_fast"):
         units = v["work"] / per                      # far point pairs of the kernel's tiles, per launch
         fp64 = cat == "assembly"
-        prof = ("k_assemble_fp64_superellipse_n4096_mixed.md" if fp64
-                else "k_assemble_fast_superellipse_n4096_zfast9.md")
+        prof = ("k_assemble_near_superellipse_n4096_mixed.md" if fp64
+                else "k_assemble_far_superellipse_n4096_mixed.md")
         fpu, fsrc = profile_figure(prof, "fp64_flops_per_far_point_pair" if fp64 else "fp32_flops_per_far_point_pair")
         bpu, _ = profile_figure(prof, "dram_bytes_per_far_point_pair")
         busy, _ = profile_figure(prof, "pipe_active_frac")
         peak = fma.get(64 if fp64 else 32)
-        name = ("k_assemble<1> (FP64 point-pair integration, tiles within k R < zfast)" if fp64
-                else "k_assemble_fast (FP32 far point pairs, k R >= zfast)")
+        name = ("k_assemble_near (FP64 point-pair integration, tiles with pairs below k R = 20)" if fp64
+                else "k_assemble_far (FP32 far point pairs)")
         if not units:
             return None
         if not fpu or not peak:

@@ -50,7 +50,8 @@ typedef enum wcs_precision {
   WCS_PREC_MIXED = 1        /* operator products on the tensor cores (split-bf16, FP32
                                accumulation; exact fixed-point products for the residual
                                with exact_residual), element-pair integrals in FP64 except
-                               far pairs beyond zfast (FP32); FP64 circulant eigenvalues,
+                               far pairs (FP32 corrections around a float-float reference,
+                               ~1e-9 of the entry; see zfast); FP64 circulant eigenvalues,
                                capacitance matrix and refinement vectors */
 } wcs_precision;
 
@@ -69,22 +70,18 @@ typedef struct wcs_options {
   int rhs_chunk;      /* right-hand sides processed per pass (default 256) */
   int mixed_planes;   /* mixed form: bf16 planes per operator entry (default 3, max 3) */
   int rhs_planes;     /* mixed form: bf16 planes per staged vector entry (= mixed_planes) */
-  double zfast;       /* mixed form: far pairs with k R >= zfast + 2 k h are integrated in FP32
-                         around float-float element-centre phases (9 is the smallest safe value),
-                         nearer ones in FP64; 0: every pair in FP64.  Default -1 = automatic:
-                         1000 in the mixed form.  Measured at N = 32768 (superellipse, k = 3642)
-                         against the FP64 form, for incidence grazing the flat faces: 9.8e-7 with
-                         zfast = 9, 7.8e-7 with 500, 6.1e-7 with 1000 (assembly 1.7 s), 3.8e-7
-                         with 2000 (2.3 s), 2.4e-7 with 0.  The FP32 part loses accuracy where the two terms of the
-                         Maue form of N cancel (pairs on one flat face), and there its roundings
-                         repeat along each diagonal of the operator. */
+  double zfast;       /* mixed form: > 0: far pairs on the FP32 pipe, as small corrections around a
+                         float-float value at the element centres (3e-9 to 7e-9 of the entry),
+                         from k R = 20 + k h where k h <= 0.9 and beyond zfast + 2 k h on coarser
+                         meshes; nearer ones in FP64.  0: every pair in FP64.  Default -1 =
+                         automatic: 1000 in the mixed form. */
   int sample_planes;  /* mixed form: bf16 planes of each operand in the skeleton's sampling
                          products (default 0 = 2; 1 = one product per pass, ~4e-3 relative) */
-  int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x exactly (fixed-
-                         point slices of the operator planes and of x, integer products on the
-                         tensor cores, float-float and FP64 sums; see wcs_gemm_exact), so
+  int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x exactly (8-bit
+                         digits of the operator planes and of x below each row's largest entry,
+                         integer products on the tensor cores, 64-bit integer sums), so
                          refinement reaches refine_tol down to ~1e-11 against the stored operator;
-                         costs 6 bf16 slices of each operator (96 N^2 bytes in all, built at the
+                         costs 6 digits of each operator as bf16 (96 N^2 bytes in all, built at the
                          first such solve).  Adjoint solves keep the drained residual.  0
                          (default): residuals in split-bf16 with FP32 accumulation, which floor
                          near 2e-7. */
@@ -184,7 +181,7 @@ int wcs_geometry_sample(wcs_ctx* ctx, int64_t count, const double* s_host, doubl
 /* Assemble the Galerkin matrices S^k~, D^k, D^k~, N^k of Eq. (4)/(5) on gamma
  * (device-resident: dense complex FP64 in the FP64 form; in the mixed form
  * split-bf16 planes of each operator and of its transpose, from entries
- * integrated in FP64, or for far pairs in FP32 when zfast > 0) and the
+ * integrated in FP64, or for far pairs on the FP32 pipe when zfast > 0) and the
  * circulant eigenvalues of the same operators on gamma_c (always FP64), from
  * which mu_C of C_c (Eq. 6 on the circle) follows. */
 int wcs_assemble(wcs_ctx* ctx);
@@ -407,9 +404,7 @@ int wcs_gemm_split_bf16_noalloc(int64_t M, int64_t Nc, int64_t K, const double* 
                                 int64_t ldd, void* stream);
 
 /* Exact real contraction D (M x Nc) = A (M x K) * B (Nc x K)^T on the tensor
- * cores, all FP64 row-major device arrays (lda, ldb >= K, ldd >= Nc).  The
- * operator products of the refinement residual (Eq. 5 with C of Eq. 6) in
- * the mixed form's exact_residual mode use the same method: each row is cut
+ * cores, all FP64 row-major device arrays (lda, ldb >= K, ldd >= Nc).  Each row is cut
  * into chunks of 1024 K values, each chunk scaled by a power of two so its
  * entries lie in (-1, 1) and written as six 7-bit fixed-point slices (bf16
  * integers); the 21 slice pairs of combined order < 6 are multiplied with

@@ -1,10 +1,8 @@
-// Exact operator products for the refinement residual of the mixed form.
+// Exact real contraction on the tensor cores (wcs_gemm_exact); the solver's own exact
+// products run in fxgemm.cu.
 //
-// Iterative refinement converges to the operator that its residual evaluates
-// (Eq. 5 solved through Eq. 9 as an approximate inverse), and a split-bf16
-// product accumulated in FP32 carries ~1e-7 relative error, so the residual
-// b - C x of the mixed form stalls there.  This file evaluates the operator
-// products of C (Eq. 6) without rounding error on the same tensor cores:
+// A split-bf16 product accumulated in FP32 carries ~1e-7 relative error.  This file
+// evaluates a product without rounding error on the same tensor cores:
 //
 //  * every row of an operand is cut into chunks of EX_CHUNK consecutive K
 //    elements; each chunk gets a power-of-two scale 2^E (its largest entry
@@ -22,11 +20,7 @@
 //    2^-7(s+t+2), is added to the FP64 output.
 //
 // Pairs with s + t < EX_LEVELS are formed (21 of the 36); the dropped ones are
-// below 2^-56 of the chunk scales.  The operator's slices describe its
-// split-bf16 planes (the operator of the rest of the mixed form) to ~2^-42 of
-// each chunk's largest entry.  With five slices the chunk that holds the
-// log-singular diagonal left its ~500 far entries at ~2^-35 of the diagonal,
-// a residual floor near 7e-10 at N = 32768; six put it below 1e-11.
+// below 2^-56 of the chunk scales.
 #include <cuda_bf16.h>
 
 #include "gemm_tc.h"

@@ -888,11 +888,8 @@ static int create_context(wcs_ctx** out, const wcs_options* opt, void* stream, c
   if (o.q_far == 0) o.q_far = (o.precision == WCS_PREC_MIXED) ? 4 : 6;
   if (o.q_near == 0) o.q_near = (o.precision == WCS_PREC_MIXED) ? 8 : 12;
   if (o.sample_planes == 0) o.sample_planes = 2;
-  // FP32 far pairs beyond k R = 1000: at N = 32768 (k = 3642, superellipse)
-  // this keeps the error against the FP64 form at 6.1e-7 for grazing
-  // incidence (2000: 3.8e-7; all far pairs in FP32: 9.8e-7) with 1.7 s of
-  // assembly (2000: 2.3 s); smaller problems have few pairs that far and stay
-  // mostly in FP64
+  // any value > 0 takes the FP32 route of farpair.cuh from k R = 20 + k h on where
+  // k h <= 0.9 (its entries are good to ~1e-9); 1000 is the threshold on coarser meshes
   if (o.zfast < 0.0) o.zfast = (o.precision == WCS_PREC_MIXED) ? 1000.0 : 0.0;
   if (o.sample_planes < 1 || o.sample_planes > 2) { set_error("sample_planes must be 1 or 2"); return WCS_ERR_ARG; }
   if (o.exact_residual != 0 && o.exact_residual != 1) { set_error("exact_residual must be 0 or 1"); return WCS_ERR_ARG; }
