@@ -249,8 +249,8 @@ static int launch_tile(const zd* in, int64_t in_es, int64_t in_ss, int64_t in_cs
 
 static int pow2_transform(Pow2& P, zd* x, int64_t ld, int64_t cols, int sign, cudaStream_t s) {
   const int64_t n = P.n;
-  if (n <= FFT_SMEM_MAX && n >= 512 && cols <= 76 && cols <= P.scratch_cols) {
-    // fewer columns than half the SMs: two halves over several CTAs per column
+  if (n <= FFT_SMEM_MAX && n >= 512 && cols <= 65535 && cols <= P.scratch_cols) {
+    // two halves over several CTAs per column (192 columns of 2048: 67 us with one CTA each, 51 so; 768: 185 and 160)
     const int lg = ilog2(n), a = lg / 2, b = lg - a;
     const size_t smem = sizeof(zd) * FH_SETS * ((size_t)1 << b);
     k_fft_half<<<dim3((unsigned)((n >> a) / FH_SETS), (unsigned)cols), 256, smem, s>>>(x, ld, P.scratch, n, (int)n, lg, a,
@@ -400,7 +400,7 @@ __global__ void k_conv_kernel(const zd* c, int64_t n, int64_t m, zd* k) {
 // convolution of n <= 1.5 * 2^a values takes 3 * 2^a points instead of 4 * 2^a, and M
 // fits one CTA's shared memory up to n = 6144 (R = 2: 4096), where a power of two
 // twice as long went through memory a second time: at n = 2777 (3 x 2048 for 8192 points)
-// 256 columns took 4 x 143 us of transforms, 2 x 185 now.
+// 256 columns took 4 x 143 us of transforms, 2 x 160 now.
 template <int R>
 __device__ __forceinline__ void conv_mix(const zd (&x)[3], double dir, zd (&y)[3]) {
   if (R == 2) {
