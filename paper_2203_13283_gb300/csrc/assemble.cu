@@ -786,7 +786,8 @@ __global__ void __launch_bounds__(ASM_THREADS) k_assemble(AsmArgs A, int64_t nt,
 // images, as split-bf16 planes in both layouts.  S~ and N are symmetric and the Hankel
 // values of a pair (e, f) serve (f, e) too, so a listed tile and its mirror are one pass
 // (six sums per node pair) and a diagonal tile walks the pairs el <= fl only: that is 5%
-// more work a pair on half the pairs (3.1 -> 2.2 ms at N = 2777).  The sums of a diagonal
+// more work a pair on half the pairs (3.1 -> 2.2 ms at N = 2777, 1.5 with the
+// pairs in the order of their offset, so that the lanes of a warp take one route).  The sums of a diagonal
 // tile's lower half are those of its upper half, as of a tile and its mirror.
 // Bound: FP64 pipe.  A listed tile is two jobs of 16 rows, 561 pairs like a diagonal
 // tile's, so that a few hundred equal jobs spread evenly over the GPU; 192 threads fill
@@ -822,6 +823,17 @@ __global__ void __launch_bounds__(NEAR_THREADS, 2) k_assemble_near(AsmArgs A, in
   const int64_t N = A.N;
   const int64_t jobs = nt + 2 * ((int64_t)A.tile_list[0] - nt);
   const int span = TILE + 1;
+  // the pairs of a half tile in the order of their offset fl - el = k - TILE / 2, so that
+  // the lanes of a warp take one route (tabulated, far or near band)
+  __shared__ uint16_t order[(TILE / 2 + 1) * (TILE + 1)];
+  for (int t = threadIdx.x; t < (TILE / 2 + 1) * span; t += NEAR_THREADS) {
+    constexpr int H = TILE / 2;              // diagonals of 1 .. H + 1, H times H + 1, H + 1 .. 1 pairs
+    const int el = t / span, fl = t - el * span, k = fl - el + H;
+    const int before = k <= H ? k * (k + 1) / 2
+                              : (k <= TILE ? H * (H + 1) / 2 + (H + 1) * (k - H)
+                                           : (H + 1) * (TILE + 1) - (TILE + H + 1 - k) * (TILE + H + 2 - k) / 2);
+    order[before + min(el, fl)] = (uint16_t)t;
+  }
   for (int64_t u = blockIdx.x; u < jobs; u += gridDim.x) {
     const bool diag = u < nt;
     const int64_t tile = diag ? u * nt + u : A.tile_list[1 + nt + ((u - nt) >> 1)];
@@ -834,14 +846,16 @@ __global__ void __launch_bounds__(NEAR_THREADS, 2) k_assemble_near(AsmArgs A, in
     for (int base = 0; base < npairs; base += NEAR_THREADS) {
       const int idx = base + threadIdx.x;
       int el, fl;
-      if (diag) {
-        fl = (int)((sqrtf(8.f * (float)idx + 1.f) - 1.f) * 0.5f);
-        while (fl * (fl + 1) / 2 > idx) --fl;
-        while ((fl + 1) * (fl + 2) / 2 <= idx) ++fl;
-        el = idx - fl * (fl + 1) / 2;
+      if (diag) {   // offsets fl - el = 32 .. 0 hold 1 .. 33 pairs
+        int d = (int)((sqrtf(8.f * (float)idx + 1.f) - 1.f) * 0.5f);
+        while (d * (d + 1) / 2 > idx) --d;
+        while ((d + 1) * (d + 2) / 2 <= idx) ++d;
+        el = idx - d * (d + 1) / 2;
+        fl = el + TILE - d;
       } else {
-        el = idx / span;
-        fl = idx - el * span;
+        const int t = idx < npairs ? order[idx] : 0;
+        el = t / span;
+        fl = t - el * span;
       }
       // element row e = i0 - 1 + el feeds tile rows el - 1 (a = 1) and el (a = 0)
       const bool valid = idx < npairs;
