@@ -621,7 +621,7 @@ __device__ __forceinline__ void tile_sums(const AsmArgs& A, int64_t i0, int64_t 
 // every branch that one of its lanes takes: near-band rule, recurrence, two expansions.
 // So the lanes of a warp hold pairs of one element offset: the near band as a table of
 // its own, the tile's far pairs sorted by offset (54 ms at N = 1024 with the pairs in
-// tile order, 14 sorted).  The values stay those of the tile order, whose
+// tile order, 15 sorted).  The values stay those of the tile order, whose
 // recurrences start at the largest index of 32 consecutive pairs: k_pair_starts tables
 // these, and in the near band every point below x = 4 starts at 28 in any company
 // (band_sorts; otherwise the tile order stays).  The circle's row, a chain of one near-band
@@ -1331,21 +1331,25 @@ int assemble_entries(const AsmArgs& A, int64_t count, const int64_t* rows, const
 // Only far pairs are differentiated here; the near band keeps its singular
 // product rules and is differenced (shape_near_forms).
 // ---------------------------------------------------------------------------
-constexpr int SH_E = 8;       // element rows per block
+constexpr int SH_E = 2;       // element rows per block
 constexpr int SH_W = 4;       // warps per block, 32 element columns each
 
 // Bound: FP64 pipe.  The pair's coefficients are folded into the Hankel values first
 // (k into D's, k~ into D~'s, so H1' = H0 - H1 / z needs no division), the common factor
 // i/4 is applied to the sums, and the eight row sums of a point pair cross the warp by a
 // halving exchange (9 additions instead of 40) into the warp's own accumulators:
-// 111 -> 76 ms at N = 1024, q = 6.
+// 111 -> 76 ms at N = 1024, q = 6, and 47 with blocks of two rows, the longest first.
 __global__ void __launch_bounds__(32 * SH_W) k_shape_far(ShapeArgs S) {
   const AsmArgs& A = S.A;
   const int64_t N = A.N;
   const int q = A.q_far;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t e0 = (int64_t)blockIdx.y * SH_E;
-  const int64_t f = (int64_t)blockIdx.x * 32 * SH_W + threadIdx.x;
+  // the column blocks in the order of their distance from the diagonal, whose pairs (the
+  // recurrences below x = 17) take several times longer than the others, 27 ms a warp at
+  // eight rows: short blocks, the long ones first
+  const int64_t e0 = (int64_t)blockIdx.x * SH_E, nf = gridDim.y;
+  const int64_t off = (blockIdx.y & 1) ? (int64_t)(blockIdx.y + 1) / 2 : nf - (int64_t)blockIdx.y / 2;
+  const int64_t f = (e0 / (32 * SH_W) + off) % nf * (32 * SH_W) + threadIdx.x;
   const bool fvalid = f < N;
   __shared__ double rowacc[SH_W][SH_E][16][8];
   __shared__ double red[SH_W][4];
@@ -1534,7 +1538,7 @@ __global__ void __launch_bounds__(128) k_shape_near_sum(const zd* pairs, int64_t
 
 int shape_far_forms(const ShapeArgs& a, cudaStream_t s) {
   if (a.A.q_far > 16) { set_error("shape derivative: q_far <= 16"); return 1; }
-  dim3 grid((unsigned)((a.A.N + 32 * SH_W - 1) / (32 * SH_W)), (unsigned)((a.A.N + SH_E - 1) / SH_E));
+  dim3 grid((unsigned)((a.A.N + SH_E - 1) / SH_E), (unsigned)((a.A.N + 32 * SH_W - 1) / (32 * SH_W)));
   k_shape_far<<<grid, 32 * SH_W, 0, s>>>(a);
   note_launch();
   cudaError_t err = cudaGetLastError();
