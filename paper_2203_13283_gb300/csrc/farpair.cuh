@@ -80,10 +80,6 @@ WCS_HD ff ff_mul(ff a, ff b) {
   ff p = ff_two_prod(a.hi, b.hi);
   return ff_quick(p.hi, p.lo + fmaf(a.hi, b.lo, a.lo * b.hi));
 }
-WCS_HD ff ff_mul_f(ff a, float b) {
-  const ff p = ff_two_prod(a.hi, b);
-  return ff_quick(p.hi, fmaf(a.lo, b, p.lo));
-}
 WCS_HD ff ff_of(double x) {
   const float h = (float)x;
   return ff{h, (float)(x - (double)h)};

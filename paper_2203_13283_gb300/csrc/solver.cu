@@ -837,21 +837,6 @@ __global__ void k_add_identity(zd* K, int64_t r) {
   if (i < r) K[i * r + i] += mkz(1.0);
 }
 
-// per-column squared norms of an N x cols block
-__global__ void k_colnorm2(const zd* X, int64_t ld, int64_t m, double* out) {
-  __shared__ double red[256];
-  const int64_t c = blockIdx.x;
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < m; i += blockDim.x) s += abs2(X[c * ld + i]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[c] = red[0];
-}
-
 // ----------------------------------------------------------------------------- C ABI
 extern "C" {
 
