@@ -23,6 +23,8 @@
 // FX_SLICES / 2 boxes per operand and the swizzle atom is that of the other
 // tensor-core kernels, the second slice 64 bytes into it.
 //
+// Operators of the exact residual are stored as six digits (the 26 pairs s + t < 7).
+//
 // Tile 128 x 64: eight levels of 64 columns fill the 512 TMEM columns.  The MMAs
 // of a stage run from the highest level down; each level is committed by itself,
 // so the eight drain warps empty it while the next levels run.  Warp 8 loads,
@@ -45,11 +47,15 @@ template <int NS>
 struct Fx {
   static constexpr int TOP = 8 * (NS - 1) + 6;        // fixed-point position: |v| 2^(TOP - E) < 2^TOP
   static constexpr int ROW = NS * FX_BK;              // bf16 values of one row and stage
+  // digit-pair levels formed.  Six digits take one level past their own: without it the
+  // dropped pairs, 2^-46 of the row scales each, left an exact-residual solve at N = 16384
+  // at 1.4e-11 where the entries' own 2^-48 leave 6e-13
+  static constexpr int LEVELS = NS == 8 ? 8 : NS + 1;
   static constexpr int A_BYTES = FX_BM * ROW * 2, B_BYTES = FX_BN * ROW * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = NS == 8 ? 2 : 3;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 512;
-  static_assert(NS % 2 == 0 && NS * FX_BN <= 512, "two slices per TMA row, one TMEM accumulator per level");
+  static_assert(NS % 2 == 0 && LEVELS * FX_BN <= 512, "two slices per TMA row, one TMEM accumulator per level");
   static_assert((int64_t)NS * FX_CHUNK * FX_BK * (1 << 14) <= (1 << 24), "level sums stay exact in FP32");
 };
 
@@ -257,8 +263,8 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
   uint64_t* full = (uint64_t*)(smem + L::STAGES * L::STAGE_BYTES);
   uint64_t* empty = full + L::STAGES;
   uint64_t* tfull = empty + L::STAGES;        // [level] MMA -> drain
-  uint64_t* tempty = tfull + NS;       // [level] drain -> MMA
-  uint32_t* tslot = (uint32_t*)(tempty + NS);
+  uint64_t* tempty = tfull + L::LEVELS;       // [level] drain -> MMA
+  uint32_t* tslot = (uint32_t*)(tempty + L::LEVELS);
   volatile int* abort_flag = (volatile int*)(tslot + 1);
   volatile int* issued = (volatile int*)(tslot + 2);
   volatile int* consumed = (volatile int*)(tslot + 3);
@@ -271,7 +277,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
 
   if (threadIdx.x == 0) {
     for (int q = 0; q < L::STAGES; ++q) { mbar_init(&full[q], 1); mbar_init(&empty[q], 1); }
-    for (int q = 0; q < NS; ++q) { mbar_init(&tfull[q], 1); mbar_init(&tempty[q], 8); }
+    for (int q = 0; q < L::LEVELS; ++q) { mbar_init(&tfull[q], 1); mbar_init(&tempty[q], 8); }
     *abort_flag = 0;
     *issued = 0;
     *consumed = 0;
@@ -329,19 +335,19 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
         const uint64_t da = sw128_desc(sp), db = sw128_desc(sp + L::A_BYTES);
         const bool last = (in == FX_CHUNK - 1) || (kb == nk - 1);
 #pragma unroll
-        for (int lev = NS - 1; lev >= 0; --lev) {
+        for (int lev = L::LEVELS - 1; lev >= 0; --lev) {
           if (in == 0 && ch > 0) {
             if (!mbar_wait(&tempty[lev], (ch - 1) & 1, WAIT_LIMIT, args.err)) { *abort_flag = 45; ok = false; break; }
             tc_fence_after();
           }
           const uint32_t dt = tmem + (uint32_t)(lev * FX_BN);
 #pragma unroll
-          for (int s = 0; s <= lev; ++s) {
+          for (int s = lev < NS ? 0 : lev - NS + 1; s <= (lev < NS ? lev : NS - 1); ++s) {
             // slice s of a tile: box s / 2, 64 bytes into the 128-byte rows when odd (descriptors count 16 bytes)
             const int t = lev - s;
             const uint64_t a = da + (uint64_t)(((s >> 1) * (FX_BM * 128) + (s & 1) * 64) >> 4);
             const uint64_t b = db + (uint64_t)(((t >> 1) * (FX_BN * 128) + (t & 1) * 64) >> 4);
-            mma_bf16(dt, a, b, idesc, (in > 0 || s > 0) ? 1u : 0u);
+            mma_bf16(dt, a, b, idesc, (in > 0 || s > (lev < NS ? 0 : lev - NS + 1)) ? 1u : 0u);
             mma_bf16(dt, a + 2, b + 2, idesc, 1u);
           }
           if (last) mma_commit(&tfull[lev]);
@@ -354,7 +360,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
     bool ok = true;
     for (int ch = 0; ch < nchunks && ok; ++ch) {
 #pragma unroll
-      for (int lev = NS - 1; lev >= 0; --lev) {
+      for (int lev = L::LEVELS - 1; lev >= 0; --lev) {
         bool got = mbar_wait_sleep(&tfull[lev], ch & 1, WAIT_LIMIT, args.err, 64u);
         got = __all_sync(0xffffffffu, got) && (__shfl_sync(0xffffffffu, *abort_flag, 0) == 0);
         if (!got) { if (lane == 0) atomicCAS((int*)abort_flag, 0, 44); ok = false; break; }
