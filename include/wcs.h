@@ -80,7 +80,7 @@ typedef struct wcs_options {
   int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x exactly (8-bit
                          digits of the operator planes and of x below each row's largest entry,
                          integer products on the tensor cores, 64-bit integer sums), so
-                         refinement reaches refine_tol down to ~1e-11 against the stored operator;
+                         refinement reaches refine_tol down to ~1e-12 against the stored operator;
                          costs 6 digits of each operator as bf16 (96 N^2 bytes in all, built at the
                          first such solve).  Adjoint solves keep the drained residual.  0
                          (default): residuals in split-bf16 with FP32 accumulation, which floor
