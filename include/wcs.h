@@ -40,7 +40,7 @@ typedef enum wcs_status {
   WCS_ERR_SINGULAR = 5,     /* capacitance matrix numerically singular */
   WCS_ERR_RANK_CAP = 6,     /* skeleton reached max_rank before the tolerance */
   WCS_ERR_NOT_CONVERGED = 7,/* iterative refinement did not reach its tolerance */
-  WCS_ERR_TIMEOUT = 8,      /* reserved: a bounded device wait gave up */
+  WCS_ERR_TIMEOUT = 8,      /* a bounded device wait gave up: the call's results are not valid */
   WCS_ERR_STATE = 9,        /* call made out of order */
   WCS_ERR_UNSUPPORTED = 10  /* option combination not built */
 } wcs_status;
@@ -452,6 +452,13 @@ typedef struct wcs_batch_stats {
 int wcs_batch_solve_fourier(const wcs_options* opt, int count, int nf, const double* cos_c, const double* sin_c,
                             const int64_t* N, const double* k, int64_t B, const double* angles_host, double tol,
                             int rank_div, uint64_t seed, int workers, double* j_host, wcs_batch_stats* stats);
+
+/* Raises the error flag of ctx's bounded device waits, as an expired wait does: tensor-core
+ * products are skipped while it is set, and the next call that reads it returns
+ * WCS_ERR_TIMEOUT, with its results not valid; that report clears it and later calls run as
+ * before.
+ * For testing a program's handling of the status; nothing waits or fails on the device. */
+int wcs_inject_timeout(wcs_ctx* ctx);
 
 /* Number of CUDA kernel launches the library has issued in this process. */
 uint64_t wcs_launch_count(void);

@@ -105,7 +105,8 @@ struct wcs_ctx {
   DevBuf tiles;                           // list of the tiles assembled in FP64
   DevBuf stage0, stage1, stage2;          // staged right-hand blocks (bf16 planes)
   int64_t stage_cols = 0;
-  DevBuf tcerr;
+  DevBuf tcerr;                           // error flag of the bounded waits
+  bool flagged = false;                   // a kernel that may raise it was launched since it was last read
   DevBuf gW;                 // split-K workspace of the small contractions (FP32)
   DevBuf qh, qt;             // skeleton basis as resident bf16 planes: rows conj(q_i); rows of Q
   DevBuf gA, gB;                          // staging for general complex tensor products
@@ -188,11 +189,15 @@ static int ensure_work(wcs_ctx* c, int64_t cols) {
   return 0;
 }
 
-// the device flag of the bounded waits in the tensor-core kernels: zeroed when allocated
+// The device flag of the bounded waits in the tensor-core kernels, zeroed when allocated.
+// Called before every launch that may raise it: the call that launches has to read it
+// (check_tc, settle) before it reports success.
 static int ensure_tcerr(wcs_ctx* c) {
-  if (c->tcerr.p) return 0;
-  TRY(c->tcerr.ensure(sizeof(int)));
-  cudaMemsetAsync(c->tcerr.p, 0, sizeof(int), c->s);
+  if (!c->tcerr.p) {
+    TRY(c->tcerr.ensure(sizeof(int)));
+    cudaMemsetAsync(c->tcerr.p, 0, sizeof(int), c->s);
+  }
+  c->flagged = true;
   return 0;
 }
 
@@ -231,7 +236,6 @@ static int ensure_stage(wcs_ctx* c, int64_t cols) {
   TRY(c->stage0.ensure(b));
   TRY(c->stage1.ensure(b));
   TRY(c->stage2.ensure(b));
-  TRY(ensure_tcerr(c));
   c->stage_cols = cols;
   return 0;
 }
@@ -293,6 +297,7 @@ static int tc_apply(wcs_ctx* c, int op, bool adjoint, DevBuf& buf, int64_t cols,
   B.ld = c->ldp;
   const int64_t per = 2 * c->stage_cols * c->ldp;
   for (int p = 0; p < P; ++p) B.plane[p] = (uint16_t*)buf.p + p * per;
+  TRY(ensure_tcerr(c));
   TcArgs t;
   t.M = (int)c->N;
   t.Nc = (int)(2 * cols);
@@ -323,6 +328,9 @@ static int tc_apply(wcs_ctx* c, int op, bool adjoint, DevBuf& buf, int64_t cols,
   return 0;
 }
 
+// Synchronises and reads the flag of the bounded waits.  A raised flag is cleared with
+// the report: the kernels return at once while it is set, so it would fail every later
+// call of the context as well.
 static int check_tc(wcs_ctx* c) {
   int e = 0;
   // the flag exists once a tensor-core product has run on this context
@@ -332,9 +340,18 @@ static int check_tc(wcs_ctx* c) {
   }
   cudaError_t r = cudaStreamSynchronize(c->s);
   if (r != cudaSuccess) { set_error(std::string("device: ") + cudaGetErrorString(r)); return WCS_ERR_CUDA; }
-  if (e) { set_error("tensor-core contraction: a bounded wait expired"); return WCS_ERR_TIMEOUT; }
+  c->flagged = false;
+  if (e) {
+    cudaMemsetAsync(c->tcerr.p, 0, sizeof(int), c->s);
+    set_error("tensor-core contraction: a bounded wait expired");
+    return WCS_ERR_TIMEOUT;
+  }
   return 0;
 }
+
+// check_tc where a launch since the last one may have raised the flag.  Also asked before
+// a result is called not finite or not converged: that may be what the wait left.
+static int settle(wcs_ctx* c) { return c->flagged ? check_tc(c) : 0; }
 
 // C (m x n, column-major ldc) = alpha * A (m x k view) * X (k x n, column-major) + beta * C.
 // Mixed form: on the tensor cores through staged split-bf16 planes; FP64 form: zgemm.
@@ -1367,8 +1384,7 @@ int wcs_apply(wcs_ctx* c, int op, int64_t B, const double* X, int64_t ldx, doubl
       default: set_error("unknown operator"); return WCS_ERR_ARG;
     }
   }
-  if (c->mixed) TRY(check_tc(c));
-  return WCS_OK;
+  return c->mixed ? check_tc(c) : settle(c);
 }
 
 int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_out) {
@@ -1443,12 +1459,12 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
     TRY(column_norms(Y, N, N, b, Nb.d(), c->s));
     cudaMemcpyAsync(norms.data(), Nb.p, sizeof(double) * b, cudaMemcpyDeviceToHost, c->s);
     TRY(sync(c));
+    TRY(settle(c));
     double mx = 0;
     for (int j = 0; j < b; ++j) {
       if (!std::isfinite(norms[j])) { set_error("skeleton: non-finite sample (block at rank " + std::to_string(ell) + ")"); return WCS_ERR_CUDA; }
       mx = std::max(mx, norms[j]);
     }
-    if (c->mixed) TRY(check_tc(c));
     if (mx <= thr) break;
     // orthonormalise the block twice (pivoted CholeskyQR)
     ProfScope ps_orth(c, CAT_ORTH, 0.0, 0.0);
@@ -1587,7 +1603,7 @@ int wcs_factor(wcs_ctx* c) {
           note_launch();
           cudaMemcpyAsync(&res, cs + 2 * r, sizeof(double), cudaMemcpyDeviceToHost, c->s);
           TRY(sync(c));
-          if (!(res == res)) { set_error("capacitance iteration diverged"); return WCS_ERR_SINGULAR; }
+          if (!(res == res)) { TRY(settle(c)); set_error("capacitance iteration diverged"); return WCS_ERR_SINGULAR; }
           // converged, or stalled at the contraction's rounding level
           if (res < target || (res < 0.1 * std::sqrt((double)r) && res > 0.8 * prev)) break;
           prev = res;
@@ -1598,7 +1614,7 @@ int wcs_factor(wcs_ctx* c) {
         TRY(cgemm(c, r, r, r, mkz(1.0), blk(X, r), T.z(), r, mkz(0.0), Xn, r));
         std::swap(X, Xn);
       }
-      if (!(res < 0.1 * std::sqrt((double)r))) { set_error("capacitance iteration did not converge"); return WCS_ERR_SINGULAR; }
+      if (!(res < 0.1 * std::sqrt((double)r))) { TRY(settle(c)); set_error("capacitance iteration did not converge"); return WCS_ERR_SINGULAR; }
       // The two-plane iteration stalls near 1e-4 per direction.  One step with
       // the drained three-plane product (~1e-7) and then exact steps (each
       // squares the residual; the exact products carry 42 bits below each
@@ -1630,7 +1646,7 @@ int wcs_factor(wcs_ctx* c) {
           c->kinv_res = res / std::sqrt((double)r);
           if (!(c->kinv_res >= 1e-10)) break;
         }
-        if (!(c->kinv_res < 1e-6)) { set_error("capacitance iteration did not reach FP64 accuracy"); return WCS_ERR_SINGULAR; }
+        if (!(c->kinv_res < 1e-6)) { TRY(settle(c)); set_error("capacitance iteration did not reach FP64 accuracy"); return WCS_ERR_SINGULAR; }
       }
       if (X != Kinv.z())
         cudaMemcpyAsync(Kinv.p, X, sizeof(zd) * r * r, cudaMemcpyDeviceToDevice, c->s);
@@ -1896,7 +1912,7 @@ int wcs_woodbury_apply(wcs_ctx* c, int64_t B, const double* b, int64_t ldb, doub
     const int64_t cc = std::min(chunk, B - c0);
     TRY(woodbury(c, (const zd*)b + c0 * ldb, ldb, (zd*)x + c0 * ldx, ldx, cc));
   }
-  return WCS_OK;
+  return settle(c);
 }
 
 int wcs_planewave_rhs(wcs_ctx* c, int64_t B, const double* angles, double* e, double* hv, int64_t ld) {
@@ -2021,10 +2037,12 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
     worst = 0;
     for (int64_t j = 0; j < cc; ++j) {
       if (!std::isfinite(bn[j])) {
+        TRY(settle(c));
         set_error("right-hand side column " + std::to_string(j) + " of the block is not finite");
         return WCS_ERR_ARG;
       }
       if (!std::isfinite(rn[j])) {
+        TRY(settle(c));
         set_error("solve: the residual of column " + std::to_string(j) + " of the block is not finite");
         finish(INFINITY);
         return WCS_ERR_NOT_CONVERGED;
@@ -2148,7 +2166,7 @@ static int solve_block(wcs_ctx* c, const zd* b, int64_t ldb, zd* x, int64_t ldx,
       floor = worst > 10.0 * upd;
     }
   }
-  TRY(check_tc(c));
+  TRY(settle(c));
   finish(worst);
   return (worst <= c->opt.refine_tol) ? 0 : WCS_ERR_NOT_CONVERGED;
 }
@@ -2498,6 +2516,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
     return 0;
   };
   TRY(shape_forms(c, W, M, i0, i1, delta, T_ops.data(), tp, tm, per_param));
+  TRY(settle(c));   // the operators' products of the mixed form
   return status;
 }
 
@@ -2722,6 +2741,13 @@ int wcs_gemm_exact(int64_t M, int64_t Nc, int64_t K, const double* A, int64_t ld
   if (e != cudaSuccess) { set_error(std::string("gemm: ") + cudaGetErrorString(e)); return WCS_ERR_CUDA; }
   if (errh) { set_error("tensor-core contraction: a bounded wait expired"); return WCS_ERR_TIMEOUT; }
   return WCS_OK;
+}
+
+int wcs_inject_timeout(wcs_ctx* c) {
+  if (!c) { set_error("null context"); return WCS_ERR_ARG; }
+  TRY(ensure_tcerr(c));
+  cudaMemsetAsync(c->tcerr.p, 1, sizeof(int), c->s);
+  return sync(c);
 }
 
 uint64_t wcs_launch_count(void) { return (uint64_t)g_launches; }
