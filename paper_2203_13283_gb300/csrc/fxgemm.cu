@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
     k_gemm_fx(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, FxArgs args) {
   using L = Fx<NS>;
   extern __shared__ uint8_t smem_raw[];
-  if (*(volatile int*)args.err != 0) return;
+  if (tc_given_up(args.err)) return;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + L::STAGES * L::STAGE_BYTES);
   uint64_t* empty = full + L::STAGES;

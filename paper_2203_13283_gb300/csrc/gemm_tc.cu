@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int kb0 = (args.kper > 0) ? (int)blockIdx.z * args.kper : 0;
   const int nk = (args.kper > 0) ? min(args.kper, nk_all - kb0) : nk_all;
 
-  if (*(volatile int*)args.err != 0) return;  // another CTA already gave up: do nothing
+  if (tc_given_up(args.err)) return;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     mbar_init(done, 1);
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 1)
                   const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2, TcArgs args) {
   using L = AccSmem<PA, PB, STAGES>;
   extern __shared__ uint8_t smem_raw[];
-  if (*(volatile int*)args.err != 0) return;
+  if (tc_given_up(args.err)) return;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + STAGES * L::STAGE_BYTES);
   uint64_t* empty = full + STAGES;
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(PER_THREADS, 1)
                   const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1, TcArgs args) {
   using L = PerSmem<STAGES>;
   extern __shared__ uint8_t smem_raw[];
-  if (*(volatile int*)args.err != 0) return;
+  if (tc_given_up(args.err)) return;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + STAGES * L::STAGE_BYTES);
   uint64_t* empty = full + STAGES;

@@ -58,6 +58,12 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity, 
   }
 }
 
+// True for every thread of a CTA, or for none, when another CTA has raised the error flag:
+// a CTA of which some warps alone left would run on without its barriers or TMEM set up.
+__device__ __forceinline__ bool tc_given_up(const int* gerr) {
+  return __syncthreads_or(*(const volatile int*)gerr != 0) != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
