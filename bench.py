@@ -348,7 +348,8 @@ def main():
                     help="bracket the last timed step's solve with cudaProfilerStart/Stop "
                          "(for ncu --profile-from-start off)")
     ap.add_argument("--zfast", type=float, default=None,
-                    help="mixed form: FP32 far pairs above k R = zfast (default: library default)")
+                    help="mixed form: element pairs beyond k R = zfast on the FP32 pipe, nearer ones in FP64, 0: all "
+                         "in FP64 (default: the library's choice, k R = 20 + k h up to k h = 0.9)")
     ap.add_argument("--sample-planes", type=int, default=0,
                     help="mixed form: bf16 planes in the skeleton's sampling products (0: library default)")
     ap.add_argument("--fp64-rhs", type=int, default=16,

@@ -70,11 +70,11 @@ typedef struct wcs_options {
   int rhs_chunk;      /* right-hand sides processed per pass (default 256) */
   int mixed_planes;   /* mixed form: bf16 planes per operator entry (default 3, max 3) */
   int rhs_planes;     /* mixed form: bf16 planes per staged vector entry (= mixed_planes) */
-  double zfast;       /* mixed form: > 0: far pairs on the FP32 pipe, as small corrections around a
-                         float-float value at the element centres (3e-9 to 7e-9 of the entry),
-                         from k R = 20 + k h where k h <= 0.9 and beyond zfast + 2 k h on coarser
-                         meshes; nearer ones in FP64.  0: every pair in FP64.  Default -1 =
-                         automatic: 1000 in the mixed form. */
+  double zfast;       /* mixed form: element pairs with k R0 >= zfast + 2 k h (R0: distance of their
+                         centres; 20 + k h at least) run on the FP32 pipe, as small corrections
+                         around a float-float value at the centres (3e-9 to 7e-9 of the entry);
+                         nearer ones in FP64.  0: every pair in FP64.  Default -1 = automatic:
+                         from 20 + k h on where k h <= 0.9, as 1000 on coarser meshes. */
   int sample_planes;  /* mixed form: bf16 planes of each operand in the skeleton's sampling
                          products (default 0 = 2; 1 = one product per pass, ~4e-3 relative) */
   int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x exactly (8-bit
@@ -97,7 +97,8 @@ typedef struct wcs_info {
   int rank;           /* skeleton rank (after wcs_skeleton), else -1 */
   double norm_cc;     /* ||C_c||_2 = max |mu_C| (after wcs_assemble) */
   double min_curvature; /* minimum curvature found by the convexity check */
-  double zfast;       /* far-pair FP32 threshold in effect (mixed form; 0 in the FP64 form) */
+  double zfast;       /* k R0 from which element pairs run on the FP32 pipe (mixed form; 0: none do,
+                         as in the FP64 form) */
   double capacitance_residual; /* ||I - K K^-1||_F / sqrt(rank) of the last wcs_factor, measured
                          with exact products when K^-1 came from the tensor-core iteration
                          (mixed form, rank >= 256); -1 when not measured */

@@ -96,6 +96,7 @@ struct wcs_ctx {
   // mixed-precision form
   bool ordered = false;                   // FP64 products sum over k in order (see OrderedScope)
   bool mixed = false;
+  bool zfast_auto = false;                // zfast was left to the library
   int planes = 2, rhs_planes = 2;
   int64_t ldp = 0;                        // plane leading dimension (bf16 elements)
   DevBuf opplanes;                        // [op][layout][plane] N x ldp bf16
@@ -874,7 +875,7 @@ int wcs_default_options(wcs_options* o) {
   o->rhs_chunk = 256;
   o->mixed_planes = 3;
   o->rhs_planes = 3;
-  o->zfast = -1.0;  // automatic: 1000 in the mixed form (FP32 far pairs beyond k R = 1000), unused in FP64
+  o->zfast = -1.0;  // automatic (see far_threshold); unused in FP64
   return WCS_OK;
 }
 
@@ -890,9 +891,10 @@ static int create_context(wcs_ctx** out, const wcs_options* opt, void* stream, c
   if (o.q_far == 0) o.q_far = (o.precision == WCS_PREC_MIXED) ? 4 : 6;
   if (o.q_near == 0) o.q_near = (o.precision == WCS_PREC_MIXED) ? 8 : 12;
   if (o.sample_planes == 0) o.sample_planes = 2;
-  // any value > 0 takes the FP32 route of farpair.cuh from k R = 20 + k h on where
-  // k h <= 0.9 (its entries are good to ~1e-9); 1000 is the threshold on coarser meshes
-  if (o.zfast < 0.0) o.zfast = (o.precision == WCS_PREC_MIXED) ? 1000.0 : 0.0;
+  // automatic: the threshold of coarse meshes stands in the options (and in checkpoints,
+  // which compare them)
+  const bool zfast_auto = o.zfast < 0.0;
+  if (zfast_auto) o.zfast = (o.precision == WCS_PREC_MIXED) ? 1000.0 : 0.0;
   if (o.sample_planes < 1 || o.sample_planes > 2) { set_error("sample_planes must be 1 or 2"); return WCS_ERR_ARG; }
   if (o.exact_residual != 0 && o.exact_residual != 1) { set_error("exact_residual must be 0 or 1"); return WCS_ERR_ARG; }
   if (o.q_far < 2 || o.q_far > 16 || o.q_near < 4 || o.q_near > 16 || o.near_band < 1 ||
@@ -904,6 +906,7 @@ static int create_context(wcs_ctx** out, const wcs_options* opt, void* stream, c
   c->opt = o;
   c->s = (cudaStream_t)stream;
   c->mixed = (o.precision == WCS_PREC_MIXED);
+  c->zfast_auto = zfast_auto;
   c->planes = o.mixed_planes;
   c->rhs_planes = o.rhs_planes;
   if (rules) {
@@ -1074,6 +1077,24 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   return WCS_OK;
 }
 
+// k~ = k (1 + i t) with 0 <= t <= 0.1: both Hankel evaluations of a point pair come from a real one
+static bool kt_paired(const wcs_ctx* c) {
+  const double t = c->kt.y / c->k;
+  return c->kt.x == c->k && t >= 0.0 && t <= 0.1;
+}
+
+// k R0 (R0: distance of the element centres) from which element pairs of the mixed form
+// take the FP32 route of farpair.cuh; 0: none do.  A caller's zfast is the distance below
+// which pairs stay in FP64, whatever the mesh.  Left to the library it is where the route's
+// Hankel series holds, k R0 = 20, when k h <= 0.9: entries then carry 3e-9 to 7e-9, those of
+// FP64 quadrature 2.6e-9 after their split into bf16 planes.  On coarser meshes the route's
+// corrections are larger (5e-8 at k h = 2.5), and it only takes the pairs beyond 1000.
+static double far_threshold(const wcs_ctx* c) {
+  if (!c->mixed || !(c->opt.zfast > 0.0) || !kt_paired(c)) return 0.0;
+  const double kh = c->k * c->h, least = 20.0 + kh;
+  return (c->zfast_auto && kh <= 0.9) ? least : std::max(least, c->opt.zfast + 2.0 * kh);
+}
+
 int wcs_query(const wcs_ctx* c, wcs_info* info) {
   if (!c || !info) { set_error("null argument"); return WCS_ERR_ARG; }
   if (c->stage < ST_MESH) { set_error("no mesh yet"); return WCS_ERR_STATE; }
@@ -1082,7 +1103,7 @@ int wcs_query(const wcs_ctx* c, wcs_info* info) {
   info->rank = c->stage >= ST_SKELETON ? c->rank : -1;
   info->norm_cc = c->stage >= ST_ASSEMBLED ? c->norm_cc : 0.0;
   info->min_curvature = c->kmin;
-  info->zfast = c->mixed ? c->opt.zfast : 0.0;
+  info->zfast = far_threshold(c);
   info->capacitance_residual = c->kinv_res;
   return WCS_OK;
 }
@@ -1099,9 +1120,8 @@ static AsmArgs asm_args(wcs_ctx* c, bool circle) {
   A.near = circle ? c->near_c : c->near;
   A.wlog = c->wlog.d();
   A.ld = c->ld;
-  // k~ = k (1 + i t): both Hankel evaluations of a point pair from one real one
   const double t = c->kt.y / c->k;
-  if (c->kt.x == c->k && t >= 0.0 && t <= 0.1) {
+  if (kt_paired(c)) {
     const std::complex<double> z(1.0, t);
     const std::complex<double> c1 = 1.0 / z, c2 = 1.0 / std::sqrt(z);
     A.kt_pair = 1;
@@ -1119,17 +1139,10 @@ static AsmArgs asm_args(wcs_ctx* c, bool circle) {
   return A;
 }
 
-// Constants of the mixed form's far-pair route.  Pairs take it from k R0 = 20 on
-// (where its Hankel series holds) when k h <= 0.9: entries then carry ~5e-9, as
-// the FP64 quadrature's do after their split into bf16 planes (2.6e-9).  On
-// coarser meshes its corrections are larger (5e-8 at k h = 2.5) and it only
-// takes the pairs beyond zfast.  zfast <= 0: every pair in FP64.
+// Constants of the mixed form's far-pair route.
 static void set_far_consts(wcs_ctx* c, AsmArgs& A) {
-  const double kh = A.k * A.h;
-  double xmin = 1e300;
-  if (c->opt.zfast > 0.0 && A.kt_pair)
-    xmin = (kh <= 0.9) ? 20.0 + kh : std::max(20.0 + kh, c->opt.zfast + 2.0 * kh);
-  far_consts(A.fc, A.q_far, c->quad.xf, c->quad.wf, A.k, A.kt.y, A.h, xmin);
+  const double xmin = far_threshold(c);
+  far_consts(A.fc, A.q_far, c->quad.xf, c->quad.wf, A.k, A.kt.y, A.h, xmin > 0.0 ? xmin : 1e300);
   const std::complex<double> kt(A.kt.x, A.kt.y), I4(0.0, 0.25);
   const std::complex<double> ck = std::sqrt((2.0 / WCS_PI) / kt);
   const double ampk = std::sqrt(2.0 / (WCS_PI * A.k)), h2 = A.h * A.h;
