@@ -46,7 +46,8 @@ typedef enum wcs_status {
 } wcs_status;
 
 typedef enum wcs_precision {
-  WCS_PREC_FP64 = 0,        /* every stage in complex FP64 */
+  WCS_PREC_FP64 = 0,        /* every stage in complex FP64; products of 3e6 multiply-adds and more as
+                               exact integer products of 63 bits (see wcs_zgemm_fixed) */
   WCS_PREC_MIXED = 1        /* operator products on the tensor cores (split-bf16, FP32
                                accumulation; exact fixed-point products for the residual
                                with exact_residual), element-pair integrals in FP64 except
@@ -77,9 +78,9 @@ typedef struct wcs_options {
                          from 20 + k h on where k h <= 0.9, as 1000 on coarser meshes. */
   int sample_planes;  /* mixed form: bf16 planes of each operand in the skeleton's sampling
                          products (default 0 = 2; 1 = one product per pass, ~4e-3 relative) */
-  int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x exactly (8-bit
-                         digits of the operator planes and of x below each row's largest entry,
-                         integer products on the tensor cores, 64-bit integer sums), so
+  int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x with integer
+                         products (six 8-bit digits, 47 bits, of the operator planes below each
+                         row's and of x below each column's largest entry, 64-bit integer sums), so
                          refinement reaches refine_tol down to ~1e-12 against the stored operator;
                          costs 6 digits of each operator as bf16 (96 N^2 bytes in all, built at the
                          first such solve).  Adjoint solves keep the drained residual.  0
@@ -202,7 +203,10 @@ int wcs_circulant_eigs(wcs_ctx* ctx, int op, double* out_dev);
  * the FP64 eigenvalues mu_C.  In the mixed form, for power-of-two N in
  * [1024, 65536], the transform itself runs in FP32 (relative error ~1e-6:
  * these applies serve the Woodbury approximate inverse of Eq. 9 and the
- * sampling of C - C_c, both corrected by refinement); otherwise in FP64. */
+ * sampling of C - C_c, both corrected by refinement); otherwise in FP64.  Operator products
+ * of the FP64 form with 6 and more columns and 3e6 multiply-adds a column block err by at most
+ * N 2^-55 of the largest entry of the operator's row times that of X's column (see
+ * wcs_zgemm_fixed): relative to a column's largest entry, not entry by entry. */
 int wcs_apply(wcs_ctx* ctx, int op, int64_t B, const double* X_dev, int64_t ldx, double* Y_dev,
               int64_t ldy);
 
@@ -222,7 +226,7 @@ int wcs_skeleton(wcs_ctx* ctx, double tol, int max_rank, uint64_t seed, int* ran
  * closed by one step with the drained three-plane product and then by steps
  * with exact fixed-point products until ||I - K K^-1||_F / sqrt(rank),
  * measured with an exact product after each, is below 1e-10 (at most three;
- * ~3e-11 at rank 4096; reported in wcs_info.capacitance_residual).  Returns
+ * 7.6e-14 at rank 4096; reported in wcs_info.capacitance_residual).  Returns
  * WCS_ERR_SINGULAR when K is singular, the iteration does not converge, or
  * the closing steps leave that residual at 1e-6 or above. */
 int wcs_factor(wcs_ctx* ctx);
@@ -420,6 +424,20 @@ int wcs_gemm_split_bf16_noalloc(int64_t M, int64_t Nc, int64_t K, const double* 
  * WCS_ERR_TIMEOUT (a bounded device wait expired). */
 int wcs_gemm_exact(int64_t M, int64_t Nc, int64_t K, const double* A_dev, int64_t lda, const double* B_dev,
                    int64_t ldb, double* D_dev, int64_t ldd, void* stream);
+
+/* Complex product C (m x n, column-major, ldc) = A B + beta C on the tensor cores through
+ * signed 8-bit digits (A: m x k row-major, lda; B: k x n column-major, ldb; complex FP64,
+ * device), the product behind the FP64 form's operators (digits = 8) and behind the mixed
+ * form's exact residual (digits = 6: A as three bf16 planes first, like a stored operator).
+ * Rows of A and columns of B are cut below their largest entries a_i, b_j (63 or 47 bits
+ * below the next power of two).  Error of C_ij, beside the rounding of the result: k a_i b_j
+ * 2^-55 (1 + k / 64) with eight digits (the k / 64 only where all digits are coherent), k a_i
+ * b_j 2^-43 with six.
+ * panel_bytes: slices of each operand that are held at a time with digits = 8 (0: 512 MB).
+ * k <= 2^20.  Allocates its buffers; ordered on `stream`; synchronises.  Errors: WCS_ERR_ARG,
+ * WCS_ERR_OOM, WCS_ERR_CUDA, WCS_ERR_TIMEOUT. */
+int wcs_zgemm_fixed(int64_t m, int64_t n, int64_t k, const double* A_dev, int64_t lda, const double* B_dev, int64_t ldb,
+                    double beta, double* C_dev, int64_t ldc, int digits, int64_t panel_bytes, void* stream);
 
 /* Per-contour outcome of wcs_batch_solve_fourier. */
 typedef struct wcs_batch_stats {

@@ -88,6 +88,7 @@ SIGNATURES = {
     "wcs_quadrature_tables": (I, [I, P]),
     "wcs_fma_rate": (I, [I, I, P, C.POINTER(C.c_double)]),
     "wcs_gemm_exact": (I, [I64, I64, I64, P, I64, P, I64, P, I64, P]),
+    "wcs_zgemm_fixed": (I, [I64, I64, I64, P, I64, P, I64, D, P, I64, I, I64, P]),
     "wcs_shape_operator_forms": (I, [P, I, I64, P, P, I64, I, C.c_double, I, I, P]),
     "wcs_batch_solve_fourier": (I, [C.POINTER(Options), I, I, P, P, P, P, I64, P, C.c_double, I, U64, I, P,
                                     P]),

@@ -6,34 +6,43 @@
 // cores sum integer products exactly: a bf16 product of integers |a|, |b| <= 128
 // is exact and the FP32 accumulator holds sums up to 2^24.  So each row of an
 // operand is scaled by a power of two (its largest entry below 2^E) and written
-// as FX_SLICES signed 8-bit digits, v = sum_s d_s 2^(E - 6 - 8 s), |d_s| <= 128:
-// 63 bits below the row's largest entry, which keeps entries down to 2^-10 of it
-// to all 53 bits.  The product is the sum over the digit pairs s + t < FX_SLICES
-// (36 pairs; the dropped ones are below 2^-62 of the row scales) of exact
-// integer products.  Every level L = s + t has its own TMEM accumulator; it is
-// drained every FX_CHUNK stages (K = 128, where FX_SLICES pairs of 128 products
-// of 2^14 just reach 2^24) into 64-bit integers, so the sums over K are exact
-// and the result is rounded about twice.  The error is below that of an FP64
-// dot product, whose partial sums are rounded K times.
+// as NS signed 8-bit digits, v = sum_s d_s 2^(E - 6 - 8 s), |d_s| <= 128.
+//
+//             digits NS  error of v    levels s + t  digit pairs  dropped pairs
+//   products      8      2^(E - 63)       0 .. 7         36        7 2^-62
+//   operators     6      2^(E - 47)       0 .. 6         26        4 2^-54   (times 2^(EA + EB) per term)
+//
+// Every level has its own TMEM accumulator, exact over FX_CHUNK stages (K = 128, where
+// eight pairs of 128 products of 2^14 just reach 2^24).  Then it is drained: levels 0 .. 4
+// into 64-bit integers, exact over any K, the three (six digits: two) levels below them
+// into FP32 sums; rounded to FP64 once per split of K.
+//
+// The error of an entry is thus relative to the largest entries a of its row of A and b of
+// its column of B.  Eight digits: k a b 2^-55 from the digits, whatever the order of the
+// sum, and at most k a b 2^-55 (k / 64) from the FP32 sums, a bound that takes all lower
+// digits coherent and every rounding one way; with digits as they come it is their roundings
+// of ~sqrt(k) 2^-62 a b.  Six digits: k a b 2^-43.  The error of an FP64 dot product is up
+// to 2 k 2^-53 sum_k |A_ik| |B_kj|.  For entries of similar size the digits' is the smaller
+// one; entries below 2^-10 of their row's or column's largest keep fewer than 53
+// bits, so where the large entries of a column meet small ones of the row (a column that
+// spans many orders of magnitude), an FP64 product is the more accurate one.
 //
 // The complex product runs as the real product of A (m x 2k, re and im
 // interleaved) with B' (2n x 2k; row 2j = (Re x, -Im x), row 2j + 1 =
 // (Im x, Re x)).  Operands lie in memory as [row][K / 32][slice][32] bf16: one
 // 128-byte row of a TMA box is two slices of 32 K-values, so a stage is
-// FX_SLICES / 2 boxes per operand and the swizzle atom is that of the other
+// NS / 2 boxes per operand and the swizzle atom is that of the other
 // tensor-core kernels, the second slice 64 bytes into it.
 //
-// Operators of the exact residual are stored as six digits (the 26 pairs s + t < 7).
+// Tile 128 x 64: the levels, 64 columns each, fill 512 TMEM columns (seven with six
+// digits: 448).  The MMAs of a stage run from the highest level down; each level is
+// committed by itself, so the eight drain warps empty it while the next levels run.
+// Warp 8 loads, warp 9 issues.  K is split over the grid (FP64 partials, summed in
+// order) when the tiles alone do not fill the GPU.
 //
-// Tile 128 x 64: eight levels of 64 columns fill the 512 TMEM columns.  The MMAs
-// of a stage run from the highest level down; each level is committed by itself,
-// so the eight drain warps empty it while the next levels run.  Warp 8 loads,
-// warp 9 issues.  K is split over the grid (FP64 partials, summed in order) when
-// the tiles alone do not fill the GPU.
-//
-// Bound: 72 MMAs of 128 x 64 x 16 per 32 K-values, limited by the shared-memory
-// reads of A (6 KB per MMA, 48 clocks); for few columns the slicing of A, which
-// reads 16 and writes 32 bytes per complex entry.
+// Bound: with eight digits 72 MMAs of 128 x 64 x 16 per 32 K-values (52 with six),
+// limited by the shared-memory reads of A (6 KB per MMA, 48 clocks); for few columns
+// the slicing of A, which reads 16 and writes 32 bytes per complex entry.
 #include <algorithm>
 
 #include "fxgemm.h"
@@ -48,7 +57,7 @@ struct Fx {
   static constexpr int TOP = 8 * (NS - 1) + 6;        // fixed-point position: |v| 2^(TOP - E) < 2^TOP
   static constexpr int ROW = NS * FX_BK;              // bf16 values of one row and stage
   // digit-pair levels formed.  Six digits take one level past their own: without it the
-  // dropped pairs, 2^-46 of the row scales each, left an exact-residual solve at N = 16384
+  // dropped pairs, five of 2^-46 of the row scales a term, left an exact-residual solve at N = 16384
   // at 1.4e-11 where the entries' own 2^-48 leave 6e-13
   static constexpr int LEVELS = NS == 8 ? 8 : NS + 1;
   static constexpr int A_BYTES = FX_BM * ROW * 2, B_BYTES = FX_BN * ROW * 2;
@@ -295,9 +304,9 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(FX_BN >> 3) << 17) |
                          ((uint32_t)(FX_BM >> 4) << 24);
 
-  // drained sums of this thread's row and 32 columns, in units of the digit
-  // weight of level 4: levels 0..4 exactly, levels 5..7 (below one unit of
-  // level 4 per product) in FP32
+  // drained sums of this thread's row and 32 columns, in units of the digit weight of level 4:
+  // levels 0..4 exactly, the lower ones in FP32 (integers across all levels cost 32 registers
+  // or the carries between two words, 1% of a product)
   long long hi[32];
   float lo[32];
 #pragma unroll
@@ -445,17 +454,17 @@ struct FxPlan {
   int64_t kb, mp, np;        // stages; rows and complex columns of a panel
   size_t a_bytes, b_bytes, e_bytes, ws_bytes;
 };
-constexpr size_t FX_PANEL = (size_t)512 << 20, FX_PARTIALS = (size_t)64 << 20;
+constexpr size_t FX_PARTIALS = (size_t)64 << 20;
 
 static size_t fx_up(size_t b) { return (b + 255) & ~(size_t)255; }
 
-static FxPlan fx_plan(int64_t m, int64_t n, int64_t k) {
+static FxPlan fx_plan(int64_t m, int64_t n, int64_t k, size_t panel) {
   FxPlan p;
   p.kb = (2 * k + FX_BK - 1) / FX_BK;
   const size_t row = (size_t)p.kb * Fx<FX_SLICES>::ROW * 2;
-  p.mp = std::max<int64_t>(FX_BM, (int64_t)(FX_PANEL / row) / FX_BM * FX_BM);
+  p.mp = std::max<int64_t>(FX_BM, (int64_t)(panel / row) / FX_BM * FX_BM);
   p.mp = std::min(p.mp, std::min<int64_t>(m, 65535 * FX_BM));
-  p.np = std::max<int64_t>(FX_BN / 2, (int64_t)(FX_PANEL / (2 * row)) / (FX_BN / 2) * (FX_BN / 2));
+  p.np = std::max<int64_t>(FX_BN / 2, (int64_t)(panel / (2 * row)) / (FX_BN / 2) * (FX_BN / 2));
   p.np = std::min(p.np, n);
   p.a_bytes = fx_up(row * p.mp);
   p.b_bytes = fx_up(2 * row * p.np);
@@ -464,8 +473,8 @@ static FxPlan fx_plan(int64_t m, int64_t n, int64_t k) {
   return p;
 }
 
-size_t zgemm_fx_bytes(int64_t m, int64_t n, int64_t k) {
-  const FxPlan p = fx_plan(m, n, k);
+size_t zgemm_fx_bytes(int64_t m, int64_t n, int64_t k, size_t panel) {
+  const FxPlan p = fx_plan(m, n, k, panel);
   return p.a_bytes + p.b_bytes + p.e_bytes + p.ws_bytes;
 }
 
@@ -536,9 +545,9 @@ static int fx_panel(const uint16_t* da, const uint16_t* db, FxArgs a, zd* part, 
 }
 
 int zgemm_fx(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc, void* ws,
-             int* err, cudaStream_t s) {
+             int* err, cudaStream_t s, size_t panel) {
   if (m <= 0 || n <= 0 || k <= 0) return 0;
-  const FxPlan P = fx_plan(m, n, k);
+  const FxPlan P = fx_plan(m, n, k, panel);
   char* base = (char*)ws;
   uint16_t* da = (uint16_t*)base;
   uint16_t* db = (uint16_t*)(base + P.a_bytes);

@@ -9,14 +9,16 @@ constexpr int FX_SLICES = 8;   // 8-bit digits per value: 63 bits below each row
 
 // True when zgemm_fx is the faster route for the shape (see fxgemm.cu).
 bool zgemm_fx_wanted(int64_t m, int64_t n, int64_t k);
+// Slices of each operand that lie in device memory at a time, at most (or one tile's).
+constexpr size_t FX_PANEL = (size_t)512 << 20;
 // Device workspace of one call (bounded: large operands go through in panels).
-size_t zgemm_fx_bytes(int64_t m, int64_t n, int64_t k);
-// C (m x n, column-major ldc) = alpha * A (m x k) * B (k x n) + beta * C, with
-// the accuracy of an FP64 product.  ws: zgemm_fx_bytes of device memory; err:
+size_t zgemm_fx_bytes(int64_t m, int64_t n, int64_t k, size_t panel = FX_PANEL);
+// C (m x n, column-major ldc) = alpha * A (m x k) * B (k x n) + beta * C, each entry
+// to k max |A_i.| max |B_.j| 2^-55 and the rounding of the result (see fxgemm.cu).  ws: zgemm_fx_bytes of device memory; err:
 // device flag of the bounded waits (zero before the first use).  C must not
 // overlap A or B.
 int zgemm_fx(int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc, void* ws,
-             int* err, cudaStream_t s);
+             int* err, cudaStream_t s, size_t panel = FX_PANEL);
 
 // The mixed form's operators for exact residuals: rows kept as six digits (47 bits
 // below each row's largest entry; their entries carry 24) plus an exponent.
@@ -32,8 +34,8 @@ void fx_operand_bytes(int64_t rows, int64_t K, int64_t* kb, size_t* digits, size
 int fx_slice_planes(const uint16_t* const* planes, int nplanes, int64_t rows, int64_t K, int64_t ld,
                     const FxOperand& out, cudaStream_t s);
 // Y (m x n, ldy) = alpha * A X + beta * Y for a sliced A (m x k complex) and FP64
-// X (k x n, ldx), X as six digits below each column's largest entry; exact up to
-// their 2^-47 and the rounding of the result.  ws: fx_apply_bytes(n, 2 k).
+// X (k x n, ldx), X as six digits below each column's largest entry: errors of 2^-47 of
+// the column's and the row's largest entries a term, and the rounding of the result.  ws: fx_apply_bytes(n, 2 k).
 size_t fx_apply_bytes(int64_t n, int64_t K);
 int fx_apply(const FxOperand& A, int64_t m, int64_t n, int64_t k, zd alpha, const zd* X, int64_t ldx, zd beta, zd* Y,
              int64_t ldy, void* ws, int* err, cudaStream_t s);

@@ -265,9 +265,9 @@ static int check_tc(wcs_ctx* c);
 //                  kernel is also the faster one at these widths)
 //   PREC_FAST1     leading plane only, one product (~4e-3): optional skeleton
 //                  sampling (sample_planes = 1)
-//   PREC_EXACT     fixed-point slices of operator and vector, integer
-//                  products, FP64 sums (exact.cu): residuals of refinement
-//                  below the accurate floor (forward products only)
+//   PREC_EXACT     six digits of operator and vector, integer products and
+//                  sums (fxgemm.cu): residuals of refinement below the
+//                  accurate floor (forward products only)
 enum { PREC_FAST = 0, PREC_ACCURATE = 1, PREC_PERIODIC = 2, PREC_FAST1 = 3, PREC_EXACT = 4 };
 
 // K = 16 steps per drain of the accurate product: one shared-memory stage
@@ -459,7 +459,8 @@ static int ensure_exact_ops(wcs_ctx* c) {
   return 0;
 }
 
-// Y = alpha * op X + beta * Y, exactly up to FP64 rounding of the result (op 0 S~, 1 D, 2 D~, 3 N).
+// Y = alpha * op X + beta * Y (op 0 S~, 1 D, 2 D~, 3 N) with six digits of X below each column's
+// largest entry and of the operators below each row's, where their 24-bit entries keep 47 bits.
 static int ex_apply(wcs_ctx* c, int op, const zd* X, int64_t ldx, int64_t cols, zd alpha, zd beta, zd* Y,
                     int64_t ldy) {
   if (cols <= 0) return 0;
@@ -1630,8 +1631,8 @@ int wcs_factor(wcs_ctx* c) {
       if (!(res < 0.1 * std::sqrt((double)r))) { TRY(settle(c)); set_error("capacitance iteration did not converge"); return WCS_ERR_SINGULAR; }
       // The two-plane iteration stalls near 1e-4 per direction.  One step with
       // the drained three-plane product (~1e-7) and then exact steps (each
-      // squares the residual; the exact products carry 42 bits below each
-      // chunk's scale, ~1e-11 per direction) close it: an exact product
+      // squares the residual; eight digits, 63 bits below the largest entries of
+      // K's rows and X's columns, leave ~1e-13 per direction) close it: an exact product
       // measures ||I - K X||_F after every exact step, and a step is added
       // while that is above 1e-10 per direction (at most three).
       auto eye_residual = [&](double& out) -> int {
@@ -2753,6 +2754,57 @@ int wcs_gemm_exact(int64_t M, int64_t Nc, int64_t K, const double* A, int64_t ld
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) { set_error(std::string("gemm: ") + cudaGetErrorString(e)); return WCS_ERR_CUDA; }
   if (errh) { set_error("tensor-core contraction: a bounded wait expired"); return WCS_ERR_TIMEOUT; }
+  return WCS_OK;
+}
+
+int wcs_zgemm_fixed(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
+                    double beta, double* C, int64_t ldc, int digits, int64_t panel_bytes, void* stream) {
+  if (m < 0 || n < 0 || k < 0 || (digits != FX_SLICES && digits != FX_OP_SLICES) || panel_bytes < 0 ||
+      m > ((int64_t)1 << 24) || n > ((int64_t)1 << 24) || k > ((int64_t)1 << 20) || (m > 0 && (lda < k || (k > 0 && !A))) ||
+      (n > 0 && (ldb < k || (k > 0 && !B))) || (m > 0 && n > 0 && (!C || ldc < m))) {
+    set_error("bad argument");
+    return WCS_ERR_ARG;
+  }
+  if (m == 0 || n == 0) return WCS_OK;
+  cudaStream_t s = (cudaStream_t)stream;
+  zd* c = (zd*)C;
+  if (k == 0) {   // an empty product
+    TRY(axpby(m, n, mkz(0.0), c, ldc, mkz(beta), c, ldc, s));
+  } else {
+    DevBuf err, ws, planes, digits_a;
+    TRY(err.ensure(sizeof(int)));
+    cudaError_t e = cudaMemsetAsync(err.p, 0, sizeof(int), s);
+    if (e != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(e)); return WCS_ERR_CUDA; }
+    if (digits == FX_SLICES) {
+      const size_t panel = panel_bytes > 0 ? (size_t)panel_bytes : FX_PANEL;
+      TRY(ws.ensure(zgemm_fx_bytes(m, n, k, panel)));
+      TRY(zgemm_fx(m, n, k, mkz(1.0), ZView{(const zd*)A, lda, 1, false}, blk((const zd*)B, ldb), mkz(beta), c, ldc, ws.p,
+                   (int*)err.p, s, panel));
+    } else {   // as the stored operators of the mixed form: three bf16 planes first
+      const int64_t ldp = ((2 * k + 63) / 64) * 64;
+      TRY(planes.ensure(sizeof(uint16_t) * 3 * (size_t)m * ldp));
+      uint16_t* P[3];
+      for (int q = 0; q < 3; ++q) P[q] = (uint16_t*)planes.p + q * m * ldp;
+      TRY(split_complex_rows((const zd*)A, m, k, lda, 3, P, ldp, s));
+      FxOperand op;
+      size_t db = 0, eb = 0;
+      fx_operand_bytes(m, 2 * k, &op.kb, &db, &eb);
+      TRY(digits_a.ensure(db + eb));
+      op.d = (uint16_t*)digits_a.p;
+      op.e = (int*)((char*)digits_a.p + db);
+      TRY(fx_slice_planes(P, 3, m, 2 * k, ldp, op, s));
+      TRY(ws.ensure(fx_apply_bytes(n, 2 * k)));
+      TRY(fx_apply(op, m, n, k, mkz(1.0), (const zd*)B, ldb, mkz(beta), c, ldc, ws.p, (int*)err.p, s));
+    }
+    int errh = 0;
+    e = cudaMemcpyAsync(&errh, err.p, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(e)); return WCS_ERR_CUDA; }
+    if (errh) { set_error("tensor-core contraction: a bounded wait expired"); return WCS_ERR_TIMEOUT; }
+    return WCS_OK;
+  }
+  cudaError_t e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(e)); return WCS_ERR_CUDA; }
   return WCS_OK;
 }
 

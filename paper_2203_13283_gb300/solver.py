@@ -311,6 +311,21 @@ def gemm_exact(A, B):
     return D
 
 
+def zgemm_fixed(A, B, add=None, digits=8, panel_bytes=0):
+    """A @ B (+ add), complex128, cuda, through integer products of 8-bit digits (see wcs_zgemm_fixed)."""
+    A = torch.as_tensor(A, dtype=torch.complex128, device="cuda").contiguous()
+    Bc = torch.as_tensor(B, dtype=torch.complex128, device=A.device).t().contiguous()
+    (m, k), n = A.shape, Bc.shape[0]
+    if add is None:
+        out = torch.empty((n, m), dtype=torch.complex128, device=A.device)
+    else:
+        out = torch.as_tensor(add, dtype=torch.complex128, device=A.device).t().contiguous().clone()
+    st = torch.cuda.current_stream(A.device)
+    check(load().wcs_zgemm_fixed(m, n, k, _ptr(A), k, _ptr(Bc), k, 0.0 if add is None else 1.0, _ptr(out), m,
+                                 int(digits), int(panel_bytes), C.c_void_p(st.cuda_stream)))
+    return out.t()
+
+
 def batch_solve_fourier(contours, angles, tol=1e-6, rank_div=8, seed=1, workers=2, allow_unconverged=False,
                         **options):
     """Batched form: contours is a list of dicts {"cos": [...], "sin": [...], "N": int, "k": float or None}
