@@ -198,8 +198,34 @@ static int launch_tc(const TcOperand& A, const TcOperand& B, TcArgs& args, cudaS
   return 0;
 }
 
-// Sum of the split-K partials in a fixed order (FP64, or float-float for complex
-// output) and the epilogue.
+// A sum of FP32 values as FP32 terms (Knuth's error-free TwoSum).  Converting and adding
+// every value on the FP64 pipe took 50 us for the partials of 4096 x 256 and seven splits.
+// Three terms lose no value's last bit: FP64's sum or better, for the one-accumulator
+// products, whose partials FP64 summed.  Two terms (~48 bits) for the drained products,
+// whose parts of K were FP32 register sums before they were split; the third would cost
+// 1.2% of a solve of 360 columns at N = 4096.
+template <bool THREE>
+struct FloatSum {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = a + x, u = s - a, e = (a - (s - u)) + (x - u);
+    a = s;
+    const float t = b + e;
+    if (THREE) {
+      const float v = t - b;
+      c += (b - (t - v)) + (e - v);
+    }
+    b = t;
+  }
+  // infinities, NaN and sums beyond the FP32 range are left to an FP64 sum
+  __device__ __forceinline__ bool ok() const { return fabsf(a) <= 3.402823466e38f; }
+  __device__ __forceinline__ double value() const {
+    return epi_f32_to_f64(a) + (THREE ? epi_f32_to_f64(b) + epi_f32_to_f64(c) : epi_f32_to_f64(b));
+  }
+};
+
+// Sum of the split-K partials in a fixed order and the epilogue.
+template <bool DRAINED>
 __global__ void k_splitk_reduce(TcArgs a, int splits) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t plane = (int64_t)a.Nc * a.M;
@@ -217,22 +243,33 @@ __global__ void k_splitk_reduce(TcArgs a, int splits) {
   if (t >= (int64_t)a.M * ncols) return;
   const int row = (int)(t % a.M), j = (int)(t / a.M);
   const float* w = a.ws + (int64_t)(2 * j) * a.M + row;
-  // float-float sums (TwoSum keeps ~48 bits; the partials carry 24): converting
-  // and adding every partial on the FP64 pipe took 50 us at 4096 x 256 and seven splits
-  float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+  FloatSum<!DRAINED> r, s;
 #pragma unroll 8
   for (int z = 0; z < splits; ++z) {
-    const float x = w[z * plane], y = w[z * plane + a.M];
-    const float sx = rh + x, bx = sx - rh, sy = ih + y, by = sy - ih;
-    rl += (rh - (sx - bx)) + (x - bx);
-    il += (ih - (sy - by)) + (y - by);
-    rh = sx;
-    ih = sy;
+    r.add(w[z * plane]);
+    s.add(w[z * plane + a.M]);
   }
-  const double re = epi_f32_to_f64(rh) + epi_f32_to_f64(rl), im = epi_f32_to_f64(ih) + epi_f32_to_f64(il);
-  zd p = mkz(re, a.conj_out ? -im : im);
-  p = a.alpha * p;
+  double re = r.value(), im = s.value();
+  if (!r.ok() || !s.ok()) {
+    re = im = 0.0;
+    for (int z = 0; z < splits; ++z) {
+      re += (double)w[z * plane];
+      im += (double)w[z * plane + a.M];
+    }
+  }
+  if (a.conj_out) im = -im;
   zd* o = (zd*)a.out + (int64_t)j * a.ldo + row;
+  if (epi_unit(a)) {   // as epilogue_store: an infinite part must not meet the zero of alpha
+    zd p = a.alpha.x < 0.0 ? mkz(-re, -im) : mkz(re, im);
+    if (a.beta.x == 1.0) {
+      const zd q = *o;
+      p.x += q.x;
+      p.y += q.y;
+    }
+    *o = p;
+    return;
+  }
+  zd p = a.alpha * mkz(re, im);
   if (!(a.beta.x == 0.0 && a.beta.y == 0.0)) p += a.beta * (*o);
   *o = p;
 }
@@ -714,9 +751,11 @@ static int launch_tc_per(const TcOperand& A, const TcOperand& B, TcArgs& args, c
   return 0;
 }
 
-static int launch_splitk_reduce(const TcArgs& args, int splits, cudaStream_t s) {
+static int launch_splitk_reduce(const TcArgs& args, int splits, bool drained, cudaStream_t s) {
   const int64_t n = (int64_t)args.M * ((args.epi == EPI_RAW_F64) ? args.Nc : args.Nc / 2);
-  k_splitk_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(args, splits);
+  const unsigned blocks = (unsigned)((n + 255) / 256);
+  if (drained) k_splitk_reduce<true><<<blocks, 256, 0, s>>>(args, splits);
+  else k_splitk_reduce<false><<<blocks, 256, 0, s>>>(args, splits);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error(std::string("split-K reduce: ") + cudaGetErrorString(e)); return 3; }
@@ -726,7 +765,7 @@ static int launch_splitk_reduce(const TcArgs& args, int splits, cudaStream_t s) 
 // k-blocks per split of a drained product (0: no split).  A launch takes whole
 // waves of 152 CTAs, so a grid of 24 or 192 tiles leaves most of the chip idle in
 // its only or last wave; splitting K evens it out at the price of the partials
-// (written and read once, FP32, summed in float-float) and of a prologue and epilogue per
+// (written and read once, FP32) and of a prologue and epilogue per
 // CTA.  Microseconds: a K = 64 block of a 128 x 128 tile is 0.8 with three planes
 // (24 MMAs of 64 clocks) and 0.4 with two, of a 128 x 256 tile with two 0.8; about
 // 4 per CTA; 8 bytes per partial at 5 TB/s and a 4 us reduction launch.
@@ -772,7 +811,7 @@ int gemm_tc_accurate(const TcOperand& A, const TcOperand& B, TcArgs args, cudaSt
   else if (A.planes == 2 && B.planes == 2) r = launch_tc_acc<2, 2, 3>(A, B, args, s);
   else set_error("gemm_tc_accurate: plane combination not built");
   if (r || splits == 1) return r;
-  return launch_splitk_reduce(args, splits, s);
+  return launch_splitk_reduce(args, splits, true, s);
 }
 
 int gemm_tc_split_plan(int M, int Nc, int K, int planesA, int planesB, int epi, int64_t* ws_elems) {
@@ -834,7 +873,7 @@ int gemm_tc(const TcOperand& A, const TcOperand& B, TcArgs args, cudaStream_t s)
     default: set_error("gemm_tc: plane combination not built"); return 1;
   }
   if (r || args.no_reduce || splits == 1) return r;
-  return launch_splitk_reduce(args, splits, s);
+  return launch_splitk_reduce(args, splits, false, s);
 }
 
 }  // namespace wcs

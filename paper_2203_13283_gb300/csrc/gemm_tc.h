@@ -62,10 +62,15 @@ __device__ __forceinline__ double epi_f32_to_f64(float f) {
   return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | (m >> 3)), (int)((m & 7u) << 29));
 }
 
+// alpha = +-1, beta = 0 or 1 for complex output
+__device__ __forceinline__ bool epi_unit(const TcArgs& a) {
+  return a.epi == EPI_CPLX_F64 && a.alpha.y == 0.0 && (a.alpha.x == 1.0 || a.alpha.x == -1.0) && a.beta.y == 0.0 &&
+         (a.beta.x == 0.0 || a.beta.x == 1.0);
+}
+
 __device__ __forceinline__ void epilogue_store(const TcArgs& a, int row, int col0, const float (&v)[32]) {
   if (row >= a.M) return;
-  if (a.epi == EPI_CPLX_F64 && a.alpha.y == 0.0 && (a.alpha.x == 1.0 || a.alpha.x == -1.0) && a.beta.y == 0.0 &&
-      (a.beta.x == 0.0 || a.beta.x == 1.0)) {
+  if (epi_unit(a)) {
     // alpha = +-1, beta = 0 or 1 (the operator products of the solver): the
     // same values as the general complex arithmetic below (up to the sign of
     // a zero) with two exact conversions and at most two FP64 additions per
