@@ -199,9 +199,16 @@ __device__ inline Bessel01 bessel01_series_real(double x) {
   return b;
 }
 
-__device__ __forceinline__ int miller_start(double x) {
+__host__ __device__ __forceinline__ int miller_start(double x) {
   const int n0 = (int)(x + (x < 12.0 ? 25.0 : 45.0));
   return n0 + (n0 & 1);
+}
+
+// First index of the recurrence at x from a table that holds 0 where its own evaluation of x
+// lies outside the recurrence's range: at the ends of the range the two evaluations may
+// differ in the last bit, and a recurrence that never starts is 0 / 0.
+__host__ __device__ __forceinline__ int miller_start_of(int tabulated, double x) {
+  return tabulated > 0 ? tabulated : miller_start(x);
 }
 
 // The backward recurrence of hankel01_miller for real x; the threads that
@@ -210,6 +217,7 @@ __device__ __forceinline__ int miller_start(double x) {
 // thread's recurrence starts at its own `start` (zeros before it).
 template <bool FROM = false>
 __device__ inline Bessel01 bessel01_miller_real(double x, int start = 0) {
+  if (FROM) start = miller_start_of(start, x);
   const int n0 = __reduce_max_sync(__activemask(), FROM ? start : miller_start(x));
   const double iz2 = 2.0 / x;
   double jp1 = 0.0, j = FROM ? 0.0 : 1e-30, norm = 0.0, s0 = 0.0, s1 = 0.0, J1 = 0.0;
