@@ -151,9 +151,19 @@ int wcs_default_options(wcs_options* opt);
 int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream);
 
 /* Free every device buffer of ctx and the context itself (NULL is a no-op).
- * Until then a context keeps its buffers from one contour and mesh to the next
- * (growing them as needed; large ones shrink when a quarter would do). */
+ * Until then a context keeps its buffers from one contour, mesh and solve to the next and
+ * grows them as needed.  Of those of 256 MB and more it gives back: the scratch of the setup calls
+ * and of wcs_farfield when the call ends, operators and factors when the next ones need less
+ * than a quarter, and all of them when a mesh has less than a quarter of the last one's
+ * elements.  A call that finds the device full gives back every buffer that it does not use
+ * and tries again. */
 int wcs_destroy(wcs_ctx* ctx);
+
+/* Bound in bytes on the buffers that ctx keeps (0: none, the default); an allocation beyond it
+ * is treated as one that the device has no room for.  *held (optional) receives the bytes they
+ * take now.  Transform plans (up to a few hundred MB) and the scratch that a call frees when
+ * it returns are not counted. */
+int wcs_memory_limit(wcs_ctx* ctx, int64_t bytes, int64_t* held);
 
 /* --- contour gamma (Sec. II: a convex 2D contour), as r(theta) = rho(theta) (cos, sin) --- */
 /* Circle of radius a. */

@@ -81,6 +81,7 @@ SIGNATURES = {
     "wcs_gemm_split_bf16": (I, [I64, I64, I64, P, I64, P, I64, I, P, I64, P]),
     "wcs_gemm_split_bf16_ex": (I, [I64, I64, I64, P, I64, P, I64, I, I, P, I64, P]),
     "wcs_gemm_split_bf16_noalloc": (I, [I64, I64, I64, P, I64, P, I64, I, P, I64, P]),
+    "wcs_memory_limit": (I, [P, I64, C.POINTER(I64)]),
     "wcs_inject_timeout": (I, [P]),
     "wcs_launch_count": (U64, []),
     "wcs_profile": (I, [P, I]),

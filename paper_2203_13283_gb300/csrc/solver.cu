@@ -31,6 +31,11 @@ using namespace wcs;
 
 enum Stage { ST_NEW = 0, ST_CONTOUR = 1, ST_MESH = 2, ST_ASSEMBLED = 3, ST_SKELETON = 4, ST_FACTORED = 5 };
 
+// Buffers of this size and more are given back when they are idle or far larger than needed.
+constexpr size_t LARGE_BUF = (size_t)256 << 20;
+
+static int dev_alloc(void** p, size_t bytes);
+
 // Owned device buffer: grows on demand (contents not kept), freed by release()
 // or when it goes out of scope; not copyable.
 struct DevBuf {
@@ -44,19 +49,19 @@ struct DevBuf {
   }
   int ensure(size_t b) {
     if (b <= bytes) return 0;
-    cudaFree(p);
-    p = nullptr;
-    bytes = 0;
-    if (cudaMalloc(&p, b) != cudaSuccess) { set_error("out of device memory"); return WCS_ERR_OOM; }
+    release();
+    const int r = dev_alloc(&p, b);
+    if (r) { p = nullptr; return r; }
     bytes = b;
     return 0;
   }
   // ensure, giving a large buffer back first when less than a quarter of it is asked for
   int fit(size_t b) {
-    if (bytes > ((size_t)256 << 20) && b < bytes / 4) release();
+    if (bytes >= LARGE_BUF && b < bytes / 4) release();
     return ensure(b);
   }
   void release() { cudaFree(p); p = nullptr; bytes = 0; }
+  void release_large() { if (bytes >= LARGE_BUF) release(); }
   zd* z() { return (zd*)p; }
   double* d() { return (double*)p; }
 };
@@ -126,7 +131,65 @@ struct wcs_ctx {
   bool profile = false;
   struct Rec { int cat; cudaEvent_t a, b; double flops, bytes; };
   std::vector<Rec> recs;
+  size_t mem_limit = 0;      // bound on the bytes of the buffers below (0: none)
+
+  typedef std::vector<DevBuf*> Bufs;
+  // kept between calls: what the setup leaves, what the solves leave, the factors
+  Bufs setup_scratch() {
+    return {&tmp[0], &tmp[1], &tmp[2], &tmp[3], &tmp[4], &tmp[5], &tmp[6], &htab, &tiles, &offs, &centres, &qh, &qt, &far_map};
+  }
+  Bufs solve_scratch() {
+    return {&norms, &w1, &w2, &w3, &w4, &w5, &fx, &stage0, &stage1, &stage2, &gW, &gA, &gB, &sol_e, &sol_h, &sol_b,
+            &sol_ang, &sol_j, &exws};
+  }
+  Bufs factors() { return {&U, &Vw, &Wt, &pVwH.b, &pWt.b, &pUH.b, &pKinvH.b, &pWa.b, &Kinv, &Wa}; }
+  Bufs buffers() {
+    Bufs all = {&xf, &xn, &wn, &wlog, &pts_far, &pts_near, &pts_far_c, &pts_near_c, &ops, &mu, &conv, &arcbuf, &small,
+                &gwork, &opplanes, &tcerr, &exops};
+    for (const Bufs& b : {setup_scratch(), solve_scratch(), factors()}) all.insert(all.end(), b.begin(), b.end());
+    return all;
+  }
+  size_t held() {
+    size_t s = 0;
+    for (DevBuf* b : buffers()) s += b->bytes;
+    return s;
+  }
 };
+
+// A call on a context, with the buffers that it neither reads nor writes: while it runs they
+// are given back when the device (or the context's limit) has no room for another.
+struct Call {
+  wcs_ctx* c;
+  wcs_ctx::Bufs idle;
+  Call* outer;
+  static thread_local Call* top;
+  Call(wcs_ctx* c_, std::initializer_list<wcs_ctx::Bufs> lists) : c(c_), outer(top) {
+    for (const wcs_ctx::Bufs& l : lists) idle.insert(idle.end(), l.begin(), l.end());
+    top = this;
+  }
+  ~Call() { top = outer; }
+  Call(const Call&) = delete;
+  Call& operator=(const Call&) = delete;
+};
+thread_local Call* Call::top = nullptr;
+
+static int dev_alloc(void** p, size_t bytes) {
+  auto attempt = [&]() -> bool {
+    for (Call* s = Call::top; s; s = s->outer)
+      if (s->c->mem_limit > 0 && s->c->held() + bytes > s->c->mem_limit) return false;
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    (void)cudaGetLastError();   // reported here, not by the next launch
+    return false;
+  };
+  if (attempt()) return 0;
+  bool freed = false;
+  for (Call* s = Call::top; s; s = s->outer)
+    for (DevBuf* b : s->idle)
+      if (b->p) { b->release(); freed = true; }
+  if (freed && attempt()) return 0;
+  set_error("out of device memory");
+  return WCS_ERR_OOM;
+}
 
 enum StatCat { CAT_GEMM_TC = 0, CAT_ASSEMBLY = 1, CAT_FFT = 2, CAT_ZGEMM = 3, CAT_SKELETON = 4,
                CAT_FACTOR = 5, CAT_SOLVE = 6, CAT_GEMM_ACC = 7, CAT_SAMPLE = 8, CAT_PROJECT = 9,
@@ -221,9 +284,8 @@ struct OrderedScope {
 static int cz(wcs_ctx* c, int64_t m, int64_t n, int64_t k, zd alpha, ZView A, ZView B, zd beta, zd* C, int64_t ldc) {
   if (c->ordered) return zgemm_ordered(m, n, k, alpha, A, B, beta, C, ldc, c->s);
   if (zgemm_fx_wanted(m, n, k) && !ensure_tcerr(c)) {
-    if (!c->fx.ensure(zgemm_fx_bytes(m, n, k)))
+    if (!c->fx.ensure(zgemm_fx_bytes(m, n, k)))   // out of memory: not an error of this call
       return zgemm_fx(m, n, k, alpha, A, B, beta, C, ldc, c->fx.p, (int*)c->tcerr.p, c->s);
-    (void)cudaGetLastError();   // out of memory: not an error of this call
   }
   return zgemm(m, n, k, alpha, A, B, beta, C, ldc, c->s);
 }
@@ -607,8 +669,7 @@ static int apply_Cc(wcs_ctx* c, const zd* X, int64_t ldx, zd* Y, int64_t ldy, in
       }
       ProfScope ps(c, CAT_FFT, 0.0, 4.0 * 16.0 * (double)N * cols);
       return conv_apply(c->fft, khat, X, ldx, Y, ldy, cols, c->s);
-    }
-    (void)cudaGetLastError();   // no room for the kernels: Bluestein's transforms
+    }   // no room for the kernels: Bluestein's transforms
   }
   if (X != Y) {
     cudaError_t e = cudaMemcpy2DAsync(Y, sizeof(zd) * ldy, X, sizeof(zd) * ldx, sizeof(zd) * N, cols,
@@ -657,10 +718,8 @@ static int factor_gemm(wcs_ctx* c, wcs_ctx::Planes& P, int64_t m, int64_t n, int
   const int64_t ld = ((2 * k + 63) / 64) * 64, per = m * ld;
   uint16_t* pl[3] = {nullptr, nullptr, nullptr};
   if (!P.ready) {
-    if (P.b.ensure(sizeof(uint16_t) * 2 * (size_t)per)) {
-      (void)cudaGetLastError();   // no room to keep them: stage for this product
+    if (P.b.fit(sizeof(uint16_t) * 2 * (size_t)per))   // no room to keep them: stage for this product
       return cgemm(c, m, n, k, alpha, A, X, ldx, beta, C, ldc);
-    }
     pl[0] = (uint16_t*)P.b.p;
     pl[1] = pl[0] + per;
     if (ld != 2 * k) cudaMemsetAsync(P.b.p, 0, sizeof(uint16_t) * 2 * (size_t)per, c->s);
@@ -926,7 +985,8 @@ int wcs_create(wcs_ctx** out, const wcs_options* opt, void* stream) { return cre
 
 // A new contour or mesh invalidates everything built on the old one.  The device
 // buffers stay with the context for the next mesh (an allocation of gigabytes and
-// its release cost milliseconds); fit() gives them back when that is much smaller.
+// its release cost milliseconds); wcs_mesh gives the large ones back when that is
+// much smaller, and a call that finds the device full those it does not use (Call).
 static void free_mesh(wcs_ctx* c) {
   c->arc.cum = nullptr;
   c->stage_cols = 0;
@@ -1034,6 +1094,9 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   if (N < 12 || N > (int64_t)1 << 22) { set_error("N must be in [12, 4194304]"); return WCS_ERR_ARG; }
   free_mesh(c);
   c->stage = ST_CONTOUR;
+  if (N < c->N / 4)
+    for (DevBuf* b : c->buffers()) b->release_large();
+  Call call(c, {c->setup_scratch(), c->solve_scratch(), c->factors(), {&c->ops, &c->opplanes, &c->mu, &c->conv, &c->exops, &c->gwork}});
   TRY(c->arcbuf.ensure(sizeof(double) * arc_table_doubles()));
   TRY(arc_table_build(c->contour, c->arc, c->arcbuf.d(), c->s, c->mixed));
   c->L = c->arc.L;
@@ -1186,6 +1249,17 @@ int wcs_geometry_sample(wcs_ctx* c, int64_t count, const double* s_host, double*
 int wcs_assemble(wcs_ctx* c) {
   if (!c) { set_error("null context"); return WCS_ERR_ARG; }
   if (c->stage < ST_MESH) { set_error("mesh first"); return WCS_ERR_STATE; }
+  // what the old operators carried goes first: a call that fails leaves a mesh
+  c->stage = ST_MESH;
+  c->rank = -1;
+  c->stage_cols = 0;
+  drop_planes(c);
+  c->Kinv.release(); c->Wa.release();
+  for (bool& r : c->conv_ready) r = false;
+  c->circ.ready = false;   // the circulant tables follow mu_C
+  c->exact_ready = false;
+  Call call(c, {{&c->tmp[0], &c->tmp[1], &c->tmp[2], &c->tmp[3], &c->tmp[4], &c->tmp[5], &c->tmp[6], &c->qh, &c->qt, &c->far_map},
+                c->solve_scratch(), c->factors(), {&c->conv, &c->exops}});
   const int64_t N = c->N, ld = c->ld;
   bool near_tab = false;
   TRY(c->mu.ensure(sizeof(zd) * 6 * N));
@@ -1198,7 +1272,7 @@ int wcs_assemble(wcs_ctx* c) {
     AsmArgs A = asm_args(c, false);
     A.S = c->S; A.D = c->D; A.Dt = c->Dt; A.Nk = c->Nk;
     ProfScope ps(c, CAT_ASSEMBLY, (double)N * N * c->opt.q_far * c->opt.q_far, 0.0);
-    if (c->htab.ensure(assemble_dense_bytes(A))) (void)cudaGetLastError();   // no room: without it
+    (void)c->htab.fit(assemble_dense_bytes(A));   // no room: without it
     TRY(assemble_dense(A, B, c->gwork.z(), c->htab.bytes >= assemble_dense_bytes(A) ? c->htab.p : nullptr, c->s));
   } else {
     c->ldp = ((2 * N + 63) / 64) * 64;
@@ -1220,11 +1294,11 @@ int wcs_assemble(wcs_ctx* c) {
     AsmArgs A = asm_args(c, false);
     TRY(far_tables(A, cp, fe, fp, c->s));
     // Hankel table and near-band blocks (N (2 near_band + 1) of 256 bytes);
-    // without them (k~ off the table's form, a band of more than 1 GB) the tile
-    // kernel integrates those pairs itself
+    // without them (k~ off the table's form, a band of more than 1 GB or no room for
+    // it) the tile kernel integrates those pairs itself
     const int64_t band = N * (2 * c->opt.near_band + 1), band_row = 2 * (2 * c->opt.near_band + 1);
     near_tab = A.kt_pair && 2 * c->opt.near_band + 1 <= N && 256 * band <= ((int64_t)1 << 30);
-    if (near_tab) TRY(c->htab.ensure(sizeof(double) * (hankel_table_doubles() + 32 * (band + band_row))));
+    if (near_tab && c->htab.fit(sizeof(double) * (hankel_table_doubles() + 32 * (band + band_row)))) near_tab = false;
     A.planes = c->planes;
     A.ldp = c->ldp;
     for (int op = 0; op < 4; ++op)
@@ -1273,16 +1347,12 @@ int wcs_assemble(wcs_ctx* c) {
   TRY(fft_columns(c->fft, mu_ptr(c, MU_S), N, 4, +1, c->s));
   k_mu_finish<<<(unsigned)((N + 255) / 256), 256, 0, c->s>>>(c->mu.z(), N, c->h);
   note_launch();
-  c->circ.ready = false;   // the circulant tables follow mu_C
-  for (bool& r : c->conv_ready) r = false;
   TRY(c->small.ensure(sizeof(double) * 8));
   k_absmax<<<1, 256, 0, c->s>>>(mu_ptr(c, MU_C), N, c->small.d());
   note_launch();
   cudaMemcpyAsync(&c->norm_cc, c->small.p, sizeof(double), cudaMemcpyDeviceToHost, c->s);
   TRY(sync(c));
-  c->Kinv.release(); c->Wa.release();
-  drop_planes(c);
-  c->rank = -1;
+  c->htab.release_large();
   c->stage = ST_ASSEMBLED;
   return WCS_OK;
 }
@@ -1349,6 +1419,7 @@ int wcs_apply(wcs_ctx* c, int op, int64_t B, const double* X, int64_t ldx, doubl
   TRY(check_block(c, B, X, ldx));
   TRY(check_block(c, B, Y, ldy));
   if (B == 0) return WCS_OK;
+  Call call(c, {c->setup_scratch()});
   const int64_t N = c->N;
   const zd* x = (const zd*)X;
   zd* y = (zd*)Y;
@@ -1405,6 +1476,13 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   if (!c) { set_error("null context"); return WCS_ERR_ARG; }
   if (c->stage < ST_ASSEMBLED) { set_error("assemble first"); return WCS_ERR_STATE; }
   if (!(tol >= 0)) { set_error("tolerance must be >= 0"); return WCS_ERR_ARG; }
+  // the old skeleton and its factors go first: a call that fails leaves the operators
+  c->stage = ST_ASSEMBLED;
+  drop_planes(c);
+  c->Kinv.release(); c->Wa.release();
+  Call call(c, {{&c->tmp[5], &c->tmp[6], &c->htab, &c->tiles, &c->offs, &c->centres, &c->far_map, &c->norms, &c->fx, &c->sol_e,
+                 &c->sol_h, &c->sol_b, &c->sol_ang, &c->sol_j, &c->exws, &c->Wt, &c->pVwH.b, &c->pWt.b, &c->pUH.b, &c->pKinvH.b,
+                 &c->pWa.b}});
   const int64_t N = c->N;
   OrderedScope ordered(c);
   const int64_t cap = (max_rank <= 0 || max_rank > N) ? N : max_rank;
@@ -1416,7 +1494,7 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   // stream, so the basis is the one of the b-column loop
   const int64_t SB = std::min<int64_t>(8 * (int64_t)b, ((cap + b - 1) / b) * b);
   TRY(ensure_work(c, SB));
-  TRY(c->U.ensure(sizeof(zd) * N * (cap + b)));
+  TRY(c->U.fit(sizeof(zd) * N * (cap + b)));
   zd* Q = c->U.z();
   const double thr = tol * c->norm_cc / (10.0 * std::sqrt(2.0 / WCS_PI));
   // small scratch: Z (cap x b), Gram (b x b), perm, rank, norms
@@ -1519,11 +1597,10 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
     ell += rk;
     if (ell > cap) ell = cap;
   }
-  for (DevBuf* q : {&c->qh, &c->qt})
-    if (q->bytes > ((size_t)256 << 20)) q->release();
+  for (DevBuf* q : {&c->qh, &c->qt, &GW, &Zb, &Gb, &Ib, &Nb}) q->release_large();
   c->rank = (int)ell;
   // V^T = Q^H (C - C_c)  <=>  Vw = (C - C_c)^H Q  (V = conj(Vw))
-  TRY(c->Vw.ensure(sizeof(zd) * N * std::max<int64_t>(ell, 1)));
+  TRY(c->Vw.fit(sizeof(zd) * N * std::max<int64_t>(ell, 1)));
   ProfScope ps_vw(c, CAT_VW, 0.0, 0.0);
   const int64_t wide = std::max<int64_t>(b, std::min<int64_t>(c->opt.rhs_chunk, 1024));
   TRY(ensure_work(c, wide));
@@ -1533,8 +1610,6 @@ int wcs_skeleton(wcs_ctx* c, double tol, int max_rank, uint64_t seed, int* rank_
   }
   TRY(check_tc(c));
   if (rank_out) *rank_out = (int)ell;
-  c->Kinv.release(); c->Wa.release();
-  drop_planes(c);
   c->stage = ST_SKELETON;
   return status;
 }
@@ -1553,11 +1628,14 @@ int wcs_factor(wcs_ctx* c) {
   if (c->stage < ST_SKELETON) { set_error("skeleton first"); return WCS_ERR_STATE; }
   const int64_t N = c->N, r = c->rank;
   OrderedScope ordered(c);
+  c->stage = ST_SKELETON;
   c->kinv_res = -1.0;
   drop_planes(c);
+  Call call(c, {{&c->htab, &c->tiles, &c->offs, &c->centres, &c->far_map, &c->qh, &c->qt, &c->norms, &c->sol_e, &c->sol_h, &c->sol_b,
+                 &c->sol_ang, &c->sol_j, &c->exws, &c->pVwH.b, &c->pWt.b, &c->pUH.b, &c->pKinvH.b, &c->pWa.b}});
   ProfScope whole(c, CAT_FACTOR, 8.0 / 3.0 * r * (double)r * r, 0.0);
   if (r > 0) {
-    TRY(c->Wt.ensure(sizeof(zd) * N * r));
+    TRY(c->Wt.fit(sizeof(zd) * N * r));
     // W = C_c^{-1} U  (held in Wt until the inverse is applied)
     DevBuf &Wb = c->tmp[0], &Kb = c->tmp[1], &info = c->tmp[2];
     DevBuf& Kinv = c->Kinv;   // kept for adjoint solves
@@ -1668,6 +1746,7 @@ int wcs_factor(wcs_ctx* c) {
     // Wt = W K^{-1}
     TRY(cgemm(c, N, r, r, mkz(1.0), blk(Wb.z(), N), Kinv.z(), r, mkz(0.0), c->Wt.z(), N));
     TRY(check_tc(c));
+    for (DevBuf& b : c->tmp) b.release_large();
   }
   c->stage = ST_FACTORED;
   return WCS_OK;
@@ -1896,6 +1975,7 @@ int wcs_load(wcs_ctx* c, const char* path) {
   if (!r) r = set_contour(c, hd.contour);
   if (!r) r = wcs_mesh(c, hd.N, hd.k);
   if (!r) r = wcs_assemble(c);
+  Call call(c, {c->setup_scratch()});
   if (!r && hd.rank > 0) {
     const size_t b = sizeof(zd) * (size_t)hd.N * hd.rank;
     r = c->U.ensure(b);
@@ -1920,6 +2000,7 @@ int wcs_woodbury_apply(wcs_ctx* c, int64_t B, const double* b, int64_t ldb, doub
   if (c->stage < ST_FACTORED) { set_error("factor first"); return WCS_ERR_STATE; }
   TRY(check_block(c, B, b, ldb));
   TRY(check_block(c, B, x, ldx));
+  Call call(c, {c->setup_scratch()});
   const int64_t chunk = c->opt.rhs_chunk;
   TRY(ensure_work(c, std::min(B, chunk)));
   for (int64_t c0 = 0; c0 < B; c0 += chunk) {
@@ -2192,6 +2273,7 @@ int wcs_solve_rhs(wcs_ctx* c, int64_t B, const double* e, const double* hv, int6
   TRY(check_block(c, B, e, ld));
   TRY(check_block(c, B, hv, ld));
   TRY(check_block(c, B, j, ldj));
+  Call call(c, {c->setup_scratch()});
   const int64_t chunk = c->opt.rhs_chunk, N = c->N;
   TRY(ensure_work(c, std::min(B, chunk)));
   DevBuf& bb = c->sol_b;
@@ -2221,6 +2303,7 @@ static int solve_general(wcs_ctx* c, int64_t B, const double* b, int64_t ldb, do
   TRY(check_block(c, B, b, ldb));
   TRY(check_block(c, B, x, ldx));
   if (B == 0) return WCS_OK;
+  Call call(c, {c->setup_scratch()});
   const int64_t chunk = c->opt.rhs_chunk;
   TRY(ensure_work(c, std::min(B, chunk)));
   int status = WCS_OK;
@@ -2411,6 +2494,7 @@ int wcs_shape_gradient_range(wcs_ctx* c, int64_t B, const double* angles, int np
   if (!(delta > 0)) delta = 1e-6;
   const int64_t N = c->N;
   OrderedScope ordered(c);
+  Call call(c, {c->setup_scratch()});
   DevBuf j, lam, E, F, G, ang, phd, dots;
   TRY(j.ensure(sizeof(zd) * N * B));
   TRY(lam.ensure(sizeof(zd) * N * B));
@@ -2547,6 +2631,7 @@ int wcs_shape_operator_forms(wcs_ctx* c, int op, int64_t B, const double* u_dev,
   if (!(delta > 0)) delta = 1e-6;
   const int64_t N = c->N;
   OrderedScope ordered(c);
+  Call call(c, {c->setup_scratch()});
   DevBuf Wb;
   TRY(Wb.ensure(sizeof(zd) * 4 * N * N));
   cudaMemsetAsync(Wb.p, 0, Wb.bytes, c->s);
@@ -2575,6 +2660,7 @@ int wcs_solve_planewaves(wcs_ctx* c, int64_t B, const double* angles, double* j,
   TRY(check_block(c, B, j, ldj));
   if (B == 0) return WCS_OK;
   TRY(check_angles(B, angles, "solve_planewaves"));
+  Call call(c, {c->setup_scratch()});
   const int64_t chunk = c->opt.rhs_chunk, N = c->N;
   TRY(ensure_work(c, std::min(B, chunk)));
   DevBuf &eb = c->sol_e, &hb = c->sol_h, &bb = c->sol_b, &ang = c->sol_ang;
@@ -2604,6 +2690,7 @@ int wcs_solve_planewaves_host(wcs_ctx* c, int64_t B, const double* angles, doubl
                               int64_t ldj, wcs_solve_info* info) {
   if (!c || (B > 0 && (!angles || !j_host)) || ldj < (c ? c->N : 0)) { set_error("bad argument"); return WCS_ERR_ARG; }
   if (B == 0) return WCS_OK;
+  Call call(c, {c->setup_scratch()});
   DevBuf& jd = c->sol_j;
   TRY(jd.ensure(sizeof(zd) * c->N * B));
   int r = wcs_solve_planewaves(c, B, angles, jd.d(), c->N, info);
@@ -2621,6 +2708,8 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
   TRY(check_block(c, B, j, ldj));
   if (B == 0 || nphi == 0) return WCS_OK;
   TRY(check_angles(nphi, phi, "farfield"));
+  Call call(c, {{&c->tmp[0], &c->tmp[1], &c->tmp[2], &c->tmp[3], &c->tmp[4], &c->tmp[5], &c->tmp[6], &c->htab, &c->tiles, &c->offs,
+                 &c->centres, &c->qh, &c->qt}});
   DevBuf &E = c->far_map, &ang = c->sol_ang;
   TRY(E.fit(sizeof(zd) * ((int64_t)nphi * c->N + farfield_moments(c->N))));
   TRY(ang.ensure(sizeof(double) * nphi));
@@ -2629,7 +2718,9 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
                       nphi, E.z(), nphi, c->s, E.z() + (int64_t)nphi * c->N));
   TRY(cz(c, nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
          (zd*)F, ldf));
-  return check_tc(c);
+  TRY(check_tc(c));
+  E.release_large();
+  return WCS_OK;
 }
 
 static int gemm_split_impl(int64_t M, int64_t Nc, int64_t K, const double* A, int64_t lda, const double* B,
@@ -2805,6 +2896,13 @@ int wcs_zgemm_fixed(int64_t m, int64_t n, int64_t k, const double* A, int64_t ld
   }
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) { set_error(std::string("zgemm: ") + cudaGetErrorString(e)); return WCS_ERR_CUDA; }
+  return WCS_OK;
+}
+
+int wcs_memory_limit(wcs_ctx* c, int64_t bytes, int64_t* held) {
+  if (!c || bytes < 0) { set_error("bad argument"); return WCS_ERR_ARG; }
+  c->mem_limit = (size_t)bytes;
+  if (held) *held = (int64_t)c->held();
   return WCS_OK;
 }
 

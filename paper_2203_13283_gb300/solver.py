@@ -62,6 +62,12 @@ class Solver:
         except Exception:
             pass
 
+    def memory(self, limit=0):
+        """Bytes of the device buffers the context keeps; limit: bound on them (0: none)."""
+        held = C.c_int64(0)
+        check(self.lib.wcs_memory_limit(self.h, int(limit), C.byref(held)))
+        return held.value
+
     # ---- contour and mesh
     def contour(self, family, **p):
         if family == "circle":
