@@ -161,8 +161,8 @@ int wcs_destroy(wcs_ctx* ctx);
 
 /* Bound in bytes on the buffers that ctx keeps (0: none, the default); an allocation beyond it
  * is treated as one that the device has no room for.  *held (optional) receives the bytes they
- * take now.  Transform plans (up to a few hundred MB) and the scratch that a call frees when
- * it returns are not counted. */
+ * take now.  Transform plans and the scratch that a call frees when it returns are asked the
+ * same question but are not part of *held. */
 int wcs_memory_limit(wcs_ctx* ctx, int64_t bytes, int64_t* held);
 
 /* --- contour gamma (Sec. II: a convex 2D contour), as r(theta) = rho(theta) (cos, sin) --- */

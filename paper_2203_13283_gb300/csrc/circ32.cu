@@ -381,7 +381,7 @@ int circ32_prepare(Circ32& p, const zd* mu, int64_t n, cudaStream_t s) {
     cudaFree(p.scale);
     p.scale = nullptr;
     p.scale_n = 0;
-    if (cudaMalloc(&p.scale, sizeof(float2) * 4 * n) != cudaSuccess) { set_error("oom (circ32 scale)"); return WCS_ERR_OOM; }
+    if (const int r = device_alloc((void**)&p.scale, sizeof(float2) * 4 * n)) { p.scale = nullptr; return r; }
     p.scale_n = n;
   }
   k_circ_scale<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(mu, n, p.n1, p.n2, p.n1 / 32, p.scale);
@@ -403,7 +403,7 @@ int circ32_apply(Circ32& p, const zd* x, int64_t ldx, zd* y, int64_t ldy, int64_
     cudaFree(p.work);
     p.work = nullptr;
     p.work_elems = 0;
-    if (cudaMalloc(&p.work, sizeof(float2) * n * cap) != cudaSuccess) { set_error("oom (circ32 work)"); return WCS_ERR_OOM; }
+    if (const int r = device_alloc((void**)&p.work, sizeof(float2) * n * cap)) { p.work = nullptr; return r; }
     p.work_elems = n * cap;
   }
   float2* S = p.work;

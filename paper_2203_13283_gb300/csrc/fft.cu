@@ -298,26 +298,20 @@ int fft_plan_create(FFTPlan& p, int64_t n, cudaStream_t s) {
     p.m = m;
     len = m;
   }
-  if (cudaMalloc(&p.twiddle, sizeof(zd) * len) != cudaSuccess) { set_error("oom (fft)"); return 4; }
+  if (const int r = device_alloc((void**)&p.twiddle, sizeof(zd) * len)) return r;
   k_twiddles<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(p.twiddle, len);
   note_launch();
   p.work_cols = std::max<int64_t>(1, std::min<int64_t>(256, (int64_t(1) << 27) / len));
-  if (cudaMalloc(&p.work, sizeof(zd) * len * p.work_cols * (p.pow2 ? 1 : 2)) != cudaSuccess) {
-    set_error("oom (fft work)");
-    return 4;
-  }
+  if (const int r = device_alloc((void**)&p.work, sizeof(zd) * len * p.work_cols * (p.pow2 ? 1 : 2))) return r;
   if (!p.pow2) {
     const int64_t m = p.m;
-    if (cudaMalloc(&p.chirp, sizeof(zd) * n) != cudaSuccess ||
-        cudaMalloc(&p.chirp_hat, sizeof(zd) * m) != cudaSuccess) {
-      set_error("oom (bluestein)");
-      return 4;
-    }
+    if (const int r = device_alloc((void**)&p.chirp, sizeof(zd) * n)) return r;
+    if (const int r = device_alloc((void**)&p.chirp_hat, sizeof(zd) * m)) return r;
     // linear convolution of n values needs 2 n - 1: three quarters of m where that is enough
     p.conv_r = 3 * (m / 4) >= 2 * n - 1 ? 3 : 2;
     p.conv_m = p.conv_r == 3 ? m / 4 : m / 2;
     const int64_t c = p.conv_r * p.conv_m;
-    if (cudaMalloc(&p.conv_tw, sizeof(zd) * (c + p.conv_m)) != cudaSuccess) { set_error("oom (convolution)"); return 4; }
+    if (const int r = device_alloc((void**)&p.conv_tw, sizeof(zd) * (c + p.conv_m))) return r;
     k_twiddles<<<(unsigned)((c + 255) / 256), 256, 0, s>>>(p.conv_tw, c);
     note_launch();
     k_twiddles<<<(unsigned)((p.conv_m + 255) / 256), 256, 0, s>>>(p.conv_tw + c, p.conv_m);

@@ -32,6 +32,10 @@ struct DeviceOnce {
   }
 };
 
+// Device memory for the running call: where there is no room, the kept buffers that the call
+// does not use are given back first.  0, or WCS_ERR_OOM with its message.
+int device_alloc(void** p, size_t bytes);
+
 // ---------------------------------------------------------------- geometry
 enum ContourFamily { FAM_CIRCLE = 0, FAM_ELLIPSE = 1, FAM_SUPERELLIPSE = 2, FAM_FOURIER = 3 };
 constexpr int kMaxFourier = 64;

@@ -34,8 +34,6 @@ enum Stage { ST_NEW = 0, ST_CONTOUR = 1, ST_MESH = 2, ST_ASSEMBLED = 3, ST_SKELE
 // Buffers of this size and more are given back when they are idle or far larger than needed.
 constexpr size_t LARGE_BUF = (size_t)256 << 20;
 
-static int dev_alloc(void** p, size_t bytes);
-
 // Owned device buffer: grows on demand (contents not kept), freed by release()
 // or when it goes out of scope; not copyable.
 struct DevBuf {
@@ -50,7 +48,7 @@ struct DevBuf {
   int ensure(size_t b) {
     if (b <= bytes) return 0;
     release();
-    const int r = dev_alloc(&p, b);
+    const int r = device_alloc(&p, b);
     if (r) { p = nullptr; return r; }
     bytes = b;
     return 0;
@@ -173,7 +171,7 @@ struct Call {
 };
 thread_local Call* Call::top = nullptr;
 
-static int dev_alloc(void** p, size_t bytes) {
+int wcs::device_alloc(void** p, size_t bytes) {
   auto attempt = [&]() -> bool {
     for (Call* s = Call::top; s; s = s->outer)
       if (s->c->mem_limit > 0 && s->c->held() + bytes > s->c->mem_limit) return false;
@@ -1094,8 +1092,10 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   if (N < 12 || N > (int64_t)1 << 22) { set_error("N must be in [12, 4194304]"); return WCS_ERR_ARG; }
   free_mesh(c);
   c->stage = ST_CONTOUR;
-  if (N < c->N / 4)
+  if (N < c->N / 4) {
     for (DevBuf* b : c->buffers()) b->release_large();
+    circ32_release(c->circ);
+  }
   Call call(c, {c->setup_scratch(), c->solve_scratch(), c->factors(), {&c->ops, &c->opplanes, &c->mu, &c->conv, &c->exops, &c->gwork}});
   TRY(c->arcbuf.ensure(sizeof(double) * arc_table_doubles()));
   TRY(arc_table_build(c->contour, c->arc, c->arcbuf.d(), c->s, c->mixed));

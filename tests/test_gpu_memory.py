@@ -104,3 +104,17 @@ def test_large_buffers_are_given_back():
     currents(s, 1000, 4)
     assert s.memory() < 2e9
     s.close()
+
+
+def test_transform_plan_after_a_full_mesh():
+    """The plan of a new length finds the room of the old mesh's operators."""
+    s = new(0)
+    s.mesh(1000).assemble()
+    s.memory(s.memory() + (1 << 20))          # the operators of N = 1000 take 64 MB, the plan of N = 997 17 MB
+    s.mesh(997)
+    s.memory(0)
+    x = torch.randn(997, 3, dtype=torch.complex128, device="cuda")
+    s.assemble()
+    f = np.fft.fft(to_np(x), axis=0) * to_np(s.circulant_eigs("CC"))[:, None]
+    assert colrel(to_np(s.apply("CC", x)), np.fft.ifft(f, axis=0)) < 1e-12
+    s.close()
