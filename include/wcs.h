@@ -73,9 +73,10 @@ typedef struct wcs_options {
   int rhs_planes;     /* mixed form: bf16 planes per staged vector entry (= mixed_planes) */
   double zfast;       /* mixed form: element pairs with k R0 >= zfast + 2 k h (R0: distance of their
                          centres; 20 + k h at least) run on the FP32 pipe, as small corrections
-                         around a float-float value at the centres (3e-9 to 7e-9 of the entry);
+                         around a float-float value at the centres (3e-9 to 7e-9 of the entry rms);
                          nearer ones in FP64.  0: every pair in FP64.  Default -1 = automatic:
-                         from 20 + k h on where k h <= 0.9, as 1000 on coarser meshes. */
+                         from 20 + k h on where k h <= 0.9 and no element turns by more than a
+                         radian, as 1000 on coarser meshes. */
   int sample_planes;  /* mixed form: bf16 planes of each operand in the skeleton's sampling
                          products (default 0 = 2; 1 = one product per pass, ~4e-3 relative) */
   int exact_residual; /* mixed form: 1 = evaluate the refinement residual b - C x with integer

@@ -229,9 +229,10 @@ __global__ void k_points(Contour c, const double* cum, int P, double L, int64_t 
   if (out.kappa) out.kappa[idx] = kap;
 }
 
-__global__ void k_min_curv(Contour c, const double* cum, int P, double L, int64_t M, double* kmin) {
-  __shared__ double red[256];
-  double m = 1e300;
+// Extremes of the curvature, each block's minimum and maximum
+__global__ void k_curvature_range(Contour c, int64_t M, double* out) {
+  __shared__ double red[2][256];
+  double lo = 1e300, hi = -1e300;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M;
        i += (int64_t)gridDim.x * blockDim.x) {
     // a dense uniform grid in theta covers the curve as well as one in arc
@@ -240,15 +241,21 @@ __global__ void k_min_curv(Contour c, const double* cum, int P, double L, int64_
     double r0, r1, r2;
     rho_derivs(c, th, r0, r1, r2);
     const double sp2 = r0 * r0 + r1 * r1;
-    m = fmin(m, (r0 * r0 + 2.0 * r1 * r1 - r0 * r2) / (sp2 * sqrt(sp2)));
+    const double kap = (r0 * r0 + 2.0 * r1 * r1 - r0 * r2) / (sp2 * sqrt(sp2));
+    lo = fmin(lo, kap);
+    hi = fmax(hi, kap);
   }
-  red[threadIdx.x] = m;
+  red[0][threadIdx.x] = lo;
+  red[1][threadIdx.x] = hi;
   __syncthreads();
   for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] = fmin(red[threadIdx.x], red[threadIdx.x + o]);
+    if (threadIdx.x < o) {
+      red[0][threadIdx.x] = fmin(red[0][threadIdx.x], red[0][threadIdx.x + o]);
+      red[1][threadIdx.x] = fmax(red[1][threadIdx.x], red[1][threadIdx.x + o]);
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) kmin[blockIdx.x] = red[0];
+  if (threadIdx.x < 2) out[gridDim.x * threadIdx.x + blockIdx.x] = red[threadIdx.x][0];
 }
 
 static DeviceOnce g_gl16_ready;   // __constant__ tables are per device
@@ -301,18 +308,20 @@ int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const
   return 0;
 }
 
-int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, double* d,
-                  cudaStream_t s) {
-  const int blocks = 304;
-  k_min_curv<<<blocks, 256, 0, s>>>(c, t.cum, t.P, t.L, samples, d);
+int curvature_range(const Contour& c, int64_t samples, double* kmin, double* kmax, double* d, cudaStream_t s) {
+  constexpr int blocks = CURVATURE_WORK / 2;
+  k_curvature_range<<<blocks, 256, 0, s>>>(c, samples, d);
   note_launch();
-  double h[blocks];
+  double h[2 * blocks];
   cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) { set_error(cudaGetErrorString(err)); return 3; }
-  double m = 1e300;
-  for (int i = 0; i < blocks; ++i) m = fmin(m, h[i]);
-  *kmin = m;
+  *kmin = 1e300;
+  *kmax = -1e300;
+  for (int i = 0; i < blocks; ++i) {
+    *kmin = fmin(*kmin, h[i]);
+    *kmax = fmax(*kmax, h[blocks + i]);
+  }
   return 0;
 }
 

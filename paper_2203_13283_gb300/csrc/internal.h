@@ -79,9 +79,10 @@ struct PointSet {
 };
 int points_build(const Contour& c, const ArcTable& t, int64_t N, double h, const PointSet& s0, const PointSet& s1,
                  cudaStream_t s, double tol);
-// Minimum curvature over a dense sample of the contour (convexity check).
-// (work: 304 doubles of device memory)
-int min_curvature(const Contour& c, const ArcTable& t, int64_t samples, double* kmin, double* work, cudaStream_t s);
+// Smallest (convexity check) and largest curvature over a dense sample of the contour;
+// work: CURVATURE_WORK doubles of device memory.
+constexpr int CURVATURE_WORK = 608;
+int curvature_range(const Contour& c, int64_t samples, double* kmin, double* kmax, double* work, cudaStream_t s);
 
 // ---------------------------------------------------------------- quadrature
 struct QuadTables {

@@ -71,7 +71,7 @@ struct wcs_ctx {
   Contour contour{}, circle{};
   ArcTable arc{}, arc_c{};
   int64_t N = 0, ld = 0;
-  double L = 0, h = 0, a = 0, k = 0, kmin = 0;
+  double L = 0, h = 0, a = 0, k = 0, kmin = 0, kmax = 0;
   zd kt = mkz(0.0);
   QuadTables quad;
   DevBuf xf, xn, wn, wlog;                // device rule nodes / weights
@@ -1107,8 +1107,8 @@ int wcs_mesh(wcs_ctx* c, int64_t N, double k) {
   c->k = (k > 0) ? k : 2.0 * WCS_PI * ((double)N / 10.0) / c->L;
   if (c->k * c->h > 2.5) { set_error("k h > 2.5: mesh too coarse for the wavenumber"); return WCS_ERR_ARG; }
   c->kt = mkz(c->k, 0.4 * cbrt(c->k) * pow(c->a, -2.0 / 3.0));
-  TRY(c->small.ensure(sizeof(double) * 304));
-  TRY(min_curvature(c->contour, c->arc, std::max<int64_t>(16 * N, 65536), &c->kmin, c->small.d(), c->s));
+  TRY(c->small.ensure(sizeof(double) * CURVATURE_WORK));
+  TRY(curvature_range(c->contour, std::max<int64_t>(16 * N, 65536), &c->kmin, &c->kmax, c->small.d(), c->s));
   if (c->kmin < -1e-9) { set_error("contour is not convex (negative curvature)"); return WCS_ERR_NOT_CONVEX; }
   // equivalent circle
   c->circle = Contour{};
@@ -1150,13 +1150,15 @@ static bool kt_paired(const wcs_ctx* c) {
 // k R0 (R0: distance of the element centres) from which element pairs of the mixed form
 // take the FP32 route of farpair.cuh; 0: none do.  A caller's zfast is the distance below
 // which pairs stay in FP64, whatever the mesh.  Left to the library it is where the route's
-// Hankel series holds, k R0 = 20, when k h <= 0.9: entries then carry 3e-9 to 7e-9, those of
-// FP64 quadrature 2.6e-9 after their split into bf16 planes.  On coarser meshes the route's
-// corrections are larger (5e-8 at k h = 2.5), and it only takes the pairs beyond 1000.
+// Hankel series holds, k R0 = 20, when k h <= 0.9 and no element turns by more than a
+// radian: entries then carry 3e-9 to 7e-9 rms and 2^-24.7 of their kernel at worst, those
+// of FP64 quadrature 2.6e-9 after their split into bf16 planes.  On coarser meshes the
+// route's corrections are larger (5e-8 at k h = 2.5; 2^-23.9 at worst where the tip of an
+// ellipse 1 : 0.05 turns through one element), and it only takes the pairs beyond 1000.
 static double far_threshold(const wcs_ctx* c) {
   if (!c->mixed || !(c->opt.zfast > 0.0) || !kt_paired(c)) return 0.0;
   const double kh = c->k * c->h, least = 20.0 + kh;
-  return (c->zfast_auto && kh <= 0.9) ? least : std::max(least, c->opt.zfast + 2.0 * kh);
+  return (c->zfast_auto && kh <= 0.9 && c->kmax * c->h <= 1.0) ? least : std::max(least, c->opt.zfast + 2.0 * kh);
 }
 
 int wcs_query(const wcs_ctx* c, wcs_info* info) {

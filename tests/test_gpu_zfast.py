@@ -49,3 +49,15 @@ def test_distance_in_effect(kh, options, want):
     s.mesh(ELL["N"], kh / s.info()["h"])
     assert s.info()["zfast"] == pytest.approx(want, rel=1e-12)
     s.close()
+
+
+@pytest.mark.parametrize("ay,N,want", [(0.2, 300, "route"), (0.1, 420, "route"), (0.1, 380, "coarse"), (0.05, 400, "coarse")])
+def test_elements_that_turn_by_a_radian(ay, N, want):
+    """Curvature at the tip 1 / ay^2: the route starts at k R0 = 20 + k h while an element turns by
+    less than a radian, and as on a coarse mesh beyond."""
+    s = make_solver(dict(family="ellipse", params={"ax": 1.0, "ay": ay}, N=N, k=None), precision=1)
+    i = s.info()
+    s.close()
+    kh = i["k"] * i["h"]
+    assert (i["h"] / ay ** 2 <= 1.0) == (want == "route")
+    assert i["zfast"] == pytest.approx(20 + kh if want == "route" else 1000 + 2 * kh, rel=1e-12)
