@@ -1195,7 +1195,10 @@ static AsmArgs asm_args(wcs_ctx* c, bool circle) {
     A.ktp.c1 = mkz(c1.real(), c1.imag());
     A.ktp.c2 = mkz(c2.real(), c2.imag());
     // the mixed form stores entries to 24 bits: its expansion stops at 1e-13;
-    // the FP64 form and the circle rows (the eigenvalues) keep 1e-16
+    // the FP64 form and the circle rows (the eigenvalues) keep 1e-16.  (Below
+    // k R = 24 the mixed form's circle row takes the run's table: its eigenvalues
+    // are the FP64 form's to 2e-15, those of N to 1e-13 of the largest, which is
+    // the cancellation in its terms.)
     fill_asymptotic(A.ktp, (c->mixed && !circle) ? 1e-13 : 1e-16);
     // the reference-phase route of the far pairs needs |k R - x0| <= 1.05
     // (points within 0.45 h of their element's reference point) and
