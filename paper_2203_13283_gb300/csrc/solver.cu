@@ -1222,8 +1222,6 @@ static void set_far_consts(wcs_ctx* c, AsmArgs& A) {
   A.fN = mkz(fN.real(), fN.imag());
 }
 
-__global__ void k_geom_sample_dummy() {}
-
 int wcs_geometry_sample(wcs_ctx* c, int64_t count, const double* s_host, double* out_host) {
   if (!c || !s_host || !out_host || count < 0) { set_error("bad argument"); return WCS_ERR_ARG; }
   if (c->stage < ST_MESH) { set_error("no mesh yet"); return WCS_ERR_STATE; }
@@ -1240,9 +1238,7 @@ int wcs_geometry_sample(wcs_ctx* c, int64_t count, const double* s_host, double*
   P.x = b; P.y = b + count; P.nx = b + 2 * count; P.ny = b + 3 * count; P.kappa = b + 4 * count;
   P.n = count;
   // one "element" with count local nodes
-  const int64_t savedN = c->N;
   int r = points_build(c->contour, c->arc, 1, c->h, PointSet{sb.d(), (int)count, P}, PointSet{}, c->s, 1e-16);
-  (void)savedN;
   if (r) { sb.release(); pb.release(); return r; }
   cudaMemcpyAsync(out_host, pb.p, sizeof(double) * count * 5, cudaMemcpyDeviceToHost, c->s);
   r = sync(c);
