@@ -275,11 +275,12 @@ int lu_inverse(zd* A, int64_t n, zd* Ainv, zd* work, int* info_dev, double* minp
 int planewave_rhs(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                   double h, double k, const double* angles, int B, zd* e, zd* hv, int64_t ld,
                   cudaStream_t s, bool split_phase = false);
-// mom: farfield_moments(N) values of scratch; without it (the map of a central
-// difference) every k h takes one evaluation
+// mom: farfield_moments values of scratch, or null: every point by itself (a central difference
+// keeps that one evaluation at every size)
 int farfield_matrix(const Points& near, const double* wn, const double* xn, int q, int64_t N,
                     double h, double k, const double* phi, int nphi, zd* E, int64_t lde,
                     cudaStream_t s, zd* mom);
-int64_t farfield_moments(int64_t N);
+// Complex values of scratch for the map by moments; 0 where the points are the faster route.
+int64_t farfield_moments(int64_t N, int nphi, double kh);
 
 }  // namespace wcs

@@ -2712,11 +2712,12 @@ int wcs_farfield(wcs_ctx* c, int64_t B, const double* j, int64_t ldj, int nphi, 
   Call call(c, {{&c->tmp[0], &c->tmp[1], &c->tmp[2], &c->tmp[3], &c->tmp[4], &c->tmp[5], &c->tmp[6], &c->htab, &c->tiles, &c->offs,
                  &c->centres, &c->qh, &c->qt}});
   DevBuf &E = c->far_map, &ang = c->sol_ang;
-  TRY(E.fit(sizeof(zd) * ((int64_t)nphi * c->N + farfield_moments(c->N))));
+  const int64_t map = (int64_t)nphi * c->N, mom = farfield_moments(c->N, nphi, c->k * c->h);
+  TRY(E.fit(sizeof(zd) * (map + mom)));
   TRY(ang.ensure(sizeof(double) * nphi));
   cudaMemcpyAsync(ang.p, phi, sizeof(double) * nphi, cudaMemcpyHostToDevice, c->s);
   TRY(farfield_matrix(c->near, c->quad.wn, c->quad.xn, c->opt.q_near, c->N, c->h, c->k, ang.d(),
-                      nphi, E.z(), nphi, c->s, E.z() + (int64_t)nphi * c->N));
+                      nphi, E.z(), nphi, c->s, mom > 0 ? E.z() + map : nullptr));
   TRY(cz(c, nphi, B, c->N, mkz(1.0), ZView{E.z(), 1, nphi, false}, blk((const zd*)j, ldj), mkz(0.0),
          (zd*)F, ldf));
   TRY(check_tc(c));

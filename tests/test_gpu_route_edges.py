@@ -114,3 +114,29 @@ def test_circle_eigenvalues_of_both_forms(N, kh):
     R = np.maximum(2.0 * i["a"] * np.sin(np.pi * np.arange(N) / N), 0.5 * i["h"])
     terms = np.sum(np.abs(hankel1(0, i["k"] * R)))
     assert np.max(np.abs(mu[0]["N"] - mu[1]["N"])) < 1e-15 * terms
+
+
+# both sides of the map's rule (16 angles, 65536 of N times angles), meshes and rules of the moments
+@pytest.mark.parametrize("N,nphi,kh,q", [(12, 1, 0.63, 8), (63, 100, 0.63, 8), (1023, 64, 0.63, 8), (1024, 64, 0.63, 8),
+                                         (4400, 15, 0.63, 8), (4097, 16, 0.63, 8), (730, 90, 0.89, 4), (2200, 33, 0.85, 16),
+                                         (301, 219, 0.2, 5), (911, 73, 0.89, 7)])
+def test_farfield_map_around_its_rule(N, nphi, kh, q):
+    """Against the same quadrature in numpy (positions from the library's arc-length inversion,
+    ~1e-12: 1e-9)."""
+    s = make_solver(dict(ELL, N=N, k=None), q_near=q)
+    s.mesh(N, kh / s.info()["h"])
+    i = s.info()
+    k, h = i["k"], i["h"]
+    x, w = np.polynomial.legendre.leggauss(q)
+    x, w = (x + 1) / 2, w / 2
+    g = s.geometry_sample(((np.arange(N)[:, None] + x) * h).ravel())
+    J = randn(N, 4)
+    j = to_np(J)
+    phi = np.arange(nphi) * 0.7 + 0.1
+    cur = np.tile(w, N)[:, None] * h * (np.tile(1 - x, N)[:, None] * np.repeat(j, q, axis=0)
+                                        + np.tile(x, N)[:, None] * np.repeat(np.roll(j, -1, axis=0), q, axis=0))
+    d = np.cos(phi)[:, None] * g["x"] + np.sin(phi)[:, None] * g["y"]
+    n = np.cos(phi)[:, None] * g["nx"] + np.sin(phi)[:, None] * g["ny"]
+    want = 1j * k * np.exp(0.25j * np.pi) / np.sqrt(8 * np.pi * k) * ((n * np.exp(-1j * k * d)) @ cur)
+    assert colrel(to_np(s.farfield(J, phi)), want) < 1e-9
+    s.close()
