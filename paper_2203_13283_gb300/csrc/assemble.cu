@@ -361,6 +361,9 @@ int hankel_table(double t, double* T, cudaStream_t s) {
 // 33 lanes of a diagonal tile's warps on the heaviest path in the program, 60 ms
 // of FP64 pipe per tile); the 32 sums are joined by a halving exchange that
 // leaves sum l in lane l.  Bound: FP64 pipe, ~300 operations a point.
+// TAB: Hankel functions from the run's table; without one (k~ off its form, small k a) from
+// the full expansions.
+template <bool TAB>
 __global__ void __launch_bounds__(128) k_near_band(AsmArgs A, int64_t e0, int64_t ne, double* out) {
   const int64_t N = A.N;
   const int64_t pair = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -398,7 +401,9 @@ __global__ void __launch_bounds__(128) k_near_band(AsmArgs A, int64_t e0, int64_
     } else {
       const double R2 = dx * dx + dy * dy, ri = rsqrt(R2), R = R2 * ri, gg = (dx * nxs + dy * nys) * ri, x = k * R;
       Hankel01 Hk, Ht;
-      if (x < HT_X0) {
+      if (!TAB) {
+        hankel_k_kt(A, R, Hk, Ht);
+      } else if (x < HT_X0) {
         hankel_tab_series(A.htab, x, log(0.5 * x), Hk, Ht);
       } else if (kind >= 0 || x >= HT_X1) {
         hankel01_pair(x, A.ktp, Hk, Ht);
@@ -462,7 +467,8 @@ __global__ void __launch_bounds__(128) k_near_band(AsmArgs A, int64_t e0, int64_
 
 int near_band_pairs(const AsmArgs& A, int64_t e0, int64_t ne, double* out, cudaStream_t s) {
   const int64_t pairs = ne * (2 * A.near_band + 1);
-  k_near_band<<<(unsigned)((pairs + 3) / 4), 128, 0, s>>>(A, e0, ne, out);
+  if (A.htab) k_near_band<true><<<(unsigned)((pairs + 3) / 4), 128, 0, s>>>(A, e0, ne, out);
+  else k_near_band<false><<<(unsigned)((pairs + 3) / 4), 128, 0, s>>>(A, e0, ne, out);
   note_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) { set_error(std::string("near band: ") + cudaGetErrorString(err)); return 3; }
@@ -799,7 +805,7 @@ __device__ __forceinline__ void pair_both(const AsmArgs& A, int64_t e, int64_t f
   const int64_t N = A.N;
   const bool band = A.near_buf && periodic_dist(e, f, N) <= A.near_band;
   if (!band && pair_is_far(A, e, f)) { pair_far(A, e, f, o); return; }
-  if (!band && A.near_buf && pair_is_mid(A, e, f)) { pair_mid<6>(A, A.htab, e, f, o); return; }
+  if (!band && A.htab && pair_is_mid(A, e, f)) { pair_mid<6>(A, A.htab, e, f, o); return; }
   PairOut p;
   for (int m = 0; m < 2; ++m) {
     const int64_t x = m ? f : e, y = m ? e : f;
@@ -955,7 +961,7 @@ __global__ void k_circle_row_part(AsmArgs A, zd* part) {
   circle_pair(t, N, e, f);
   PairOut o;
   if (A.near_buf && periodic_dist(e, f, N) <= A.near_band) pair_near(A.near_buf, N - 1, 2, A.near_band, N, e, f, o);
-  else if (A.near_buf && pair_is_mid(A, e, f)) pair_mid<4>(A, A.htab, e, f, o);
+  else if (A.htab && pair_is_mid(A, e, f)) pair_mid<4>(A, A.htab, e, f, o);
   else pair_integrals(A, e, f, o);
   circle_store(o, t, N, part);
 }

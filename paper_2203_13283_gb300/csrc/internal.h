@@ -123,7 +123,7 @@ struct AsmArgs {
   // constant rounded to FP32 would bias every far entry of an operator alike)
   zd fS, fD, fDt, fN;              // S~, D, D~, N (see FarPair)
   // mixed form: Hankel table of the run (hankeltab.cuh) and the near-band pairs'
-  // blocks (near_band_pairs; null: pair integrals without either)
+  // blocks (near_band_pairs); null: pair integrals without it
   const double* htab = nullptr;
   const double* near_buf = nullptr;
   int* tile_list = nullptr;        // count, then the diagonal tiles and the tiles above them that hold a pair nearer than the far route
@@ -148,7 +148,7 @@ int far_tables(const AsmArgs& a, const Points& cen, FarElem* fe, FarPoint* fp, c
 int64_t hankel_table_doubles();
 int hankel_table(double t, double* T, cudaStream_t s);
 // Blocks of the near-band element pairs of elements e0 .. e0 + ne - 1 (mod N):
-// 32 doubles for each of ne (2 near_band + 1) pairs.  Needs a.htab.
+// 32 doubles for each of ne (2 near_band + 1) pairs (with a.htab from the table).
 int near_band_pairs(const AsmArgs& a, int64_t e0, int64_t ne, double* out, cudaStream_t s);
 // First row of the four circulant operators on the circle (row 0, N entries each).
 // (part: 16 N values of scratch).

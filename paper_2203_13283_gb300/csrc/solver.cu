@@ -1295,10 +1295,10 @@ int wcs_assemble(wcs_ctx* c) {
     AsmArgs A = asm_args(c, false);
     TRY(far_tables(A, cp, fe, fp, c->s));
     // Hankel table and near-band blocks (N (2 near_band + 1) of 256 bytes);
-    // without them (k~ off the table's form, a band of more than 1 GB or no room for
-    // it) the tile kernel integrates those pairs itself
+    // without the band (more than 1 GB of it, or no room) the tile kernel integrates those
+    // pairs itself; without the table (k~ off its form) every pair by the full expansions
     const int64_t band = N * (2 * c->opt.near_band + 1), band_row = 2 * (2 * c->opt.near_band + 1);
-    near_tab = A.kt_pair && 2 * c->opt.near_band + 1 <= N && 256 * band <= ((int64_t)1 << 30);
+    near_tab = 2 * c->opt.near_band + 1 <= N && 256 * band <= ((int64_t)1 << 30);
     if (near_tab && c->htab.fit(sizeof(double) * (hankel_table_doubles() + 32 * (band + band_row)))) near_tab = false;
     A.planes = c->planes;
     A.ldp = c->ldp;
@@ -1312,8 +1312,10 @@ int wcs_assemble(wcs_ctx* c) {
     A.tile_list = (int*)c->tiles.p;
     set_far_consts(c, A);
     if (near_tab) {
-      TRY(hankel_table(A.ktp.t, c->htab.d(), c->s));
-      A.htab = c->htab.d();
+      if (A.kt_pair) {
+        TRY(hankel_table(A.ktp.t, c->htab.d(), c->s));
+        A.htab = c->htab.d();
+      }
       TRY(near_band_pairs(A, 0, N, c->htab.d() + hankel_table_doubles(), c->s));
       A.near_buf = c->htab.d() + hankel_table_doubles();
     }
@@ -1339,7 +1341,7 @@ int wcs_assemble(wcs_ctx* c) {
   // circle: first rows -> eigenvalues
   if (near_tab) {   // the same wavenumbers: the table serves the circle as well
     double* row = c->htab.d() + hankel_table_doubles() + 32 * N * (2 * c->opt.near_band + 1);
-    B.htab = c->htab.d();
+    if (B.kt_pair) B.htab = c->htab.d();
     TRY(near_band_pairs(B, N - 1, 2, row, c->s));
     B.near_buf = row;
   }

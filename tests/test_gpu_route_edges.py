@@ -61,6 +61,19 @@ def test_near_bands(N, band, precision):
     s.close()
 
 
+@pytest.mark.parametrize("N", [12, 13, 20, 60])
+@pytest.mark.parametrize("options", [dict(precision=0), dict(precision=1), dict(precision=1, near_band=6)])
+def test_small_k_a(N, options):
+    """k~ off the tables' form (Im k~ above a tenth of k): near bands by the full expansions, or,
+    where they cover the contour, pair by pair."""
+    s = make_solver(dict(ELL, N=N, k=None), **options)
+    i = s.info()
+    assert i["kt_im"] > 0.1 * i["k"]
+    s.assemble()
+    check_columns(s, 2e-6 if options["precision"] else 1e-12)
+    s.close()
+
+
 def test_coarse_mesh_with_a_sorted_band():
     # k h (near_band + 1) below 3.9: the FP64 form's sorted pairs on a coarse mesh
     s = make_solver(dict(ELL, N=300, k=None), near_band=1)
