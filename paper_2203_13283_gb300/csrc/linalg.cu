@@ -634,11 +634,15 @@ constexpr int GRAM_ROWS = 256;
 // Hermitian b x b result is formed (pair index p -> column j = row of the
 // triangular numbers, row i = p - j (j + 1) / 2); both halves are written.  A CTA
 // takes GRAM_PAIRS pairs, two lanes each (real and imaginary part), so that the
-// FP64 work of a row chunk (528 pairs at b = 32) spreads over 17 CTAs instead of
-// one: at N = 2777 eleven CTAs took 185 us.  With plain loads between the tiles'
-// barriers 187 CTAs took 91 us, most of it the loads' latency: GRAM_STAGES tiles are
-// in flight (cp.async), and what is left is the chain of 512 dependent FMA (17 us).
-constexpr int GRAM_PAIRS = 32, GRAM_TILE = 32, GRAM_STAGES = 4;
+// FP64 work of a row chunk (528 pairs at b = 32) spreads over nine CTAs instead of
+// one: at N = 2777 eleven CTAs took 185 us a product, 38 so.  GRAM_STAGES tiles are in
+// flight (cp.async): with plain loads between the tiles' barriers most of the time was
+// the loads' latency.  Bound: the chain of 512 dependent FMA (17 us) for few rows, the FP64
+// pipe for many, which needs warps on all four quarters of the SM and nothing on the pipe
+// but the FMA.  32 pairs a CTA, four stages (one CTA of two warps a SM at b = 64) and the
+// sign of the imaginary part as an FP64 negation took 2338 us at N = 32768, b = 64, where
+// one CTA a chunk took 593; now 521 (435 is the pipe's time for it), 162 at b = 32.
+constexpr int GRAM_PAIRS = 64, GRAM_TILE = 32, GRAM_STAGES = 2;
 __global__ void __launch_bounds__(2 * GRAM_PAIRS) k_gram_partial(const zd* X, int64_t ld, int64_t m, int b, zd* part) {
   extern __shared__ zd gram_s[];   // [stage][column][GRAM_TILE + 1]
   const int64_t r0 = (int64_t)blockIdx.x * GRAM_ROWS, r1 = min(m, r0 + GRAM_ROWS);
@@ -672,17 +676,20 @@ __global__ void __launch_bounds__(2 * GRAM_PAIRS) k_gram_partial(const zd* X, in
   };
   for (int t = 0; t < GRAM_STAGES - 1; ++t) fetch(t);
   double acc = 0.0;
+  const int sgn = im ? (int)0x80000000 : 0;
   for (int t = 0; t < tiles; ++t) {
     asm volatile("cp.async.wait_group %0;" ::"n"(GRAM_STAGES - 2) : "memory");
     __syncthreads();               // tile t is there; tile t - 1's stage is free
     fetch(t + GRAM_STAGES - 1);
     const zd* xi = gram_s + ((size_t)(t % GRAM_STAGES) * b + i) * (GRAM_TILE + 1);
     const zd* xj = gram_s + ((size_t)(t % GRAM_STAGES) * b + j) * (GRAM_TILE + 1);
-    // conj(x_i) x_j with the operations of zfma: re: fma(x, u, fma(y, v, re)); im: fma(x, v, fma(-y, u, im))
+    // conj(x_i) x_j with the operations of zfma: re: fma(x, u, fma(y, v, re)); im: fma(x, v, fma(-y, u, im)),
+    // -y by its sign bit (a selected negation would run on the FP64 pipe)
 #pragma unroll 8
     for (int r = 0; r < GRAM_TILE; ++r) {
       const zd a = xi[r], c = xj[r];
-      acc = fma(a.x, im ? c.y : c.x, fma(im ? -a.y : a.y, im ? c.x : c.y, acc));
+      const double y = __hiloint2double(__double2hiint(a.y) ^ sgn, __double2loint(a.y));
+      acc = fma(a.x, im ? c.y : c.x, fma(y, im ? c.x : c.y, acc));
     }
   }
   const double other = __shfl_xor_sync(0xffffffffu, acc, 1);
