@@ -373,6 +373,7 @@ __global__ void k_gram_bwd(const zd* __restrict__ U, zd* __restrict__ Y, int64_t
 // filter starts in the next one, behind a short last chunk in the one after it: with more
 // than GI_SLOTS chunks a CTA also runs the forward filter of the two that follow its own.
 constexpr int GI_SLOTS = 32, GI_LD = GI_CH + GI_WARM + 1;   // odd stride: no bank conflicts
+constexpr int64_t GI_FUSED_CHUNKS = 16384, GI_FUSED_CTAS = 2560;
 
 __global__ void __launch_bounds__(2 * GI_SLOTS) k_gram_inverse(const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t n,
                                                                int per, double rho, double scale) {
@@ -448,9 +449,16 @@ int gram_inverse(const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t n, int64_
   const double rho = sqrt(3.0) - 2.0;
   const int64_t chunks = (n + GI_CH - 1) / GI_CH;
   const bool apart = Y + (cols - 1) * ldy + n <= X || X + (cols - 1) * ldx + n <= Y;
-  // in place only where one CTA holds the whole column
-  if (chunks <= GI_SLOTS || apart) {
-    const int per = chunks <= GI_SLOTS ? (int)chunks : GI_SLOTS - 2;
+  const int per = chunks <= GI_SLOTS ? (int)chunks : GI_SLOTS - 2;
+  const int64_t ctas = cols * ((chunks + per - 1) / per);
+  // One kernel while its CTAs, four to an SM for their shared memory, go round few times;
+  // the two passes where all their chains run at once anyway.  us for both, N = 2777:
+  // 42 and 64 at 12288 chunks, 55 and 62 at 16384, 70 and 72 at 24576, 177 and 136 at
+  // 65536; N = 32768: 46 and 62, 78 and 72 at 24576, 674 and 473 at 262144.  Columns of few
+  // chunks leave lanes idle, so the CTAs count too: N = 64, 40 and 57 at 2048, 72 and 57 at
+  // 4096, 525 and 72 at 32768; N = 200, 42 and 59 at 2048, 60 and 59 at 3072.
+  // In place only where one CTA holds the whole column.
+  if (chunks * cols <= GI_FUSED_CHUNKS && ctas <= GI_FUSED_CTAS && (chunks <= GI_SLOTS || apart)) {
     const size_t smem = sizeof(zd) * GI_LD * (chunks <= GI_SLOTS ? chunks : GI_SLOTS);
     static DeviceOnce attr;
     if (attr.need()) {
@@ -459,7 +467,7 @@ int gram_inverse(const zd* X, int64_t ldx, zd* Y, int64_t ldy, int64_t n, int64_
       if (e != cudaSuccess) { set_error(std::string("gram: ") + cudaGetErrorString(e)); return 3; }
       attr.done();
     }
-    k_gram_inverse<<<dim3((unsigned)cols, (unsigned)((chunks + per - 1) / per)), 2 * GI_SLOTS, smem, s>>>(
+    k_gram_inverse<<<dim3((unsigned)cols, (unsigned)(ctas / cols)), 2 * GI_SLOTS, smem, s>>>(
         X, ldx, Y, ldy, n, per, rho, -rho * 6.0 / h);
     note_launch();
     cudaError_t err = cudaGetLastError();

@@ -50,6 +50,17 @@ def test_gram_inverse(N):
     assert torch.equal(Y.t(), s.apply("GINV", X))
 
 
+# on both sides of the one kernel's range: 16384 chunks of 64 samples (256 columns of 64
+# chunks, 496 of 33) and 2560 CTAs; every column has the values that it has by itself
+@pytest.mark.parametrize("N, B", [(64, 2560), (64, 2561), (4096, 256), (4096, 257), (2100, 496), (2100, 497)])
+def test_gram_inverse_of_many_columns(N, B):
+    s = assembled(N, False)
+    X = randn(N, B)
+    Y = s.apply("GINV", X)
+    for c in (0, B // 2, B - 1):
+        assert torch.equal(Y[:, c:c + 1], s.apply("GINV", X[:, c:c + 1])), c
+
+
 # lengths on both sides of the two-half transform's range, column counts on both sides
 # of its limit
 @pytest.mark.parametrize("N", [256, 512, 1024, 4096, 8192])
